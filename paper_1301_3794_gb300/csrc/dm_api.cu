@@ -263,7 +263,14 @@ struct OpLevel {
     int sd_nsub = 0, sd_ncopies = 0, sd_maxrows = 0, sd_maxbox = 0;
     int sd_cls_first[kSchwarzClasses] = {}, sd_cls_count[kSchwarzClasses] = {};
     long long sd_cls_copies[kSchwarzClasses] = {}, sd_cls_owned[kSchwarzClasses] = {};
-    bool sd_fixed = false;
+    // the same for bricks of up to 8 nodes, which the node kernels smooth
+    bool by_node = false;
+    DBuf<int> bn_off, bn_node, bn_info, bn_org, bn_uidx;
+    DBuf<double> bn_v64;
+    DBuf<float> bn_v32;
+    int bn_nsub = 0, bn_ncopies = 0;
+    int bn_cls_first[kNodeClasses] = {}, bn_cls_count[kNodeClasses] = {};
+    long long bn_cls_copies[kNodeClasses] = {};
 };
 
 // FGMRES workspace: the Arnoldi basis V and the work vector wf in
@@ -360,12 +367,30 @@ BandSchwarz<TC> schwarz_view(const OpLevel& o, const TC* vals) {
     b.ncopies = o.sd_ncopies;
     b.maxrows = o.sd_maxrows;
     b.maxbox = o.sd_maxbox;
-    b.fixed = o.sd_fixed;
     for (int k = 0; k < kSchwarzClasses; ++k) {
         b.cls_first[k] = o.sd_cls_first[k];
         b.cls_count[k] = o.sd_cls_count[k];
         b.cls_copies[k] = o.sd_cls_copies[k];
         b.cls_owned[k] = o.sd_cls_owned[k];
+    }
+    return b;
+}
+
+template <typename TC>
+BandNodes<TC> nodes_view(const OpLevel& o, const TC* vals) {
+    BandNodes<TC> b;
+    b.off = o.bn_off.get();
+    b.node = o.bn_node.get();
+    b.info = o.bn_info.get();
+    b.org = o.bn_org.get();
+    b.uidx = o.bn_uidx.get();
+    b.vals = vals;
+    b.nsub = o.bn_nsub;
+    b.ncopies = o.bn_ncopies;
+    for (int k = 0; k < kNodeClasses; ++k) {
+        b.cls_first[k] = o.bn_cls_first[k];
+        b.cls_count[k] = o.bn_cls_count[k];
+        b.cls_copies[k] = o.bn_cls_copies[k];
     }
     return b;
 }
@@ -378,6 +403,7 @@ template <> struct Pick<double, double> {
     static const double* iD(const OpLevel& o) { return o.invD.get(); }
     static const double* iDs(const OpLevel& o) { return o.invDs.get(); }
     static BandSchwarz<double> bs(const OpLevel& o) { return schwarz_view<double>(o, o.sd_v64.get()); }
+    static BandNodes<double> bn(const OpLevel& o) { return nodes_view<double>(o, o.bn_v64.get()); }
 };
 template <typename T> struct Pick<T, float> {
     static const float* A(const GeoLevel& g) { return g.A32.get(); }
@@ -386,6 +412,7 @@ template <typename T> struct Pick<T, float> {
     static const float* iD(const OpLevel& o) { return o.invD32.get(); }
     static const float* iDs(const OpLevel& o) { return o.invDs32.get(); }
     static BandSchwarz<float> bs(const OpLevel& o) { return schwarz_view<float>(o, o.sd_v32.get()); }
+    static BandNodes<float> bn(const OpLevel& o) { return nodes_view<float>(o, o.bn_v32.get()); }
 };
 
 template <typename T, typename TC>
@@ -405,6 +432,19 @@ ScalOp<T, TC> sop(const dm_operator* op, int l) {
 // band smoother sweeps of level l: the fine level, or the coarser ones
 int band_sweeps_of(const dm_operator* op, int l) { return l == 0 ? op->mg.band_sweeps : op->mg.band_sweeps_coarse; }
 
+// the band smoother on level l
+template <typename T, typename TC>
+void smooth_band(const dm_operator* op, int l, const TC* invD, const T* f, T* x, const Fork* fk) {
+    const GeoLevel& g = glv(op, l);
+    const OpLevel& o = op->ol[l];
+    if (o.by_node)
+        band_nodes<T, TC>(Pick<T, TC>::bn(o), g.g, g.band.get(), g.nband, f, x, op->band_u.get(), o.omega,
+                          band_sweeps_of(op, l), l == 0, op->ctx->stream, fk);
+    else
+        band_schwarz<T, TC>(Pick<T, TC>::bs(o), invD, g.g, g.band.get(), g.nband, f, x, op->band_u.get(), o.omega,
+                            band_sweeps_of(op, l), l == 0, op->ctx->stream, fk);
+}
+
 // ---- vector V-cycle: result in rbuf ------------------------------------------------
 template <typename T, typename TC>
 void vcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
@@ -420,8 +460,6 @@ void vcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
     }
     const VecOp<T, TC> o = vop<T, TC>(op, l);
     const double om = op->ol[l].omega;
-    double* u = op->band_u.get();
-    const int sweeps = band_sweeps_of(op, l);
     const int nu = op->mg.jacobi_sweeps;
     // the iterate and the other work buffer swap roles at every Jacobi sweep
     T* it = ebuf;
@@ -439,8 +477,7 @@ void vcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
         vec_stencil(o, ST_JACOBI, it, f, tmp, om, s);
         std::swap(it, tmp);
     }
-    band_schwarz<T, TC>(Pick<T, TC>::bs(op->ol[l]), o.invD, g.g, g.band.get(), g.nband, f, it, u, om, sweeps, l == 0,
-                        s, fork_of(op));
+    smooth_band<T, TC>(op, l, o.invD, f, it, fork_of(op));
     vec_stencil(o, ST_RESID, it, f, tmp, 0.0, s);
     const GeoLevel& gc = glv(op, l + 1);
     WorkLevel& wc = op->wk[l + 1];
@@ -456,8 +493,7 @@ void vcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
         vec_stencil(o, ST_JACOBI, it, f, tmp, om, s);
         std::swap(it, tmp);
     }
-    band_schwarz<T, TC>(Pick<T, TC>::bs(op->ol[l]), o.invD, g.g, g.band.get(), g.nband, f, it, u, om, sweeps, l == 0,
-                        s, fork_of(op));
+    smooth_band<T, TC>(op, l, o.invD, f, it, fork_of(op));
     // the cycle's result goes in rbuf
     if (it != rbuf) DM_CUDA(cudaMemcpyAsync(rbuf, it, sizeof(T) * 3 * (size_t)g.g.np, cudaMemcpyDeviceToDevice, s));
 }
@@ -1125,7 +1161,7 @@ void setup_operator(dm_operator* op) {
     op->wk.resize(nl);
     const bool lowp = op->mg.precision != DM_PREC_F64;
     const size_t ts = tsize(op->mg.precision);
-    int max_band = 1;
+    size_t max_band = 1;   // scratch of the band smoother, in doubles
     for (int l = 0; l < nl; ++l) {
         GeoLevel& g = *geom->lv[l];
         if (lowp) {
@@ -1149,14 +1185,50 @@ void setup_operator(dm_operator* op) {
             convert_coeff<float>(n3, o.invD.get(), o.invD32.get(), s);
             convert_coeff<float>(n1, o.invDs.get(), o.invDs32.get(), s);
         }
-        if (g.nband > 0 && l + 1 < nl) {
+        auto upload = [&](DBuf<int>& d, const std::vector<int>& h) {
+            d.alloc(h.size(), false);
+            DM_CUDA(cudaMemcpyAsync(d.get(), h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, s));
+        };
+        if (g.nband > 0 && l + 1 < nl && band_nodes_fit(op->mg.band_brick)) {
+            NodeLayout nl_;
+            // (the FP64 kernel splits a subdomain by box order and is not bound by shared memory)
+            band_nodes_setup(g.g, g.band.get(), g.nband, op->mg.band_brick, lowp, nl_, s);
+            o.by_node = true;
+            o.bn_nsub = (int)nl_.off.size() - 1;
+            o.bn_ncopies = (int)nl_.node.size();
+            for (int k = 0; k < kNodeClasses; ++k) {
+                o.bn_cls_first[k] = nl_.cls_first[k];
+                o.bn_cls_count[k] = nl_.cls_count[k];
+                o.bn_cls_copies[k] = nl_.cls_copies[k];
+            }
+            upload(o.bn_off, nl_.off);
+            upload(o.bn_node, nl_.node);
+            upload(o.bn_info, nl_.info);
+            upload(o.bn_org, nl_.org);
+            o.bn_uidx.alloc(g.nband);
+            DBuf<double> rows(kBandSlots * (size_t)g.nband, false);
+            DBuf<int> tmap(n3, false);
+            band_slots(g.g, g.A.get(), g.L.get(), g.invV.get(), op->sigma, g.band.get(), g.nband, rows.get(), s);
+            compact_map(n3, g.band.get(), g.nband, tmap.get(), s);
+            const size_t nv = 45 * (size_t)o.bn_ncopies;
+            if (lowp) {
+                o.bn_v32.alloc(nv, false);
+                band_node_vals<float>(o.bn_node.get(), o.bn_info.get(), o.bn_ncopies, g.g, tmap.get(), rows.get(),
+                                      g.nband, o.invD.get(), o.bn_v32.get(), o.bn_uidx.get(), s);
+            } else {
+                o.bn_v64.alloc(nv, false);
+                band_node_vals<double>(o.bn_node.get(), o.bn_info.get(), o.bn_ncopies, g.g, tmap.get(), rows.get(),
+                                       g.nband, o.invD.get(), o.bn_v64.get(), o.bn_uidx.get(), s);
+            }
+            max_band = std::max(max_band, 3 * (size_t)o.bn_ncopies);
+            Sync::stream(s);   // the host layout and the row buffer are released on return
+        } else if (g.nband > 0 && l + 1 < nl) {
             SchwarzLayout sl;
             band_schwarz_setup(g.g, g.band.get(), g.nband, op->mg.band_brick, sl, s);
             o.sd_nsub = (int)sl.off.size() - 1;
             o.sd_ncopies = (int)sl.copy.size();
             o.sd_maxrows = sl.maxrows;
             o.sd_maxbox = sl.maxbox;
-            o.sd_fixed = sl.fixed;
             for (int k = 0; k < kSchwarzClasses; ++k) {
                 o.sd_cls_first[k] = sl.cls_first[k];
                 o.sd_cls_count[k] = sl.cls_count[k];
@@ -1168,10 +1240,6 @@ void setup_operator(dm_operator* op) {
                 case DM_PREC_F32: band_schwarz_prepare<float, float>(sl); break;
                 default: band_schwarz_prepare<__nv_bfloat16, float>(sl);
             }
-            auto upload = [&](DBuf<int>& d, const std::vector<int>& h) {
-                d.alloc(h.size(), false);
-                DM_CUDA(cudaMemcpyAsync(d.get(), h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, s));
-            };
             upload(o.sd_off, sl.off);
             upload(o.sd_copy, sl.copy);
             upload(o.sd_pos, sl.pos);
@@ -1195,9 +1263,9 @@ void setup_operator(dm_operator* op) {
         w.sf.alloc(ts * n1);
         w.se.alloc(ts * n1);
         w.sr.alloc(ts * n1);
-        max_band = std::max(max_band, g.nband);
+        max_band = std::max(max_band, (size_t)g.nband);
     }
-    op->band_u.alloc((size_t)max_band);
+    op->band_u.alloc(max_band);
     {
         note_allocation();
         DM_CUDA(cudaEventCreateWithFlags(&op->fork.fork, cudaEventDisableTiming));
@@ -1821,7 +1889,6 @@ dm_status dm_operator_smooth(dm_operator* op, int level, const double* f, double
         double* pads[3] = {fp.get(), xp.get(), yp.get()};
         cudaStream_t s = op->ctx->stream;
         const double om = op->ol[level].omega;
-        double* u = op->band_u.get();
         auto run = [&](auto** p) {
             using T = std::remove_pointer_t<std::remove_reference_t<decltype(*p)>>;
             using TC = std::conditional_t<std::is_same<T, double>::value, double, float>;
@@ -1832,8 +1899,7 @@ dm_status dm_operator_smooth(dm_operator* op, int level, const double* f, double
                 vec_stencil(o, ST_JACOBI, it, p[0], tmp, om, s);
                 std::swap(it, tmp);
             }
-            band_schwarz<T, TC>(Pick<T, TC>::bs(op->ol[level]), o.invD, g.g, g.band.get(), g.nband, p[0], it, u, om,
-                                band_sweeps_of(op, level), level == 0, s);
+            smooth_band<T, TC>(op, level, o.invD, p[0], it, nullptr);
             if (it != p[2]) DM_CUDA(cudaMemcpyAsync(p[2], it, sizeof(T) * (size_t)n3, cudaMemcpyDeviceToDevice, s));
         };
         if (op->mg.precision == DM_PREC_F64) run(reinterpret_cast<double**>(pads));

@@ -10,12 +10,15 @@
 // on the owned faces.  With one brick covering the grid this is plain
 // band-restricted Jacobi.
 //
-// One thread block per subdomain.  The correction d lives in shared memory on
-// the subdomain's local box of nodes (all three components, zero wherever the
-// subdomain has no row), so a row's couplings are reached at fixed offsets:
-// the 15 slots of band_slot.  Each thread keeps the coefficients of its rows in
-// registers, so every sweep after the first touches only registers and shared
-// memory, with one block barrier per sweep and none across the grid.
+// Bricks of up to 8 nodes (the default is 8) take k_band_node: one thread per
+// node of the subdomain, which holds the rows of the node's three faces.
+// Larger bricks take k_band_schwarz, one thread per few rows, one block per
+// subdomain.  In both the correction d lives in shared memory on the
+// subdomain's local box of nodes (all three components, zero wherever the
+// subdomain has no row), so a row's couplings are reached at fixed offsets: the
+// 15 slots of band_slot.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -60,38 +63,11 @@ __device__ __forceinline__ C row_dot(const C* v, C self, const C* d, const RowAd
     return acc;
 }
 
-// The default brick (8 nodes) uses one fixed local box for every subdomain:
-// nodes B b - 2 .. B b + 9 on each axis (12 nodes; x padded to 13 to spread
-// shared-memory banks), so every coupling offset is a compile-time constant.
-constexpr int kFixedBrick = 8, kFX = 13, kFY = 12, kFZ = 12, kFXY = kFX * kFY, kF3 = kFXY * kFZ;
-
-template <typename C, int c>
-__device__ __forceinline__ C row_dot_fixed(const C* v, C self, const C* d, int p) {
-    constexpr int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
-    constexpr int sc = c == 0 ? 1 : (c == 1 ? kFX : kFXY);
-    constexpr int s1 = c1 == 0 ? 1 : (c1 == 1 ? kFX : kFXY);
-    constexpr int s2 = c2 == 0 ? 1 : (c2 == 1 ? kFX : kFXY);
-    constexpr int o1 = (c1 - c) * kF3 - sc, o2 = (c2 - c) * kF3 - sc;
-    const C* q = d + p;
-    C acc = v[0] * self;
-    acc += v[1] * q[-1] + v[2] * q[1];
-    acc += v[3] * q[-kFX] + v[4] * q[kFX];
-    acc += v[5] * q[-kFXY] + v[6] * q[kFXY];
-    acc += v[7] * q[o1] + v[8] * q[o1 + s1] + v[9] * q[o1 + sc] + v[10] * q[o1 + sc + s1];
-    acc += v[11] * q[o2] + v[12] * q[o2 + s2] + v[13] * q[o2 + sc] + v[14] * q[o2 + sc + s2];
-    return acc;
-}
-template <typename C>
-__device__ __forceinline__ C row_dot_fixed(int c, const C* v, C self, const C* d, int p) {
-    return c == 0 ? row_dot_fixed<C, 0>(v, self, d, p)
-                  : (c == 1 ? row_dot_fixed<C, 1>(v, self, d, p) : row_dot_fixed<C, 2>(v, self, d, p));
-}
-
 // R > 0: each thread owns up to R rows (row r = threadIdx.x + k blockDim.x) with
 // their coefficients and addresses in registers.  R == 0: any row count; r0
 // and omega/D in shared memory and the coefficients re-read on every sweep.
 // Block b handles subdomain sub0 + b.
-template <typename T, typename TC, int R, int NT, bool FIXED>
+template <typename T, typename TC, int R, int NT>
 __global__ void __launch_bounds__(NT)
     k_band_schwarz(int sub0, const int* __restrict__ off, const int* __restrict__ copy, const int* __restrict__ pos,
                    const int* __restrict__ dims, const int* __restrict__ org, const TC* __restrict__ vals, int ncopies,
@@ -108,7 +84,7 @@ __global__ void __launch_bounds__(NT)
     const int b0 = off[sd];
     const int nr = off[sd + 1] - b0;
     const int dm = dims[sd];
-    const int lx = FIXED ? kFX : dm & 1023, ly = FIXED ? kFY : (dm >> 10) & 1023, lz = FIXED ? kFZ : dm >> 20;
+    const int lx = dm & 1023, ly = (dm >> 10) & 1023, lz = dm >> 20;
     const int lxy = lx * ly, l3 = lxy * lz;
     // x over the local box (nodes org + local coordinates; outside the padded
     // grid's -1 .. n+1 it is zero), so that the start residuals read it from
@@ -131,7 +107,7 @@ __global__ void __launch_bounds__(NT)
     C v[RR][kBandSlots];
     C r0[RR], w[RR], dself[RR];   // dself: the row's current correction (R > 0)
     RowAddr ad[RR];
-    int cm[RR];
+    bool cm[RR];
     // residual of the full row at the start values, and the first sweep from d = 0
     auto start_row = [&](int r, C* ve, C& rr, C& ww) {
         const int ct = copy[b0 + r];
@@ -147,8 +123,7 @@ __global__ void __launch_bounds__(NT)
         const int ps = pos[b0 + r];
 #pragma unroll
         for (int e = 0; e < kBandSlots; ++e) ve[e] = (C)vals[(size_t)e * ncopies + b0 + r];
-        const C acc = FIXED ? row_dot_fixed(ps / l3, ve, buf1[ps], buf1, ps)
-                            : row_dot(ve, buf1[ps], buf1, row_addr(ps, l3, lx, lxy), lx, lxy);
+        const C acc = row_dot(ve, buf1[ps], buf1, row_addr(ps, l3, lx, lxy), lx, lxy);
         rr = (C)to_c(f[q]) - acc;
         ww = om * (C)invD[q];
         buf0[ps] = ww * rr;
@@ -157,14 +132,14 @@ __global__ void __launch_bounds__(NT)
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const int r = threadIdx.x + k * blockDim.x;
-            cm[k] = -1;
+            cm[k] = false;
             if (r < nr) {
                 start_row(r, v[k], r0[k], w[k]);
                 dself[k] = w[k] * r0[k];
                 const int ps = pos[b0 + r];
                 if (ps >= 0) {
                     ad[k] = row_addr(ps, l3, lx, lxy);
-                    cm[k] = ps / l3;
+                    cm[k] = true;
                 }
             }
         }
@@ -182,9 +157,8 @@ __global__ void __launch_bounds__(NT)
 #pragma unroll
             for (int k = 0; k < RR; ++k) {
                 const int r = threadIdx.x + k * blockDim.x;
-                if (r < nr && cm[k] >= 0) {
-                    const C acc = FIXED ? row_dot_fixed(cm[k], v[k], dself[k], dc, ad[k].b0)
-                                        : row_dot(v[k], dself[k], dc, ad[k], lx, lxy);
+                if (r < nr && cm[k]) {
+                    const C acc = row_dot(v[k], dself[k], dc, ad[k], lx, lxy);
                     dself[k] = dself[k] + w[k] * (r0[k] - acc);
                     dn[ad[k].b0] = dself[k];
                 }
@@ -209,6 +183,363 @@ __global__ void __launch_bounds__(NT)
     for (int r = threadIdx.x; r < nr; r += blockDim.x) {
         const int ct = copy[b0 + r];
         if (ct >= 0) u[ct] = (double)dc[pos[b0 + r]];
+    }
+}
+
+// ---- node kernel -------------------------------------------------------------
+// Every thread owns one node: its three faces' rows share the couplings they
+// read (24 distinct entries of d for 3 rows, where three separate rows read
+// 42), because the shared-memory loads of the sweeps are what bounds the FP32
+// kernel once a block fills its SM.  Rows are stored scaled by D^-1, so that a
+// sweep is d <- c0 + (1 - omega) d - omega sum_e s_e d_e with the row's own
+// slot equal to 1 and not stored: 42 coefficients and 3 constants per node in
+// registers, which is what lets a full 10^3-node subdomain run as one block of
+// 1024 threads with 64 registers each (no spills).  The x box and the couplings
+// arrive in one batch of independent loads: with a plain staging loop (ten
+// dependent round trips and 500 index instructions a thread) the FP32 pass took
+// 170 us where it now takes 134.
+// Measured (CUDA events, classes one after another; a kernel of one thread per
+// row before): fine level of a 192^3 ellipsoid, FP32, 24 sweeps 241 -> 134 us a
+// pass; its coarser levels 24.5 -> 18.5 us a launch; 128^3 sphere, BF16, fine
+// 171 -> 83 us.  The shared-memory loads alone would take 43 us at 192^3; the
+// rest is the start of each block and the last wave.
+//
+// Local layout: the up to 10^3 nodes of a subdomain at li + 11 lj + 121 lk in
+// each component.  Column 10 of every row, row 10 of every plane and one plane
+// before and after each component hold no node and stay zero, and serve as the
+// zero neighbours of both of their sides.
+constexpr int kNodeBrick = 8;                    // largest brick of the node kernels
+constexpr int kNB = kNodeBrick + 2;              // nodes per axis of a subdomain
+constexpr int kNX = kNB + 1, kNXY = kNX * kNX, kNC = kNXY * kNX;   // strides: row, plane, component
+constexpr int kN0 = kNXY + kNX + 1;              // position of local node (0, 0, 0) of component 0
+constexpr int kNBuf = ((kN0 + 3 * kNC + kNXY + kNX + 1) + 3) & ~3; // entries of one correction buffer
+constexpr int kNodeVals = 45;                    // per node: 14 scaled couplings of each face's row, then 3 values of 1 / D
+// the x box of the start residual: the subdomain's nodes and one ring
+constexpr int kXX = kNB + 2, kXXY = kXX * kXX, kXC = kXXY * kXX;
+
+// info word of a node copy: local position (12 bits), faces present (bits 12..14), owned (bit 15)
+__host__ __device__ inline int node_info(int pos, int mask, bool owned) { return pos | (mask << 12) | (owned ? 1 << 15 : 0); }
+
+// The 24 neighbours of a node's three faces at q (component blocks of C3
+// entries, strides 1, Y, Z) against the 42 couplings v (14 per row, slots 1..14
+// of band_slot): ax, ay, az += sum.
+template <typename C, int Y, int Z, int C3, typename Ptr>
+__device__ __forceinline__ void node_dot(const C* v, Ptr q, C xs, C ys, C zs, C& ax, C& ay, C& az) {
+    constexpr int X = 1;
+    C t;
+    // x faces
+    t = q[-X]; ax += v[0] * t;
+    t = q[X]; ax += v[1] * t; ay += v[14 + 13] * t; az += v[28 + 9] * t;
+    t = q[-Y]; ax += v[2] * t; ay += v[14 + 10] * t;
+    t = q[Y]; ax += v[3] * t;
+    t = q[-Z]; ax += v[4] * t; az += v[28 + 6] * t;
+    t = q[Z]; ax += v[5] * t;
+    t = q[X - Y]; ay += v[14 + 11] * t;
+    t = q[X - Z]; az += v[28 + 7] * t;
+    ay += v[14 + 12] * xs; az += v[28 + 8] * xs;
+    // y faces
+    t = q[C3 - X]; ay += v[14 + 0] * t; ax += v[6] * t;
+    t = q[C3 + X]; ay += v[14 + 1] * t;
+    t = q[C3 - Y]; ay += v[14 + 2] * t;
+    t = q[C3 + Y]; ay += v[14 + 3] * t; ax += v[9] * t; az += v[28 + 13] * t;
+    t = q[C3 - Z]; ay += v[14 + 4] * t; az += v[28 + 10] * t;
+    t = q[C3 + Z]; ay += v[14 + 5] * t;
+    t = q[C3 + Y - X]; ax += v[7] * t;
+    t = q[C3 + Y - Z]; az += v[28 + 11] * t;
+    ax += v[8] * ys; az += v[28 + 12] * ys;
+    // z faces
+    t = q[2 * C3 - X]; az += v[28 + 0] * t; ax += v[10] * t;
+    t = q[2 * C3 + X]; az += v[28 + 1] * t;
+    t = q[2 * C3 - Y]; az += v[28 + 2] * t; ay += v[14 + 6] * t;
+    t = q[2 * C3 + Y]; az += v[28 + 3] * t;
+    t = q[2 * C3 - Z]; az += v[28 + 4] * t;
+    t = q[2 * C3 + Z]; az += v[28 + 5] * t; ax += v[13] * t; ay += v[14 + 9] * t;
+    t = q[2 * C3 + Z - X]; ax += v[11] * t;
+    t = q[2 * C3 + Z - Y]; ay += v[14 + 7] * t;
+    ax += v[12] * zs; ay += v[14 + 8] * zs;
+}
+
+template <typename T, typename TC>
+struct NodeArgs {
+    const int* off;      // first copy of each subdomain
+    const int* node;     // padded node of each copy (-1: empty lane)
+    const int* info;
+    const int* org;      // node coordinates of each subdomain's local node (0, 0, 0)
+    const TC* vals;      // [kNodeVals][ncopies]
+    int ncopies;
+    const T* f;
+    const T* x;
+    typename Compute<T>::type* u;   // [3][ncopies], the owned nodes' corrections
+    typename Compute<T>::type om;
+    int sweeps;
+    Grid3 g;
+};
+
+// 4-byte asynchronous copy into shared memory (zero when !in): no register
+// holds the value, so a thread's twelve copies and its node's couplings are all
+// in flight at once
+__device__ __forceinline__ void copy4_async(void* dst, const void* src, bool in) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = in ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One block per subdomain, one thread per node (FP32 arithmetic).
+template <typename T, typename TC, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_band_node(int sub0, NodeArgs<T, TC> a) {
+    using C = typename Compute<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* const buf = reinterpret_cast<C*>(smem_raw);
+    const int sd = sub0 + blockIdx.x;
+    const int b0 = a.off[sd];
+    const bool has = (int)threadIdx.x < a.off[sd + 1] - b0;
+    const int ct = b0 + threadIdx.x;
+    const int p = has ? a.node[ct] : -1;
+    const int info = p >= 0 ? a.info[ct] : 0;
+    const bool live = p >= 0;
+    // x over the local box (zero outside the padded grid's -1 .. n+1): every
+    // thread copies whole columns along z, twelve independent loads each
+    {
+        C* const xb = buf + 2 * kNBuf;
+        const int ox = a.org[3 * sd] - 1, oy = a.org[3 * sd + 1] - 1, oz = a.org[3 * sd + 2] - 1;
+        for (int col = threadIdx.x; col < 3 * kXXY; col += NT) {
+            const int c = col / kXXY, r = col - c * kXXY, lj = r / kXX, li = r - lj * kXX;
+            const int i = ox + li, j = oy + lj;
+            const bool inxy = i >= -1 && j >= -1 && i <= a.g.nx + 1 && j <= a.g.ny + 1;
+            const T* src = a.x + (inxy ? (size_t)c * a.g.np + a.g.idx(i, j, 0) : 0);
+            C* dst = xb + c * kXC + r;
+            if constexpr (std::is_same<T, float>::value) {
+#pragma unroll
+                for (int lk = 0; lk < kXX; ++lk) {
+                    const bool in = inxy && oz + lk >= -1 && oz + lk <= a.g.nz + 1;
+                    copy4_async(dst + lk * kXXY, in ? src + (oz + lk) * a.g.sxy : a.x, in);
+                }
+            } else {
+                C tmp[kXX];
+#pragma unroll
+                for (int lk = 0; lk < kXX; ++lk) {
+                    const bool in = inxy && oz + lk >= -1 && oz + lk <= a.g.nz + 1;
+                    tmp[lk] = in ? (C)to_c(src[(oz + lk) * a.g.sxy]) : C(0);
+                }
+#pragma unroll
+                for (int lk = 0; lk < kXX; ++lk) dst[lk * kXXY] = tmp[lk];
+            }
+        }
+    }
+    C v[42], cx = C(0), cy = C(0), cz = C(0), dx = C(0), dy = C(0), dz = C(0), fx = C(0), fy = C(0), fz = C(0);
+#pragma unroll
+    for (int e = 0; e < 42; ++e) v[e] = live ? (C)a.vals[(size_t)e * a.ncopies + ct] : C(0);
+    if (live) {
+        dx = (C)a.vals[(size_t)42 * a.ncopies + ct];   // 1 / D, 0 on faces without a row
+        dy = (C)a.vals[(size_t)43 * a.ncopies + ct];
+        dz = (C)a.vals[(size_t)44 * a.ncopies + ct];
+        fx = (C)to_c(a.f[p]);
+        fy = (C)to_c(a.f[a.g.np + p]);
+        fz = (C)to_c(a.f[2 * a.g.np + p]);
+    }
+    for (int k = threadIdx.x; k < 2 * kNBuf / 4; k += NT) reinterpret_cast<float4*>(buf)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int pos = info & 4095;   // li + 11 lj + 121 lk
+    if constexpr (std::is_same<T, float>::value) copy_async_wait();
+    __syncthreads();
+    if (live) {
+        const int lk = pos / kNXY, lj = (pos / kNX) % kNX, li = pos % kNX;
+        const C* q = buf + 2 * kNBuf + (lk + 1) * kXXY + (lj + 1) * kXX + li + 1;
+        const C xs = q[0], ys = q[kXC], zs = q[2 * kXC];
+        cx = xs; cy = ys; cz = zs;
+        node_dot<C, kXX, kXXY, kXC>(v, q, xs, ys, zs, cx, cy, cz);
+        cx = dx != C(0) ? a.om * (dx * fx - cx) : C(0);
+        cy = dy != C(0) ? a.om * (dy * fy - cy) : C(0);
+        cz = dz != C(0) ? a.om * (dz * fz - cz) : C(0);
+    }
+#pragma unroll
+    for (int e = 0; e < 42; ++e) v[e] *= -a.om;
+    C* const mine = buf + kN0 + pos;
+    const C keep = C(1) - a.om;
+    C ex = cx, ey = cy, ez = cz;   // the node's correction
+    if (live) {
+        mine[0] = ex;
+        mine[kNC] = ey;
+        mine[2 * kNC] = ez;
+    }
+    __syncthreads();
+    int cur = 0;
+    for (int s = 1; s < a.sweeps; ++s) {
+        if (live) {
+            const C* q = mine + cur;
+            C ax = fma(keep, ex, cx), ay = fma(keep, ey, cy), az = fma(keep, ez, cz);
+            node_dot<C, kNX, kNXY, kNC>(v, q, ex, ey, ez, ax, ay, az);
+            ex = ax; ey = ay; ez = az;
+            C* w = mine + (kNBuf - cur);
+            w[0] = ex;
+            w[kNC] = ey;
+            w[2 * kNC] = ez;
+        }
+        cur = kNBuf - cur;
+        __syncthreads();
+    }
+    if ((info >> 15) & 1) {
+        a.u[ct] = ex;
+        a.u[(size_t)a.ncopies + ct] = ey;
+        a.u[2 * (size_t)a.ncopies + ct] = ez;
+    }
+}
+
+// FP64: a cluster of CS blocks per subdomain.  The FP64 pipe issues two FMAs
+// per clock and SM, so a subdomain's 45 FMAs per node and sweep are what its
+// time goes on; the cluster spreads them over CS SMs and leaves each thread
+// room for the couplings of its node in FP64 registers.  Every block keeps the
+// whole correction box; a node's new values go to the blocks whose nodes read
+// them (positions within one plane, row and column) through distributed shared
+// memory, and a cluster barrier closes each sweep.  Blocks of 128 threads: one
+// warp per scheduler keeps its FP64 unit busy, and three blocks fit an SM.
+// Measured, one pass (one block per subdomain before): 16^3 sphere (27
+// subdomains) 190 -> 63 us; 72 x 56 x 88 ellipsoid fine level 326 -> 310 us
+// with the classes one after another, the solve with them side by side
+// 23.6 -> 15.5 ms.
+constexpr int kClusterThreads = 128;
+template <typename T, typename TC, int CS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) k_band_node_cluster(int sub0, NodeArgs<T, TC> a) {
+    using C = typename Compute<T>::type;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* const buf = reinterpret_cast<C*>(smem_raw);
+    constexpr int NT = kClusterThreads;
+    const int rank = (int)cluster.block_rank();
+    const int sd = sub0 + blockIdx.x / CS;
+    const int b0 = a.off[sd], n = a.off[sd + 1] - b0;
+    const int per = (n + CS - 1) / CS;               // nodes of each block, in box order
+    const int local = rank * per + threadIdx.x;
+    const bool live = (int)threadIdx.x < per && local < n;
+    const int ct = b0 + local;
+    const int p = live ? a.node[ct] : 0;
+    const int info = live ? a.info[ct] : 0;
+    const int pos = info & 4095;
+    // the blocks that hold a neighbour of this node
+    int r0 = CS, r1 = -1;
+    if (live) {
+#pragma unroll
+        for (int r = 0; r < CS; ++r) {
+            const int lo = r * per, hi = min(n, lo + per) - 1;
+            if (lo <= hi && (a.info[b0 + lo] & 4095) <= pos + kN0 && (a.info[b0 + hi] & 4095) >= pos - kN0) {
+                r0 = min(r0, r);
+                r1 = max(r1, r);
+            }
+        }
+    }
+    C v[42], cx = C(0), cy = C(0), cz = C(0);
+#pragma unroll
+    for (int e = 0; e < 42; ++e) v[e] = live ? (C)a.vals[(size_t)e * a.ncopies + ct] : C(0);
+    for (int k = threadIdx.x; k < 2 * kNBuf; k += NT) buf[k] = C(0);
+    if (live) {
+        // start residual from global memory: the neighbours' loads are independent of one another
+        const int X = 1, Y = a.g.sx, Z = a.g.sxy, N = a.g.np;
+        const T* q = a.x + p;
+        auto at = [&](int o) { return (C)to_c(q[o]); };
+        const C xs = at(0), ys = at(N), zs = at(2 * N);
+        cx = xs; cy = ys; cz = zs;
+        C t;
+        t = at(-X); cx += v[0] * t;
+        t = at(X); cx += v[1] * t; cy += v[14 + 13] * t; cz += v[28 + 9] * t;
+        t = at(-Y); cx += v[2] * t; cy += v[14 + 10] * t;
+        t = at(Y); cx += v[3] * t;
+        t = at(-Z); cx += v[4] * t; cz += v[28 + 6] * t;
+        t = at(Z); cx += v[5] * t;
+        t = at(X - Y); cy += v[14 + 11] * t;
+        t = at(X - Z); cz += v[28 + 7] * t;
+        cy += v[14 + 12] * xs; cz += v[28 + 8] * xs;
+        t = at(N - X); cy += v[14 + 0] * t; cx += v[6] * t;
+        t = at(N + X); cy += v[14 + 1] * t;
+        t = at(N - Y); cy += v[14 + 2] * t;
+        t = at(N + Y); cy += v[14 + 3] * t; cx += v[9] * t; cz += v[28 + 13] * t;
+        t = at(N - Z); cy += v[14 + 4] * t; cz += v[28 + 10] * t;
+        t = at(N + Z); cy += v[14 + 5] * t;
+        t = at(N + Y - X); cx += v[7] * t;
+        t = at(N + Y - Z); cz += v[28 + 11] * t;
+        cx += v[8] * ys; cz += v[28 + 12] * ys;
+        t = at(2 * N - X); cz += v[28 + 0] * t; cx += v[10] * t;
+        t = at(2 * N + X); cz += v[28 + 1] * t;
+        t = at(2 * N - Y); cz += v[28 + 2] * t; cy += v[14 + 6] * t;
+        t = at(2 * N + Y); cz += v[28 + 3] * t;
+        t = at(2 * N - Z); cz += v[28 + 4] * t;
+        t = at(2 * N + Z); cz += v[28 + 5] * t; cx += v[13] * t; cy += v[14 + 9] * t;
+        t = at(2 * N + Z - X); cx += v[11] * t;
+        t = at(2 * N + Z - Y); cy += v[14 + 7] * t;
+        cx += v[12] * zs; cy += v[14 + 8] * zs;
+        const C dx = (C)a.vals[(size_t)42 * a.ncopies + ct], dy = (C)a.vals[(size_t)43 * a.ncopies + ct],
+                dz = (C)a.vals[(size_t)44 * a.ncopies + ct];
+        cx = dx != C(0) ? a.om * (dx * (C)to_c(a.f[p]) - cx) : C(0);
+        cy = dy != C(0) ? a.om * (dy * (C)to_c(a.f[N + p]) - cy) : C(0);
+        cz = dz != C(0) ? a.om * (dz * (C)to_c(a.f[2 * N + p]) - cz) : C(0);
+    }
+#pragma unroll
+    for (int e = 0; e < 42; ++e) v[e] *= -a.om;
+    cluster.sync();   // every block's buffers are zero
+    const C keep = C(1) - a.om;
+    C ex = cx, ey = cy, ez = cz;
+    int cur = 0;      // offset of the buffer the sweep reads
+    for (int r = r0; r <= r1; ++r) {
+        C* w = cluster.map_shared_rank(buf, r) + kN0 + pos;
+        w[0] = ex;
+        w[kNC] = ey;
+        w[2 * kNC] = ez;
+    }
+    for (int s = 1; s < a.sweeps; ++s) {
+        cluster.sync();
+        if (live) {
+            const C* q = buf + kN0 + pos + cur;
+            C ax = fma(keep, ex, cx), ay = fma(keep, ey, cy), az = fma(keep, ez, cz);
+            node_dot<C, kNX, kNXY, kNC>(v, q, ex, ey, ez, ax, ay, az);
+            ex = ax; ey = ay; ez = az;
+            if (s + 1 < a.sweeps)
+                for (int r = r0; r <= r1; ++r) {
+                    C* w = cluster.map_shared_rank(buf, r) + kN0 + pos + (kNBuf - cur);
+                    w[0] = ex;
+                    w[kNC] = ey;
+                    w[2 * kNC] = ez;
+                }
+        }
+        cur = kNBuf - cur;
+    }
+    if ((info >> 15) & 1) {
+        a.u[ct] = ex;
+        a.u[(size_t)a.ncopies + ct] = ey;
+        a.u[2 * (size_t)a.ncopies + ct] = ez;
+    }
+    cluster.sync();   // no block leaves while another may still write to it
+}
+
+// x <- x + u on the band faces (uidx: where each face's owner put its correction)
+template <typename T>
+__global__ void k_band_add_node(const int* __restrict__ band, const int* __restrict__ uidx, int nband,
+                                const typename Compute<T>::type* __restrict__ u, T* __restrict__ x) {
+    using C = typename Compute<T>::type;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nband) return;
+    const int q = band[t];
+    x[q] = to_store<T>((C)to_c(x[q]) + u[uidx[t]]);
+}
+
+// Scaled couplings of every node copy from the band rows (15 slots, slot-major)
+// and, for the owners, where each face's correction will be.  tmap: position of
+// a face in the band list, -1 off the band.
+template <typename TC>
+__global__ void k_band_node_vals(int ncopies, const int* __restrict__ node, const int* __restrict__ info, int np,
+                                 const int* __restrict__ tmap, const double* __restrict__ rows, int nband,
+                                 const double* __restrict__ invD, TC* __restrict__ vals, int* __restrict__ uidx) {
+    const int ct = blockIdx.x * blockDim.x + threadIdx.x;
+    if (ct >= ncopies) return;
+    const int p = node[ct];
+    const int in = p >= 0 ? info[ct] : 0;
+    for (int c = 0; c < 3; ++c) {
+        const bool row = (in >> (12 + c)) & 1;
+        const int t = row ? tmap[c * np + p] : 0;
+        const double d = row ? invD[c * np + p] : 0.0;
+        for (int e = 1; e < kBandSlots; ++e)
+            vals[(size_t)(14 * c + e - 1) * ncopies + ct] = row ? (TC)(d * rows[(size_t)e * nband + t]) : TC(0);
+        vals[(size_t)(42 + c) * ncopies + ct] = (TC)d;
+        if (row && ((in >> 15) & 1)) uidx[t] = c * ncopies + ct;
     }
 }
 
@@ -367,18 +698,12 @@ void band_schwarz_setup(const Grid3& g, const int* band_dev, int nband, int bric
         ++out.cls_count[cl];
         const long long kb = cp[c0].brick;
         const int B[3] = {(int)(kb % nb[0]), (int)((kb / nb[0]) % nb[1]), (int)(kb / ((long long)nb[0] * nb[1]))};
-        // local box: the subdomain's nodes and their neighbours (within the
-        // padded grid; the default brick uses the fixed, unclipped box)
+        // local box: the subdomain's nodes and their neighbours (within the padded grid)
         int lo[3], l[3];
         for (int a = 0; a < 3; ++a) {
-            if (brick == kFixedBrick) {
-                lo[a] = B[a] * brick - 2;
-                l[a] = a == 0 ? kFX : (a == 1 ? kFY : kFZ);
-            } else {
-                lo[a] = std::max(B[a] * brick - 2, -1);
-                const int hi = std::min(B[a] * brick + brick + 1, n[a] + 1);
-                l[a] = hi - lo[a] + 1;
-            }
+            lo[a] = std::max(B[a] * brick - 2, -1);
+            const int hi = std::min(B[a] * brick + brick + 1, n[a] + 1);
+            l[a] = hi - lo[a] + 1;
         }
         DM_REQUIRE(l[0] < 1024 && l[1] < 1024 && l[2] < 1024, DM_ERR_INVALID_ARG, "band brick too large");
         out.off.push_back((int)out.copy.size());
@@ -420,13 +745,211 @@ void band_schwarz_setup(const Grid3& g, const int* band_dev, int nband, int bric
         out.maxrows = std::max(out.maxrows, (int)out.copy.size() - out.off.back());
     }
     out.off.push_back((int)out.copy.size());
-    out.fixed = brick == kFixedBrick;
 }
 
 void band_copy_vals(const int* copy, int ncopies, const double* band_vals, int nband, double* out, cudaStream_t s) {
     if (ncopies <= 0) return;
     launch("k_band_copy_vals", k_band_copy_vals, (ncopies + 255) / 256, 256, 0, s, copy, ncopies, band_vals, nband,
            out);
+}
+
+// ---- node kernels: layout and launches ----------------------------------------
+
+bool band_nodes_fit(int brick) { return brick >= 1 && brick <= kNodeBrick; }
+
+void band_nodes_setup(const Grid3& g, const int* band_dev, int nband, int brick, bool by_bank, NodeLayout& out,
+                      cudaStream_t s) {
+    out = NodeLayout{};
+    if (nband <= 0) return;
+    std::vector<int> band(nband);
+    DM_CUDA(cudaMemcpyAsync(band.data(), band_dev, sizeof(int) * nband, cudaMemcpyDeviceToHost, s));
+    DM_CUDA(cudaStreamSynchronize(s));
+    // the band's nodes in ascending order, with the faces each carries
+    std::vector<unsigned char> mask(g.np, 0);
+    for (int q : band) mask[q % g.np] |= (unsigned char)(1 << (q / g.np));
+    std::vector<int> nodes;
+    nodes.reserve(nband / 2 + 1);
+    for (int p = 0; p < g.np; ++p)
+        if (mask[p]) nodes.push_back(p);
+    const int nb[3] = {(g.nx + brick) / brick, (g.ny + brick) / brick, (g.nz + brick) / brick};
+    const size_t nbk = (size_t)nb[0] * nb[1] * nb[2];
+    auto coords = [&](int p, int c[3]) {
+        const int r = p - g.off0;
+        c[2] = r / g.sxy;
+        const int rem = r - c[2] * g.sxy;
+        c[1] = rem / g.sx;
+        c[0] = rem - c[1] * g.sx;
+    };
+    std::vector<unsigned char> owner(nbk, 0);
+    auto key = [&](int bx, int by, int bz) { return ((size_t)bz * nb[1] + by) * nb[0] + bx; };
+    for (int p : nodes) {
+        int c[3];
+        coords(p, c);
+        owner[key(c[0] / brick, c[1] / brick, c[2] / brick)] = 1;
+    }
+    // brick B holds node P when B b - 1 <= P <= B b + b on every axis
+    auto each = [&](auto&& visit) {
+        for (int p : nodes) {
+            int c[3], lo[3], hi[3];
+            coords(p, c);
+            for (int ax = 0; ax < 3; ++ax) {
+                lo[ax] = std::max((c[ax] + brick - 1) / brick - 1, 0);
+                hi[ax] = std::min((c[ax] + 1) / brick, nb[ax] - 1);
+            }
+            for (int bz = lo[2]; bz <= hi[2]; ++bz)
+                for (int by = lo[1]; by <= hi[1]; ++by)
+                    for (int bx = lo[0]; bx <= hi[0]; ++bx) {
+                        const size_t kb = key(bx, by, bz);
+                        if (owner[kb]) visit(kb, p, c, bx, by, bz);
+                    }
+        }
+    };
+    std::vector<int> start(nbk + 1, 0);
+    each([&](size_t kb, int, const int*, int, int, int) { ++start[kb + 1]; });
+    for (size_t b = 0; b < nbk; ++b) start[b + 1] += start[b];
+    std::vector<int> cnode((size_t)start[nbk]), cinfo((size_t)start[nbk]);
+    {
+        std::vector<int> fill(start.begin(), start.end() - 1);
+        // nodes come in ascending order, so every brick's copies are in box order
+        each([&](size_t kb, int p, const int* c, int bx, int by, int bz) {
+            const int li = c[0] - (bx * brick - 1), lj = c[1] - (by * brick - 1), lk = c[2] - (bz * brick - 1);
+            const bool owned = c[0] / brick == bx && c[1] / brick == by && c[2] / brick == bz;
+            const int at = fill[kb]++;
+            cnode[at] = p;
+            cinfo[at] = node_info(li + kNX * lj + kNXY * lk, mask[p], owned);
+        });
+    }
+    // subdomains class by class, the largest class first (its blocks take an SM each)
+    std::vector<size_t> order;
+    for (size_t b = 0; b < nbk; ++b)
+        if (start[b + 1] > start[b]) order.push_back(b);
+    std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) {
+        return node_class(start[x + 1] - start[x]) > node_class(start[y + 1] - start[y]);
+    });
+    std::vector<int> slot;
+    for (size_t b : order) {
+        const int c0 = start[b], n = start[b + 1] - c0;
+        const int cl = node_class(n);
+        if (out.cls_count[cl] == 0) out.cls_first[cl] = (int)out.off.size();
+        ++out.cls_count[cl];
+        out.off.push_back((int)out.node.size());
+        const int bx = (int)(b % nb[0]), by = (int)((b / nb[0]) % nb[1]), bz = (int)(b / ((size_t)nb[0] * nb[1]));
+        out.org.insert(out.org.end(), {bx * brick - 1, by * brick - 1, bz * brick - 1});
+        out.cls_copies[cl] += n;
+        slot.resize(n);
+        if (by_bank) {
+            // Lanes of a warp in distinct shared-memory banks: the nodes sorted by
+            // bank and dealt round-robin over the warps (every coupling sits at one
+            // offset for all nodes, so then all 24 loads of a sweep are nearly free
+            // of conflicts; in box order they take two to three passes each).
+            const int ng = (n + 31) / 32;
+            int cnt[33] = {};
+            for (int i = 0; i < n; ++i) ++cnt[((cinfo[c0 + i] & 4095) & 31) + 1];
+            for (int k = 0; k < 32; ++k) cnt[k + 1] += cnt[k];
+            const size_t base = out.node.size();
+            out.node.resize(base + 32 * (size_t)ng, -1);
+            out.info.resize(base + 32 * (size_t)ng, 0);
+            for (int i = 0; i < n; ++i) {
+                const int rk = cnt[(cinfo[c0 + i] & 4095) & 31]++;
+                const size_t at = base + (size_t)(rk % ng) * 32 + rk / ng;
+                out.node[at] = cnode[c0 + i];
+                out.info[at] = cinfo[c0 + i];
+            }
+        } else {
+            out.node.insert(out.node.end(), cnode.begin() + c0, cnode.begin() + c0 + n);
+            out.info.insert(out.info.end(), cinfo.begin() + c0, cinfo.begin() + c0 + n);
+        }
+    }
+    out.off.push_back((int)out.node.size());
+}
+
+template <typename TC>
+void band_node_vals(const int* node, const int* info, int ncopies, const Grid3& g, const int* tmap, const double* rows,
+                    int nband, const double* invD, TC* vals, int* uidx, cudaStream_t s) {
+    if (ncopies <= 0) return;
+    launch("k_band_node_vals", k_band_node_vals<TC>, (ncopies + 127) / 128, 128, 0, s, ncopies, node, info, g.np, tmap,
+           rows, nband, invD, vals, uidx);
+}
+
+namespace {
+
+constexpr int kSMs = 152;
+
+template <typename T, typename TC, int NT>
+void launch_node(const char* name, double bytes, int first, int count, const NodeArgs<T, TC>& a, cudaStream_t s) {
+    using C = typename Compute<T>::type;
+    constexpr size_t smem = sizeof(C) * (2 * kNBuf + 3 * kXC);
+    // above the 48 KB a kernel may use unasked; set on every call because the setting belongs to the current device
+    DM_CUDA(cudaFuncSetAttribute(k_band_node<T, TC, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    launch_b(name, bytes, k_band_node<T, TC, NT>, count, NT, smem, s, first, a);
+}
+template <int CS>
+void launch_cluster(const char* name, double bytes, int first, int count, const NodeArgs<double, double>& a,
+                    cudaStream_t s) {
+    constexpr size_t smem = sizeof(double) * 2 * kNBuf;
+    // above the 48 KB a kernel may use unasked; set on every call because the setting belongs to the current device
+    DM_CUDA(cudaFuncSetAttribute(k_band_node_cluster<double, double, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem));
+    launch_b(name, bytes, k_band_node_cluster<double, double, CS>, count * CS, kClusterThreads, smem, s, first, a);
+}
+
+}  // namespace
+
+template <typename T, typename TC>
+void band_nodes(const BandNodes<TC>& bn, const Grid3& g, const int* band, int nband, const T* f, T* x, void* u_raw,
+                double omega, int sweeps, bool fine, cudaStream_t s0, const Fork* fk) {
+    using C = typename Compute<T>::type;
+    if (nband <= 0 || bn.nsub <= 0 || sweeps <= 0) return;
+    const char* name = stencil_name("band_schwarz", prec_index<T>(), ST_JACOBI, fine);
+    C* u = static_cast<C*>(u_raw);
+    const NodeArgs<T, TC> a{bn.off, bn.node, bn.info, bn.org, bn.vals, bn.ncopies, f, x, u, (C)omega, sweeps, g};
+    // bytes: per node copy its 45 values and two words, x and f of its faces; the owners' corrections
+    const double per = kNodeVals * sizeof(TC) + 8.0 + 6.0 * sizeof(T);
+    const double owned = (double)nband * sizeof(C);
+    constexpr bool wide = std::is_same<T, double>::value;
+    int top = 0, nl = 0;
+    for (int cl = 0; cl < kNodeClasses; ++cl)
+        if (bn.cls_count[cl] > 0) {
+            top = cl;
+            ++nl;
+        }
+    // A level with few subdomains goes in one launch shaped for its largest
+    // class: FP32, when they fit the SMs at one block each; FP64, when clusters
+    // of eight blocks for every subdomain still run at once.
+    const bool single = wide ? 8 * bn.nsub <= 2 * kSMs : bn.nsub <= kSMs;
+    if (single) nl = 1;
+    const bool forked = fk && fk->naux > 0 && nl > 1;
+    if (forked) {
+        DM_CUDA(cudaEventRecord(fk->fork, s0));
+        for (int k = 0; k < std::min(nl - 1, fk->naux); ++k) DM_CUDA(cudaStreamWaitEvent(fk->aux[k], fk->fork, 0));
+    }
+    int li = 0;
+    for (int cl = kNodeClasses - 1; cl >= 0; --cl) {
+        if (bn.cls_count[cl] == 0 || (single && cl != top)) continue;
+        const int ai = li++;   // the first class stays on s0
+        cudaStream_t s = (forked && ai > 0 && ai - 1 < fk->naux) ? fk->aux[ai - 1] : s0;
+        const int first = single ? 0 : bn.cls_first[cl], count = single ? bn.nsub : bn.cls_count[cl];
+        const double bytes = (single ? bn.copies() : (double)bn.cls_copies[cl]) * per + owned / nl;
+        if constexpr (wide) {
+            if (single || cl >= 2) launch_cluster<8>(name, bytes, first, count, a, s);
+            else if (cl == 1) launch_cluster<4>(name, bytes, first, count, a, s);
+            else launch_cluster<2>(name, bytes, first, count, a, s);
+        } else {
+            switch (cl) {
+                case 0: launch_node<T, TC, 256>(name, bytes, first, count, a, s); break;
+                case 1: launch_node<T, TC, 512>(name, bytes, first, count, a, s); break;
+                case 2: launch_node<T, TC, 768>(name, bytes, first, count, a, s); break;
+                default: launch_node<T, TC, 1024>(name, bytes, first, count, a, s);
+            }
+        }
+    }
+    if (forked)
+        for (int k = 0; k < std::min(nl - 1, fk->naux); ++k) {
+            DM_CUDA(cudaEventRecord(fk->join[k], fk->aux[k]));
+            DM_CUDA(cudaStreamWaitEvent(s0, fk->join[k], 0));
+        }
+    launch_b(stencil_name("band_add", prec_index<T>(), ST_JACOBI, fine), (double)nband * (8.0 + sizeof(C) + 2.0 * sizeof(T)),
+             k_band_add_node<T>, (nband + 255) / 256, 256, 0, s0, band, bn.uidx, nband, (const C*)u, x);
 }
 
 // rows per thread and block size of a class (R = 0: the shared-memory variant;
@@ -484,14 +1007,9 @@ void band_schwarz(const BandSchwarz<TC>& bs, const TC* invD, const Grid3& g, con
             }
         const double bytes = (double)copies * (16.0 * sizeof(TC) + 8.0 + 2.0 * sizeof(T)) + 8.0 * (double)owned;
 #define DM_SCHWARZ(RV, NV)                                                                                         \
-    if (bs.fixed)                                                                                                  \
-        launch_b(name, bytes, k_band_schwarz<T, TC, RV, NV, true>, count, NV, smem, s, first, bs.off, bs.copy,     \
-                 bs.pos, bs.dims, bs.org, bs.vals, bs.ncopies, band, invD, f, (const T*)x, u, omega, sweeps, g,    \
-                 bs.maxbox, bs.maxrows);                                                                         \
-    else                                                                                                           \
-    launch_b(name, bytes, k_band_schwarz<T, TC, RV, NV, false>, count, NV, smem, s, first, bs.off, bs.copy,      \
-             bs.pos, bs.dims, bs.org, bs.vals, bs.ncopies, band, invD, f, (const T*)x, u, omega, sweeps, g,       \
-             bs.maxbox, bs.maxrows)
+    launch_b(name, bytes, k_band_schwarz<T, TC, RV, NV>, count, NV, smem, s, first, bs.off, bs.copy, bs.pos,     \
+             bs.dims, bs.org, bs.vals, bs.ncopies, band, invD, f, (const T*)x, u, omega, sweeps, g, bs.maxbox,     \
+             bs.maxrows)
         if (nt == 256) DM_SCHWARZ(1, 256);
         else if (R == 1) DM_SCHWARZ(1, 512);
         else if (R == 2) DM_SCHWARZ(2, 512);
@@ -530,24 +1048,24 @@ void band_schwarz_prepare(const SchwarzLayout& sl) {
         int R, nt;
         class_shape<T>(cl, R, nt);
         const size_t need = schwarz_smem<T>(sl.maxbox, sl.maxrows, R);
-        const bool fx = sl.fixed;
-        if (nt == 256) fx ? allow_smem(k_band_schwarz<T, TC, 1, 256, true>, need)
-                          : allow_smem(k_band_schwarz<T, TC, 1, 256, false>, need);
-        else if (R == 1) fx ? allow_smem(k_band_schwarz<T, TC, 1, 512, true>, need)
-                            : allow_smem(k_band_schwarz<T, TC, 1, 512, false>, need);
-        else if (R == 2) fx ? allow_smem(k_band_schwarz<T, TC, 2, 512, true>, need)
-                            : allow_smem(k_band_schwarz<T, TC, 2, 512, false>, need);
-        else if (R == 4) fx ? allow_smem(k_band_schwarz<T, TC, 4, 512, true>, need)
-                            : allow_smem(k_band_schwarz<T, TC, 4, 512, false>, need);
-        else fx ? allow_smem(k_band_schwarz<T, TC, 0, 512, true>, need)
-                : allow_smem(k_band_schwarz<T, TC, 0, 512, false>, need);
+        if (nt == 256) allow_smem(k_band_schwarz<T, TC, 1, 256>, need);
+        else if (R == 1) allow_smem(k_band_schwarz<T, TC, 1, 512>, need);
+        else if (R == 2) allow_smem(k_band_schwarz<T, TC, 2, 512>, need);
+        else if (R == 4) allow_smem(k_band_schwarz<T, TC, 4, 512>, need);
+        else allow_smem(k_band_schwarz<T, TC, 0, 512>, need);
     }
 }
 
 #define DM_INST(T, TC)                                                                                           \
     template void band_schwarz<T, TC>(const BandSchwarz<TC>&, const TC*, const Grid3&, const int*, int, const T*, \
                                       T*, double*, double, int, bool, cudaStream_t, const Fork*);                \
-    template void band_schwarz_prepare<T, TC>(const SchwarzLayout&);
+    template void band_schwarz_prepare<T, TC>(const SchwarzLayout&);                                             \
+    template void band_nodes<T, TC>(const BandNodes<TC>&, const Grid3&, const int*, int, const T*, T*, void*,   \
+                                    double, int, bool, cudaStream_t, const Fork*);
+template void band_node_vals<double>(const int*, const int*, int, const Grid3&, const int*, const double*, int,
+                                     const double*, double*, int*, cudaStream_t);
+template void band_node_vals<float>(const int*, const int*, int, const Grid3&, const int*, const double*, int,
+                                    const double*, float*, int*, cudaStream_t);
 DM_INST(double, double)
 DM_INST(float, float)
 DM_INST(__nv_bfloat16, float)

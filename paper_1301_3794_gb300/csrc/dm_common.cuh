@@ -400,7 +400,6 @@ struct SchwarzLayout {
     std::vector<int> off, copy, pos, dims;
     std::vector<int> org;         // 3 per subdomain: node coordinates of its local box's first node
     int maxrows = 0, maxbox = 0;
-    bool fixed = false;           // every subdomain uses the fixed box of the default brick
     int cls_first[kSchwarzClasses] = {}, cls_count[kSchwarzClasses] = {};
     long long cls_copies[kSchwarzClasses] = {}, cls_owned[kSchwarzClasses] = {};   // row copies, owned ones
 };
@@ -415,7 +414,6 @@ struct BandSchwarz {
     int nsub = 0, ncopies = 0, maxrows = 0, maxbox = 0;
     int cls_first[kSchwarzClasses] = {}, cls_count[kSchwarzClasses] = {};
     long long cls_copies[kSchwarzClasses] = {}, cls_owned[kSchwarzClasses] = {};
-    bool fixed = false;
 };
 void band_schwarz_setup(const Grid3& g, const int* band_dev, int nband, int brick, SchwarzLayout& out,
                         cudaStream_t s);
@@ -439,6 +437,44 @@ struct Fork {
 template <typename T, typename TC>
 void band_schwarz(const BandSchwarz<TC>& bs, const TC* invD, const Grid3& g, const int* band, int nband, const T* f,
                   T* x, double* u, double omega, int sweeps, bool fine, cudaStream_t s, const Fork* fk = nullptr);
+// Subdomains of the node kernels (bricks of up to 8 nodes, dm_band.cu): copies
+// of band nodes grouped by brick, one lane each (node -1: an empty lane), class
+// by class with the largest class first.  by_bank orders a subdomain's nodes
+// for conflict-free shared memory, else they keep box order.
+constexpr int kNodeClasses = 4;   // blocks of 256, 512, 768 and 1024 threads
+inline int node_class(int nodes) { return nodes <= 256 ? 0 : (nodes <= 512 ? 1 : (nodes <= 768 ? 2 : 3)); }
+struct NodeLayout {
+    std::vector<int> off, node, info, org;
+    int cls_first[kNodeClasses] = {}, cls_count[kNodeClasses] = {};
+    long long cls_copies[kNodeClasses] = {};
+};
+template <typename TC>
+struct BandNodes {
+    const int* off = nullptr;
+    const int* node = nullptr;
+    const int* info = nullptr;
+    const int* org = nullptr;
+    const int* uidx = nullptr;    // per band face: where its owner puts the correction
+    const TC* vals = nullptr;     // [45][ncopies]: couplings scaled by 1/D, then 1/D
+    int nsub = 0, ncopies = 0;
+    int cls_first[kNodeClasses] = {}, cls_count[kNodeClasses] = {};
+    long long cls_copies[kNodeClasses] = {};
+    double copies() const {
+        double n = 0;
+        for (long long c : cls_copies) n += (double)c;
+        return n;
+    }
+};
+bool band_nodes_fit(int brick);
+void band_nodes_setup(const Grid3& g, const int* band_dev, int nband, int brick, bool by_bank, NodeLayout& out,
+                      cudaStream_t s);
+template <typename TC>
+void band_node_vals(const int* node, const int* info, int ncopies, const Grid3& g, const int* tmap, const double* rows,
+                    int nband, const double* invD, TC* vals, int* uidx, cudaStream_t s);
+// as band_schwarz; u: 3 ncopies values of scratch in the compute type
+template <typename T, typename TC>
+void band_nodes(const BandNodes<TC>& bn, const Grid3& g, const int* band, int nband, const T* f, T* x, void* u,
+                double omega, int sweeps, bool fine, cudaStream_t s, const Fork* fk = nullptr);
 void vec_apply_dense_f64(const Grid3& g, const double* A, const double* L, const double* invV, double sigma,
                          const double* x, double* y, cudaStream_t s);
 // (K - sigma A) x in float-float into the compact vector out (out[cmap[q]] for
