@@ -1342,7 +1342,7 @@ void setup_operator(dm_operator* op) {
         DM_REQUIRE(n <= 6000, DM_ERR_INVALID_ARG, "coarsest level too large for the dense solve; raise max_coarse");
         op->c_inv.alloc((size_t)n * n);
         vec_dense_assemble(g.g, g.A.get(), g.L.get(), g.invV.get(), op->sigma, op->c_list.get(), n, op->c_inv.get(), s);
-        DBuf<double> work(2ull * n * n + n);
+        DBuf<double> work(dense_inverse_work(n), false);
         DBuf<int> flag(1);
         DM_REQUIRE(dense_inverse(op->c_inv.get(), n, work.get(), flag.get(), s), DM_ERR_NO_CONVERGENCE,
                    "coarsest K - sigma A is singular (sigma is an eigenvalue of the coarsest grid)");
@@ -1367,7 +1367,7 @@ void setup_operator(dm_operator* op) {
         cell_components_pin(g.g, g.A.get(), op->s_list.get(), n, label.get(), op->s_pinned.get(), s);
         op->s_inv.alloc((size_t)n * n);
         scal_dense_assemble(g.g, g.A.get(), op->s_list.get(), op->s_pinned.get(), n, op->s_inv.get(), s);
-        DBuf<double> work(2ull * n * n + n);
+        DBuf<double> work(dense_inverse_work(n), false);
         DBuf<int> flag(1);
         DM_REQUIRE(dense_inverse(op->s_inv.get(), n, work.get(), flag.get(), s), DM_ERR_NO_CONVERGENCE,
                    "coarsest scalar Laplacian is singular after pinning");

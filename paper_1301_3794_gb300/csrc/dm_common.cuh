@@ -542,8 +542,9 @@ void cell_prolong_add(const Grid3& gf, const Grid3& gc, const unsigned char* act
                       const int* tiles_f, int ntiles_f, cudaStream_t s);
 
 // dense (dm_dense.cu)
-// in-place inverse of the n x n row-major FP64 matrix M (work: 2 n^2 + n doubles).
-// Returns false if a pivot fell below tiny * max|M|.
+// in-place inverse of the n x n row-major FP64 matrix M, n <= 6144 (work:
+// dense_inverse_work(n) doubles).  Returns false if a column had no pivot above 1e-300.
+size_t dense_inverse_work(int n);
 bool dense_inverse(double* M, int n, double* work, int* d_flag, cudaStream_t s);
 template <typename T>
 void dense_coarse_solve(const double* Minv64, const float* Minv32, int n, const int* list, const unsigned char* zero_rows,

@@ -1,82 +1,275 @@
-// Dense kernels of the coarsest multigrid level: Gauss-Jordan inversion with
-// partial pivoting, the gather / dense matvec / scatter of the coarsest solve,
+// Dense kernels of the coarsest multigrid level: blocked Gauss-Jordan inversion
+// with partial pivoting, the gather / dense matvec / scatter of the coarsest solve,
 // and connected components of the active coarsest cells (the scalar Laplacian
 // D A D^T has one constant null vector per component; the lowest-index cell of
 // each component is pinned to zero).
+#include <cooperative_groups.h>
+
 #include "dm_common.cuh"
 
 namespace dm {
 
 namespace {
 
-// pivot search, row swap, pivot-row scaling and factor column of step k on the
-// augmented n x 2n matrix W (one block)
-__global__ void k_gj_pivot(double* __restrict__ W, int n, int k, double* __restrict__ fac, int* __restrict__ flag) {
-    __shared__ double best[1024];
-    __shared__ int bidx[1024];
-    const int t = threadIdx.x;
-    const int n2 = 2 * n;
-    double bv = -1.0;
-    int bi = k;
-    for (int i = k + t; i < n; i += blockDim.x) {
-        const double v = fabs(W[(long long)i * n2 + k]);
-        if (v > bv) { bv = v; bi = i; }
+// ---- in-place inverse by blocked Gauss-Jordan elimination ---------------------
+// The steps of a panel of NB columns act on the rest of the matrix as one
+// update: with E the product of the panel's elimination steps and J its rows,
+// E v = (v with its J entries zeroed) + M v_J, and the in-place panel holds M.
+// So one block eliminates within the panel (its rows in registers), the row
+// swaps are carried to the other columns, and one rank-NB update over the whole
+// chip follows.  The n^3 FP64 FMAs of the updates bound it (two per clock and
+// SM); a step per column instead, as an n x 2n elimination of [A | I], did twice
+// those FMAs and two launches for each of the n columns, every launch waiting
+// on one block's pivot search.
+// Measured (CUDA events), both coarsest inverses of an operator: 96^3 ellipsoid (2,600
+// columns in all) 80 -> 31.5 ms, 16^3 sphere (920 columns) 20 -> 7.1 ms.
+
+// The panel goes to a cluster of eight blocks, an eighth of the rows each: its
+// own n NB^2 FMAs on one SM's FP64 pipe took 180-290 us, more than the update.
+constexpr int kPanelBlocks = 8, kPanelThreads = 256, kPanel = 16;
+
+// Eliminate the panel of columns k0 .. k0 + nb - 1 (nb <= kPanel) of the n x n
+// row-major W in place, with partial pivoting over the rows k0 + p and below;
+// RPT rows per thread.  piv[k0 + p]: the row swapped with k0 + p.
+// Mt[p n + r]: the panel after it; swaps[0 .. 2 nb): destination rows of the
+// swaps, swaps[2 kPanel .. 2 kPanel + 2 nb): the rows their contents come from.
+template <int RPT>
+__global__ void __cluster_dims__(kPanelBlocks, 1, 1) __launch_bounds__(kPanelThreads)
+    k_gj_panel(double* __restrict__ W, int n, int k0, int nb, int* __restrict__ piv, double* __restrict__ Mt,
+               int* __restrict__ swaps, int* __restrict__ flag) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    constexpr int NB = kPanel, NW = kPanelThreads / 32, NC = kPanelBlocks * NW;   // NC candidates per column
+    // by column parity: a block may write the next column's entries while another still reads this one's
+    __shared__ double s_best[2][NC];
+    __shared__ int s_idx[2][NC];
+    __shared__ double s_prow[2][NB], s_krow[2][NB];   // the scaled pivot row, and row k0 + p
+    __shared__ int s_piv[NB];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, rank = (int)cluster.block_rank();
+    const int per = (n + kPanelBlocks - 1) / kPanelBlocks;
+    const int rend = min(n, (rank + 1) * per);
+    const int r0 = rank * per + t;   // this thread's rows: r0 + i kPanelThreads, below rend
+    double a[RPT][NB];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        const int r = r0 + i * kPanelThreads;
+#pragma unroll
+        for (int q = 0; q < NB; ++q) a[i][q] = (r < rend && q < nb) ? W[(size_t)r * n + k0 + q] : 0.0;
     }
-    best[t] = bv;
-    bidx[t] = bi;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (t < s) {
-            if (best[t + s] > best[t] || (best[t + s] == best[t] && bidx[t + s] < bidx[t])) {
-                best[t] = best[t + s];
-                bidx[t] = bidx[t + s];
+    cluster.sync();   // every block runs before another writes to its shared memory
+#pragma unroll
+    for (int p = 0; p < NB; ++p) {
+        if (p < nb) {
+            const int buf = p & 1;
+            double bv = -1.0;
+            int bi = k0 + p;
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const int r = r0 + i * kPanelThreads;
+                const double v = fabs(a[i][p]);
+                if (r >= k0 + p && r < rend && v > bv) {
+                    bv = v;
+                    bi = r;
+                }
+            }
+            auto best = [&](int o) {
+                const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (ov > bv || (ov == bv && oi < bi)) {
+                    bv = ov;
+                    bi = oi;
+                }
+            };
+            for (int o = 16; o > 0; o >>= 1) best(o);
+            if (lane < kPanelBlocks) {
+                *cluster.map_shared_rank(&s_best[buf][rank * NW + wid], lane) = bv;
+                *cluster.map_shared_rank(&s_idx[buf][rank * NW + wid], lane) = bi;
+            }
+            cluster.sync();
+            bv = s_best[buf][lane];
+            bi = s_idx[buf][lane];
+#pragma unroll
+            for (int e = 32; e < NC; e += 32) {
+                const double ov = s_best[buf][e + lane];
+                const int oi = s_idx[buf][e + lane];
+                if (ov > bv || (ov == bv && oi < bi)) {
+                    bv = ov;
+                    bi = oi;
+                }
+            }
+            for (int o = 16; o > 0; o >>= 1) best(o);
+            const int pr = bi;   // the same in every thread of the cluster
+            const bool found = bv > 1e-300;
+            if (!found) {   // every thread alike: no block is left waiting
+                if (rank == 0 && t == 0) *flag = 1;
+                return;
+            }
+            if (t == 0) s_piv[p] = pr;
+            // the warps that hold the pivot row and row k0 + p send them to every block
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const int w0 = rank * per + i * kPanelThreads + 32 * wid;   // this warp's rows: w0 .. w0 + 31, below rend
+                const int wend = min(rend, w0 + 32);
+                if (pr >= w0 && pr < wend) {
+                    const double inv = 1.0 / __shfl_sync(0xffffffffu, a[i][p], pr - w0);
+#pragma unroll
+                    for (int q = 0; q < NB; ++q) {
+                        const double v = __shfl_sync(0xffffffffu, a[i][q], pr - w0);
+                        if (lane < kPanelBlocks) *cluster.map_shared_rank(&s_prow[buf][q], lane) = q == p ? inv : v * inv;
+                    }
+                }
+                if (k0 + p >= w0 && k0 + p < wend) {
+#pragma unroll
+                    for (int q = 0; q < NB; ++q) {
+                        const double v = __shfl_sync(0xffffffffu, a[i][q], k0 + p - w0);
+                        if (lane < kPanelBlocks) *cluster.map_shared_rank(&s_krow[buf][q], lane) = v;
+                    }
+                }
+            }
+            cluster.sync();
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                const int r = r0 + i * kPanelThreads;
+                if (r == k0 + p && r < rend) {
+#pragma unroll
+                    for (int q = 0; q < NB; ++q) a[i][q] = s_prow[buf][q];
+                } else if (r < rend) {
+                    if (r == pr) {
+#pragma unroll
+                        for (int q = 0; q < NB; ++q) a[i][q] = s_krow[buf][q];
+                    }
+                    const double f = -a[i][p];
+                    a[i][p] = 0.0;
+#pragma unroll
+                    for (int q = 0; q < NB; ++q) a[i][q] = fma(f, s_prow[buf][q], a[i][q]);
+                }
             }
         }
-        __syncthreads();
     }
-    const int piv = bidx[0];
-    if (!(best[0] > 1e-300)) {
-        if (t == 0) *flag = 1;
-        return;
-    }
-    if (piv != k) {
-        for (int j = t; j < n2; j += blockDim.x) {
-            const double a = W[(long long)k * n2 + j];
-            W[(long long)k * n2 + j] = W[(long long)piv * n2 + j];
-            W[(long long)piv * n2 + j] = a;
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        const int r = r0 + i * kPanelThreads;
+        if (r < rend) {
+#pragma unroll
+            for (int q = 0; q < NB; ++q)
+                if (q < nb) {
+                    W[(size_t)r * n + k0 + q] = a[i][q];
+                    Mt[(size_t)q * n + r] = a[i][q];
+                }
         }
     }
     __syncthreads();
-    const double inv = 1.0 / W[(long long)k * n2 + k];
-    __syncthreads();
-    for (int j = t; j < n2; j += blockDim.x) W[(long long)k * n2 + j] *= inv;
-    __syncthreads();
-    for (int i = t; i < n; i += blockDim.x) fac[i] = (i == k) ? 0.0 : W[(long long)i * n2 + k];
-}
-
-__global__ void k_gj_eliminate(double* __restrict__ W, int n, int k, const double* __restrict__ fac,
-                               const int* __restrict__ flag) {
-    if (*flag) return;
-    const int n2 = 2 * n;
-    const int i = blockIdx.y;
-    const double f = fac[i];
-    if (f == 0.0) return;
-    for (int j = k + blockIdx.x * blockDim.x + threadIdx.x; j < n2; j += gridDim.x * blockDim.x)
-        W[(long long)i * n2 + j] -= f * W[(long long)k * n2 + j];
-}
-
-__global__ void k_gj_init(const double* __restrict__ M, double* __restrict__ W, int n) {
-    const long long tot = 2ll * n * n;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(t / (2 * n)), j = (int)(t % (2 * n));
-        W[t] = j < n ? M[(long long)i * n + j] : (j - n == i ? 1.0 : 0.0);
+    if (rank == 0 && t < nb) piv[k0 + t] = s_piv[t];
+    if (rank == 0 && t < 2 * nb) {
+        // the row a destination's content comes from: follow the swaps backwards
+        const int d = t < nb ? k0 + t : s_piv[t - nb];
+        int from = d;
+        for (int p = nb - 1; p >= 0; --p) {
+            if (from == k0 + p) from = s_piv[p];
+            else if (from == s_piv[p]) from = k0 + p;
+        }
+        swaps[t] = d;
+        swaps[2 * NB + t] = from;
     }
 }
-__global__ void k_gj_extract(const double* __restrict__ W, double* __restrict__ M, int n) {
-    const long long tot = (long long)n * n;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(t / n), j = (int)(t % n);
-        M[t] = W[(long long)i * 2 * n + n + j];
+
+// Carry the panel's row swaps to the other columns (one thread each) and copy
+// their rows k0 .. k0 + nb - 1 to B[p n + j].
+__global__ void k_gj_swap(double* __restrict__ W, int n, int k0, int nb, const int* __restrict__ swaps,
+                          double* __restrict__ B, const int* __restrict__ flag) {
+    constexpr int NB = kPanel;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (*flag || j >= n || (j >= k0 && j < k0 + nb)) return;
+    double v[2 * NB];
+#pragma unroll
+    for (int e = 0; e < 2 * NB; ++e)
+        if (e < 2 * nb) v[e] = W[(size_t)swaps[2 * NB + e] * n + j];
+#pragma unroll
+    for (int e = 0; e < 2 * NB; ++e)
+        if (e < 2 * nb) W[(size_t)swaps[e] * n + j] = v[e];
+#pragma unroll
+    for (int e = 0; e < NB; ++e)
+        if (e < nb) B[(size_t)e * n + j] = v[e];
+}
+
+// W(i, j) <- (0 in the panel's rows, else W(i, j)) + sum_p M(i, p) B(p, j) off
+// the panel's columns; 64 x 64 tiles, 4 x 4 per thread
+__global__ void __launch_bounds__(256) k_gj_update(double* __restrict__ W, int n, int k0, int nb,
+                                                   const double* __restrict__ Mt, const double* __restrict__ B,
+                                                   const int* __restrict__ flag) {
+    constexpr int NB = kPanel;
+    if (*flag) return;
+    __shared__ double sm[NB][64], sb[NB][64];
+    const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    for (int e = t; e < NB * 64; e += 256) {
+        const int p = e >> 6, c = e & 63;
+        sm[p][c] = (p < nb && i0 + c < n) ? Mt[(size_t)p * n + i0 + c] : 0.0;
+        sb[p][c] = (p < nb && j0 + c < n) ? B[(size_t)p * n + j0 + c] : 0.0;
+    }
+    double acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
+            acc[a][b] = (i < n && j < n && !(i >= k0 && i < k0 + nb)) ? W[(size_t)i * n + j] : 0.0;
+        }
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < NB; ++p) {
+        double m[4], v[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            m[a] = sm[p][ty + 16 * a];
+            v[a] = sb[p][tx + 16 * a];
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[a][b] = fma(m[a], v[b], acc[a][b]);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
+            if (i < n && j < n && !(j >= k0 && j < k0 + nb)) W[(size_t)i * n + j] = acc[a][b];
+        }
+}
+
+// The row swaps of the elimination are column swaps of the inverse, in reverse
+// order: src[d] = the column of W that belongs in column d.
+__global__ void k_gj_columns(int n, const int* __restrict__ piv, int* __restrict__ src) {
+    __shared__ int sp[1024];
+    const int d = blockIdx.x * blockDim.x + threadIdx.x;
+    int from = d;
+    for (int k0 = 0; k0 < n; k0 += 1024) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < 1024; e += blockDim.x) sp[e] = k0 + e < n ? piv[k0 + e] : k0 + e;
+        __syncthreads();
+        const int m = min(1024, n - k0);
+        for (int e = 0; e < m; ++e) {
+            const int k = k0 + e, q = sp[e];
+            from = from == k ? q : (from == q ? k : from);
+        }
+    }
+    if (d < n) src[d] = from;
+}
+__global__ void k_gj_gather(const double* __restrict__ W, double* __restrict__ M, int n, const int* __restrict__ src) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n) M[(size_t)blockIdx.y * n + j] = W[(size_t)blockIdx.y * n + src[j]];
+}
+
+template <int RPT>
+void gj_eliminate(double* W, int n, int* piv, double* Mt, double* B, int* swaps, int* d_flag, cudaStream_t s) {
+    const int nt = (n + 63) / 64;
+    for (int k0 = 0; k0 < n; k0 += kPanel) {
+        const int nb = std::min(kPanel, n - k0);
+        launch("k_gj_panel", k_gj_panel<RPT>, kPanelBlocks, kPanelThreads, 0, s, W, n, k0, nb, piv, Mt, swaps, d_flag);
+        launch("k_gj_swap", k_gj_swap, (n + 63) / 64, 64, 0, s, W, n, k0, nb, (const int*)swaps, B, (const int*)d_flag);
+        launch("k_gj_update", k_gj_update, dim3(nt, nt), 256, 0, s, W, n, k0, nb, (const double*)Mt, (const double*)B,
+               (const int*)d_flag);
     }
 }
 
@@ -175,21 +368,28 @@ __global__ void k_components(Grid3 g, const double* __restrict__ A, const int* _
 
 }  // namespace
 
+size_t dense_inverse_work(int n) { return (size_t)n * n + (2 * kPanel + 1) * (size_t)n + 2 * kPanel; }
+
 bool dense_inverse(double* M, int n, double* work, int* d_flag, cudaStream_t s) {
     double* W = work;
-    double* fac = work + 2ll * n * n;
+    double* Mt = W + (size_t)n * n;
+    double* B = Mt + kPanel * (size_t)n;
+    int* piv = reinterpret_cast<int*>(B + kPanel * (size_t)n);
+    int* src = piv + n;
+    int* swaps = src + n;   // 4 kPanel entries
     DM_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
-    launch("k_gj_init", k_gj_init, 256, 256, 0, s, M, W, n);
-    const int bx = std::max(1, std::min(8, (2 * n + 255) / 256));
-    for (int k = 0; k < n; ++k) {
-        launch("k_gj_pivot", k_gj_pivot, 1, 1024, 0, s, W, n, k, fac, d_flag);
-        launch("k_gj_eliminate", k_gj_eliminate, dim3(bx, n), 256, 0, s, W, n, k, fac, d_flag);
-    }
-    launch("k_gj_extract", k_gj_extract, 256, 256, 0, s, W, M, n);
+    DM_CUDA(cudaMemcpyAsync(W, M, sizeof(double) * (size_t)n * n, cudaMemcpyDeviceToDevice, s));
+    constexpr int rows = kPanelBlocks * kPanelThreads;   // of one row per thread
+    if (n <= rows) gj_eliminate<1>(W, n, piv, Mt, B, swaps, d_flag, s);
+    else if (n <= 2 * rows) gj_eliminate<2>(W, n, piv, Mt, B, swaps, d_flag, s);
+    else gj_eliminate<3>(W, n, piv, Mt, B, swaps, d_flag, s);
     int h = 0;
     DM_CUDA(cudaMemcpyAsync(&h, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
-    return h == 0;
+    if (h) return false;   // the pivots after the failing one were never written
+    launch("k_gj_columns", k_gj_columns, (n + 127) / 128, 128, 0, s, n, (const int*)piv, src);
+    launch("k_gj_gather", k_gj_gather, dim3((n + 127) / 128, n), 128, 0, s, (const double*)W, M, n, (const int*)src);
+    return true;
 }
 
 template <typename T>
