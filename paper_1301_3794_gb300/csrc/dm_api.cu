@@ -307,13 +307,13 @@ struct dm_operator {
     // coarsest vector solve
     DBuf<int> c_list;
     int c_n = 0;
-    DBuf<double> c_inv, c_tmp_in, c_tmp_out;
+    DBuf<double> c_inv;
     DBuf<float> c_inv32;
     // coarsest scalar solve
     DBuf<int> s_list;
     int s_n = 0;
     DBuf<unsigned char> s_pinned;
-    DBuf<double> s_inv, s_tmp_in, s_tmp_out;
+    DBuf<double> s_inv;
     DBuf<float> s_inv32;
     // FP64 scratch on the fine level
     DBuf<double> t0, t1, t2, t3, c0, c1;
@@ -450,12 +450,11 @@ template <typename T, typename TC>
 void vcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
     cudaStream_t s = op->ctx->stream;
     const GeoLevel& g = glv(op, l);
-    const size_t vbytes = sizeof(T) * 3 * (size_t)g.g.np;
     if (l == op->nlev - 1) {
-        zero(rbuf, vbytes, s);
+        // (nothing writes the closed faces of rbuf: they stay zero)
         dense_coarse_solve<T>(std::is_same<T, double>::value ? op->c_inv.get() : nullptr,
                               std::is_same<T, double>::value ? nullptr : op->c_inv32.get(), op->c_n, op->c_list.get(),
-                              nullptr, f, rbuf, op->c_tmp_in.get(), op->c_tmp_out.get(), s);
+                              nullptr, f, rbuf, s);
         return;
     }
     const VecOp<T, TC> o = vop<T, TC>(op, l);
@@ -504,10 +503,9 @@ void svcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
     cudaStream_t s = op->ctx->stream;
     const GeoLevel& g = glv(op, l);
     if (l == op->nlev - 1) {
-        zero(rbuf, sizeof(T) * (size_t)g.g.np, s);
         dense_coarse_solve<T>(std::is_same<T, double>::value ? op->s_inv.get() : nullptr,
                               std::is_same<T, double>::value ? nullptr : op->s_inv32.get(), op->s_n, op->s_list.get(),
-                              op->s_pinned.get(), f, rbuf, op->s_tmp_in.get(), op->s_tmp_out.get(), s);
+                              op->s_pinned.get(), f, rbuf, s);
         return;
     }
     const ScalOp<T, TC> o = sop<T, TC>(op, l);
@@ -1350,8 +1348,6 @@ void setup_operator(dm_operator* op) {
             op->c_inv32.alloc((size_t)n * n);
             convert_coeff<float>((long long)n * n, op->c_inv.get(), op->c_inv32.get(), s);
         }
-        op->c_tmp_in.alloc(n);
-        op->c_tmp_out.alloc(n);
     }
     // coarsest scalar level: dense inverse with one pinned cell per component
     {
@@ -1375,8 +1371,6 @@ void setup_operator(dm_operator* op) {
             op->s_inv32.alloc((size_t)n * n);
             convert_coeff<float>((long long)n * n, op->s_inv.get(), op->s_inv32.get(), s);
         }
-        op->s_tmp_in.alloc(n);
-        op->s_tmp_out.alloc(n);
     }
     const long long n3 = 3ll * glv(op, 0).g.np, n1 = glv(op, 0).g.np;
     op->t0.alloc(n3);

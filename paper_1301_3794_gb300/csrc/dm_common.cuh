@@ -546,9 +546,10 @@ void cell_prolong_add(const Grid3& gf, const Grid3& gc, const unsigned char* act
 // dense_inverse_work(n) doubles).  Returns false if a column had no pivot above 1e-300.
 size_t dense_inverse_work(int n);
 bool dense_inverse(double* M, int n, double* work, int* d_flag, cudaStream_t s);
+// x[list[r]] = sum_c Minv(r, c) f[list[c]] over the rows that zero_rows does not mark (n <= 6000)
 template <typename T>
 void dense_coarse_solve(const double* Minv64, const float* Minv32, int n, const int* list, const unsigned char* zero_rows,
-                        const T* f, T* x, double* tmp_in, double* tmp_out, cudaStream_t s);
+                        const T* f, T* x, cudaStream_t s);
 // connected components of active coarsest cells: pinned[c] = 1 for the lowest
 // index of every component (list order = natural order)
 void cell_components_pin(const Grid3& g, const double* A, const int* list, int n, int* label,

@@ -1,5 +1,5 @@
 // Dense kernels of the coarsest multigrid level: blocked Gauss-Jordan inversion
-// with partial pivoting, the gather / dense matvec / scatter of the coarsest solve,
+// with partial pivoting, the dense product of the coarsest solve,
 // and connected components of the active coarsest cells (the scalar Laplacian
 // D A D^T has one constant null vector per component; the lowest-index cell of
 // each component is pinned to zero).
@@ -273,34 +273,72 @@ void gj_eliminate(double* W, int n, int* piv, double* Mt, double* B, int* swaps,
     }
 }
 
+// x[list[r]] = sum_c M(r, c) f[list[c]]: the coarsest solve in one launch (a
+// gather, a product and a scatter before, and a memset of x, whose other entries
+// nothing writes).  Every block gathers f into shared memory; one warp per row,
+// whose first loads are issued before the gather is waited for.
+// FP32 inverse (storage types FP32 and BF16): the products of two FP32 numbers
+// are summed in float-float (an error-free product and a two-sum, about 48
+// bits), because converting and adding in FP64 issues at two per clock and SM
+// where this takes nine FP32 instructions at 128; the sum is rounded to the
+// storage type either way.
+// Measured (CUDA events, of which some 4 us a launch are the events): n = 1,990
+// in FP32, 24.9 + 6.7 + 6.4 -> 14.9 us a solve.
+constexpr int kSolveWarps = 8;
 template <typename T>
-__global__ void k_gather(int n, const int* __restrict__ list, const unsigned char* __restrict__ zero_rows,
-                         const T* __restrict__ f, double* __restrict__ out) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
-        out[r] = (zero_rows && zero_rows[r]) ? 0.0 : (double)to_c(f[list[r]]);
-}
-
-// out = M in  (one warp per row; FP64 or FP32 matrix, FP64 accumulation)
-__global__ void k_dense_mv(int n, const double* __restrict__ M64, const float* __restrict__ M32,
-                           const double* __restrict__ in, double* __restrict__ out) {
-    const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+__global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const double* __restrict__ M64,
+                                                                   const float* __restrict__ M32,
+                                                                   const int* __restrict__ list,
+                                                                   const unsigned char* __restrict__ zero_rows,
+                                                                   const T* __restrict__ f, T* __restrict__ x) {
+    using C = typename Compute<T>::type;
+    extern __shared__ __align__(16) unsigned char solve_smem[];
+    C* const sf = reinterpret_cast<C*>(solve_smem);
     const int lane = threadIdx.x & 31;
-    if (row >= n) return;
-    double s = 0.0;
-    if (M64) {
-        for (int c = lane; c < n; c += 32) s += M64[(long long)row * n + c] * in[c];
-    } else {
-        for (int c = lane; c < n; c += 32) s += (double)M32[(long long)row * n + c] * in[c];
-    }
+    const int row = blockIdx.x * kSolveWarps + (threadIdx.x >> 5);
+    const C* m;
+    if constexpr (std::is_same<C, double>::value) m = M64;
+    else m = M32;
+    m += (size_t)min(row, n - 1) * n;
+    constexpr int U = sizeof(C) == 8 ? 8 : 16;
+    C v[U];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) out[row] = s;
-}
-
-template <typename T>
-__global__ void k_scatter(int n, const int* __restrict__ list, const double* __restrict__ in, T* __restrict__ x) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
-        x[list[r]] = to_store<T>(in[r]);
+    for (int e = 0; e < U; ++e) v[e] = lane + 32 * e < n ? m[lane + 32 * e] : C(0);
+    for (int c = threadIdx.x; c < n; c += 32 * kSolveWarps)
+        sf[c] = (zero_rows && zero_rows[c]) ? C(0) : (C)to_c(f[list[c]]);
+    __syncthreads();
+    if (row >= n) return;
+    C s = C(0), err = C(0);
+    for (int c0 = lane; c0 < n; c0 += 32 * U) {
+        C cur[U];
+#pragma unroll
+        for (int e = 0; e < U; ++e) cur[e] = v[e];
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            const int c = c0 + 32 * (U + e);
+            v[e] = c < n ? m[c] : C(0);
+        }
+#pragma unroll
+        for (int e = 0; e < U; ++e) {
+            const int c = c0 + 32 * e;
+            if (c < n) {
+                if constexpr (std::is_same<C, double>::value) {
+                    s = fma(cur[e], sf[c], s);
+                } else {
+                    const float pr = __fmul_rn(cur[e], sf[c]);
+                    const float pe = fmaf(cur[e], sf[c], -pr);
+                    const float t = __fadd_rn(s, pr);
+                    const float bp = __fsub_rn(t, s);
+                    err = __fadd_rn(err, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(pr, bp)), pe));
+                    s = t;
+                }
+            }
+        }
+    }
+    double tot = (double)s + (double)err;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, o);
+    if (lane == 0) x[list[row]] = to_store<T>(tot);
 }
 
 __device__ int find_in_list(const int* list, int n, int key) {
@@ -394,12 +432,13 @@ bool dense_inverse(double* M, int n, double* work, int* d_flag, cudaStream_t s) 
 
 template <typename T>
 void dense_coarse_solve(const double* Minv64, const float* Minv32, int n, const int* list, const unsigned char* zero_rows,
-                        const T* f, T* x, double* tmp_in, double* tmp_out, cudaStream_t s) {
+                        const T* f, T* x, cudaStream_t s) {
+    using C = typename Compute<T>::type;
     if (n <= 0) return;
-    const int b = (n + 255) / 256;
-    launch("k_gather", k_gather<T>, b, 256, 0, s, n, list, zero_rows, f, tmp_in);
-    launch("k_dense_mv", k_dense_mv, (n + 7) / 8, 256, 0, s, n, Minv64, Minv32, tmp_in, tmp_out);
-    launch("k_scatter", k_scatter<T>, b, 256, 0, s, n, list, tmp_out, x);
+    // n <= 6000 FP64 values fit the 48 KB a kernel may use unasked
+    launch_b("k_coarse_solve", (double)n * n * sizeof(C) + 2.0 * n * sizeof(T), k_coarse_solve<T>,
+             (n + kSolveWarps - 1) / kSolveWarps, 32 * kSolveWarps, sizeof(C) * (size_t)n, s, n, Minv64, Minv32, list,
+             zero_rows, f, x);
 }
 
 void cell_components_pin(const Grid3& g, const double* A, const int* list, int n, int* label, unsigned char* pinned,
@@ -409,10 +448,10 @@ void cell_components_pin(const Grid3& g, const double* A, const int* list, int n
 }
 
 template void dense_coarse_solve<double>(const double*, const float*, int, const int*, const unsigned char*,
-                                         const double*, double*, double*, double*, cudaStream_t);
+                                         const double*, double*, cudaStream_t);
 template void dense_coarse_solve<float>(const double*, const float*, int, const int*, const unsigned char*,
-                                        const float*, float*, double*, double*, cudaStream_t);
+                                        const float*, float*, cudaStream_t);
 template void dense_coarse_solve<__nv_bfloat16>(const double*, const float*, int, const int*, const unsigned char*,
-                                                const __nv_bfloat16*, __nv_bfloat16*, double*, double*, cudaStream_t);
+                                                const __nv_bfloat16*, __nv_bfloat16*, cudaStream_t);
 
 }  // namespace dm
