@@ -270,14 +270,15 @@ dm_status dm_operator_apply_ff(dm_operator* op, const double* x, double* y, int 
  *  - x, y: device pointers, natural face layout of `level`.
  *  - Scratch: a static device array of 6,291,456 doubles (48 MiB) inside the
  *    library, held by every GPU that loads the library until the process exits.
- *    A call needs 6 * np doubles (np = padded node count of the level: about
+ *    A call may need 6 * np doubles (np = padded node count of the level: about
  *    1.0 M nodes, i.e. grids up to roughly 100^3); larger levels are rejected
- *    with DM_ERR_INVALID_ARG and an explanatory dm_last_error().
+ *    with DM_ERR_INVALID_ARG and an explanatory dm_last_error().  It is used
+ *    when x and y share memory (x is then copied there first).
  *  - The first call on each device looks up the scratch's device address
  *    (cudaGetSymbolAddress) with that device current.
- *  - Every call shares the one scratch array: calls that overlap on the GPU
- *    (other threads, other contexts or streams) race and corrupt each other's
- *    results; serialise them. */
+ *  - Every call may use the one scratch array: calls that overlap on the GPU
+ *    (other threads, other contexts or streams) can race and corrupt each
+ *    other's results; serialise them. */
 dm_status dm_operator_apply_noalloc(dm_operator* op, int level, const double* x, double* y);
 /* Diagonal of K - sigma A on `level` (natural face layout, 0 on closed faces). */
 dm_status dm_operator_diagonal(dm_operator* op, int level, double* d, int on_device);

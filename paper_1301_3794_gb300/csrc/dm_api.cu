@@ -1398,6 +1398,9 @@ void stage_out(dm_context* ctx, const double* dev, double* dst, int on_device, s
     DM_CUDA(cudaStreamSynchronize(ctx->stream));
 }
 
+// whether two arrays of n doubles share memory
+bool overlap(const double* a, const double* b, size_t n) { return a < b + n && b < a + n; }
+
 __global__ void k_mask_open(long long n, const double* __restrict__ A, double* __restrict__ x) {
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x)
         if (!(A[r] > 0.0)) x[r] = 0.0;
@@ -1836,11 +1839,22 @@ dm_status dm_operator_set_omega(dm_operator* op, int level, int scalar, double o
 dm_status dm_operator_apply(dm_operator* op, int level, const double* x, double* y, int on_device) {
     if (!op || !x || !y || level < 0 || level >= op->nlev) return DM_ERR_INVALID_ARG;
     return guarded(op->ctx, [&] {
-        const Grid3& g = glv(op, level).g;
-        DBuf<double> xp(3ll * g.np), yp(3ll * g.np);
-        faces_in(op, level, x, on_device, xp.get());
-        apply_vec64(op, level, xp.get(), yp.get());
-        faces_out(op, level, yp.get(), y, on_device);
+        const size_t nf = (size_t)natural_faces(glv(op, level).g);
+        const VecOp<double, double> o = vop<double, double>(op, level);
+        cudaStream_t s = op->ctx->stream;
+        DBuf<double> xt, yt;
+        const double* xd = nullptr;
+        stage_in(op->ctx, x, on_device, nf, xt, &xd);
+        if (on_device && overlap(x, y, nf)) {
+            xt.alloc(nf, false);
+            DM_CUDA(cudaMemcpyAsync(xt.get(), x, sizeof(double) * nf, cudaMemcpyDeviceToDevice, s));
+            xd = xt.get();
+        }
+        if (!on_device) yt.alloc(nf, false);
+        double* yd = on_device ? y : yt.get();
+        vec_apply_natural(o, xd, yd, true, s);
+        if (on_device) Sync::stream(s);
+        else stage_out(op->ctx, yd, y, 0, nf);
     });
 }
 
@@ -2045,32 +2059,45 @@ void dm_eig_params_default(dm_eig_params* p) {
 
 namespace {
 
-// k^2, rho, delta, rq of the eigenvectors in the padded FP64 columns X (ld = 3 np)
-void certify_padded(dm_context* ctx, const GeoLevel& g0, int n, const double* X, double* k2_io, bool set_k2, double* rho,
-                    double* delta, double* rq) {
+// rho, delta, rq of n vectors X, ld apart (padded, or natural), at k2_io; with
+// set_k2, k2_io holds estimates of the Rayleigh quotients and receives them, and
+// rho is taken there.  One pass over each vector: the operator, the products and
+// the norms in one kernel (a launch each and five synchronisations per vector before).
+void certify_columns(dm_context* ctx, const GeoLevel& g0, int n, const double* X, long long ld, bool natural,
+                     double* k2_io, bool set_k2, double* rho, double* delta, double* rq) {
     cudaStream_t s = ctx->stream;
-    const long long n3 = 3ll * g0.g.np;
-    const Domain D = g0.vdom(), Dc = g0.sdom();
-    DBuf<double> kb(n3), ab(n3), dv(g0.g.np);
-    const VecOp<double, double> o{g0.g, g0.A.get(), g0.L.get(), g0.invV.get(), nullptr, 0.0, 0};
     const double h = std::min(g0.g.hx, std::min(g0.g.hy, g0.g.hz));
+    int sy, sz;
+    constexpr int shape = 3;   // 32x8x8
+    stencil_shape_dims(shape, sy, sz);
+    const int nt = ((g0.g.nx + TX) / TX) * ((g0.g.ny + sy) / sy) * ((g0.g.nz + sz) / sz);
+    DBuf<int> tl(nt, false), flags(nt, false), cnt(1);
+    const int ntiles = geom_tiles_shape(g0.g, sy, sz, g0.A.get(), g0.active.get(), tl.get(), flags.get(), cnt.get(), s);
+    std::vector<double> sums((size_t)n * kCertSums, 0.0);
+    if (ntiles > 0) {
+        VecOp<double, double> o{g0.g, g0.A.get(), g0.L.get(), g0.invV.get(), nullptr, 0.0, 0};
+        o.stiles = tl.get();
+        o.nstiles = ntiles;
+        o.shape = shape;
+        DBuf<double> part((size_t)n * ntiles * kCertSums, false), out((size_t)n * kCertSums, false), kd(n, false);
+        DM_CUDA(cudaMemcpyAsync(kd.get(), k2_io, sizeof(double) * n, cudaMemcpyHostToDevice, s));
+        vec_cert_sums(o, natural, n, X, ld, kd.get(), part.get(), out.get(), s);
+        DM_CUDA(cudaMemcpyAsync(sums.data(), out.get(), sizeof(double) * sums.size(), cudaMemcpyDeviceToHost, s));
+        Sync::stream(s);
+    }
     for (int i = 0; i < n; ++i) {
-        const double* b = X + (size_t)i * n3;
-        vec_stencil<double, double>(o, ST_APPLY, b, nullptr, kb.get(), 0.0, s);
-        hadamard(D, g0.A.get(), b, ab.get(), s);
-        // K b and A b vanish on closed faces, so the sums run over the open ones
-        const double bkb = face_dot(ctx, g0, b, kb.get()), bab = face_dot(ctx, g0, b, ab.get());
-        const double r = bkb / bab;
+        const double* q = &sums[(size_t)i * kCertSums];
+        const double r = q[0] / q[1], abn = std::sqrt(std::max(q[2], 0.0));
+        double rn2 = q[3];
         if (rq) rq[i] = r;
-        const double k2 = set_k2 ? r : k2_io[i];
-        if (set_k2) k2_io[i] = r;
-        const double abn = face_norm(ctx, g0, ab.get());
-        axpby(D, -k2, ab.get(), 1.0, kb.get(), s);
-        const double rn = face_norm(ctx, g0, kb.get());
-        if (rho) rho[i] = rn / (std::fabs(k2) * abn);
-        dm_div_a(g0.g, g0.A.get(), b, dv.get(), g0.tiles.get(), g0.ntiles, s);
-        const double dn = norm2(ctx, Dc, dv.get());
-        if (delta) delta[i] = dn * h / abn;
+        if (set_k2) {
+            // |K b - r A b|^2 from the residual at the nearby estimate: every term is of the residual's own size
+            const double d = r - k2_io[i];
+            rn2 += d * (d * q[2] - 2.0 * q[4]);
+            k2_io[i] = r;
+        }
+        if (rho) rho[i] = std::sqrt(std::max(rn2, 0.0)) / (std::fabs(k2_io[i]) * abn);
+        if (delta) delta[i] = std::sqrt(std::max(q[5], 0.0)) * h / abn;
     }
 }
 
@@ -2222,6 +2249,8 @@ dm_status dm_eigensolve(dm_context* ctx, const dm_geometry* geom, const dm_eig_p
         // certificate rho (the residual of K b = k^2 A b itself) misses rho_tol
         double tol_eff = p.tol, inner_eff = p.inner_tol;
         int cert_retries = 0;
+        // k^2 of the c-th Ritz pair by |theta|
+        auto ritz_k2 = [&](int c) { return theta[order[c]] != 0.0 ? p.sigma + 1.0 / theta[order[c]] : p.sigma; };
         // rho of the wanted Ritz pairs (|theta| order) from the current basis
         auto certify_wanted = [&](std::vector<double>& rho_out) {
             std::vector<double> Yw((size_t)m * p.nev), kk(p.nev);
@@ -2231,7 +2260,8 @@ dm_status dm_eigensolve(dm_context* ctx, const dm_geometry* geom, const dm_eig_p
             DM_CUDA(cudaMemcpyAsync(Yd.get(), Yw.data(), sizeof(double) * m * p.nev, cudaMemcpyHostToDevice, s));
             vgemm(D, m, p.nev, V, n, Yd.get(), m, tmp.get(), n, s);
             rho_out.assign(p.nev, 0.0);
-            certify_padded(ctx, g0, p.nev, tmp.get(), kk.data(), true, rho_out.data(), nullptr, nullptr);
+            for (int c = 0; c < p.nev; ++c) kk[c] = ritz_k2(c);
+            certify_columns(ctx, g0, p.nev, tmp.get(), n, false, kk.data(), true, rho_out.data(), nullptr, nullptr);
         };
         while (true) {
             for (int j = k; j < m; ++j) {
@@ -2389,7 +2419,8 @@ dm_status dm_eigensolve(dm_context* ctx, const dm_geometry* geom, const dm_eig_p
                    (const long long*)pi.get(), (const double*)b, sign.get());
             launch("k_sign_fix", k_sign_fix, (int)std::min<long long>((n + 255) / 256, 1216), 256, 0, s, n, b, sign.get());
         }
-        certify_padded(ctx, g0, nev, tmp.get(), k2.data(), true, rho.data(), delta.data(), rq.data());
+        for (int c = 0; c < nev; ++c) k2[c] = ritz_k2(c);
+        certify_columns(ctx, g0, nev, tmp.get(), n, false, k2.data(), true, rho.data(), delta.data(), rq.data());
         if (p.rho_tol > 0.0) {
             // the converged prefix (|theta| order) also needs its certificate
             int nc = 0;
@@ -2459,8 +2490,8 @@ dm_status dm_eigensolve(dm_context* ctx, const dm_geometry* geom, const dm_eig_p
 
 namespace {
 
-// Scratch of dm_operator_apply_noalloc: the padded input and output vectors of
-// one call.  It lives in the library's own device image, so every GPU that
+// Scratch of dm_operator_apply_noalloc: a copy of the input when input and output
+// share memory.  It lives in the library's own device image, so every GPU that
 // loads the library holds it until the process exits.
 constexpr long long kNoAllocDoubles = 6ll * 1024 * 1024;   // 48 MiB
 __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
@@ -2501,16 +2532,13 @@ dm_status dm_operator_apply_noalloc(dm_operator* op, int level, const double* x,
                                                 std::to_string(2 * n3) + " doubles of scratch; the static scratch holds " +
                                                 std::to_string(kNoAllocDoubles) + " (use dm_operator_apply)");
         cudaStream_t s = op->ctx->stream;
-        double* xp = noalloc_scratch(op->ctx->device);
-        double* yp = xp + n3;
-        // the scratch keeps the previous call's contents: the padded input must
-        // start at zero (ghost and non-face entries are read by the stencil)
-        DM_CUDA(cudaMemsetAsync(xp, 0, sizeof(double) * (size_t)n3, s));
-        pack_faces(g.g, x, xp, s);
-        launch("k_mask_open", k_mask_open, (int)std::min<long long>((n3 + 255) / 256, 1216), 256, 0, s, n3, g.A.get(),
-               xp);
-        vec_apply_dense_f64(g.g, g.A.get(), g.L.get(), g.invV.get(), op->sigma, xp, yp, s);
-        unpack_faces(g.g, yp, y, s);
+        const size_t nf = (size_t)natural_faces(g.g);
+        if (overlap(x, y, nf)) {   // the kernel's blocks read their neighbours' x: take it from a copy
+            double* xs = noalloc_scratch(op->ctx->device);
+            DM_CUDA(cudaMemcpyAsync(xs, x, sizeof(double) * nf, cudaMemcpyDeviceToDevice, s));
+            x = xs;
+        }
+        vec_apply_natural(vop<double, double>(op, level), x, y, false, s);
         DM_CUDA(cudaStreamSynchronize(s));
     });
 }
@@ -2861,19 +2889,12 @@ dm_status dm_certify(dm_context* ctx, const dm_geometry* geom, int n, const doub
     if (!ctx || !geom || !b || !k2 || n < 1) return DM_ERR_INVALID_ARG;
     return guarded(ctx, [&] {
         const GeoLevel& g0 = *geom->lv[0];
-        cudaStream_t s = ctx->stream;
-        const long long n3 = 3ll * g0.g.np;
         const size_t nf = (size_t)natural_faces(g0.g);
-        DBuf<double> X((size_t)n * n3);
-        for (int i = 0; i < n; ++i) {
-            DBuf<double> tmpb;
-            const double* d = nullptr;
-            stage_in(ctx, b + i * nf, on_device, nf, tmpb, &d);
-            pack_faces(g0.g, d, X.get() + (size_t)i * n3, s);
-            Sync::stream(s);
-        }
+        DBuf<double> tmp;
+        const double* X = nullptr;
+        stage_in(ctx, b, on_device, (size_t)n * nf, tmp, &X);
         std::vector<double> kk(k2, k2 + n);
-        certify_padded(ctx, g0, n, X.get(), kk.data(), false, rho, delta, rq);
+        certify_columns(ctx, g0, n, X, (long long)nf, true, kk.data(), false, rho, delta, rq);
     });
 }
 

@@ -475,8 +475,15 @@ void band_node_vals(const int* node, const int* info, int ncopies, const Grid3& 
 template <typename T, typename TC>
 void band_nodes(const BandNodes<TC>& bn, const Grid3& g, const int* band, int nband, const T* f, T* x, void* u,
                 double omega, int sweeps, bool fine, cudaStream_t s, const Fork* fk = nullptr);
-void vec_apply_dense_f64(const Grid3& g, const double* A, const double* L, const double* invV, double sigma,
-                         const double* x, double* y, cudaStream_t s);
+// y = (K - sigma A) x on vectors in the natural layout, closed faces of x taken
+// as zero (x and y must not overlap; no allocation when !traced)
+void vec_apply_natural(const VecOp<double, double>& op, const double* x, double* y, bool traced, cudaStream_t s);
+// Sums for the certificates of n vectors (natural or padded, `stride` apart):
+// out[v] = [x.Kx, x.Ax, |Ax|^2, |r|^2, r.Ax, |D A x|^2] with r = K x - k2[v] A x.
+// op.stiles: 32x8x8 tiles; k2, part (n * nstiles * kCertSums) and out on the device.
+constexpr int kCertSums = 6;
+void vec_cert_sums(const VecOp<double, double>& op, bool natural, int n, const double* x, long long stride,
+                   const double* k2, double* part, double* out, cudaStream_t s);
 // (K - sigma A) x in float-float into the compact vector out (out[cmap[q]] for
 // the open faces q), over the level's 32 x 4 x 2 active tiles; A, L, invV:
 // float-float copies of the level's coefficients (to_ff)

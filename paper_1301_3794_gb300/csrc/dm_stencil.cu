@@ -102,32 +102,6 @@ __device__ __forceinline__ C cell_psi(const Coef<C, TC>& cf, const Acc& b, int p
     return cf.iv(p) * (fx * rdx + fy * rdy + fz * rdz);
 }
 
-// (K - sigma A) b at the three faces of node p
-template <typename C, typename TC, typename Acc>
-__device__ __forceinline__ void node_K(const Coef<C, TC>& cf, const Acc& b, int p, int X, int Y, int Z, C rdx, C rdy,
-                                       C rdz, C sigma, C out[3]) {
-    const C ex0 = edge_x(cf, b, p, Y, Z, rdy, rdz);
-    const C exZ = edge_x(cf, b, p + Z, Y, Z, rdy, rdz);
-    const C exY = edge_x(cf, b, p + Y, Y, Z, rdy, rdz);
-    const C ey0 = edge_y(cf, b, p, X, Z, rdx, rdz);
-    const C eyZ = edge_y(cf, b, p + Z, X, Z, rdx, rdz);
-    const C eyX = edge_y(cf, b, p + X, X, Z, rdx, rdz);
-    const C ez0 = edge_z(cf, b, p, X, Y, rdx, rdy);
-    const C ezY = edge_z(cf, b, p + Y, X, Y, rdx, rdy);
-    const C ezX = edge_z(cf, b, p + X, X, Y, rdx, rdy);
-    const C ps0 = cell_psi(cf, b, p, X, Y, Z, rdx, rdy, rdz);
-    const C psX = cell_psi(cf, b, p - X, X, Y, Z, rdx, rdy, rdz);
-    const C psY = cell_psi(cf, b, p - Y, X, Y, Z, rdx, rdy, rdz);
-    const C psZ = cell_psi(cf, b, p - Z, X, Y, Z, rdx, rdy, rdz);
-    const C ax = cf.a(0, p), ay = cf.a(1, p), az = cf.a(2, p);
-    const C yx = (ezY - ez0) * rdy - (eyZ - ey0) * rdz + ax * ((psX - ps0) * rdx - sigma * b(0, p));
-    const C yy = (exZ - ex0) * rdz - (ezX - ez0) * rdx + ay * ((psY - ps0) * rdy - sigma * b(1, p));
-    const C yz = (eyX - ey0) * rdx - (exY - ex0) * rdy + az * ((psZ - ps0) * rdz - sigma * b(2, p));
-    out[0] = ax > C(0) ? yx : C(0);
-    out[1] = ay > C(0) ? yy : C(0);
-    out[2] = az > C(0) ? yz : C(0);
-}
-
 // (K - sigma A) b at one face (component c, node p)
 template <typename C, typename TC, typename Acc>
 __device__ __forceinline__ C face_K(const Coef<C, TC>& cf, const Acc& b, int c, int p, int X, int Y, int Z, C rdx,
@@ -153,41 +127,11 @@ __device__ __forceinline__ C face_K(const Coef<C, TC>& cf, const Acc& b, int c, 
     }
 }
 
-template <typename T, typename TC, int MODE>
-__global__ void k_vec_stencil(Grid3 g, const TC* __restrict__ A, const TC* __restrict__ L,
-                              const TC* __restrict__ invV, const TC* __restrict__ invD,
-                              typename Compute<T>::type sigma, const T* __restrict__ x, const T* __restrict__ f,
-                              T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles) {
-    using C = typename Compute<T>::type;
-    int i, j, k;
-    block_node(g, tiles, i, j, k);
-    if (i > g.nx || j > g.ny || k > g.nz) return;
-    const int p = g.idx(i, j, k);
-    const int N = g.np;
-    Coef<C, TC> cf{A, L, invV, N};
-    const auto b = x_acc<T, TC, C, MODE>(x, f, invD, omega, N);
-    C out[3];
-    node_K(cf, b, p, 1, g.sx, g.sxy, inv_h<C>(g, 0), inv_h<C>(g, 1), inv_h<C>(g, 2), sigma, out);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int q = c * N + p;
-        C v = out[c];
-        if (MODE == ST_RESID) {
-            v = (C)to_c(f[q]) - v;
-        } else if (MODE == ST_JACOBI) {
-            v = (C)to_c(x[q]) + omega * (C)invD[q] * ((C)to_c(f[q]) - v);
-        } else if (MODE == ST_JACOBI2Z) {
-            v = b(c, p) + omega * (C)invD[q] * ((C)to_c(f[q]) - v);
-        }
-        y[q] = to_store<T>(v);
-    }
-}
-
-// Tiled form of k_vec_stencil: one active tile of TX x SY x SZ nodes per
+// One-node-per-thread form of the operator: one active tile of TX x SY x SZ nodes per
 // block.  The L-weighted edge curls and cell divergences the tile's faces need
 // are computed once into shared memory (ex, ey, ez on the tile plus one layer
 // above, psi on the tile plus one layer below), then every thread forms its
-// node's three face outputs from them.  Same arithmetic as node_K.  The tile
+// node's three face outputs from them.  Same arithmetic as face_K.  The tile
 // shape (SY, SZ) is chosen per level by the autotuner.
 template <typename T, typename TC, int MODE, int SY, int SZ>
 __global__ void __launch_bounds__(TX * SY * SZ) k_vec_stencil_tiled(
@@ -290,11 +234,28 @@ __global__ void __launch_bounds__(TX * SY * SZ) k_vec_stencil_tiled(
 // latency overlaps that work.  Entries outside [-1, n+1] along x or y are taken
 // as zero; inside that box the padded layout already holds zeros at every
 // position that is not an element of the grid.
-template <typename T, typename TC, int MODE, int SY, int KZ>
+//
+// IN says where x comes from: the padded layout (IN_PADDED), or the caller's
+// natural layout, whole (IN_NATURAL) or with its closed faces taken as zero
+// (IN_OPEN); an apply from the natural layout also writes it.  So a product on
+// a caller's vectors is this one kernel, bound by the FP64 pipe: staging them
+// through padded copies took four more passes, two allocations and two memsets.
+// Measured, a whole call: 128^3 ellipsoid 547 -> 215 us (kernel 203), 32^3
+// sphere 52 -> 29 us; the certificates of 8 vectors on 88 x 72 x 104, 4.1 -> 0.73 ms.
+// MODE ST_CERT forms no vector: each block sums what the certificates of x need
+// (CertSums) and leaves them in ca.part; blockIdx.y counts the vectors.
+enum StencilInput { IN_PADDED = 0, IN_NATURAL = 1, IN_OPEN = 2 };
+constexpr int ST_CERT = kStencilModes;
+struct CertArgs {
+    const double* k2 = nullptr;   // per vector
+    long long stride = 0;         // between the vectors
+    double* part = nullptr;       // [vector][block][kCertSums]
+};
+template <typename T, typename TC, int MODE, int SY, int KZ, int IN = IN_PADDED>
 __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512 : 768) / (TX * SY)) k_vec_stencil_march(
     Grid3 g, const TC* __restrict__ A, const TC* __restrict__ L, const TC* __restrict__ invV,
     const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* __restrict__ x, const T* __restrict__ f,
-    T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles) {
+    T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles, CertArgs ca) {
     using C = typename Compute<T>::type;
     constexpr int RW = TX + 2, RH = SY + 2, RP = RW * RH;   // ring plane: i0-1 .. i0+TX, j0-1 .. j0+SY
     constexpr int NT = TX * SY;
@@ -356,6 +317,26 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
     const int dp0 = dval ? g.idx(di, dj, 0) : 0;
     // ring entry of array a (0..2: b, 3..5: A) at node (ii, jj) of the plane in `slot`
     auto R = [&](int slot, int a, int ii, int jj) -> C { return s_ring[slot][a * RP + (jj - j0 + 1) * RW + (ii - i0 + 1)]; };
+    const C k2 = MODE == ST_CERT ? (C)ca.k2[blockIdx.y] : C(0);
+    if (MODE == ST_CERT) x += blockIdx.y * ca.stride;
+    C sum[kCertSums];
+#pragma unroll
+    for (int e = 0; e < kCertSums; ++e) sum[e] = C(0);
+    // natural layout: index at k = 0 of component c of the node and of the border entry (-1: no such face), and its
+    // plane stride
+    int nown[3], nbor[3], npl[3];
+    if constexpr (IN != IN_PADDED) {
+        int base = 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const int w = g.nx + (c == 0), h = g.ny + (c == 1), d = g.nz + (c == 2);
+            const int bi = i0 - 1 + hli, bj = j0 - 1 + hlj;
+            npl[c] = w * h;
+            nown[c] = i < w && j < h ? base + j * w + i : -1;
+            nbor[c] = hval && bi >= 0 && bj >= 0 && bi < w && bj < h ? base + bj * w + bi : -1;
+            base += npl[c] * d;
+        }
+    }
     const auto xa = x_acc<T, TC, C, MODE>(x, f, invD, omega, N);
     // prefetch registers: ring entries of the node and of the border entry, coefficients, f and 1/D
     C pn[6], ph[6], cv = C(0), cz = C(0), cx = C(0), cy = C(0), hc = C(0), he = C(0), pf[3], pd[3];
@@ -363,10 +344,20 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
         const int pn_ = p0 + k * Z, ph_ = hp0 + k * Z;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            pn[c] = inb ? xa(c, pn_) : C(0);
             pn[3 + c] = inb ? (C)A[c * N + pn_] : C(0);
-            ph[c] = hval ? xa(c, ph_) : C(0);
             ph[3 + c] = hval ? (C)A[c * N + ph_] : C(0);
+            if constexpr (IN == IN_PADDED) {
+                pn[c] = inb ? xa(c, pn_) : C(0);
+                ph[c] = hval ? xa(c, ph_) : C(0);
+            } else {
+                const bool ink = k >= 0 && k < g.nz + (c == 2);
+                pn[c] = ink && nown[c] >= 0 ? (C)to_c(x[nown[c] + k * npl[c]]) : C(0);
+                ph[c] = ink && nbor[c] >= 0 ? (C)to_c(x[nbor[c] + k * npl[c]]) : C(0);
+                if (IN == IN_OPEN) {
+                    if (!(pn[3 + c] > C(0))) pn[c] = C(0);
+                    if (!(ph[3 + c] > C(0))) ph[c] = C(0);
+                }
+            }
         }
     };
     auto store_ring = [&](int slot) {
@@ -397,7 +388,7 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
         for (int c = 0; c < 3; ++c) {
             pf[c] = C(0);
             pd[c] = C(0);
-            if (MODE != ST_APPLY && own) {
+            if (MODE != ST_APPLY && MODE != ST_CERT && own) {
                 pf[c] = (C)to_c(f[c * N + p0 + k * Z]);
                 if (MODE == ST_JACOBI || MODE == ST_JACOBI2Z) pd[c] = (C)invD[c * N + p0 + k * Z];
             }
@@ -413,12 +404,14 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
     auto ez_at = [&](int ii, int jj, int s0, C lz) -> C {
         return lz * ((R(s0, 0, ii, jj - 1) - R(s0, 0, ii, jj)) * rdy + (R(s0, 1, ii, jj) - R(s0, 1, ii - 1, jj)) * rdx);
     };
-    auto psi_at = [&](int ii, int jj, int s0, int s1, C iv) -> C {
+    auto div_at = [&](int ii, int jj, int s0, int s1) -> C {
         const C fx = R(s0, 3, ii + 1, jj) * R(s0, 0, ii + 1, jj) - R(s0, 3, ii, jj) * R(s0, 0, ii, jj);
         const C fy = R(s0, 4, ii, jj + 1) * R(s0, 1, ii, jj + 1) - R(s0, 4, ii, jj) * R(s0, 1, ii, jj);
         const C fz = R(s1, 5, ii, jj) * R(s1, 2, ii, jj) - R(s0, 5, ii, jj) * R(s0, 2, ii, jj);
-        return iv * (fx * rdx + fy * rdy + fz * rdz);
+        return fx * rdx + fy * rdy + fz * rdz;
     };
+    auto psi_at = [&](int ii, int jj, int s0, int s1, C iv) -> C { return iv * div_at(ii, jj, s0, s1); };
+    C divn = C(0);   // ST_CERT: the node's cell divergence on the current plane
     // x- and y-edge curls of plane kp (ring slots: sm = plane kp-1, sp = plane kp) into edge slot es
     auto edges_xy = [&](int sm, int sp, int es) {
         s_ex[es][ty * TX + tx] = inb ? ex_at(i, j, sm, sp, cx) : C(0);
@@ -428,7 +421,12 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
     };
     // cell divergences and z-edge curls of plane k (ring slots: s0 = plane k, s1 = plane k+1)
     auto psi_ez = [&](int s0, int s1) {
-        s_psi[(ty + 1) * W1 + tx + 1] = inb ? psi_at(i, j, s0, s1, cv) : C(0);
+        if constexpr (MODE == ST_CERT) {
+            divn = inb ? div_at(i, j, s0, s1) : C(0);
+            s_psi[(ty + 1) * W1 + tx + 1] = cv * divn;
+        } else {
+            s_psi[(ty + 1) * W1 + tx + 1] = inb ? psi_at(i, j, s0, s1, cv) : C(0);
+        }
         s_ez[ty * W1 + tx] = inb ? ez_at(i, j, s0, cz) : C(0);
         if (role == 0) s_psi[dsm] = dval ? psi_at(di, dj, s0, s1, hc) : C(0);
         if (role == 1) s_ez[dsm] = dval ? ez_at(di, dj, s0, hc) : C(0);
@@ -484,10 +482,62 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
                 } else if (MODE == ST_JACOBI || MODE == ST_JACOBI2Z) {
                     v = bv[c] + omega * pd[c] * (pf[c] - v);
                 }
-                y[c * N + p] = to_store<T>(v);
+                if constexpr (MODE == ST_CERT) {
+                    const C ab = av[c] * bv[c], r = v - k2 * ab;
+                    sum[0] += bv[c] * v;
+                    sum[1] += bv[c] * ab;
+                    sum[2] += ab * ab;
+                    sum[3] += r * r;
+                    sum[4] += r * ab;
+                } else if constexpr (IN != IN_PADDED) {
+                    if (nown[c] >= 0 && k < g.nz + (c == 2)) y[nown[c] + k * npl[c]] = to_store<T>(v);
+                } else {
+                    y[c * N + p] = to_store<T>(v);
+                }
             }
+            if (MODE == ST_CERT && i < g.nx && j < g.ny && k < g.nz) sum[5] += divn * divn;
             psi_below = ps0;
         }
+    }
+    if constexpr (MODE == ST_CERT) {
+        __shared__ double red[TX * SY / 32][kCertSums];
+#pragma unroll
+        for (int e = 0; e < kCertSums; ++e) {
+            double v = sum[e];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (tx == 0) red[ty][e] = v;
+        }
+        __syncthreads();
+        if (tid < kCertSums) {
+            double v = 0.0;
+            for (int w = 0; w < SY; ++w) v += red[w][tid];
+            ca.part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kCertSums + tid] = v;
+        }
+    }
+}
+
+// out[vector][e] = sum of the blocks' sums, in a fixed order (one block per vector)
+__global__ void k_cert_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
+    __shared__ double red[8][kCertSums];
+    const double* p = part + (size_t)blockIdx.x * nb * kCertSums;
+    double s[kCertSums];
+#pragma unroll
+    for (int e = 0; e < kCertSums; ++e) s[e] = 0.0;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x)
+#pragma unroll
+        for (int e = 0; e < kCertSums; ++e) s[e] += p[(size_t)b * kCertSums + e];
+#pragma unroll
+    for (int e = 0; e < kCertSums; ++e) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[e] += __shfl_down_sync(0xffffffffu, s[e], o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][e] = s[e];
+    }
+    __syncthreads();
+    if (threadIdx.x < kCertSums) {
+        double v = 0.0;
+        for (int w = 0; w < 8; ++w) v += red[w][threadIdx.x];
+        out[blockIdx.x * kCertSums + threadIdx.x] = v;
     }
 }
 
@@ -887,52 +937,73 @@ template <typename T, typename TC>
 void vec_stencil(const VecOp<T, TC>& op, int mode, const T* x, const T* f, T* y, double omega, cudaStream_t s) {
     const Grid3& g = op.g;
     const double bytes = vec_stencil_bytes<T, TC>(g, mode);
-    if (op.tiles) {
-        const int* tl = op.stiles ? op.stiles : op.tiles;
-        const int nt = op.stiles ? op.nstiles : op.ntiles;
-        if (nt <= 0) return;
-        const char* nm = stencil_name("vec_stencil", prec_index<T>(), mode, op.level == 0);
-        // tile shape: 0 = 32x4x2 (the level's active tiles), 1 = 32x2x4, 2 = 32x8x1; 3 = 32x8x8,
-        // 4 = 32x4x8, 5 = 32x8x4 by the z-marching kernel (op.stiles is the active-tile list of that shape)
-        switch (op.shape * kStencilModes + mode) {
+    const int* tl = op.stiles ? op.stiles : op.tiles;
+    const int nt = op.stiles ? op.nstiles : op.ntiles;
+    if (nt <= 0) return;
+    const char* nm = stencil_name("vec_stencil", prec_index<T>(), mode, op.level == 0);
+    // tile shape: 0 = 32x4x2 (the level's active tiles), 1 = 32x2x4, 2 = 32x8x1; 3 = 32x8x8,
+    // 4 = 32x4x8, 5 = 32x8x4 by the z-marching kernel (op.stiles is the active-tile list of that shape)
+    switch (op.shape * kStencilModes + mode) {
 #define DM_TILED(SH, MD, SY, SZ)                                                                              \
     case SH * kStencilModes + MD:                                                                                         \
-        launch_b(nm, bytes, k_vec_stencil_tiled<T, TC, MD, SY, SZ>, nt, dim3(TX, SY, SZ), 0, s, g, op.A, op.L,  \
-                 op.invV, op.invD, op.sigma, x, f, y, omega, tl);                                             \
-        break;
-            DM_TILED(0, ST_APPLY, 4, 2) DM_TILED(0, ST_RESID, 4, 2) DM_TILED(0, ST_JACOBI, 4, 2) DM_TILED(0, ST_JACOBI2Z, 4, 2)
-            DM_TILED(1, ST_APPLY, 2, 4) DM_TILED(1, ST_RESID, 2, 4) DM_TILED(1, ST_JACOBI, 2, 4) DM_TILED(1, ST_JACOBI2Z, 2, 4)
-            DM_TILED(2, ST_APPLY, 8, 1) DM_TILED(2, ST_RESID, 8, 1) DM_TILED(2, ST_JACOBI, 8, 1) DM_TILED(2, ST_JACOBI2Z, 8, 1)
+    launch_b(nm, bytes, k_vec_stencil_tiled<T, TC, MD, SY, SZ>, nt, dim3(TX, SY, SZ), 0, s, g, op.A, op.L,  \
+             op.invV, op.invD, op.sigma, x, f, y, omega, tl);                                             \
+    break;
+        DM_TILED(0, ST_APPLY, 4, 2) DM_TILED(0, ST_RESID, 4, 2) DM_TILED(0, ST_JACOBI, 4, 2) DM_TILED(0, ST_JACOBI2Z, 4, 2)
+        DM_TILED(1, ST_APPLY, 2, 4) DM_TILED(1, ST_RESID, 2, 4) DM_TILED(1, ST_JACOBI, 2, 4) DM_TILED(1, ST_JACOBI2Z, 2, 4)
+        DM_TILED(2, ST_APPLY, 8, 1) DM_TILED(2, ST_RESID, 8, 1) DM_TILED(2, ST_JACOBI, 8, 1) DM_TILED(2, ST_JACOBI2Z, 8, 1)
 #undef DM_TILED
 #define DM_MARCH(SH, MD, SY, KZ)                                                                                \
     case SH * kStencilModes + MD:                                                                                         \
-        launch_b(nm, bytes, k_vec_stencil_march<T, TC, MD, SY, KZ>, nt, dim3(TX, SY, 1), 0, s, g, op.A, op.L,  \
-                 op.invV, op.invD, op.sigma, x, f, y, omega, tl);                                             \
-        break;
-            DM_MARCH(3, ST_APPLY, 8, 8) DM_MARCH(3, ST_RESID, 8, 8) DM_MARCH(3, ST_JACOBI, 8, 8) DM_MARCH(3, ST_JACOBI2Z, 8, 8)
-            DM_MARCH(4, ST_APPLY, 4, 8) DM_MARCH(4, ST_RESID, 4, 8) DM_MARCH(4, ST_JACOBI, 4, 8) DM_MARCH(4, ST_JACOBI2Z, 4, 8)
-            DM_MARCH(5, ST_APPLY, 8, 4) DM_MARCH(5, ST_RESID, 8, 4) DM_MARCH(5, ST_JACOBI, 8, 4) DM_MARCH(5, ST_JACOBI2Z, 8, 4)
+    launch_b(nm, bytes, k_vec_stencil_march<T, TC, MD, SY, KZ>, nt, dim3(TX, SY, 1), 0, s, g, op.A, op.L,  \
+             op.invV, op.invD, op.sigma, x, f, y, omega, tl, CertArgs{});                                 \
+    break;
+        DM_MARCH(3, ST_APPLY, 8, 8) DM_MARCH(3, ST_RESID, 8, 8) DM_MARCH(3, ST_JACOBI, 8, 8) DM_MARCH(3, ST_JACOBI2Z, 8, 8)
+        DM_MARCH(4, ST_APPLY, 4, 8) DM_MARCH(4, ST_RESID, 4, 8) DM_MARCH(4, ST_JACOBI, 4, 8) DM_MARCH(4, ST_JACOBI2Z, 4, 8)
+        DM_MARCH(5, ST_APPLY, 8, 4) DM_MARCH(5, ST_RESID, 8, 4) DM_MARCH(5, ST_JACOBI, 8, 4) DM_MARCH(5, ST_JACOBI2Z, 8, 4)
 #undef DM_MARCH
-            default: throw Error(DM_ERR_INVALID_ARG, "unknown stencil tile shape");
-        }
-        return;
+        default: throw Error(DM_ERR_INVALID_ARG, "unknown stencil tile shape");
     }
-    if (mode == ST_APPLY)
-        launch_b(stencil_name("vec_stencil", prec_index<T>(), ST_APPLY, op.level == 0), bytes, k_vec_stencil<T, TC, ST_APPLY>, tile_grid(g, op.tiles, op.ntiles, 1), kBlock, 0, s, g, op.A, op.L, op.invV, op.invD, op.sigma, x, f, y, omega, op.tiles);
-    else if (mode == ST_RESID)
-        launch_b(stencil_name("vec_stencil", prec_index<T>(), ST_RESID, op.level == 0), bytes, k_vec_stencil<T, TC, ST_RESID>, tile_grid(g, op.tiles, op.ntiles, 1), kBlock, 0, s, g, op.A, op.L, op.invV, op.invD, op.sigma, x, f, y, omega, op.tiles);
-    else if (mode == ST_JACOBI2Z)
-        launch_b(stencil_name("vec_stencil", prec_index<T>(), ST_JACOBI2Z, op.level == 0), bytes, k_vec_stencil<T, TC, ST_JACOBI2Z>, tile_grid(g, op.tiles, op.ntiles, 1), kBlock, 0, s, g, op.A, op.L, op.invV, op.invD, op.sigma, x, f, y, omega, op.tiles);
-    else
-        launch_b(stencil_name("vec_stencil", prec_index<T>(), ST_JACOBI, op.level == 0), bytes, k_vec_stencil<T, TC, ST_JACOBI>, tile_grid(g, op.tiles, op.ntiles, 1), kBlock, 0, s, g, op.A, op.L, op.invV, op.invD, op.sigma, x, f, y, omega, op.tiles);
 }
 
-// y = (K - sigma A) x in FP64 over every node of the level (dense grid of
-// blocks), launched under a fixed name: makes no host or device allocation.
-void vec_apply_dense_f64(const Grid3& g, const double* A, const double* L, const double* invV, double sigma,
-                         const double* x, double* y, cudaStream_t s) {
-    launch("vec_stencil_f64_apply_noalloc", k_vec_stencil<double, double, ST_APPLY>, node_grid(g), kBlock, 0, s, g, A, L,
-           invV, (const double*)nullptr, sigma, x, (const double*)nullptr, y, 0.0, (const int*)nullptr);
+void vec_apply_natural(const VecOp<double, double>& op, const double* x, double* y, bool traced, cudaStream_t s) {
+    const Grid3& g = op.g;
+    // off the active tiles there is no open face
+    DM_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * (size_t)natural_faces(g), s));
+    const bool march = op.stiles && op.shape >= 3;   // the level's tuned z-marching shape, else its 32x4x2 tiles
+    const int* tl = march ? op.stiles : op.tiles;
+    const int nt = march ? op.nstiles : op.ntiles;
+    if (nt <= 0) return;
+    const char* nm = traced ? stencil_name("vec_stencil", 0, ST_APPLY, op.level == 0) : "";   // (the name may allocate)
+    const double bytes = traced ? vec_stencil_bytes<double, double>(g, ST_APPLY) : 0.0;
+    switch (march ? op.shape : 0) {
+#define DM_NAT(SH, SY, KZ)                                                                                        \
+    case SH:                                                                                                      \
+        launch_b(nm, bytes, k_vec_stencil_march<double, double, ST_APPLY, SY, KZ, IN_OPEN>, nt, dim3(TX, SY, 1), 0, s, \
+                 g, op.A, op.L, op.invV, (const double*)nullptr, op.sigma, x, (const double*)nullptr, y, 0.0, tl,   \
+                 CertArgs{});                                                                                      \
+        break;
+        DM_NAT(0, 4, 2) DM_NAT(3, 8, 8) DM_NAT(4, 4, 8) DM_NAT(5, 8, 4)
+#undef DM_NAT
+    }
+}
+
+void vec_cert_sums(const VecOp<double, double>& op, bool natural, int n, const double* x, long long stride,
+                   const double* k2, double* part, double* out, cudaStream_t s) {
+    // op.stiles: 32x8x8 tiles
+    constexpr int kRows = 32768;   // vectors per launch (grid.y)
+    for (int v0 = 0; v0 < n; v0 += kRows) {
+        const int m = std::min(kRows, n - v0);
+        const CertArgs ca{k2 + v0, stride, part + (size_t)v0 * op.nstiles * kCertSums};
+        auto go = [&](auto kern) {
+            launch_b("vec_cert_sums", m * vec_stencil_bytes<double, double>(op.g, ST_APPLY), kern, dim3(op.nstiles, m),
+                     dim3(TX, 8, 1), 0, s, op.g, op.A, op.L, op.invV, (const double*)nullptr, 0.0, x + v0 * stride,
+                     (const double*)nullptr, (double*)nullptr, 0.0, op.stiles, ca);
+        };
+        if (natural) go(k_vec_stencil_march<double, double, ST_CERT, 8, 8, IN_NATURAL>);
+        else go(k_vec_stencil_march<double, double, ST_CERT, 8, 8, IN_PADDED>);
+    }
+    launch("k_cert_final", k_cert_final, n, 256, 0, s, op.nstiles, (const double*)part, out);
 }
 
 void band_slots(const Grid3& g, const double* A, const double* L, const double* invV, double sigma, const int* band,
