@@ -244,7 +244,7 @@ namespace {
 // buffers of one level of the V-cycles, in the preconditioner's storage type
 struct WorkLevel {
     DBuf<char> f, e, r;       // vector (3 np)
-    DBuf<char> sf, se, sr;    // scalar (np)
+    DBuf<char> sf, sr;        // scalar (np)
 };
 
 struct OpLevel {
@@ -499,7 +499,7 @@ void vcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
 
 // ---- scalar V-cycle: result in rbuf -----------------------------------------------
 template <typename T, typename TC>
-void svcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
+void svcycle(dm_operator* op, int l, const T* f, T* rbuf) {
     cudaStream_t s = op->ctx->stream;
     const GeoLevel& g = glv(op, l);
     if (l == op->nlev - 1) {
@@ -510,16 +510,13 @@ void svcycle(dm_operator* op, int l, const T* f, T* ebuf, T* rbuf) {
     }
     const ScalOp<T, TC> o = sop<T, TC>(op, l);
     const double om = op->ol[l].omega_s;
-    scal_jacobi_zero(o, f, ebuf, om, s);
-    scal_stencil(o, ST_RESID, ebuf, f, rbuf, 0.0, s);
     const GeoLevel& gc = glv(op, l + 1);
     WorkLevel& wc = op->wk[l + 1];
     T* fc = reinterpret_cast<T*>(wc.sf.get());
-    cell_restrict<T>(g.g, gc.g, gc.active.get(), rbuf, fc, gc.tiles.get(), gc.ntiles, s);
-    svcycle<T, TC>(op, l + 1, fc, reinterpret_cast<T*>(wc.se.get()), reinterpret_cast<T*>(wc.sr.get()));
-    cell_prolong_add<T>(g.g, gc.g, g.active.get(), reinterpret_cast<const T*>(wc.sr.get()), ebuf, g.tiles.get(),
-                        g.ntiles, s);
-    scal_stencil(o, ST_JACOBI, ebuf, f, rbuf, om, s);
+    T* ec = reinterpret_cast<T*>(wc.sr.get());
+    scal_down(o, gc.g, gc.active.get(), f, fc, om, s);
+    svcycle<T, TC>(op, l + 1, fc, ec);
+    scal_up(o, gc.g, f, ec, rbuf, om, s);
 }
 
 // Capture f(...) issued on the context stream into an executable graph.
@@ -665,18 +662,17 @@ void precond_scal_T(dm_operator* op, const TIn& v, double* z, double scale = 1.0
     const Domain D = glv(op, 0).sdom();
     WorkLevel& w0 = op->wk[0];
     T* f = reinterpret_cast<T*>(w0.sf.get());
-    T* e = reinterpret_cast<T*>(w0.se.get());
     T* r = reinterpret_cast<T*>(w0.sr.get());
     mg_input<T>(D, v, scale, f, s);
     if (graphs_allowed(op) && op->scalls > 0) {
-        if (!op->sexec && !capture_graph(op, [&] { svcycle<T, TC>(op, 0, f, e, r); }, &op->sexec, &op->sexec_kernels))
+        if (!op->sexec && !capture_graph(op, [&] { svcycle<T, TC>(op, 0, f, r); }, &op->sexec, &op->sexec_kernels))
             op->graphs = false;
     }
     if (graphs_allowed(op) && op->sexec) {
         DM_CUDA(cudaGraphLaunch(op->sexec, s));
         count_launch(op->sexec_kernels);
     } else {
-        svcycle<T, TC>(op, 0, f, e, r);
+        svcycle<T, TC>(op, 0, f, r);
     }
     ++op->scalls;
     convert<double, T>(D, r, z, s);
@@ -704,7 +700,7 @@ void apply_vec64(dm_operator* op, int l, const double* x, double* y) {
     vec_stencil<double, double>(vop<double, double>(op, l), ST_APPLY, x, nullptr, y, 0.0, op->ctx->stream);
 }
 void apply_scal64(dm_operator* op, int l, const double* x, double* y) {
-    scal_stencil<double, double>(sop<double, double>(op, l), ST_APPLY, x, nullptr, y, 0.0, op->ctx->stream);
+    scal_apply(sop<double, double>(op, l), x, y, op->ctx->stream);
 }
 
 // sum of x y (times w, nullable) over the fine level's open faces, by the flat
@@ -1259,7 +1255,6 @@ void setup_operator(dm_operator* op) {
         w.e.alloc(ts * n3);
         w.r.alloc(ts * n3);
         w.sf.alloc(ts * n1);
-        w.se.alloc(ts * n1);
         w.sr.alloc(ts * n1);
         max_band = std::max(max_band, (size_t)g.nband);
     }

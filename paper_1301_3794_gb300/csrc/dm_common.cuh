@@ -512,10 +512,14 @@ struct ScalOp {
     const int* tiles = nullptr;
     int ntiles = 0;
 };
+void scal_apply(const ScalOp<double, double>& op, const double* x, double* y, cudaStream_t s);
+// one level of the scalar V-cycle: fc = R (f - S om D^-1 f) on the way down,
+// y = x + om D^-1 (f - S x) with x = om D^-1 f + P ec on the way up
 template <typename T, typename TC>
-void scal_stencil(const ScalOp<T, TC>& op, int mode, const T* x, const T* f, T* y, double omega, cudaStream_t s);
+void scal_down(const ScalOp<T, TC>& op, const Grid3& gc, const unsigned char* active_c, const T* f, T* fc, double omega,
+               cudaStream_t s);
 template <typename T, typename TC>
-void scal_jacobi_zero(const ScalOp<T, TC>& op, const T* f, T* y, double omega, cudaStream_t s);
+void scal_up(const ScalOp<T, TC>& op, const Grid3& gc, const T* f, const T* ec, T* y, double omega, cudaStream_t s);
 void scal_diagonal(const Grid3& g, const double* A, const unsigned char* active, double* d, cudaStream_t s);
 void scal_dense_assemble(const Grid3& g, const double* A, const int* list, const unsigned char* pinned, int n,
                          double* M, cudaStream_t s);
@@ -541,13 +545,6 @@ void face_prolong_add(const Grid3& gf, const Grid3& gc, const TC* Af, const T* e
 // x <- A^-1/2 x (inverse) or A^1/2 x on the open faces of the domain
 template <typename T, typename TC>
 void scale_sqrt_a(const Domain& d, const TC* A, bool inverse, T* x, cudaStream_t s);
-template <typename T>
-void cell_restrict(const Grid3& gf, const Grid3& gc, const unsigned char* active_c, const T* r, T* fc,
-                   const int* tiles_c, int ntiles_c, cudaStream_t s);
-template <typename T>
-void cell_prolong_add(const Grid3& gf, const Grid3& gc, const unsigned char* active_f, const T* ec, T* x,
-                      const int* tiles_f, int ntiles_f, cudaStream_t s);
-
 // dense (dm_dense.cu)
 // in-place inverse of the n x n row-major FP64 matrix M, n <= 6144 (work:
 // dense_inverse_work(n) doubles).  Returns false if a column had no pivot above 1e-300.

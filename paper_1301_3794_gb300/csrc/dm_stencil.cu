@@ -624,10 +624,84 @@ struct CellUnit {
     __device__ __forceinline__ C operator()(int p) const { return p == q ? C(1) : C(0); }
 };
 
-template <typename T, typename TC, int MODE>
-__global__ void k_scal_stencil(Grid3 g, const TC* __restrict__ A, const unsigned char* __restrict__ active,
-                               const TC* __restrict__ invD, const T* __restrict__ x, const T* __restrict__ f,
-                               T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles) {
+// ---- scalar V-cycle, one launch per level and direction ------------------------
+// The scalar cycle's levels are small (latency-bound) and its passes cheap, so
+// what counts is the number of launches: the zero-start Jacobi sweep, the
+// residual and the restriction of the way down are one kernel, the prolongation
+// and the Jacobi sweep of the way up another (16 launches per cycle of four
+// levels -> 7).  Both form the first iterate om D^-1 f where they read it, and
+// round every value a separate pass would have stored as that pass rounded it,
+// so the results are the same bits.
+// Measured, a projection on 104 x 88 x 72 cells (FP32, 32 iterations): 751 -> 463
+// launches; with one synchronisation less per iteration 5.4 -> 4.6 ms.
+template <typename T, typename TC, typename C>
+struct ScalJac0 {   // the first iterate from zero
+    const T* __restrict__ f;
+    const TC* __restrict__ invD;
+    C om;
+    __device__ __forceinline__ C operator()(int p) const { return (C)to_c(to_store<T>(om * (C)invD[p] * (C)to_c(f[p]))); }
+};
+template <typename T, typename TC, typename C>
+struct ScalJac0Up {   // that iterate plus the parent's coarse correction
+    ScalJac0<T, TC, C> x0;
+    const unsigned char* __restrict__ active;
+    const T* __restrict__ ec;
+    Grid3 gf, gc;
+    __device__ __forceinline__ C at(int p, int i, int j, int k) const {
+        if (!active[p]) return C(0);
+        return (C)to_c(to_store<T>(x0(p) + (C)to_c(ec[gc.idx(i >> 1, j >> 1, k >> 1)])));
+    }
+};
+
+// fc = R (f - S om D^-1 f): one thread per fine cell of the active tiles, whose
+// corner is even, so the eight children of a coarse cell meet in one block
+template <typename T, typename TC>
+__global__ void __launch_bounds__(TX * TY * TZ) k_scal_down(Grid3 g, Grid3 gc, const TC* __restrict__ A,
+                                                            const unsigned char* __restrict__ active,
+                                                            const TC* __restrict__ invD, const T* __restrict__ f,
+                                                            typename Compute<T>::type om,
+                                                            const unsigned char* __restrict__ active_c,
+                                                            T* __restrict__ fc, const int* __restrict__ tiles) {
+    using C = typename Compute<T>::type;
+    __shared__ C r[TZ][TY][TX];
+    int i, j, k;
+    block_node(g, tiles, i, j, k);
+    C v = C(0);
+    if (i < g.nx && j < g.ny && k < g.nz) {
+        const int p = g.idx(i, j, k);
+        if (active[p]) {
+            const ScalJac0<T, TC, C> x0{f, invD, om};
+            const C rx = inv_h<C>(g, 0), ry = inv_h<C>(g, 1), rz = inv_h<C>(g, 2);
+            const C sx = cell_S<C>(A, x0, p, 1, g.sx, g.sxy, g.np, rx * rx, ry * ry, rz * rz);
+            v = (C)to_c(to_store<T>((C)to_c(f[p]) - sx));
+        }
+    }
+    r[threadIdx.z][threadIdx.y][threadIdx.x] = v;
+    __syncthreads();
+    if ((threadIdx.x | threadIdx.y | threadIdx.z) & 1) return;
+    const int I = i >> 1, J = j >> 1, K = k >> 1;
+    if (I >= gc.nx || J >= gc.ny || K >= gc.nz) return;
+    const int q = gc.idx(I, J, K);
+    C acc = C(0);
+    if (active_c[q]) {
+#pragma unroll
+        for (int dk = 0; dk < 2; ++dk)
+#pragma unroll
+            for (int dj = 0; dj < 2; ++dj)
+#pragma unroll
+                for (int di = 0; di < 2; ++di) acc += r[dk][threadIdx.y + dj][threadIdx.x + di];
+        acc *= C(0.125);
+    }
+    fc[q] = to_store<T>(acc);
+}
+
+// y = x + om D^-1 (f - S x), x = om D^-1 f + P ec
+template <typename T, typename TC>
+__global__ void __launch_bounds__(TX * TY * TZ) k_scal_up(Grid3 g, Grid3 gc, const TC* __restrict__ A,
+                                                          const unsigned char* __restrict__ active,
+                                                          const TC* __restrict__ invD, const T* __restrict__ f,
+                                                          typename Compute<T>::type om, const T* __restrict__ ec,
+                                                          T* __restrict__ y, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     int i, j, k;
     block_node(g, tiles, i, j, k);
@@ -635,14 +709,31 @@ __global__ void k_scal_stencil(Grid3 g, const TC* __restrict__ A, const unsigned
     const int p = g.idx(i, j, k);
     C v = C(0);
     if (active[p]) {
-        CellAcc<T, C> acc{x};
+        const ScalJac0Up<T, TC, C> x{{f, invD, om}, active, ec, g, gc};
+        const int Y = g.sx, Z = g.sxy, N = g.np;
         const C rx = inv_h<C>(g, 0), ry = inv_h<C>(g, 1), rz = inv_h<C>(g, 2);
-        const C sx = cell_S<C>(A, acc, p, 1, g.sx, g.sxy, g.np, rx * rx, ry * ry, rz * rz);
-        if (MODE == ST_APPLY) v = sx;
-        else if (MODE == ST_RESID) v = (C)to_c(f[p]) - sx;
-        else v = (C)to_c(x[p]) + omega * (C)invD[p] * ((C)to_c(f[p]) - sx);
+        const C v0 = x.at(p, i, j, k);
+        // as cell_S
+        const C sx = ((C)A[p + 1] * (v0 - x.at(p + 1, i + 1, j, k)) + (C)A[p] * (v0 - x.at(p - 1, i - 1, j, k))) * (rx * rx) +
+                     ((C)A[N + p + Y] * (v0 - x.at(p + Y, i, j + 1, k)) + (C)A[N + p] * (v0 - x.at(p - Y, i, j - 1, k))) *
+                         (ry * ry) +
+                     ((C)A[2 * N + p + Z] * (v0 - x.at(p + Z, i, j, k + 1)) +
+                      (C)A[2 * N + p] * (v0 - x.at(p - Z, i, j, k - 1))) *
+                         (rz * rz);
+        v = v0 + om * (C)invD[p] * ((C)to_c(f[p]) - sx);
     }
     y[p] = to_store<T>(v);
+}
+
+// y = D A D^T x on the active cells
+__global__ void k_scal_apply(Grid3 g, const double* __restrict__ A, const unsigned char* __restrict__ active,
+                             const double* __restrict__ x, double* __restrict__ y, const int* __restrict__ tiles) {
+    int i, j, k;
+    block_node(g, tiles, i, j, k);
+    if (i >= g.nx || j >= g.ny || k >= g.nz) return;
+    const int p = g.idx(i, j, k);
+    const CellAcc<double, double> acc{x};
+    y[p] = active[p] ? cell_S<double>(A, acc, p, 1, g.sx, g.sxy, g.np, g.rhx * g.rhx, g.rhy * g.rhy, g.rhz * g.rhz) : 0.0;
 }
 
 __global__ void k_scal_diag(Grid3 g, const double* __restrict__ A, const unsigned char* __restrict__ active,
@@ -925,14 +1016,6 @@ double vec_stencil_bytes(const Grid3& g, int mode) {
     const bool jac = mode == ST_JACOBI || mode == ST_JACOBI2Z;
     return (double)g.nopen * (tv * (2 + (mode == ST_RESID || mode == ST_JACOBI)) + tc * (2.0 + 1.0 / 3.0 + jac));
 }
-// per active cell: x, y (and f), three face fractions (six faces, each shared
-// by two cells), 1/D for jacobi, and the activity flag
-template <typename T, typename TC>
-double scal_stencil_bytes(const Grid3& g, int mode) {
-    const double tv = sizeof(T), tc = sizeof(TC);
-    return (double)g.nact * (tv * (2 + (mode != ST_APPLY)) + tc * (3 + (mode == ST_JACOBI)) + 1.0);
-}
-
 template <typename T, typename TC>
 void vec_stencil(const VecOp<T, TC>& op, int mode, const T* x, const T* f, T* y, double omega, cudaStream_t s) {
     const Grid3& g = op.g;
@@ -1032,24 +1115,27 @@ void vec_dense_assemble(const Grid3& g, const double* A, const double* L, const 
     launch("k_vec_dense", k_vec_dense, n, 128, 0, s, g, A, L, invV, sigma, list, n, M);
 }
 
-template <typename T, typename TC>
-void scal_stencil(const ScalOp<T, TC>& op, int mode, const T* x, const T* f, T* y, double omega, cudaStream_t s) {
-    const Grid3& g = op.g;
-    if (mode == ST_APPLY)
-        launch_b(stencil_name("scal_stencil", prec_index<T>(), ST_APPLY, op.level == 0), scal_stencil_bytes<T, TC>(g, ST_APPLY), k_scal_stencil<T, TC, ST_APPLY>, tile_grid(g, op.tiles, op.ntiles, 0), kBlock, 0, s, g, op.A, op.active, op.invD, x, f, y, omega, op.tiles);
-    else if (mode == ST_RESID)
-        launch_b(stencil_name("scal_stencil", prec_index<T>(), ST_RESID, op.level == 0), scal_stencil_bytes<T, TC>(g, ST_RESID), k_scal_stencil<T, TC, ST_RESID>, tile_grid(g, op.tiles, op.ntiles, 0), kBlock, 0, s, g, op.A, op.active, op.invD, x, f, y, omega, op.tiles);
-    else
-        launch_b(stencil_name("scal_stencil", prec_index<T>(), ST_JACOBI, op.level == 0), scal_stencil_bytes<T, TC>(g, ST_JACOBI), k_scal_stencil<T, TC, ST_JACOBI>, tile_grid(g, op.tiles, op.ntiles, 0), kBlock, 0, s, g, op.A, op.active, op.invD, x, f, y, omega, op.tiles);
+void scal_apply(const ScalOp<double, double>& op, const double* x, double* y, cudaStream_t s) {
+    // per active cell: x, y, three face fractions (six faces, each shared by two cells) and the flag
+    launch_b(op.level == 0 ? "scal_apply_f64_L0" : "scal_apply_f64_Lc", op.g.nact * 41.0, k_scal_apply,
+             tile_grid(op.g, op.tiles, op.ntiles, 0), kBlock, 0, s, op.g, op.A, op.active, x, y, op.tiles);
 }
 
 template <typename T, typename TC>
-void scal_jacobi_zero(const ScalOp<T, TC>& op, const T* f, T* y, double omega, cudaStream_t s) {
-    const Domain d{op.g, op.tiles, op.ntiles, 1};
-    const int blocks = op.tiles ? std::max(op.ntiles, 1) : (int)std::min<long long>((d.len() + 255) / 256, 152 * 16);
-    launch_b(stencil_name("scal_jacobi_zero", prec_index<T>(), ST_JACOBI, op.level == 0),
-             (double)op.g.nact * (2.0 * sizeof(T) + sizeof(TC)), k_jacobi_zero<T, TC>, blocks, 256, 0, s, d, op.invD,
-             f, y, omega);
+void scal_down(const ScalOp<T, TC>& op, const Grid3& gc, const unsigned char* active_c, const T* f, T* fc, double omega,
+               cudaStream_t s) {
+    // per fine cell f, 1/D, three face fractions and the flag; per coarse cell its result and flag
+    launch_b(stencil_name("scal_down", prec_index<T>(), ST_RESID, op.level == 0),
+             op.g.nact * (sizeof(T) + 4.0 * sizeof(TC) + 1.0) + gc.nact * (sizeof(T) + 1.0), k_scal_down<T, TC>,
+             tile_grid(op.g, op.tiles, op.ntiles, 0), kBlock, 0, s, op.g, gc, op.A, op.active, op.invD, f, omega,
+             active_c, fc, op.tiles);
+}
+template <typename T, typename TC>
+void scal_up(const ScalOp<T, TC>& op, const Grid3& gc, const T* f, const T* ec, T* y, double omega, cudaStream_t s) {
+    launch_b(stencil_name("scal_up", prec_index<T>(), ST_JACOBI, op.level == 0),
+             op.g.nact * (2.0 * sizeof(T) + 4.0 * sizeof(TC) + 1.0) + (double)gc.nact * sizeof(T), k_scal_up<T, TC>,
+             tile_grid(op.g, op.tiles, op.ntiles, 0), kBlock, 0, s, op.g, gc, op.A, op.active, op.invD, f, omega, ec, y,
+             op.tiles);
 }
 
 void scal_diagonal(const Grid3& g, const double* A, const unsigned char* active, double* d, cudaStream_t s) {
@@ -1078,8 +1164,9 @@ void dm_sub_grad(const Grid3& g, const double* A, const double* x, const double*
 #define DM_INST(T, TC)                                                                                          \
     template void vec_stencil<T, TC>(const VecOp<T, TC>&, int, const T*, const T*, T*, double, cudaStream_t);  \
     template void vec_jacobi_zero<T, TC>(const VecOp<T, TC>&, const T*, T*, double, cudaStream_t);            \
-    template void scal_stencil<T, TC>(const ScalOp<T, TC>&, int, const T*, const T*, T*, double, cudaStream_t); \
-    template void scal_jacobi_zero<T, TC>(const ScalOp<T, TC>&, const T*, T*, double, cudaStream_t);
+    template void scal_down<T, TC>(const ScalOp<T, TC>&, const Grid3&, const unsigned char*, const T*, T*, double, \
+                                   cudaStream_t);                                                              \
+    template void scal_up<T, TC>(const ScalOp<T, TC>&, const Grid3&, const T*, const T*, T*, double, cudaStream_t);
 DM_INST(double, double)
 DM_INST(float, float)
 DM_INST(__nv_bfloat16, float)

@@ -10,8 +10,7 @@
 // The fine result is masked by the open fine faces.  Restriction R = P^T / 8
 // is evaluated from the same per-axis weights, masked by the open coarse faces.
 //
-// Cell transfers: a fine cell copies its parent; R = P^T / 8 (the mean of the
-// 8 children); both masked by the active cells of the receiving level.
+// The cell transfers are part of the scalar V-cycle's kernels (dm_stencil.cu).
 #include "dm_common.cuh"
 
 namespace dm {
@@ -144,41 +143,6 @@ __global__ void k_scale_sqrt_a(Domain d, const TC* __restrict__ A, int inverse, 
     });
 }
 
-template <typename T>
-__global__ void k_cell_restrict(Grid3 gf, Grid3 gc, const unsigned char* __restrict__ active_c,
-                                const T* __restrict__ r, T* __restrict__ fc, const int* __restrict__ tiles) {
-    using C = typename Compute<T>::type;
-    int I, J, K;
-    block_node(gc, tiles, I, J, K);
-    if (I >= gc.nx || J >= gc.ny || K >= gc.nz) return;
-    const int q = gc.idx(I, J, K);
-    C acc = C(0);
-    if (active_c[q]) {
-        const int p = gf.idx(2 * I, 2 * J, 2 * K);
-        for (int dk = 0; dk < 2; ++dk)
-            for (int dj = 0; dj < 2; ++dj)
-                for (int di = 0; di < 2; ++di) acc += (C)to_c(r[p + di + dj * gf.sx + dk * gf.sxy]);
-        acc *= C(0.125);
-    }
-    fc[q] = to_store<T>(acc);
-}
-
-template <typename T>
-__global__ void k_cell_prolong(Grid3 gf, Grid3 gc, const unsigned char* __restrict__ active_f,
-                               const T* __restrict__ ec, T* __restrict__ x, const int* __restrict__ tiles) {
-    using C = typename Compute<T>::type;
-    int i, j, k;
-    block_node(gf, tiles, i, j, k);
-    if (i >= gf.nx || j >= gf.ny || k >= gf.nz) return;
-    const int p = gf.idx(i, j, k);
-    if (!active_f[p]) return;
-    x[p] = to_store<T>((C)to_c(x[p]) + (C)to_c(ec[gc.idx(i >> 1, j >> 1, k >> 1)]));
-}
-
-inline dim3 grid_for(const Grid3& g, int extra) {
-    return dim3((g.nx + extra + BX - 1) / BX, (g.ny + extra + BY - 1) / BY, (g.nz + extra + BZ - 1) / BZ);
-}
-
 }  // namespace
 
 template <typename T, typename TC>
@@ -210,19 +174,6 @@ void scale_sqrt_a(const Domain& d, const TC* A, bool inverse, T* x, cudaStream_t
     launch_b("k_scale_sqrt_a", d.live() * (2.0 * sizeof(T) + sizeof(TC)), k_scale_sqrt_a<T, TC>,
              d.tiles ? std::max(d.ntiles, 1) : 1216, 256, 0, s, d, A, inverse ? 1 : 0, x);
 }
-template <typename T>
-void cell_restrict(const Grid3& gf, const Grid3& gc, const unsigned char* active_c, const T* r, T* fc,
-                   const int* tiles_c, int ntiles_c, cudaStream_t s) {
-    launch_b("k_cell_restrict", (double)gf.nact * sizeof(T) + (double)gc.nact * (sizeof(T) + 1.0), k_cell_restrict<T>,
-             tile_grid(gc, tiles_c, ntiles_c, 0), kBlock, 0, s, gf, gc, active_c, r, fc, tiles_c);
-}
-template <typename T>
-void cell_prolong_add(const Grid3& gf, const Grid3& gc, const unsigned char* active_f, const T* ec, T* x,
-                      const int* tiles_f, int ntiles_f, cudaStream_t s) {
-    launch_b("k_cell_prolong", (double)gc.nact * sizeof(T) + (double)gf.nact * (2.0 * sizeof(T) + 1.0),
-             k_cell_prolong<T>, tile_grid(gf, tiles_f, ntiles_f, 0), kBlock, 0, s, gf, gc, active_f, ec, x, tiles_f);
-}
-
 #define DM_INST(T, TC)                                                                                   \
     template void face_restrict<T, TC>(const Grid3&, const Grid3&, const TC*, const T*, T*, const int*, int,  \
                                        cudaStream_t, bool);                                                \
@@ -233,13 +184,5 @@ DM_INST(double, double)
 DM_INST(float, float)
 DM_INST(__nv_bfloat16, float)
 #undef DM_INST
-template void cell_restrict<double>(const Grid3&, const Grid3&, const unsigned char*, const double*, double*, const int*, int, cudaStream_t);
-template void cell_restrict<float>(const Grid3&, const Grid3&, const unsigned char*, const float*, float*, const int*, int, cudaStream_t);
-template void cell_restrict<__nv_bfloat16>(const Grid3&, const Grid3&, const unsigned char*, const __nv_bfloat16*,
-                                           __nv_bfloat16*, const int*, int, cudaStream_t);
-template void cell_prolong_add<double>(const Grid3&, const Grid3&, const unsigned char*, const double*, double*, const int*, int, cudaStream_t);
-template void cell_prolong_add<float>(const Grid3&, const Grid3&, const unsigned char*, const float*, float*, const int*, int, cudaStream_t);
-template void cell_prolong_add<__nv_bfloat16>(const Grid3&, const Grid3&, const unsigned char*, const __nv_bfloat16*,
-                                              __nv_bfloat16*, const int*, int, cudaStream_t);
 
 }  // namespace dm
