@@ -814,7 +814,7 @@ int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long l
     int total = 0;
     bool first = true;
     double res = 1.0;
-    std::vector<double> H((size_t)(m + 1) * m), dots(2 * m + 2), coef(2 * m + 2), y;
+    std::vector<double> H((size_t)(m + 1) * m), dots(2 * m + 5), y;
     while (total < maxit) {
         // r = b - A x (FP64); V_0 = r / beta in float-float
         double beta = bnorm;
@@ -839,14 +839,10 @@ int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long l
                 apply(Z + (size_t)j * n, w);
                 ff_gather(nl, list, 1.0, w, wf, s);
             }
-            // one sweep: Q^T v, Q^T w, v.v, v.w with Q = V_0 .. V_{j-1} finished
-            dcgs_dots(ctx->red, Dc, j, V, nlp, Vj, wf, dots.data(), s);
-            double ss = 0.0, sc = 0.0;
-            for (int i = 0; i < j; ++i) {
-                ss += dots[i] * dots[i];
-                sc += dots[i] * dots[j + i];
-            }
-            const double bj = std::sqrt(std::max(dots[2 * j] - ss, 0.0));
+            // one sweep: Q^T v, Q^T w, v.v, v.w with Q = V_0 .. V_{j-1} finished; a
+            // second finishes V_j and forms the next pending vector
+            dcgs_step(ctx->red, Dc, j, V, nlp, Vj, wf, V + (size_t)(j + 1) * nlp, dots.data(), s);
+            const double bj = dots[2 * j + 2];
             if (!(bj > 0.0)) break;
             // finish column j-1: its pending vector was Q s + bj V_j
             if (j > 0) {
@@ -854,16 +850,9 @@ int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long l
                 H[(size_t)j * m + (j - 1)] = bj;
             }
             // new column: Q^T w and V_j . w for the finished V_j
-            const double hj = (dots[2 * j + 1] - sc) / bj;
-            for (int i = 0; i < j; ++i) {
-                coef[i] = dots[i];
-                coef[j + i] = dots[j + i] - hj / bj * dots[i];
-                H[(size_t)i * m + j] = dots[j + i];
-            }
-            H[(size_t)j * m + j] = hj;
-            coef[2 * j] = 1.0 / bj;
-            coef[2 * j + 1] = hj / bj;
-            const double nn2 = dcgs_update(ctx->red, Dc, j, V, nlp, coef.data(), Vj, wf, V + (size_t)(j + 1) * nlp, s);
+            for (int i = 0; i < j; ++i) H[(size_t)i * m + j] = dots[j + i];
+            H[(size_t)j * m + j] = dots[2 * j + 3];
+            const double nn2 = dots[2 * j + 4];
             nu = std::sqrt(std::max(nn2, 0.0));
             H[(size_t)(j + 1) * m + j] = nu;   // provisional until the next iteration
             k = j + 1;

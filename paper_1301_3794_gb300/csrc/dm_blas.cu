@@ -124,15 +124,61 @@ __global__ void k_dot_list(long long n, const int* __restrict__ list, const doub
     }
 }
 
-// result[c] = sum_b partial[b * ldp + c]  (one warp per column, fixed order)
-__global__ void k_mdot_final(int nb, int m, const double* __restrict__ partial, int ldp, double* __restrict__ result) {
+// result[c] = sum_b partial[b * ldb + c * ldc]  (one warp per column, fixed order)
+__global__ void k_mdot_final(int nb, int m, const double* __restrict__ partial, int ldb, int ldc,
+                             double* __restrict__ result) {
     const int c = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (c >= m) return;
     double s = 0.0;
-    for (int b = lane; b < nb; b += 32) s += partial[(long long)b * ldp + c];
+    for (int b = lane; b < nb; b += 32) s += partial[(long long)b * ldb + (long long)c * ldc];
     s = warp_sum(s);
     if (lane == 0) result[c] = s;
+}
+
+// Final sums of a dcgs_dots pass and the coefficients of its update, in one
+// block: result[0 .. 2j + 2) = the dots (as k_mdot_final sums them),
+// result[2j + 2] = b = sqrt(v.v - |s|^2), result[2j + 3] = h = (v.w - s.c) / b,
+// coef = [s (j), c - (h / b) s (j), 1 / b, h / b]; all coefficients 0 when b is
+// not positive (the caller stops there).  On the device, the update need not
+// wait for the host: one synchronisation per FGMRES iteration instead of two.
+__global__ void __launch_bounds__(1024) k_dcgs_coef(int nb, int j, const double* __restrict__ partial, int ldp,
+                                                    double* __restrict__ result, double* __restrict__ coef) {
+    __shared__ double dots[256];
+    __shared__ double bh[2];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, m = 2 * j + 2;
+    for (int c = wid; c < m; c += 32) {
+        double s = 0.0;
+        for (int b = lane; b < nb; b += 32) s += partial[(long long)c * ldp + b];
+        s = warp_sum(s);
+        if (lane == 0) dots[c] = result[c] = s;
+    }
+    __syncthreads();
+    if (wid == 0) {
+        double ss = 0.0, sc = 0.0;
+        for (int i = lane; i < j; i += 32) {
+            ss += dots[i] * dots[i];
+            sc += dots[i] * dots[j + i];
+        }
+        ss = warp_sum(ss);
+        sc = warp_sum(sc);
+        if (lane == 0) {
+            const double b = sqrt(fmax(dots[2 * j] - ss, 0.0));
+            bh[0] = result[m] = b;
+            bh[1] = result[m + 1] = b > 0.0 ? (dots[2 * j + 1] - sc) / b : 0.0;
+        }
+    }
+    __syncthreads();
+    const double b = bh[0], h = bh[1];
+    const bool ok = b > 0.0;
+    for (int i = threadIdx.x; i < j; i += blockDim.x) {
+        coef[i] = ok ? dots[i] : 0.0;
+        coef[j + i] = ok ? dots[j + i] - h / b * dots[i] : 0.0;
+    }
+    if (threadIdx.x == 0) {
+        coef[2 * j] = ok ? 1.0 / b : 0.0;
+        coef[2 * j + 1] = ok ? h / b : 0.0;
+    }
 }
 
 __global__ void k_maxpy(Domain d, int m, const double* __restrict__ V, long long ld, const double* __restrict__ h,
@@ -293,20 +339,62 @@ __device__ __forceinline__ double ff_warp_sum(float s, float e) {
     return ff_to_double(v);
 }
 
+// Sums over a warp of P float-float values per lane at once (P a power of two, at
+// most 32): at each step a lane hands half of its values to its partner and
+// keeps the other half, so all P sums take P - 1 additions (and one more per
+// step beyond log2 P) where P separate warp sums take 5 P.  Lane l ends with the
+// sum of value l >> (5 - log2 P).
+template <int P>
+__device__ __forceinline__ double ff_warp_sums(float2 (&v)[P]) {
+    const int lane = threadIdx.x & 31;
+    auto add = [](float2 a, float2 b) {
+        const float t = __fadd_rn(a.x, b.x);
+        const float bp = __fsub_rn(t, a.x);
+        const float err = __fadd_rn(__fsub_rn(a.x, __fsub_rn(t, bp)), __fsub_rn(b.x, bp));
+        return ff_norm(t, __fadd_rn(err, __fadd_rn(a.y, b.y)));
+    };
+    int n = P;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        n = P >> (o == 16 ? 0 : o == 8 ? 1 : o == 4 ? 2 : o == 2 ? 3 : 4);   // values left (0: one, summed over lanes)
+        if (n > 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < P / 2; ++i)
+                if (i < n / 2) {
+                    const float2 keep = up ? v[i + n / 2] : v[i], give = up ? v[i] : v[i + n / 2];
+                    const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, o),
+                                                   __shfl_xor_sync(0xffffffffu, give.y, o));
+                    v[i] = add(keep, got);
+                }
+        } else {
+            const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, v[0].x, o), __shfl_xor_sync(0xffffffffu, v[0].y, o));
+            v[0] = add(v[0], got);
+        }
+    }
+    return ff_to_double(v[0]);
+}
+
 // One pass of delayed classical Gram-Schmidt (DCGS2): against the finished
 // basis Q (j vectors) and the pending vector v, with the new vector w:
-//   partial[b][c] = Q_c . v, [j + c] = Q_c . w (c < j), [2j] = v . v, [2j + 1] = v . w
-// Columns go in chunks of up to 8 whose size is a compile-time constant, so the
-// accumulators stay in registers and no predicated-off column is issued.
+//   column c of partial = Q_c . v, j + c = Q_c . w (c < j), 2j = v . v, 2j + 1 = v . w,
+// partial[column * ldp + block] (so that the final sums read along it).
+// Columns go in chunks of up to 16 whose size is a compile-time constant, so the
+// accumulators stay in registers and no predicated-off column is issued; each
+// chunk re-reads v and w, which at 8 columns a chunk was a fifth of the traffic.
 // The compact vectors have an even length and stride (a zero pad entry when
 // needed), and every thread takes two entries per step with one 16-byte load
 // per vector, so twice the bytes are in flight per load instruction.
+// HBM bounds it on large vectors; on small ones the reductions did, at 80
+// float-float additions and two barriers per 8 columns (see ff_warp_sums).
+// Measured (CUDA events, some 4 us a launch of them the events): 300 k cells, 16 columns
+// on average, 34 -> 17 us; 5.65 M faces 121 -> 110 us (5.5 TB/s of the bytes needed).
+constexpr int kDotCols = 16;
 template <int NC>
 __device__ __forceinline__ void dcgs_chunk(long long n2, int j, int c0, const float4* __restrict__ Q, long long ld2,
                                            const float4* __restrict__ v, const float4* __restrict__ w, bool first,
                                            float& as, float& ae, float& ds, float& de, double* __restrict__ partial,
-                                           int ldp) {
-    __shared__ double red[kThreads / 32][16];
+                                           int ldp, double (*red)[32]) {
     constexpr int N1 = NC > 0 ? NC : 1;
     float ss[N1], se[N1], cs[N1], ce[N1];
 #pragma unroll
@@ -319,73 +407,77 @@ __device__ __forceinline__ void dcgs_chunk(long long n2, int j, int c0, const fl
             ff_madd(vv.x, vv.y, ww.x, ww.y, ds, de);
             ff_madd(vv.z, vv.w, ww.z, ww.w, ds, de);
         }
-        float4 q[N1];
+        constexpr int LB = 8;   // columns loaded at once
 #pragma unroll
-        for (int c = 0; c < NC; ++c) q[c] = Q[(c0 + c) * ld2 + r];
+        for (int b = 0; b < NC; b += LB) {
+            float4 q[LB];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            ff_madd(q[c].x, q[c].y, vv.x, vv.y, ss[c], se[c]);
-            ff_madd(q[c].z, q[c].w, vv.z, vv.w, ss[c], se[c]);
-            ff_madd(q[c].x, q[c].y, ww.x, ww.y, cs[c], ce[c]);
-            ff_madd(q[c].z, q[c].w, ww.z, ww.w, cs[c], ce[c]);
+            for (int c = 0; c < LB; ++c)
+                if (b + c < NC) q[c] = Q[(c0 + b + c) * ld2 + r];
+#pragma unroll
+            for (int c = 0; c < LB; ++c)
+                if (b + c < NC) {
+                    const int k = b + c;
+                    ff_madd(q[c].x, q[c].y, vv.x, vv.y, ss[k], se[k]);
+                    ff_madd(q[c].z, q[c].w, vv.z, vv.w, ss[k], se[k]);
+                    ff_madd(q[c].x, q[c].y, ww.x, ww.y, cs[k], ce[k]);
+                    ff_madd(q[c].z, q[c].w, ww.z, ww.w, cs[k], ce[k]);
+                }
         }
     }
     if constexpr (NC > 0) {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        constexpr int P = NC > 8 ? 32 : NC > 4 ? 16 : NC > 2 ? 8 : NC > 1 ? 4 : 2;   // 2 NC sums, padded with zeros
+        constexpr int SH = P == 32 ? 0 : P == 16 ? 1 : P == 8 ? 2 : P == 4 ? 3 : 4;
+        float2 t[P];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const double t1 = ff_warp_sum(ss[c], se[c]);
-            const double t2 = ff_warp_sum(cs[c], ce[c]);
-            if (lane == 0) {
-                red[wid][c] = t1;
-                red[wid][8 + c] = t2;
-            }
+        for (int e = 0; e < P / 2; ++e) {
+            t[e] = e < NC ? ff_norm(ss[e < NC ? e : 0], se[e < NC ? e : 0]) : make_float2(0.f, 0.f);
+            t[P / 2 + e] = e < NC ? ff_norm(cs[e < NC ? e : 0], ce[e < NC ? e : 0]) : make_float2(0.f, 0.f);
         }
+        const double s = ff_warp_sums<P>(t);
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        if ((lane & ((1 << SH) - 1)) == 0) red[wid][lane >> SH] = s;
         __syncthreads();
         if (threadIdx.x < 2 * NC) {
             const bool isv = threadIdx.x < NC;
             const int c = isv ? threadIdx.x : threadIdx.x - NC;
-            double t = 0.0;
-            for (int k = 0; k < kThreads / 32; ++k) t += red[k][isv ? c : 8 + c];
-            partial[(long long)blockIdx.x * ldp + (isv ? c0 + c : j + c0 + c)] = t;
+            double tot = 0.0;
+            for (int k = 0; k < kThreads / 32; ++k) tot += red[k][isv ? c : P / 2 + c];
+            partial[(long long)(isv ? c0 + c : j + c0 + c) * ldp + blockIdx.x] = tot;
         }
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 3) k_ff_dcgs_dots(long long n2, int j, const float4* __restrict__ Q,
+__global__ void __launch_bounds__(kThreads, 2) k_ff_dcgs_dots(long long n2, int j, const float4* __restrict__ Q,
                                                               long long ld2, const float4* __restrict__ v,
                                                               const float4* __restrict__ w, double* __restrict__ partial,
                                                               int ldp) {
-    __shared__ double red2[kThreads / 32][2];
+    __shared__ double red[kThreads / 32][32];
     float as = 0.f, ae = 0.f, ds = 0.f, de = 0.f;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int c0 = 0; c0 < (j > 0 ? j : 1); c0 += 8) {
-        const int nc = j > 0 ? min(8, j - c0) : 0;
-        const bool first = c0 == 0;
+    const int chunks = (j + kDotCols - 1) / kDotCols;   // of nearly equal size
+    int c0 = 0;
+    for (int k = 0; k < (chunks > 0 ? chunks : 1); ++k) {
+        const int nc = chunks > 0 ? (j - c0 + chunks - k - 1) / (chunks - k) : 0;
+        const bool first = k == 0;
         switch (nc) {
-            case 0: dcgs_chunk<0>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            case 1: dcgs_chunk<1>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            case 2: dcgs_chunk<2>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            case 3: dcgs_chunk<3>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            case 4: dcgs_chunk<4>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            case 5: dcgs_chunk<5>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            case 6: dcgs_chunk<6>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            case 7: dcgs_chunk<7>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp); break;
-            default: dcgs_chunk<8>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp);
+#define DM_CHUNK(NC) \
+    case NC: dcgs_chunk<NC>(n2, j, c0, Q, ld2, v, w, first, as, ae, ds, de, partial, ldp, red); break;
+            DM_CHUNK(0) DM_CHUNK(1) DM_CHUNK(2) DM_CHUNK(3) DM_CHUNK(4) DM_CHUNK(5) DM_CHUNK(6) DM_CHUNK(7) DM_CHUNK(8)
+            DM_CHUNK(9) DM_CHUNK(10) DM_CHUNK(11) DM_CHUNK(12) DM_CHUNK(13) DM_CHUNK(14) DM_CHUNK(15) DM_CHUNK(16)
+#undef DM_CHUNK
         }
+        c0 += nc;
     }
-    const double ta = ff_warp_sum(as, ae);
-    const double td = ff_warp_sum(ds, de);
-    if (lane == 0) {
-        red2[wid][0] = ta;
-        red2[wid][1] = td;
-    }
+    float2 t[2] = {ff_norm(as, ae), ff_norm(ds, de)};
+    const double s = ff_warp_sums<2>(t);
+    if ((lane & 15) == 0) red[wid][lane >> 4] = s;
     __syncthreads();
     if (threadIdx.x < 2) {
-        double t = 0.0;
-        for (int k = 0; k < kThreads / 32; ++k) t += red2[k][threadIdx.x];
-        partial[(long long)blockIdx.x * ldp + 2 * j + threadIdx.x] = t;
+        double tot = 0.0;
+        for (int k = 0; k < kThreads / 32; ++k) tot += red[k][threadIdx.x];
+        partial[(long long)(2 * j + threadIdx.x) * ldp + blockIdx.x] = tot;
     }
 }
 
@@ -552,9 +644,9 @@ void reducer_init(Reducer& r, int max_cols) {
     note_allocation();
     DM_CUDA(cudaMalloc(&r.partial, sizeof(double) * (size_t)r.cap_blocks * max_cols));
     note_allocation();
-    DM_CUDA(cudaMalloc(&r.result, sizeof(double) * (size_t)max_cols));
+    DM_CUDA(cudaMalloc(&r.result, sizeof(double) * (size_t)(2 * max_cols + 8)));   // and dcgs_step's coefficients
     note_allocation();
-    DM_CUDA(cudaMallocHost(&r.host, sizeof(double) * (size_t)max_cols));
+    DM_CUDA(cudaMallocHost(&r.host, sizeof(double) * (size_t)(max_cols + 8)));
 }
 void reducer_free(Reducer& r) {
     if (r.partial) cudaFree(r.partial);
@@ -569,7 +661,7 @@ void mdot(Reducer& red, const Domain& d, int m, const double* V, long long ld, c
     const int nb = blocks_for(d, k_mdot_partial);
     launch_b("k_mdot_partial", 8.0 * d.live() * (m + 1 + (w ? 1 : 0)), k_mdot_partial, nb, kThreads, 0, s, d, m, V,
              ld, x, w, red.partial, red.max_cols, 0);
-    launch("k_mdot_final", k_mdot_final, (m + 7) / 8, 256, 0, s, nb, m, red.partial, red.max_cols, red.result);
+    launch("k_mdot_final", k_mdot_final, (m + 7) / 8, 256, 0, s, nb, m, red.partial, red.max_cols, 1, red.result);
     DM_CUDA(cudaMemcpyAsync(red.host, red.result, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
     for (int c = 0; c < m; ++c) host_out[c] = red.host[c];
@@ -581,7 +673,7 @@ double dot_list(Reducer& red, long long n, const int* list, const double* x, con
     const int nb = (int)std::max<long long>(1, std::min<long long>((n + kThreads - 1) / kThreads, kMaxBlocks));
     launch_b("k_dot_list", (w ? 28.0 : 20.0) * (double)n, k_dot_list, nb, kThreads, 0, s, n, list, x, y, w,
              red.partial);
-    launch("k_mdot_final", k_mdot_final, 1, 256, 0, s, nb, 1, red.partial, 1, red.result);
+    launch("k_mdot_final", k_mdot_final, 1, 256, 0, s, nb, 1, red.partial, 1, 1, red.result);
     DM_CUDA(cudaMemcpyAsync(red.host, red.result, sizeof(double), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
     return red.host[0];
@@ -593,7 +685,7 @@ void mdot_self(Reducer& red, const Domain& d, int m, const double* V, long long 
     const int nb = blocks_for(d, k_mdot_partial);
     launch_b("k_mdot_partial", 8.0 * d.live() * (m + 1 + (w ? 1 : 0)), k_mdot_partial, nb, kThreads, 0, s, d, m, V,
              ld, x, w, red.partial, red.max_cols, 1);
-    launch("k_mdot_final", k_mdot_final, (m + 1 + 7) / 8, 256, 0, s, nb, m + 1, red.partial, red.max_cols, red.result);
+    launch("k_mdot_final", k_mdot_final, (m + 1 + 7) / 8, 256, 0, s, nb, m + 1, red.partial, red.max_cols, 1, red.result);
     DM_CUDA(cudaMemcpyAsync(red.host, red.result, sizeof(double) * (m + 1), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
     for (int c = 0; c < m; ++c) host_out[c] = red.host[c];
@@ -608,7 +700,7 @@ double maxpy_norm(Reducer& red, const Domain& d, int m, const double* V, long lo
     double* part = red.partial + (size_t)red.cap_blocks * (red.max_cols - 1);
     launch_b("k_maxpy_norm", 8.0 * d.live() * (m + 2 + (w ? 1 : 0)), k_maxpy_norm, nb, kThreads, 0, s, d, m, V, ld,
              red.result, x, w, part);
-    launch("k_mdot_final", k_mdot_final, 1, 256, 0, s, nb, 1, part, 1, red.result + red.max_cols - 1);
+    launch("k_mdot_final", k_mdot_final, 1, 256, 0, s, nb, 1, part, 1, 1, red.result + red.max_cols - 1);
     DM_CUDA(cudaMemcpyAsync(red.host, red.result + red.max_cols - 1, sizeof(double), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
     return red.host[0];
@@ -683,8 +775,8 @@ void dcgs_dots(Reducer& red, const Domain& d, int j, const float2* Q, long long 
     // j finished basis vectors, v and w: float-float, 8 bytes an entry
     launch_b("k_ff_dcgs_dots", 8.0 * d.live() * (j + 2), k_ff_dcgs_dots, nb, kThreads, 0, s, n2, j,
              reinterpret_cast<const float4*>(Q), ld / 2, reinterpret_cast<const float4*>(v),
-             reinterpret_cast<const float4*>(w), red.partial, red.max_cols);
-    launch("k_mdot_final", k_mdot_final, (m + 7) / 8, 256, 0, s, nb, m, red.partial, red.max_cols, red.result);
+             reinterpret_cast<const float4*>(w), red.partial, red.cap_blocks);
+    launch("k_mdot_final", k_mdot_final, (m + 7) / 8, 256, 0, s, nb, m, red.partial, 1, red.cap_blocks, red.result);
     DM_CUDA(cudaMemcpyAsync(red.host, red.result, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
     for (int c = 0; c < m; ++c) host_out[c] = red.host[c];
@@ -705,11 +797,34 @@ double dcgs_update(Reducer& red, const Domain& d, int j, const float2* Q, long l
     launch_b("k_ff_dcgs_update", 8.0 * d.live() * (j + 4), k_ff_dcgs_update, nb, kThreads, 0, s, n2, j,
              reinterpret_cast<const float4*>(Q), ld / 2, (const double*)red.result, reinterpret_cast<float4*>(v),
              reinterpret_cast<const float4*>(w), reinterpret_cast<float4*>(out), part);
-    launch("k_mdot_final", k_mdot_final, 1, 256, 0, s, nb, 1, part, 1, red.result + red.max_cols - 1);
+    launch("k_mdot_final", k_mdot_final, 1, 256, 0, s, nb, 1, part, 1, 1, red.result + red.max_cols - 1);
     DM_CUDA(cudaMemcpyAsync(red.host, red.result + red.max_cols - 1, sizeof(double), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
     return red.host[0];
 }
+void dcgs_step(Reducer& red, const Domain& d, int j, const float2* Q, long long ld, float2* v, const float2* w,
+               float2* out, double* host_out, cudaStream_t s) {
+    const int m = 2 * j + 2;
+    DM_REQUIRE(j >= 0 && j <= 120 && m < red.max_cols, DM_ERR_INVALID_ARG, "dcgs: too many columns");
+    DM_REQUIRE(d.tiles == nullptr && d.len() % 2 == 0 && ld % 2 == 0, DM_ERR_INVALID_ARG,
+               "dcgs: compact vectors need an even length and stride");
+    const long long n2 = d.len() / 2;
+    const float4* q4 = reinterpret_cast<const float4*>(Q);
+    const float4* w4 = reinterpret_cast<const float4*>(w);
+    double* coef = red.result + red.max_cols + 8;
+    int nb = std::min(pair_blocks(n2, k_ff_dcgs_dots), red.cap_blocks);
+    launch_b("k_ff_dcgs_dots", 8.0 * d.live() * (j + 2), k_ff_dcgs_dots, nb, kThreads, 0, s, n2, j, q4, ld / 2,
+             reinterpret_cast<const float4*>(v), w4, red.partial, red.cap_blocks);
+    launch("k_dcgs_coef", k_dcgs_coef, 1, 1024, 0, s, nb, j, (const double*)red.partial, red.cap_blocks, red.result, coef);
+    nb = std::min(pair_blocks(n2, k_ff_dcgs_update), red.cap_blocks);
+    launch_b("k_ff_dcgs_update", 8.0 * d.live() * (j + 4), k_ff_dcgs_update, nb, kThreads, 0, s, n2, j, q4, ld / 2,
+             (const double*)coef, reinterpret_cast<float4*>(v), w4, reinterpret_cast<float4*>(out), red.partial);
+    launch("k_mdot_final", k_mdot_final, 1, 32, 0, s, nb, 1, (const double*)red.partial, 1, 1, red.result + m + 2);
+    DM_CUDA(cudaMemcpyAsync(red.host, red.result, sizeof(double) * (m + 3), cudaMemcpyDeviceToHost, s));
+    DM_CUDA(cudaStreamSynchronize(s));
+    for (int c = 0; c < m + 3; ++c) host_out[c] = red.host[c];
+}
+
 void vgemm(const Domain& d, int m, int p, const double* V, long long ld, const double* Y_dev, int ldy, double* out,
            long long ldo, cudaStream_t s) {
     const size_t sm = sizeof(double) * (size_t)m * p;

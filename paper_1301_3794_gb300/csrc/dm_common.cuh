@@ -597,6 +597,11 @@ void dcgs_dots(Reducer& red, const Domain& d, int j, const float2* Q, long long 
                double* host_out, cudaStream_t s);
 double dcgs_update(Reducer& red, const Domain& d, int j, const float2* Q, long long ld, const double* coef_host,
                    float2* v, const float2* w, float2* out, cudaStream_t s);
+// One iteration's orthogonalisation, both passes with the coefficients formed on
+// the device: host_out = the 2j + 2 dots, b = |v - Q s|, h = the new vector's
+// component along the finished v, |out|^2 (one sync; nothing to use when b <= 0)
+void dcgs_step(Reducer& red, const Domain& d, int j, const float2* Q, long long ld, float2* v, const float2* w,
+               float2* out, double* host_out, cudaStream_t s);
 double maxpy_norm(Reducer& red, const Domain& d, int m, const double* V, long long ld, double* x, const double* w,
                   cudaStream_t s);
 // x -= sum_c h[c] V[c*ld + r]    (h host array, m <= max_cols)
