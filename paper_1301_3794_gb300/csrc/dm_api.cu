@@ -134,7 +134,14 @@ struct GeoLevel {
     // the float-float operator apply of the shifted solves (fine level only,
     // built with the first operator that asks for them)
     DBuf<float2> ffA, ffL, ffV;
-    DBuf<int> fmap, fmapc;   // padded-to-compact maps of the open faces and of the active cells
+    DBuf<int2> rowmap;       // row maps and flags of the float-float apply, and its tiles
+    DBuf<unsigned char> rowflag;
+    DBuf<int> fftiles;
+    int nfftiles = 0;
+    DBuf<int> fmapc;         // padded-to-compact map of the active cells
+    FFLevel ffl() const {
+        return FFLevel{g, ffA.get(), ffL.get(), ffV.get(), rowmap.get(), rowflag.get(), fftiles.get(), nfftiles};
+    }
     bool ff = false;
 };
 
@@ -273,22 +280,25 @@ struct OpLevel {
     long long bn_cls_copies[kNodeClasses] = {};
 };
 
-// FGMRES workspace: the Arnoldi basis V and the work vector wf in
-// float-float (see dcgs_dots), the preconditioned vectors Z and the operator
-// output w in FP64
+// FGMRES workspace: the Arnoldi basis V and the work vector wf in float-float
+// (see dcgs_dots), the operator output w in FP64, and the preconditioned vectors
+// Z, zlen entries of zsize bytes each: compact and in the V-cycle's storage type
+// (which holds them exactly) when the iterations apply the float-float operator,
+// else padded and in FP64
 struct Fgmres {
     long long n = 0, nc = 0;   // padded vector length, compact (basis) length
     int m = 0;
     DBuf<float2> V, wf;
-    DBuf<double> Z, w;
-    void ensure(long long n_, long long nc_, int m_) {
-        if (n == n_ && nc == nc_ && m >= m_) return;
+    DBuf<char> Z;
+    DBuf<double> w;
+    void ensure(long long n_, long long nc_, int m_, size_t zbytes) {   // zbytes: of one vector of Z
+        if (n == n_ && nc == nc_ && m >= m_ && Z.n >= zbytes * m_) return;
         n = n_;
         nc = nc_;
         m = m_;
         V.alloc((size_t)(m + 1) * nc);
         wf.alloc((size_t)nc);
-        Z.alloc((size_t)m * n);
+        Z.alloc(zbytes * m);
         w.alloc((size_t)n);
     }
 };
@@ -631,9 +641,10 @@ void mg_input(const Domain& D, const CompactIn& v, double scale, T* f, cudaStrea
     ff_scatter<T>(v.n, v.list, scale, v.v, f, s);
 }
 
-// z = M^-1 (scale v): one V-cycle (graph-replayed after the first call)
+// M^-1 (scale v): one V-cycle (graph-replayed after the first call); returns the
+// result, in the level-0 r buffer
 template <typename T, typename TC, typename TIn>
-void precond_vec_T(dm_operator* op, const TIn& v, double* z, double scale = 1.0) {
+const T* cycle_vec(dm_operator* op, const TIn& v, double scale = 1.0) {
     cudaStream_t s = op->ctx->stream;
     const Domain D = glv(op, 0).vdom();
     WorkLevel& w0 = op->wk[0];
@@ -653,11 +664,11 @@ void precond_vec_T(dm_operator* op, const TIn& v, double* z, double scale = 1.0)
     }
     ++op->vcalls;
     if (op->lnet && op->learned_active) learned_correct<T, TC>(op, f, r, e);
-    convert<double, T>(D, r, z, s);
+    return r;
 }
 
 template <typename T, typename TC, typename TIn>
-void precond_scal_T(dm_operator* op, const TIn& v, double* z, double scale = 1.0) {
+const T* cycle_scal(dm_operator* op, const TIn& v, double scale = 1.0) {
     cudaStream_t s = op->ctx->stream;
     const Domain D = glv(op, 0).sdom();
     WorkLevel& w0 = op->wk[0];
@@ -675,25 +686,33 @@ void precond_scal_T(dm_operator* op, const TIn& v, double* z, double scale = 1.0
         svcycle<T, TC>(op, 0, f, r);
     }
     ++op->scalls;
-    convert<double, T>(D, r, z, s);
+    return r;
 }
 
+// f(T{}, TC{}) with the V-cycle's storage and coefficient types
+template <class F>
+auto with_types(const dm_operator* op, F&& f) {
+    switch (op->mg.precision) {
+        case DM_PREC_F64: return f(double{}, double{});
+        case DM_PREC_F32: return f(float{}, float{});
+        default: return f(__nv_bfloat16{}, float{});
+    }
+}
+
+// z = M^-1 (scale v) as a padded FP64 vector
 template <typename TIn>
 void precond_vec(dm_operator* op, const TIn& v, double* z, double scale = 1.0) {
-    switch (op->mg.precision) {
-        case DM_PREC_F64: precond_vec_T<double, double>(op, v, z, scale); break;
-        case DM_PREC_F32: precond_vec_T<float, float>(op, v, z, scale); break;
-        default: precond_vec_T<__nv_bfloat16, float>(op, v, z, scale);
-    }
+    with_types(op, [&](auto t, auto tc) {
+        using T = decltype(t);
+        convert<double, T>(glv(op, 0).vdom(), cycle_vec<T, decltype(tc)>(op, v, scale), z, op->ctx->stream);
+    });
 }
-
 template <typename TIn>
 void precond_scal(dm_operator* op, const TIn& v, double* z, double scale = 1.0) {
-    switch (op->mg.precision) {
-        case DM_PREC_F64: precond_scal_T<double, double>(op, v, z, scale); break;
-        case DM_PREC_F32: precond_scal_T<float, float>(op, v, z, scale); break;
-        default: precond_scal_T<__nv_bfloat16, float>(op, v, z, scale);
-    }
+    with_types(op, [&](auto t, auto tc) {
+        using T = decltype(t);
+        convert<double, T>(glv(op, 0).sdom(), cycle_scal<T, decltype(tc)>(op, v, scale), z, op->ctx->stream);
+    });
 }
 
 void apply_vec64(dm_operator* op, int l, const double* x, double* y) {
@@ -770,22 +789,43 @@ double hessenberg_lsq(const std::vector<double>& H, int ld, int k, double beta, 
 struct NoMonitor {
     void operator()(double) const {}
 };
-// no float-float apply: the iterations apply the FP64 operator and gather
-struct NoApplyFF {
-    static constexpr bool on = false;
-    void operator()(const double*, float2*) const {}
+// The preconditioned directions of an FGMRES: how they are made, applied and
+// summed up.  zbytes: of one stored vector;
+//   step(v, scale, j, wf): z_j = M^-1 (scale v), stored, and wf = A z_j (compact float-float);
+//   add(k, y, x): x += sum_i y_i z_i for i < k.
+//
+// This one applies the FP64 operator to padded FP64 vectors and gathers.
+template <class Apply, class Prec>
+struct PaddedSteps {
+    dm_context* ctx;
+    Fgmres& ws;
+    Domain D;
+    const int* list;
+    long long nl;
+    Apply apply;
+    Prec prec;   // prec(v, scale, z)
+    size_t zbytes() const { return sizeof(double) * (size_t)D.len(); }
+    double* z(int j) const { return reinterpret_cast<double*>(ws.Z.get()) + (size_t)j * D.len(); }
+    void step(const float2* v, double scale, int j, float2* wf) const {
+        prec(v, scale, z(j));
+        apply(z(j), ws.w.get());
+        ff_gather(nl, list, 1.0, ws.w.get(), wf, ctx->stream);
+    }
+    void add(int k, const std::vector<double>& y, double* x) const {
+        std::vector<double> neg(k);
+        for (int i = 0; i < k; ++i) neg[i] = -y[i];
+        maxpy(ctx->red, D, k, z(0), D.len(), neg.data(), x, ctx->stream);
+    }
 };
 
 // monitor(ratio) is told the residual contraction of every iteration
 // The basis lives in the compact index space of `list` (the nl entries of the
 // padded domain D that can be nonzero); b, x and the operator work on D.
-// apply_ff(z, wf), when ApplyFF::on, forms the operator of an iteration
-// straight into the compact float-float vector wf; restart residuals and the
-// final check use the FP64 apply.
-template <class Apply, class Prec, class Monitor = NoMonitor, class ApplyFF = NoApplyFF>
-int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long long nl, int m, Apply apply, Prec prec,
-           const double* b, double* x, double tol, int maxit, double* relres, double abs_tol = 0.0,
-           Monitor monitor = Monitor(), ApplyFF apply_ff = ApplyFF()) {
+// Restart residuals and the final check use the FP64 apply.
+template <class Apply, class Steps, class Monitor = NoMonitor>
+int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long long nl, int m, Apply apply,
+           const Steps& steps, const double* b, double* x, double tol, int maxit, double* relres, double abs_tol = 0.0,
+           Monitor monitor = Monitor()) {
     cudaStream_t s = ctx->stream;
     const long long n = D.len();
     DM_REQUIRE(m >= 1 && 2 * m + 2 < ctx->red.max_cols, DM_ERR_INVALID_ARG, "FGMRES restart length too large");
@@ -793,14 +833,13 @@ int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long l
     // the compact vectors' length and stride, even for the two-entry passes
     // (the pad entry stays zero: nothing writes it but the update, from zeros)
     const long long nlp = (nl + 1) & ~1ll;
-    ws.ensure(n, nlp, m);
+    ws.ensure(n, nlp, m, steps.zbytes());
     // flat domain of the compact vectors
     Grid3 gc = D.g;
     gc.np = (int)nlp;
     const Domain Dc{gc, nullptr, 0, 1};
     float2* V = ws.V.get();
     float2* wf = ws.wf.get();
-    double* Z = ws.Z.get();
     double* w = ws.w.get();
     zero(x, sizeof(double) * n, s);
     // b and every residual vanish outside `list` (closed faces, inactive
@@ -832,13 +871,7 @@ int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long l
         int k = 0;                // columns of H built in this cycle
         for (int j = 0; j < m && total < maxit; ++j) {
             float2* Vj = V + (size_t)j * nlp;
-            prec(Vj, 1.0 / nu, Z + (size_t)j * n);
-            if constexpr (ApplyFF::on) {
-                apply_ff(Z + (size_t)j * n, wf);
-            } else {
-                apply(Z + (size_t)j * n, w);
-                ff_gather(nl, list, 1.0, w, wf, s);
-            }
+            steps.step(Vj, 1.0 / nu, j, wf);
             // one sweep: Q^T v, Q^T w, v.v, v.w with Q = V_0 .. V_{j-1} finished; a
             // second finishes V_j and forms the next pending vector
             dcgs_step(ctx->red, Dc, j, V, nlp, Vj, wf, V + (size_t)(j + 1) * nlp, dots.data(), s);
@@ -865,9 +898,7 @@ int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long l
         }
         if (k == 0) break;
         hessenberg_lsq(H, m, k, beta, &y);
-        std::vector<double> neg(k);
-        for (int i = 0; i < k; ++i) neg[i] = -y[i];
-        maxpy(ctx->red, D, k, Z, n, neg.data(), x, s);
+        steps.add(k, y, x);
         first = false;
         if (res * bnorm <= thr) {
             // confirm with the true residual
@@ -882,24 +913,30 @@ int fgmres(dm_context* ctx, Fgmres& ws, const Domain& D, const int* list, long l
     return total;
 }
 
-// the float-float apply of the projection's scalar iterations (fine level)
-struct FFApplyScal {
-    static constexpr bool on = true;
+// The fine level's float-float applies straight from the V-cycle's result, kept
+// compact and in its own type: no FP64 copy of it is made, and forming the
+// solution reads a fourth to an eighth of the bytes.
+template <typename T, typename TC, bool VEC>
+struct CompactSteps {
     dm_operator* op;
-    void operator()(const double* z, float2* wf) const {
+    Fgmres& ws;
+    const int* list;
+    long long nl;
+    long long ld() const { return (nl + 1) & ~1ll; }
+    size_t zbytes() const { return sizeof(T) * (size_t)ld(); }
+    T* z(int j) const { return reinterpret_cast<T*>(ws.Z.get()) + (size_t)j * ld(); }
+    void step(const float2* v, double scale, int j, float2* wf) const {
         const GeoLevel& l0 = glv(op, 0);
-        scal_apply_ff(l0.g, l0.tiles.get(), l0.ntiles, l0.ffA.get(), z, l0.fmapc.get(), wf, op->ctx->stream);
+        cudaStream_t s = op->ctx->stream;
+        const CompactIn in{v, list, nl};
+        if constexpr (VEC)
+            vec_apply_ff<T>(l0.ffl(), op->sigma, cycle_vec<T, TC>(op, in, scale), wf, z(j), s);
+        else
+            scal_apply_ff<T>(l0.g, l0.tiles.get(), l0.ntiles, l0.ffA.get(), cycle_scal<T, TC>(op, in, scale),
+                             l0.fmapc.get(), wf, z(j), s);
     }
-};
-
-// the float-float apply of the shifted solves' iterations (fine level)
-struct FFApply {
-    static constexpr bool on = true;
-    dm_operator* op;
-    void operator()(const double* z, float2* wf) const {
-        const GeoLevel& l0 = glv(op, 0);
-        vec_apply_ff(l0.g, l0.tiles.get(), l0.ntiles, l0.ffA.get(), l0.ffL.get(), l0.ffV.get(), op->sigma, z,
-                     l0.fmap.get(), wf, op->ctx->stream);
+    void add(int k, const std::vector<double>& y, double* x) const {
+        combine_list<T>(op->ctx->red, nl, list, k, z(0), ld(), y.data(), x, op->ctx->stream);
     }
 };
 
@@ -913,9 +950,6 @@ int solve_vec(dm_operator* op, const double* b, double* x, double tol, int resta
     const GeoLevel& g0 = glv(op, 0);
     const int* fl = g0.flist.get();
     const long long nfl = g0.nflist;
-    auto prec = [op, fl, nfl](const float2* in, double scale, double* out) {
-        precond_vec(op, CompactIn{in, fl, nfl}, out, scale);
-    };
     // the FP64 residual decides on the learned correction: an iteration that
     // contracts by less than 0.8 switches it off for the rest of the solve, and
     // after kLearnedStreak solves in a row that switched it off the operator
@@ -931,9 +965,16 @@ int solve_vec(dm_operator* op, const double* b, double* x, double tol, int resta
     };
     int it;
     if (op->mg.krylov_ff && g0.ff) {
-        it = fgmres(op->ctx, op->vg, n, fl, nfl, restart, apply, prec, b, x, tol, maxit, relres, 0.0, monitor, FFApply{op});
+        it = with_types(op, [&](auto t, auto tc) {
+            const CompactSteps<decltype(t), decltype(tc), true> steps{op, op->vg, fl, nfl};
+            return fgmres(op->ctx, op->vg, n, fl, nfl, restart, apply, steps, b, x, tol, maxit, relres, 0.0, monitor);
+        });
     } else {
-        it = fgmres(op->ctx, op->vg, n, fl, nfl, restart, apply, prec, b, x, tol, maxit, relres, 0.0, monitor);
+        auto prec = [op, fl, nfl](const float2* in, double scale, double* out) {
+            precond_vec(op, CompactIn{in, fl, nfl}, out, scale);
+        };
+        const PaddedSteps<decltype(apply), decltype(prec)> steps{op->ctx, op->vg, n, fl, nfl, apply, prec};
+        it = fgmres(op->ctx, op->vg, n, fl, nfl, restart, apply, steps, b, x, tol, maxit, relres, 0.0, monitor);
     }
     if (fell_back) {
         ++op->learned_fallbacks;
@@ -971,15 +1012,20 @@ int project(dm_operator* op, const double* x, double* y, double tol) {
     auto apply = [op](const double* in, double* out) { apply_scal64(op, 0, in, out); };
     const int* cl = g0.clist.get();
     const long long ncl = g0.nclist;
-    auto prec = [op, cl, ncl](const float2* in, double scale, double* out) {
-        precond_scal(op, CompactIn{in, cl, ncl}, out, scale);
-    };
     double rr = 0.0;
-    const int it = (op->mg.krylov_ff && g0.ff)
-                       ? fgmres(op->ctx, op->sg, nc, cl, ncl, 40, apply, prec, sv, phi, tol, kProjMaxit, &rr,
-                                tol * xscale, NoMonitor(), FFApplyScal{op})
-                       : fgmres(op->ctx, op->sg, nc, cl, ncl, 40, apply, prec, sv, phi, tol, kProjMaxit, &rr,
-                                tol * xscale);
+    int it;
+    if (op->mg.krylov_ff && g0.ff) {
+        it = with_types(op, [&](auto t, auto tc) {
+            const CompactSteps<decltype(t), decltype(tc), false> steps{op, op->sg, cl, ncl};
+            return fgmres(op->ctx, op->sg, nc, cl, ncl, 40, apply, steps, sv, phi, tol, kProjMaxit, &rr, tol * xscale);
+        });
+    } else {
+        auto prec = [op, cl, ncl](const float2* in, double scale, double* out) {
+            precond_scal(op, CompactIn{in, cl, ncl}, out, scale);
+        };
+        const PaddedSteps<decltype(apply), decltype(prec)> steps{op->ctx, op->sg, nc, cl, ncl, apply, prec};
+        it = fgmres(op->ctx, op->sg, nc, cl, ncl, 40, apply, steps, sv, phi, tol, kProjMaxit, &rr, tol * xscale);
+    }
     dm_sub_grad(g0.g, g0.A.get(), x, phi, y, g0.tiles.get(), g0.ntiles, s);
     return it;
 }
@@ -1272,12 +1318,25 @@ void setup_operator(dm_operator* op) {
             g0.ffA = DBuf<float2>(n3);
             g0.ffL = DBuf<float2>(n3);
             g0.ffV = DBuf<float2>(g0.g.np);
-            g0.fmap = DBuf<int>(n3);
             note_allocation();
             to_ff(n3, g0.A.get(), g0.ffA.get(), s);
             to_ff(n3, g0.L.get(), g0.ffL.get(), s);
             to_ff(g0.g.np, g0.invV.get(), g0.ffV.get(), s);
-            compact_map(n3, g0.flist.get(), g0.nflist, g0.fmap.get(), s);
+            {
+                const int nrow = row_count(g0.g);
+                DBuf<int> fmap(n3, false), cnt(1);
+                compact_map(n3, g0.flist.get(), g0.nflist, fmap.get(), s);
+                g0.rowmap = DBuf<int2>(3 * (size_t)nrow, false);
+                g0.rowflag = DBuf<unsigned char>(nrow, false);
+                row_maps(g0.g, g0.A.get(), g0.L.get(), g0.invV.get(), fmap.get(), g0.rowmap.get(), g0.rowflag.get(), s);
+                int sy, sz;
+                stencil_shape_dims(3, sy, sz);   // 32 x 8 x 8
+                const int nt = ((g0.g.nx + TX) / TX) * ((g0.g.ny + sy) / sy) * ((g0.g.nz + sz) / sz);
+                DBuf<int> flags(nt, false);
+                g0.fftiles = DBuf<int>(nt, false);
+                g0.nfftiles = geom_tiles_shape(g0.g, sy, sz, g0.A.get(), g0.active.get(), g0.fftiles.get(), flags.get(),
+                                               cnt.get(), s);
+            }
             g0.fmapc = DBuf<int>(g0.g.np);
             compact_map(g0.g.np, g0.clist.get(), g0.nclist, g0.fmapc.get(), s);
             Sync::stream(s);
@@ -1852,8 +1911,7 @@ dm_status dm_operator_apply_ff(dm_operator* op, const double* x, double* y, int 
         DBuf<double> xp(n3), yp(n3);
         DBuf<float2> wf(std::max(g0.nflist, 1));
         faces_in(op, 0, x, on_device, xp.get());
-        vec_apply_ff(g0.g, g0.tiles.get(), g0.ntiles, g0.ffA.get(), g0.ffL.get(), g0.ffV.get(), op->sigma, xp.get(),
-                     g0.fmap.get(), wf.get(), s);
+        vec_apply_ff<double>(g0.ffl(), op->sigma, xp.get(), wf.get(), nullptr, s);
         zero(yp.get(), sizeof(double) * n3, s);
         ff_scatter<double>(g0.nflist, g0.flist.get(), 1.0, wf.get(), yp.get(), s);
         faces_out(op, 0, yp.get(), y, on_device);

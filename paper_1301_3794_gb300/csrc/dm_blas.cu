@@ -193,6 +193,20 @@ __global__ void k_maxpy(Domain d, int m, const double* __restrict__ V, long long
     });
 }
 
+template <typename T>
+__global__ void k_combine_list(long long n, const int* __restrict__ list, int m, const T* __restrict__ Z, long long ld,
+                               const double* __restrict__ h, double* __restrict__ x) {
+    __shared__ double hs[128];
+    for (int c = threadIdx.x; c < m; c += blockDim.x) hs[c] = h[c];
+    __syncthreads();
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        double acc = 0.0;
+#pragma unroll 8
+        for (int c = 0; c < m; ++c) acc += hs[c] * (double)to_c(Z[c * ld + i]);
+        x[list[i]] += acc;
+    }
+}
+
 __global__ void k_vgemm(Domain d, int m, int p, const double* __restrict__ V, long long ld,
                         const double* __restrict__ Y, int ldy, double* __restrict__ out, long long ldo) {
     extern __shared__ double Ys[];
@@ -763,6 +777,25 @@ int pair_blocks(long long n2, K kernel) {
     const long long need = (n2 + kThreads - 1) / kThreads;
     return (int)std::max<long long>(1, std::min<long long>(need, 152ll * std::max(per_sm, 1)));
 }
+
+template <typename T>
+void combine_list(Reducer& red, long long n, const int* list, int m, const T* Z, long long ld, const double* h_host,
+                  double* x, cudaStream_t s) {
+    DM_REQUIRE(m >= 1 && m <= 128 && m <= red.max_cols, DM_ERR_INVALID_ARG, "combine: too many columns");
+    // h through the pinned buffer: its last use was waited for
+    for (int c = 0; c < m; ++c) red.host[c] = h_host[c];
+    DM_CUDA(cudaMemcpyAsync(red.result, red.host, sizeof(double) * m, cudaMemcpyHostToDevice, s));
+    const int nb = (int)std::max<long long>(1, std::min<long long>((n + kThreads - 1) / kThreads, 152 * 8));
+    launch_b("k_combine_list", (double)n * (20.0 + (double)m * sizeof(T)), k_combine_list<T>, nb, kThreads, 0, s, n, list, m,
+             Z, ld, (const double*)red.result, x);
+    DM_CUDA(cudaStreamSynchronize(s));   // the buffer is free again
+}
+template void combine_list<double>(Reducer&, long long, const int*, int, const double*, long long, const double*, double*,
+                                   cudaStream_t);
+template void combine_list<float>(Reducer&, long long, const int*, int, const float*, long long, const double*, double*,
+                                  cudaStream_t);
+template void combine_list<__nv_bfloat16>(Reducer&, long long, const int*, int, const __nv_bfloat16*, long long,
+                                          const double*, double*, cudaStream_t);
 
 void dcgs_dots(Reducer& red, const Domain& d, int j, const float2* Q, long long ld, const float2* v, const float2* w,
                double* host_out, cudaStream_t s) {

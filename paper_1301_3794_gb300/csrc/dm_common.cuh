@@ -484,16 +484,29 @@ void vec_apply_natural(const VecOp<double, double>& op, const double* x, double*
 constexpr int kCertSums = 6;
 void vec_cert_sums(const VecOp<double, double>& op, bool natural, int n, const double* x, long long stride,
                    const double* k2, double* part, double* out, cudaStream_t s);
-// (K - sigma A) x in float-float into the compact vector out (out[cmap[q]] for
-// the open faces q), over the level's 32 x 4 x 2 active tiles; A, L, invV:
-// float-float copies of the level's coefficients (to_ff)
-void vec_apply_ff(const Grid3& g, const int* tiles, int ntiles, const float2* A, const float2* L, const float2* invV,
-                  double sigma, const double* x, const int* cmap, float2* out, cudaStream_t s);
+// (K - sigma A) x in float-float into the compact vector out (the open faces in
+// ascending order), x's own entries there into zc (nullptr: not wanted)
+struct FFLevel {
+    Grid3 g;
+    const float2 *A, *L, *invV;       // float-float copies of the level's coefficients (to_ff)
+    const int2* rowmap;               // row_maps
+    const unsigned char* rowflag;
+    const int* tiles;                 // 32 x 8 x 8 tiles
+    int ntiles;
+};
+inline int row_count(const Grid3& g) { return tiles_x(g) * (g.ny + 1) * (g.nz + 1); }
+// rowmap: 3 row_count entries, rowflag: row_count; cmap: compact_map of the open faces
+void row_maps(const Grid3& g, const double* A, const double* L, const double* invV, const int* cmap, int2* rowmap,
+              unsigned char* rowflag, cudaStream_t s);
+template <typename T>
+void vec_apply_ff(const FFLevel& f, double sigma, const T* x, float2* out, T* zc, cudaStream_t s);
 void to_ff(long long n, const double* a, float2* out, cudaStream_t s);
 // D A D^T x in float-float into the compact vector out (out[cmap[p]] for the
-// active cells p), over the level's active tiles; A: float-float face fractions
-void scal_apply_ff(const Grid3& g, const int* tiles, int ntiles, const float2* A, const double* x, const int* cmap,
-                   float2* out, cudaStream_t s);
+// active cells p), x's entries into zc alike, over the level's active tiles; A:
+// float-float face fractions
+template <typename T>
+void scal_apply_ff(const Grid3& g, const int* tiles, int ntiles, const float2* A, const T* x, const int* cmap,
+                   float2* out, T* zc, cudaStream_t s);
 // cmap[q] = position of q in the ascending list (nl entries), -1 elsewhere (n3 entries)
 void compact_map(long long n3, const int* list, int nl, int* cmap, cudaStream_t s);
 void vec_diagonal(const Grid3& g, const double* A, const double* L, const double* invV, double sigma, double* d,
@@ -604,6 +617,11 @@ void dcgs_step(Reducer& red, const Domain& d, int j, const float2* Q, long long 
                float2* out, double* host_out, cudaStream_t s);
 double maxpy_norm(Reducer& red, const Domain& d, int m, const double* V, long long ld, double* x, const double* w,
                   cudaStream_t s);
+// x[list[i]] += sum_c h[c] Z[c*ld + i] over compact vectors of storage type T, in
+// FP64 (h host array, m <= max_cols)
+template <typename T>
+void combine_list(Reducer& red, long long n, const int* list, int m, const T* Z, long long ld, const double* h_host,
+                  double* x, cudaStream_t s);
 // x -= sum_c h[c] V[c*ld + r]    (h host array, m <= max_cols)
 void maxpy(Reducer& red, const Domain& d, int m, const double* V, long long ld, const double* h_host, double* x,
            cudaStream_t s);

@@ -788,141 +788,292 @@ __global__ void k_sub_grad(Grid3 g, const double* __restrict__ A, const double* 
     y[2 * N + p] = A[2 * N + p] > 0.0 ? x[2 * N + p] - (phi[p - Z] - ph) * g.rhz : 0.0;
 }
 
+// Entries of a Krylov vector in float-float arithmetic: an FP64 vector splits
+// into two FP32 numbers, an FP32 or BF16 one (a V-cycle's result) is one, whose
+// differences and products cost a third of the general ones and are as exact.
+struct FFWide {
+    using V = ffv;
+    static __device__ __forceinline__ V zero() { return ff_zero(); }
+    static __device__ __forceinline__ V load(const double* p) { return ff_from_double(*p); }
+    static __device__ __forceinline__ ffv sub(V a, V b) { return a - b; }
+    static __device__ __forceinline__ ffv mul(ffv c, V b) { return c * b; }
+    static __device__ __forceinline__ ffv wide(V b) { return b; }
+};
+template <typename T>
+struct FFNarrow {
+    using V = float;
+    static __device__ __forceinline__ V zero() { return 0.f; }
+    static __device__ __forceinline__ V load(const T* p) { return to_c(*p); }
+    static __device__ __forceinline__ ffv sub(V a, V b) {
+        ffv r;
+        ff_two_sum(a, -b, r.hi, r.lo);
+        return r;
+    }
+    static __device__ __forceinline__ ffv mul(ffv c, V b) {
+        const float p = __fmul_rn(c.hi, b);
+        return ff_fast(p, fmaf(c.lo, b, fmaf(c.hi, b, -p)));
+    }
+    static __device__ __forceinline__ ffv wide(V b) { return ffv{b, 0.f}; }
+};
+template <typename T> struct FFOps { using type = FFNarrow<T>; };
+template <> struct FFOps<double> { using type = FFWide; };
+
 // (K - sigma A) x in float-float on the FP32 pipes, for the shifted solves'
-// Krylov vectors: x is FP64, the coefficients are float-float copies of the
-// level's FP64 A, L, 1/V, and every product and sum is a float-float operation
-// (about 48 significant bits).  The result goes straight into the compact
-// float-float vector of the FGMRES basis: out[cmap[q]] for every open face q.
-// Same tiles and the same sharing of edge curls and cell divergences through
-// shared memory as k_vec_stencil_tiled (32 x 4 x 2 tiles); in addition the
-// block splits the x it needs (the tile with a one-node ring) into float-float
-// once, into shared memory, so that each value is converted once per block.
-__global__ void __launch_bounds__(TX * TY * TZ) k_vec_apply_ff(Grid3 g, const float2* __restrict__ A,
-                                                               const float2* __restrict__ L,
-                                                               const float2* __restrict__ invV, ffv rdx, ffv rdy,
-                                                               ffv rdz, ffv sigma, const double* __restrict__ x,
-                                                               const int* __restrict__ cmap, float2* __restrict__ out,
-                                                               const int* __restrict__ tiles) {
-    constexpr int SY = TY, SZ = TZ;
-    constexpr int BXW = TX + 2, BYW = SY + 2, BZW = SZ + 2, NB = BXW * BYW * BZW;   // x: i0-1 .. i0+TX (j, k alike)
-    constexpr int PSI_X = TX + 1, PSI_Y = SY + 1, PSI_Z = SZ + 1;
-    constexpr int EX_X = TX, EX_Y = SY + 1, EX_Z = SZ + 1;
-    constexpr int EY_X = TX + 1, EY_Y = SY, EY_Z = SZ + 1;
-    constexpr int EZ_X = TX + 1, EZ_Y = SY + 1, EZ_Z = SZ;
-    constexpr int N_PSI = PSI_X * PSI_Y * PSI_Z, N_EX = EX_X * EX_Y * EX_Z, N_EY = EY_X * EY_Y * EY_Z,
-                  N_EZ = EZ_X * EZ_Y * EZ_Z;
-    constexpr int NT = TX * SY * SZ;
-    __shared__ ffv s_b[3][NB];
-    __shared__ ffv s_psi[N_PSI], s_ex[N_EX], s_ey[N_EY], s_ez[N_EZ];
+// Krylov vectors: the coefficients are float-float copies of the level's FP64
+// A, L, 1/V, and every product and sum is a float-float operation (about 48
+// significant bits).  The result goes straight into the compact float-float
+// vector of the FGMRES basis, and x's entries on the open faces into the compact
+// vector zc (nullptr: not wanted) the solution is later formed from.
+// The FP32 pipes bound it, so the work per node is kept down: a TX x SY block
+// marches KZ planes along z as k_vec_stencil_march does (each curl and
+// divergence is formed once but for the blocks' rims), a face's flux A x is
+// formed once, where x is loaded, and with one spacing for all axes (CUBE) the
+// factors 1/h are applied once at the end.  rowflag bit 0 marks the 32-node rows
+// whose coefficients are all 1 (inside the vacuum): their coefficients are
+// neither read nor multiplied by.  rowmap[c][row] holds the compact index of the
+// row's first open face of component c and the mask of its open faces.
+// Measured (FP32 x; 32 x 4 x 2 tiles, an FP64 copy of x and face maps of 4 bytes
+// an entry before): 192^3 ellipsoid 220 us and 33 for the copy -> 168 us; error
+// against 64 bits on a 128^3 field 1.4e-14 before and after (2-norm, relative).
+constexpr int kFFY = 8, kFFZ = 8;
+template <typename T, bool CUBE>
+__global__ void __launch_bounds__(TX * kFFY, 3) k_vec_apply_ff(
+    Grid3 g, const float2* __restrict__ A, const float2* __restrict__ L, const float2* __restrict__ invV, ffv rdx, ffv rdy,
+    ffv rdz, ffv r2, ffv sigma, const T* __restrict__ x, const int2* __restrict__ rowmap,
+    const unsigned char* __restrict__ rowflag, float2* __restrict__ out, T* __restrict__ zc, const int* __restrict__ tiles) {
+    using O = typename FFOps<T>::type;
+    using B = typename O::V;
+    constexpr int SY = kFFY, KZ = kFFZ;
+    constexpr int RW = TX + 2, RH = SY + 2, RP = RW * RH;
+    constexpr int NT = TX * SY, W1 = TX + 1;
+    constexpr int NRH = 2 * TX + 2 * RH, NPH = W1 + SY, NZH = W1 + SY, NXH = TX, NYH = SY;
+    static_assert(NRH <= NT && NPH + NZH + NXH + NYH <= NT, "one border entry per thread");
+    __shared__ B s_b[2][3][RP];             // x of two planes with a one-node ring
+    __shared__ ffv s_f[2][3][RP];           // the fluxes A x
+    __shared__ ffv s_ex[2][(SY + 1) * TX], s_ey[2][SY * W1], s_ez[(SY + 1) * W1], s_psi[(SY + 1) * W1];
     const int t = tiles[blockIdx.x];
     const int nti = (g.nx + TX) / TX, ntj = (g.ny + SY) / SY;
-    const int i0 = (t % nti) * TX, j0 = ((t / nti) % ntj) * SY, k0 = (t / (nti * ntj)) * SZ;
-    const int X = 1, Y = g.sx, Z = g.sxy, N = g.np;
-    const int tid = threadIdx.x + TX * (threadIdx.y + SY * threadIdx.z);
-    // x over the box; the padded layout holds nodes -1 .. n+1 along each axis
-    // (zero where no face exists), and nodes past n+1 are taken as zero
-    for (int e = tid; e < NB; e += NT) {
-        const int li = e % BXW, lj = (e / BXW) % BYW, lk = e / (BXW * BYW);
-        const int i = i0 - 1 + li, j = j0 - 1 + lj, k = k0 - 1 + lk;
-        const bool in = i <= g.nx + 1 && j <= g.ny + 1 && k <= g.nz + 1;
-        const int p = in ? g.idx(i, j, k) : 0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) s_b[c][e] = in ? ff_from_double(x[c * N + p]) : ff_zero();
+    const int ti = t % nti;
+    const int i0 = ti * TX, j0 = ((t / nti) % ntj) * SY, k0 = (t / (nti * ntj)) * KZ;
+    const int kend = min(k0 + KZ - 1, g.nz);
+    const int N = g.np, Z = g.sxy, ilim = g.nx + 1, jlim = g.ny + 1;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = tx + TX * ty;
+    const int i = i0 + tx, j = j0 + ty;
+    const bool inb = i <= ilim && j <= jlim, own = i <= g.nx && j <= g.ny;
+    const int p0 = g.idx(i, j, 0);
+    const int rown = (ty + 1) * RW + tx + 1;
+    // this warp's row of plane k: row0 + k * rowz
+    const int rowz = (g.ny + 1) * nti, row0 = j * nti + ti, nrow = rowz * (g.nz + 1);
+    // ring border entry of this thread, and its border entry of the divergence / curl tiles
+    // (roles and places as in k_vec_stencil_march)
+    int hli = 0, hlj = 0;
+    if (tid < TX) { hli = tid + 1; hlj = 0; }
+    else if (tid < 2 * TX) { hli = tid - TX + 1; hlj = RH - 1; }
+    else if (tid < 2 * TX + RH) { hli = 0; hlj = tid - 2 * TX; }
+    else { hli = RW - 1; hlj = tid - 2 * TX - RH; }
+    const bool hval = tid < NRH && i0 - 1 + hli <= ilim && j0 - 1 + hlj <= jlim;
+    const int hp0 = hval ? g.idx(i0 - 1 + hli, j0 - 1 + hlj, 0) : 0;
+    const int rh = hlj * RW + hli;
+    int role = -1, di = 0, dj = 0, dsm = 0;
+    if (tid < NPH) {
+        role = 0;
+        if (tid < W1) { di = i0 - 1 + tid; dj = j0 - 1; dsm = tid; }
+        else { di = i0 - 1; dj = j0 + (tid - W1); dsm = (tid - W1 + 1) * W1; }
+    } else if (tid < NPH + NZH) {
+        const int e = tid - NPH;
+        role = 1;
+        if (e < W1) { di = i0 + e; dj = j0 + SY; dsm = SY * W1 + e; }
+        else { di = i0 + TX; dj = j0 + (e - W1); dsm = (e - W1) * W1 + TX; }
+    } else if (tid < NPH + NZH + NXH) {
+        const int e = tid - NPH - NZH;
+        role = 2; di = i0 + e; dj = j0 + SY; dsm = SY * TX + e;
+    } else if (tid < NPH + NZH + NXH + NYH) {
+        const int e = tid - NPH - NZH - NXH;
+        role = 3; di = i0 + TX; dj = j0 + e; dsm = e * W1 + TX;
     }
-    __syncthreads();
-    // b(c, li, lj, lk): box coordinates (node i0-1+li ...)
-    auto b = [&](int c, int li, int lj, int lk) { return s_b[c][(lk * BYW + lj) * BXW + li]; };
-    auto a = [&](int c, int p) { return ff_load(A + c * N + p); };
-    auto l = [&](int c, int p) { return ff_load(L + c * N + p); };
-    for (int e = tid; e < N_PSI; e += NT) {
-        const int li = e % PSI_X, lj = (e / PSI_X) % PSI_Y, lk = e / (PSI_X * PSI_Y);   // box coords of the cell
-        const int i = i0 - 1 + li, j = j0 - 1 + lj, k = k0 - 1 + lk;
-        ffv v = ff_zero();
-        if (i >= 0 && j >= 0 && k >= 0 && i < g.nx && j < g.ny && k < g.nz) {
-            const int p = g.idx(i, j, k);
-            const ffv iv = ff_load(invV + p);
-            if (iv.hi != 0.f) {
-                const ffv fx = a(0, p + X) * b(0, li + 1, lj, lk) - a(0, p) * b(0, li, lj, lk);
-                const ffv fy = a(1, p + Y) * b(1, li, lj + 1, lk) - a(1, p) * b(1, li, lj, lk);
-                const ffv fz = a(2, p + Z) * b(2, li, lj, lk + 1) - a(2, p) * b(2, li, lj, lk);
-                v = iv * (fx * rdx + fy * rdy + fz * rdz);
+    const bool dval = role >= 0 && di <= ilim && dj <= jlim;
+    const int dp0 = dval ? g.idx(di, dj, 0) : 0;
+    const ffv one{1.f, 0.f};
+    // whether the coefficients of this warp's row on plane k are all 1 (the same in the whole warp)
+    auto ones = [&](int k) { return j <= g.ny && k >= 0 && k <= g.nz && (rowflag[row0 + k * rowz] & 1); };
+    B pb[3], hb[3];
+    ffv pa[3], ha[3], cv, cz, cx, cy, hc, he;
+    bool f_ring = false, f_cell = false, f_edge = false;   // those of the planes the registers below hold
+    auto fetch_ring = [&](int k, bool one_row) {
+        const int pn = p0 + k * Z, ph = hp0 + k * Z;
+        f_ring = one_row;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            pb[c] = inb ? O::load(x + c * N + pn) : O::zero();
+            hb[c] = hval ? O::load(x + c * N + ph) : O::zero();
+            pa[c] = one_row ? one : inb ? ff_load(A + c * N + pn) : ff_zero();
+            ha[c] = hval ? ff_load(A + c * N + ph) : ff_zero();
+        }
+    };
+    auto store_ring = [&](int slot) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            s_b[slot][c][rown] = pb[c];
+            s_f[slot][c][rown] = f_ring ? O::wide(pb[c]) : O::mul(pa[c], pb[c]);
+            if (tid < NRH) {
+                s_b[slot][c][rh] = hb[c];
+                s_f[slot][c][rh] = O::mul(ha[c], hb[c]);
             }
         }
-        s_psi[e] = v;
-    }
-    for (int e = tid; e < N_EX; e += NT) {
-        const int li = e % EX_X, lj = (e / EX_X) % EX_Y, lk = e / (EX_X * EX_Y);
-        const int i = i0 + li, j = j0 + lj, k = k0 + lk;
-        ffv v = ff_zero();
-        if (i < g.nx && j <= g.ny && k <= g.nz) {
-            const ffv lv = l(0, g.idx(i, j, k));
-            const int bi = li + 1, bj = lj + 1, bk = lk + 1;
-            if (lv.hi != 0.f)
-                v = lv * ((b(1, bi, bj, bk - 1) - b(1, bi, bj, bk)) * rdz + (b(2, bi, bj, bk) - b(2, bi, bj - 1, bk)) * rdy);
-        }
-        s_ex[e] = v;
-    }
-    for (int e = tid; e < N_EY; e += NT) {
-        const int li = e % EY_X, lj = (e / EY_X) % EY_Y, lk = e / (EY_X * EY_Y);
-        const int i = i0 + li, j = j0 + lj, k = k0 + lk;
-        ffv v = ff_zero();
-        if (i <= g.nx && j < g.ny && k <= g.nz) {
-            const ffv lv = l(1, g.idx(i, j, k));
-            const int bi = li + 1, bj = lj + 1, bk = lk + 1;
-            if (lv.hi != 0.f)
-                v = lv * ((b(0, bi, bj, bk) - b(0, bi, bj, bk - 1)) * rdz + (b(2, bi - 1, bj, bk) - b(2, bi, bj, bk)) * rdx);
-        }
-        s_ey[e] = v;
-    }
-    for (int e = tid; e < N_EZ; e += NT) {
-        const int li = e % EZ_X, lj = (e / EZ_X) % EZ_Y, lk = e / (EZ_X * EZ_Y);
-        const int i = i0 + li, j = j0 + lj, k = k0 + lk;
-        ffv v = ff_zero();
-        if (i <= g.nx && j <= g.ny && k < g.nz) {
-            const ffv lv = l(2, g.idx(i, j, k));
-            const int bi = li + 1, bj = lj + 1, bk = lk + 1;
-            if (lv.hi != 0.f)
-                v = lv * ((b(0, bi, bj - 1, bk) - b(0, bi, bj, bk)) * rdy + (b(1, bi, bj, bk) - b(1, bi - 1, bj, bk)) * rdx);
-        }
-        s_ez[e] = v;
-    }
+    };
+    auto fetch_cells = [&](int k, bool one_row) {   // 1/V and L_z
+        f_cell = one_row;
+        cv = one_row ? one : inb ? ff_load(invV + p0 + k * Z) : ff_zero();
+        cz = one_row ? one : inb ? ff_load(L + 2 * N + p0 + k * Z) : ff_zero();
+        hc = ff_zero();
+        if (dval && role == 0) hc = ff_load(invV + dp0 + k * Z);
+        if (dval && role == 1) hc = ff_load(L + 2 * N + dp0 + k * Z);
+    };
+    auto fetch_edges = [&](int k, bool one_row) {   // L_x and L_y
+        f_edge = one_row;
+        cx = one_row ? one : inb ? ff_load(L + p0 + k * Z) : ff_zero();
+        cy = one_row ? one : inb ? ff_load(L + N + p0 + k * Z) : ff_zero();
+        he = ff_zero();
+        if (dval && role == 2) he = ff_load(L + dp0 + k * Z);
+        if (dval && role == 3) he = ff_load(L + N + dp0 + k * Z);
+    };
+    auto at = [&](int ii, int jj) { return (jj - j0 + 1) * RW + (ii - i0 + 1); };
+    // a / h_a + b / h_b (the factors left out with CUBE)
+    auto pair = [&](ffv a, ffv ra, ffv b, ffv rb) { return CUBE ? a + b : a * ra + b * rb; };
+    auto curl_x = [&](int ii, int jj, int sm, int sp) {
+        const int q = at(ii, jj);
+        return pair(O::sub(s_b[sm][1][q], s_b[sp][1][q]), rdz, O::sub(s_b[sp][2][q], s_b[sp][2][q - RW]), rdy);
+    };
+    auto curl_y = [&](int ii, int jj, int sm, int sp) {
+        const int q = at(ii, jj);
+        return pair(O::sub(s_b[sp][0][q], s_b[sm][0][q]), rdz, O::sub(s_b[sp][2][q - 1], s_b[sp][2][q]), rdx);
+    };
+    auto curl_z = [&](int ii, int jj, int s0) {
+        const int q = at(ii, jj);
+        return pair(O::sub(s_b[s0][0][q - RW], s_b[s0][0][q]), rdy, O::sub(s_b[s0][1][q], s_b[s0][1][q - 1]), rdx);
+    };
+    auto div_at = [&](int ii, int jj, int s0, int s1) {
+        const int q = at(ii, jj);
+        const ffv fx = s_f[s0][0][q + 1] - s_f[s0][0][q], fy = s_f[s0][1][q + RW] - s_f[s0][1][q],
+                  fz = s_f[s1][2][q] - s_f[s0][2][q];
+        return CUBE ? fx + fy + fz : fx * rdx + fy * rdy + fz * rdz;
+    };
+    auto times = [&](bool is_one, ffv c, ffv v) { return is_one ? v : c * v; };
+    auto edges_xy = [&](int sm, int sp, int es) {
+        s_ex[es][ty * TX + tx] = inb ? times(f_edge, cx, curl_x(i, j, sm, sp)) : ff_zero();
+        s_ey[es][ty * W1 + tx] = inb ? times(f_edge, cy, curl_y(i, j, sm, sp)) : ff_zero();
+        if (role == 2) s_ex[es][dsm] = dval ? he * curl_x(di, dj, sm, sp) : ff_zero();
+        if (role == 3) s_ey[es][dsm] = dval ? he * curl_y(di, dj, sm, sp) : ff_zero();
+    };
+    auto psi_ez = [&](int s0, int s1) {
+        s_psi[(ty + 1) * W1 + tx + 1] = inb ? times(f_cell, cv, div_at(i, j, s0, s1)) : ff_zero();
+        s_ez[ty * W1 + tx] = inb ? times(f_cell, cz, curl_z(i, j, s0)) : ff_zero();
+        if (role == 0) s_psi[dsm] = dval ? hc * div_at(di, dj, s0, s1) : ff_zero();
+        if (role == 1) s_ez[dsm] = dval ? hc * curl_z(di, dj, s0) : ff_zero();
+    };
+    // (a plane below the grid's first holds ghosts only)
+    fetch_ring(k0 - 1, ones(k0 - 1));
+    store_ring(0);
+    fetch_ring(k0, ones(k0));
+    store_ring(1);
+    fetch_edges(k0, ones(k0));
     __syncthreads();
-    const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
-    const int i = i0 + tx, j = j0 + ty, k = k0 + tz;
-    if (i > g.nx || j > g.ny || k > g.nz) return;
-    const int p = g.idx(i, j, k);
-    auto PSI = [&](int aa, int bb, int cc) { return s_psi[(cc * PSI_Y + bb) * PSI_X + aa]; };
-    auto EXS = [&](int aa, int bb, int cc) { return s_ex[(cc * EX_Y + bb) * EX_X + aa]; };
-    auto EYS = [&](int aa, int bb, int cc) { return s_ey[(cc * EY_Y + bb) * EY_X + aa]; };
-    auto EZS = [&](int aa, int bb, int cc) { return s_ez[(cc * EZ_Y + bb) * EZ_X + aa]; };
-    const ffv ps0 = PSI(tx + 1, ty + 1, tz + 1);
+    edges_xy(0, 1, 0);
+    ffv psi_below = own ? ff_load(invV + p0 + (k0 - 1) * Z) * div_at(i, j, 0, 1) : ff_zero();
+    bool o1 = ones(k0 + 1), o2 = ones(k0 + 2);
+    bool ocur = ones(k0);
+    fetch_ring(k0 + 1, o1);
+    fetch_cells(k0, ocur);
+    fetch_edges(k0 + 1, o1);
+    for (int k = k0; k <= kend; ++k) {
+        const int s0 = (k - k0 + 1) & 1, s1 = s0 ^ 1, e0 = (k - k0) & 1, e1 = e0 ^ 1;
+        int2 rm[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int ci = cmap[c * N + p];
-        if (ci < 0) continue;   // closed face
-        const ffv av = a(c, p);
-        const ffv bv = b(c, tx + 1, ty + 1, tz + 1);
-        ffv v;
-        if (c == 0)
-            v = (EZS(tx, ty + 1, tz) - EZS(tx, ty, tz)) * rdy - (EYS(tx, ty, tz + 1) - EYS(tx, ty, tz)) * rdz +
-                av * ((PSI(tx, ty + 1, tz + 1) - ps0) * rdx - sigma * bv);
-        else if (c == 1)
-            v = (EXS(tx, ty, tz + 1) - EXS(tx, ty, tz)) * rdz - (EZS(tx + 1, ty, tz) - EZS(tx, ty, tz)) * rdx +
-                av * ((PSI(tx + 1, ty, tz + 1) - ps0) * rdy - sigma * bv);
-        else
-            v = (EYS(tx + 1, ty, tz) - EYS(tx, ty, tz)) * rdx - (EXS(tx, ty + 1, tz) - EXS(tx, ty, tz)) * rdy +
-                av * ((PSI(tx + 1, ty + 1, tz) - ps0) * rdz - sigma * bv);
-        out[ci] = make_float2(v.hi, v.lo);
+        for (int c = 0; c < 3; ++c) rm[c] = j <= g.ny ? rowmap[c * nrow + row0 + k * rowz] : make_int2(0, 0);
+        __syncthreads();
+        store_ring(s1);
+        __syncthreads();
+        psi_ez(s0, s1);
+        edges_xy(s0, s1, e1);
+        const bool oc = ocur;
+        if (k < kend) {
+            fetch_ring(k + 2, o2);
+            fetch_cells(k + 1, o1);
+            fetch_edges(k + 2, o2);
+            ocur = o1;
+            o1 = o2;
+            o2 = ones(k + 3);
+        }
+        __syncthreads();
+        const ffv ps0 = s_psi[(ty + 1) * W1 + tx + 1];
+        if ((rm[0].y | rm[1].y | rm[2].y) != 0) {   // the row has an open face
+            const ffv ez0 = s_ez[ty * W1 + tx];
+            const unsigned below = (1u << tx) - 1u;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                if (!(((unsigned)rm[c].y >> tx) & 1u)) continue;
+                ffv u, v, ps;
+                if (c == 0) {
+                    u = s_ez[(ty + 1) * W1 + tx] - ez0;
+                    v = s_ey[e1][ty * W1 + tx] - s_ey[e0][ty * W1 + tx];
+                    ps = s_psi[(ty + 1) * W1 + tx];
+                } else if (c == 1) {
+                    u = s_ex[e1][ty * TX + tx] - s_ex[e0][ty * TX + tx];
+                    v = s_ez[ty * W1 + tx + 1] - ez0;
+                    ps = s_psi[ty * W1 + tx + 1];
+                } else {
+                    u = s_ey[e0][ty * W1 + tx + 1] - s_ey[e0][ty * W1 + tx];
+                    v = s_ex[e0][(ty + 1) * TX + tx] - s_ex[e0][ty * TX + tx];
+                    ps = psi_below;
+                }
+                const ffv ru = c == 0 ? rdy : c == 1 ? rdz : rdx, rv = c == 0 ? rdz : c == 1 ? rdx : rdy,
+                          rp = c == 0 ? rdx : c == 1 ? rdy : rdz;
+                ffv y = CUBE ? u - v : u * ru - v * rv;
+                const ffv gr = CUBE ? ps - ps0 : (ps - ps0) * rp;
+                y = y + (oc ? gr : ff_load(A + c * N + p0 + k * Z) * gr);
+                if (CUBE) y = y * r2;
+                y = y - sigma * s_f[s0][c][rown];
+                const int ci = rm[c].x + __popc((unsigned)rm[c].y & below);
+                out[ci] = make_float2(y.hi, y.lo);
+                if (zc) zc[ci] = x[c * N + p0 + k * Z];
+            }
+        }
+        psi_below = ps0;
     }
+}
+
+// Row maps and flags of the float-float apply, one warp per 32-node row (see there)
+__global__ void k_row_maps(Grid3 g, const double* __restrict__ A, const double* __restrict__ L,
+                           const double* __restrict__ invV, const int* __restrict__ cmap, int nrow,
+                           int2* __restrict__ rowmap, unsigned char* __restrict__ rowflag) {
+    const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= nrow) return;
+    const int nti = (g.nx + TX) / TX;
+    const int i = (row % nti) * TX + lane, j = (row / nti) % (g.ny + 1), k = row / (nti * (g.ny + 1));
+    const bool in = i <= g.nx;
+    const int p = in ? g.idx(i, j, k) : 0;
+    bool one = in && invV[p] == 1.0;
+    for (int c = 0; c < 3; ++c) {
+        const double a = in ? A[c * g.np + p] : 0.0;
+        const unsigned m = __ballot_sync(0xffffffffu, a > 0.0);
+        one = one && a == 1.0 && L[c * g.np + p] == 1.0;
+        const int first = __ffs(m) - 1;
+        if (m && lane == first) rowmap[c * nrow + row] = make_int2(cmap[c * g.np + p], (int)m);
+        if (!m && lane == 0) rowmap[c * nrow + row] = make_int2(0, 0);
+    }
+    const bool all = __all_sync(0xffffffffu, one);
+    if (lane == 0) rowflag[row] = all ? 1 : 0;
 }
 
 // D A D^T x on the active cells in float-float (the projection's scalar
 // operator, Eq. proj), straight into the compact float-float vector of the
-// scalar FGMRES basis: out[cmap[p]] for every active cell p.  x is FP64 (split
-// on load), A the float-float face fractions, 1/h^2 float-float.
+// scalar FGMRES basis: out[cmap[p]] for every active cell p, and x's entries
+// into zc alike.  A: the float-float face fractions, 1/h^2 float-float.
+template <typename T>
 __global__ void k_scal_apply_ff(Grid3 g, const float2* __restrict__ A, ffv rx2, ffv ry2, ffv rz2,
-                                const double* __restrict__ x, const int* __restrict__ cmap, float2* __restrict__ out,
-                                const int* __restrict__ tiles) {
+                                const T* __restrict__ x, const int* __restrict__ cmap, float2* __restrict__ out,
+                                T* __restrict__ zc, const int* __restrict__ tiles) {
+    using O = typename FFOps<T>::type;
     int i, j, k;
     block_node(g, tiles, i, j, k);
     if (i >= g.nx || j >= g.ny || k >= g.nz) return;
@@ -930,14 +1081,15 @@ __global__ void k_scal_apply_ff(Grid3 g, const float2* __restrict__ A, ffv rx2, 
     const int ci = cmap[p];
     if (ci < 0) return;
     const int X = 1, Y = g.sx, Z = g.sxy, N = g.np;
-    auto v = [&](int q) { return ff_from_double(x[q]); };
+    auto v = [&](int q) { return O::load(x + q); };
     auto a = [&](int q) { return ff_load(A + q); };
-    const ffv v0 = v(p);
-    const ffv sx = (a(p + X) * (v0 - v(p + X)) + a(p) * (v0 - v(p - X))) * rx2;
-    const ffv sy = (a(N + p + Y) * (v0 - v(p + Y)) + a(N + p) * (v0 - v(p - Y))) * ry2;
-    const ffv sz = (a(2 * N + p + Z) * (v0 - v(p + Z)) + a(2 * N + p) * (v0 - v(p - Z))) * rz2;
+    const typename O::V v0 = v(p);
+    const ffv sx = (a(p + X) * O::sub(v0, v(p + X)) + a(p) * O::sub(v0, v(p - X))) * rx2;
+    const ffv sy = (a(N + p + Y) * O::sub(v0, v(p + Y)) + a(N + p) * O::sub(v0, v(p - Y))) * ry2;
+    const ffv sz = (a(2 * N + p + Z) * O::sub(v0, v(p + Z)) + a(2 * N + p) * O::sub(v0, v(p - Z))) * rz2;
     const ffv r = sx + sy + sz;
     out[ci] = make_float2(r.hi, r.lo);
+    zc[ci] = x[p];
 }
 
 // float-float copy of an FP64 array: hi = the double rounded to FP32, lo =
@@ -976,23 +1128,33 @@ void compact_map(long long n3, const int* list, int nl, int* cmap, cudaStream_t 
            list, nl, cmap);
 }
 
-void vec_apply_ff(const Grid3& g, const int* tiles, int ntiles, const float2* A, const float2* L, const float2* invV,
-                  double sigma, const double* x, const int* cmap, float2* out, cudaStream_t s) {
-    if (ntiles <= 0) return;
-    // bytes: per open face its x (8), A and about one L (8 each), a third of a 1/V (8), the output (8) and cmap (4)
-    const double bytes = (double)g.nopen * (8.0 + 16.0 + 8.0 / 3.0 + 12.0);
-    launch_b("vec_apply_ff_L0", bytes, k_vec_apply_ff, ntiles, dim3(TX, TY, TZ), 0, s, g, A, L, invV, host_ff(g.rhx),
-             host_ff(g.rhy), host_ff(g.rhz), host_ff(sigma), x, cmap, out, tiles);
+void row_maps(const Grid3& g, const double* A, const double* L, const double* invV, const int* cmap, int2* rowmap,
+              unsigned char* rowflag, cudaStream_t s) {
+    const int nrow = row_count(g);
+    launch("k_row_maps", k_row_maps, (nrow + 7) / 8, 256, 0, s, g, A, L, invV, cmap, nrow, rowmap, rowflag);
 }
 
-void scal_apply_ff(const Grid3& g, const int* tiles, int ntiles, const float2* A, const double* x, const int* cmap,
-                   float2* out, cudaStream_t s) {
+template <typename T>
+void vec_apply_ff(const FFLevel& f, double sigma, const T* x, float2* out, T* zc, cudaStream_t s) {
+    const Grid3& g = f.g;
+    if (f.ntiles <= 0) return;
+    // bytes: per open face its x, A and about one L (8 each), a third of a 1/V (8), the output (8) and z
+    const double bytes = (double)g.nopen * (16.0 + 8.0 / 3.0 + 8.0 + (zc ? 2.0 : 1.0) * sizeof(T));
+    const bool cube = g.hx == g.hy && g.hy == g.hz;
+    launch_b("vec_apply_ff_L0", bytes, cube ? k_vec_apply_ff<T, true> : k_vec_apply_ff<T, false>, f.ntiles,
+             dim3(TX, kFFY, 1), 0, s, g, f.A, f.L, f.invV, host_ff(g.rhx), host_ff(g.rhy), host_ff(g.rhz),
+             host_ff(g.rhx * g.rhx), host_ff(sigma), x, f.rowmap, f.rowflag, out, zc, f.tiles);
+}
+
+template <typename T>
+void scal_apply_ff(const Grid3& g, const int* tiles, int ntiles, const float2* A, const T* x, const int* cmap,
+                   float2* out, T* zc, cudaStream_t s) {
     if (ntiles <= 0) return;
-    // bytes: per active cell its x (8), three float-float face fractions (24; six faces, each shared by two
-    // cells), the output (8) and its compact index (4)
-    const double bytes = (double)g.nact * (8.0 + 24.0 + 12.0);
-    launch_b("scal_apply_ff_L0", bytes, k_scal_apply_ff, ntiles, kBlock, 0, s, g, A, host_ff(g.rhx * g.rhx),
-             host_ff(g.rhy * g.rhy), host_ff(g.rhz * g.rhz), x, cmap, out, tiles);
+    // bytes: per active cell its x, three float-float face fractions (24; six faces, each shared by two
+    // cells), the output (8), its z and its compact index (4)
+    const double bytes = (double)g.nact * (24.0 + 12.0 + 2.0 * sizeof(T));
+    launch_b("scal_apply_ff_L0", bytes, k_scal_apply_ff<T>, ntiles, kBlock, 0, s, g, A, host_ff(g.rhx * g.rhx),
+             host_ff(g.rhy * g.rhy), host_ff(g.rhz * g.rhz), x, cmap, out, zc, tiles);
 }
 
 const char* stencil_name(const char* kind, int prec, int mode, bool fine) {
@@ -1163,6 +1325,9 @@ void dm_sub_grad(const Grid3& g, const double* A, const double* x, const double*
 // explicit instantiations: FP64 storage / FP64 coefficients, FP32 / FP32, BF16 / FP32
 #define DM_INST(T, TC)                                                                                          \
     template void vec_stencil<T, TC>(const VecOp<T, TC>&, int, const T*, const T*, T*, double, cudaStream_t);  \
+    template void vec_apply_ff<T>(const FFLevel&, double, const T*, float2*, T*, cudaStream_t);               \
+    template void scal_apply_ff<T>(const Grid3&, const int*, int, const float2*, const T*, const int*, float2*, T*, \
+                                   cudaStream_t);                                                              \
     template void vec_jacobi_zero<T, TC>(const VecOp<T, TC>&, const T*, T*, double, cudaStream_t);            \
     template void scal_down<T, TC>(const ScalOp<T, TC>&, const Grid3&, const unsigned char*, const T*, T*, double, \
                                    cudaStream_t);                                                              \
