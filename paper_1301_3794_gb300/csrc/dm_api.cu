@@ -26,6 +26,7 @@ thread_local long long* g_launch_counter = nullptr;
 thread_local cudaStream_t g_stream = nullptr;
 thread_local Tracer* g_tracer = nullptr;
 thread_local int g_untraced = 0;
+thread_local bool g_chain = true;
 
 static std::atomic<long long> g_allocations{0};
 void note_allocation() { g_allocations.fetch_add(1, std::memory_order_relaxed); }
@@ -108,6 +109,7 @@ struct dm_context {
     long long launches = 0;
     Reducer red;
     Tracer tracer;
+    bool chain = true;     // chained launches (launch_chain): off in a batch's workers
     // autotuner cache: (nx, ny, nz, precision) -> stencil tile shape
     std::vector<std::pair<std::array<int, 4>, int>> tuned;
 };
@@ -169,6 +171,7 @@ template <class F>
 dm_status guarded(const dm_context* cctx, F&& f) {
     dm_context* ctx = const_cast<dm_context*>(cctx);
     LaunchScope scope(ctx);
+    ChainScope chain(!ctx || ctx->chain);
     try {
         f();
         if (ctx) ctx->err.clear();
@@ -344,6 +347,7 @@ struct dm_operator {
     int learned_streak = 0;    // consecutive shifted solves in which the correction was switched off
     long long nopen0 = 0;
     Fork fork;                 // side streams of the band smoother's class launches
+    bool forks = false;        // whether some level's classes go on them
     ~dm_operator() {
         if (vexec) cudaGraphExecDestroy(vexec);
         if (sexec) cudaGraphExecDestroy(sexec);
@@ -652,6 +656,7 @@ const T* cycle_vec(dm_operator* op, const TIn& v, double scale = 1.0) {
     T* e = reinterpret_cast<T*>(w0.e.get());
     T* r = reinterpret_cast<T*>(w0.r.get());
     mg_input<T>(D, v, scale, f, s);
+    const ChainScope chain(!(std::is_same<T, double>::value && op->forks));
     if (graphs_allowed(op) && op->vcalls > 0) {
         if (!op->vexec && !capture_graph(op, [&] { vcycle<T, TC>(op, 0, f, e, r); }, &op->vexec, &op->vexec_kernels))
             op->graphs = false;
@@ -1230,6 +1235,7 @@ void setup_operator(dm_operator* op) {
                 o.bn_cls_count[k] = nl_.cls_count[k];
                 o.bn_cls_copies[k] = nl_.cls_copies[k];
             }
+            op->forks |= band_nodes_fork(o.bn_nsub, nl_.cls_count, !lowp);
             upload(o.bn_off, nl_.off);
             upload(o.bn_node, nl_.node);
             upload(o.bn_info, nl_.info);
@@ -2889,6 +2895,7 @@ dm_status dm_eigensolve_batched(dm_context* ctx, int n, dm_batch_item* items, in
             return st;
         }
         sub[w]->tuned = ctx->tuned;
+        sub[w]->chain = nw == 1;
     }
     std::atomic<int> next{0};
     auto worker = [&](int w) {

@@ -298,6 +298,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_band_node(int sub0, NodeArgs<
     const int p = has ? a.node[ct] : -1;
     const int info = p >= 0 ? a.info[ct] : 0;
     const bool live = p >= 0;
+    // the couplings and the zeroed buffers need nothing from the kernels before
+    C v[42], cx = C(0), cy = C(0), cz = C(0), dx = C(0), dy = C(0), dz = C(0), fx = C(0), fy = C(0), fz = C(0);
+#pragma unroll
+    for (int e = 0; e < 42; ++e) v[e] = live ? (C)a.vals[(size_t)e * a.ncopies + ct] : C(0);
+    if (live) {
+        dx = (C)a.vals[(size_t)42 * a.ncopies + ct];   // 1 / D, 0 on faces without a row
+        dy = (C)a.vals[(size_t)43 * a.ncopies + ct];
+        dz = (C)a.vals[(size_t)44 * a.ncopies + ct];
+    }
+    for (int k = threadIdx.x; k < 2 * kNBuf / 4; k += NT) reinterpret_cast<float4*>(buf)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    chain_wait();
     // x over the local box (zero outside the padded grid's -1 .. n+1): every
     // thread copies whole columns along z, twelve independent loads each
     {
@@ -327,18 +338,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_band_node(int sub0, NodeArgs<
             }
         }
     }
-    C v[42], cx = C(0), cy = C(0), cz = C(0), dx = C(0), dy = C(0), dz = C(0), fx = C(0), fy = C(0), fz = C(0);
-#pragma unroll
-    for (int e = 0; e < 42; ++e) v[e] = live ? (C)a.vals[(size_t)e * a.ncopies + ct] : C(0);
     if (live) {
-        dx = (C)a.vals[(size_t)42 * a.ncopies + ct];   // 1 / D, 0 on faces without a row
-        dy = (C)a.vals[(size_t)43 * a.ncopies + ct];
-        dz = (C)a.vals[(size_t)44 * a.ncopies + ct];
         fx = (C)to_c(a.f[p]);
         fy = (C)to_c(a.f[a.g.np + p]);
         fz = (C)to_c(a.f[2 * a.g.np + p]);
     }
-    for (int k = threadIdx.x; k < 2 * kNBuf / 4; k += NT) reinterpret_cast<float4*>(buf)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int pos = info & 4095;   // li + 11 lj + 121 lk
     if constexpr (std::is_same<T, float>::value) copy_async_wait();
     __syncthreads();
@@ -432,6 +436,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) k_
 #pragma unroll
     for (int e = 0; e < 42; ++e) v[e] = live ? (C)a.vals[(size_t)e * a.ncopies + ct] : C(0);
     for (int k = threadIdx.x; k < 2 * kNBuf; k += NT) buf[k] = C(0);
+    chain_wait();
     if (live) {
         // start residual from global memory: the neighbours' loads are independent of one another
         const int X = 1, Y = a.g.sx, Z = a.g.sxy, N = a.g.np;
@@ -513,12 +518,12 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) k_
 // x <- x + u on the band faces (uidx: where each face's owner put its correction)
 template <typename T>
 __global__ void k_band_add_node(const int* __restrict__ band, const int* __restrict__ uidx, int nband,
-                                const typename Compute<T>::type* __restrict__ u, T* __restrict__ x) {
+                                const typename Compute<T>::type* u, T* x) {
     using C = typename Compute<T>::type;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nband) return;
-    const int q = band[t];
-    x[q] = to_store<T>((C)to_c(x[q]) + u[uidx[t]]);
+    const int q = t < nband ? band[t] : 0, at = t < nband ? uidx[t] : 0;
+    chain_wait();
+    if (t < nband) x[q] = to_store<T>((C)to_c(x[q]) + u[at]);
 }
 
 // Scaled couplings of every node copy from the band rows (15 slots, slot-major)
@@ -875,25 +880,40 @@ namespace {
 
 constexpr int kSMs = 152;
 
+// A level with few subdomains goes in one launch shaped for its largest class:
+// FP32, when they fit the SMs at one block each; FP64, when clusters of eight
+// blocks for every subdomain still run at once.
+bool one_launch(int nsub, bool wide) { return wide ? 8 * nsub <= 2 * kSMs : nsub <= kSMs; }
+
 template <typename T, typename TC, int NT>
-void launch_node(const char* name, double bytes, int first, int count, const NodeArgs<T, TC>& a, cudaStream_t s) {
+void launch_node(const char* name, double bytes, int first, int count, const NodeArgs<T, TC>& a, bool chain,
+                 cudaStream_t s) {
     using C = typename Compute<T>::type;
     constexpr size_t smem = sizeof(C) * (2 * kNBuf + 3 * kXC);
     // above the 48 KB a kernel may use unasked; set on every call because the setting belongs to the current device
     DM_CUDA(cudaFuncSetAttribute(k_band_node<T, TC, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    launch_b(name, bytes, k_band_node<T, TC, NT>, count, NT, smem, s, first, a);
+    if (chain) launch_chain(name, bytes, k_band_node<T, TC, NT>, count, NT, smem, s, first, a);
+    else launch_b(name, bytes, k_band_node<T, TC, NT>, count, NT, smem, s, first, a);
 }
 template <int CS>
 void launch_cluster(const char* name, double bytes, int first, int count, const NodeArgs<double, double>& a,
-                    cudaStream_t s) {
+                    bool chain, cudaStream_t s) {
     constexpr size_t smem = sizeof(double) * 2 * kNBuf;
     // above the 48 KB a kernel may use unasked; set on every call because the setting belongs to the current device
     DM_CUDA(cudaFuncSetAttribute(k_band_node_cluster<double, double, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
-    launch_b(name, bytes, k_band_node_cluster<double, double, CS>, count * CS, kClusterThreads, smem, s, first, a);
+    const auto kern = k_band_node_cluster<double, double, CS>;
+    if (chain) launch_chain(name, bytes, kern, count * CS, kClusterThreads, smem, s, first, a);
+    else launch_b(name, bytes, kern, count * CS, kClusterThreads, smem, s, first, a);
 }
 
 }  // namespace
+
+bool band_nodes_fork(int nsub, const int cls_count[kNodeClasses], bool wide) {
+    int nl = 0;
+    for (int cl = 0; cl < kNodeClasses; ++cl) nl += cls_count[cl] > 0;
+    return nl > 1 && !one_launch(nsub, wide);
+}
 
 template <typename T, typename TC>
 void band_nodes(const BandNodes<TC>& bn, const Grid3& g, const int* band, int nband, const T* f, T* x, void* u_raw,
@@ -913,10 +933,7 @@ void band_nodes(const BandNodes<TC>& bn, const Grid3& g, const int* band, int nb
             top = cl;
             ++nl;
         }
-    // A level with few subdomains goes in one launch shaped for its largest
-    // class: FP32, when they fit the SMs at one block each; FP64, when clusters
-    // of eight blocks for every subdomain still run at once.
-    const bool single = wide ? 8 * bn.nsub <= 2 * kSMs : bn.nsub <= kSMs;
+    const bool single = one_launch(bn.nsub, wide);
     if (single) nl = 1;
     const bool forked = fk && fk->naux > 0 && nl > 1;
     if (forked) {
@@ -928,18 +945,20 @@ void band_nodes(const BandNodes<TC>& bn, const Grid3& g, const int* band, int nb
         if (bn.cls_count[cl] == 0 || (single && cl != top)) continue;
         const int ai = li++;   // the first class stays on s0
         cudaStream_t s = (forked && ai > 0 && ai - 1 < fk->naux) ? fk->aux[ai - 1] : s0;
+        // (the fork's event wait or another class's launch comes before the rest: those are ordered in full)
+        const bool chain = ai == 0 && !forked;
         const int first = single ? 0 : bn.cls_first[cl], count = single ? bn.nsub : bn.cls_count[cl];
         const double bytes = (single ? bn.copies() : (double)bn.cls_copies[cl]) * per + owned / nl;
         if constexpr (wide) {
-            if (single || cl >= 2) launch_cluster<8>(name, bytes, first, count, a, s);
-            else if (cl == 1) launch_cluster<4>(name, bytes, first, count, a, s);
-            else launch_cluster<2>(name, bytes, first, count, a, s);
+            if (single || cl >= 2) launch_cluster<8>(name, bytes, first, count, a, chain, s);
+            else if (cl == 1) launch_cluster<4>(name, bytes, first, count, a, chain, s);
+            else launch_cluster<2>(name, bytes, first, count, a, chain, s);
         } else {
             switch (cl) {
-                case 0: launch_node<T, TC, 256>(name, bytes, first, count, a, s); break;
-                case 1: launch_node<T, TC, 512>(name, bytes, first, count, a, s); break;
-                case 2: launch_node<T, TC, 768>(name, bytes, first, count, a, s); break;
-                default: launch_node<T, TC, 1024>(name, bytes, first, count, a, s);
+                case 0: launch_node<T, TC, 256>(name, bytes, first, count, a, chain, s); break;
+                case 1: launch_node<T, TC, 512>(name, bytes, first, count, a, chain, s); break;
+                case 2: launch_node<T, TC, 768>(name, bytes, first, count, a, chain, s); break;
+                default: launch_node<T, TC, 1024>(name, bytes, first, count, a, chain, s);
             }
         }
     }
@@ -948,8 +967,11 @@ void band_nodes(const BandNodes<TC>& bn, const Grid3& g, const int* band, int nb
             DM_CUDA(cudaEventRecord(fk->join[k], fk->aux[k]));
             DM_CUDA(cudaStreamWaitEvent(s0, fk->join[k], 0));
         }
-    launch_b(stencil_name("band_add", prec_index<T>(), ST_JACOBI, fine), (double)nband * (8.0 + sizeof(C) + 2.0 * sizeof(T)),
-             k_band_add_node<T>, (nband + 255) / 256, 256, 0, s0, band, bn.uidx, nband, (const C*)u, x);
+    const char* add = stencil_name("band_add", prec_index<T>(), ST_JACOBI, fine);
+    const double add_bytes = (double)nband * (8.0 + sizeof(C) + 2.0 * sizeof(T));
+    const int nb = (nband + 255) / 256;
+    if (forked) launch_b(add, add_bytes, k_band_add_node<T>, nb, 256, 0, s0, band, bn.uidx, nband, (const C*)u, x);
+    else launch_chain(add, add_bytes, k_band_add_node<T>, nb, 256, 0, s0, band, bn.uidx, nband, (const C*)u, x);
 }
 
 // rows per thread and block size of a class (R = 0: the shared-memory variant;

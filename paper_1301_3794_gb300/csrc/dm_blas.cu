@@ -125,10 +125,11 @@ __global__ void k_dot_list(long long n, const int* __restrict__ list, const doub
 }
 
 // result[c] = sum_b partial[b * ldb + c * ldc]  (one warp per column, fixed order)
-__global__ void k_mdot_final(int nb, int m, const double* __restrict__ partial, int ldb, int ldc,
+__global__ void k_mdot_final(int nb, int m, const double* partial, int ldb, int ldc,
                              double* __restrict__ result) {
     const int c = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
+    chain_wait();
     if (c >= m) return;
     double s = 0.0;
     for (int b = lane; b < nb; b += 32) s += partial[(long long)b * ldb + (long long)c * ldc];
@@ -142,11 +143,12 @@ __global__ void k_mdot_final(int nb, int m, const double* __restrict__ partial, 
 // coef = [s (j), c - (h / b) s (j), 1 / b, h / b]; all coefficients 0 when b is
 // not positive (the caller stops there).  On the device, the update need not
 // wait for the host: one synchronisation per FGMRES iteration instead of two.
-__global__ void __launch_bounds__(1024) k_dcgs_coef(int nb, int j, const double* __restrict__ partial, int ldp,
+__global__ void __launch_bounds__(1024) k_dcgs_coef(int nb, int j, const double* partial, int ldp,
                                                     double* __restrict__ result, double* __restrict__ coef) {
     __shared__ double dots[256];
     __shared__ double bh[2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, m = 2 * j + 2;
+    chain_wait();
     for (int c = wid; c < m; c += 32) {
         double s = 0.0;
         for (int b = lane; b < nb; b += 32) s += partial[(long long)c * ldp + b];
@@ -405,8 +407,8 @@ __device__ __forceinline__ double ff_warp_sums(float2 (&v)[P]) {
 // on average, 34 -> 17 us; 5.65 M faces 121 -> 110 us (5.5 TB/s of the bytes needed).
 constexpr int kDotCols = 16;
 template <int NC>
-__device__ __forceinline__ void dcgs_chunk(long long n2, int j, int c0, const float4* __restrict__ Q, long long ld2,
-                                           const float4* __restrict__ v, const float4* __restrict__ w, bool first,
+__device__ __forceinline__ void dcgs_chunk(long long n2, int j, int c0, const float4* Q, long long ld2,
+                                           const float4* v, const float4* w, bool first,
                                            float& as, float& ae, float& ds, float& de, double* __restrict__ partial,
                                            int ldp, double (*red)[32]) {
     constexpr int N1 = NC > 0 ? NC : 1;
@@ -463,11 +465,12 @@ __device__ __forceinline__ void dcgs_chunk(long long n2, int j, int c0, const fl
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 2) k_ff_dcgs_dots(long long n2, int j, const float4* __restrict__ Q,
-                                                              long long ld2, const float4* __restrict__ v,
-                                                              const float4* __restrict__ w, double* __restrict__ partial,
+__global__ void __launch_bounds__(kThreads, 2) k_ff_dcgs_dots(long long n2, int j, const float4* Q,
+                                                              long long ld2, const float4* v,
+                                                              const float4* w, double* __restrict__ partial,
                                                               int ldp) {
     __shared__ double red[kThreads / 32][32];
+    chain_wait();
     float as = 0.f, ae = 0.f, ds = 0.f, de = 0.f;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int chunks = (j + kDotCols - 1) / kDotCols;   // of nearly equal size
@@ -499,12 +502,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_ff_dcgs_dots(long long n2, int 
 //   v <- (v - Q s) / beta   (the pending vector, now finished)
 //   out <- w - Q gamma - delta v_old   and the block partial of |out|^2
 // Two entries per thread and step, as in the dots pass.
-__global__ void k_ff_dcgs_update(long long n2, int j, const float4* __restrict__ Q, long long ld2,
-                                 const double* __restrict__ coef, float4* __restrict__ v, const float4* __restrict__ w,
+__global__ void k_ff_dcgs_update(long long n2, int j, const float4* Q, long long ld2,
+                                 const double* coef, float4* v, const float4* w,
                                  float4* __restrict__ out, double* __restrict__ partial) {
     __shared__ float2 cs[128], cg[128];
     __shared__ float2 rb, dl;
     __shared__ double red[kThreads / 32];
+    chain_wait();
     for (int c = threadIdx.x; c < j; c += blockDim.x) {
         cs[c] = ff_bits(-coef[c]);
         cg[c] = ff_bits(-coef[j + c]);
@@ -611,7 +615,8 @@ __global__ void k_ff_gather(long long n, const int* __restrict__ list, double a,
 // y[list[i]] = a x[i] in storage type T   (scatter from a compact float-float vector)
 template <typename T>
 __global__ void k_ff_scatter(long long n, const int* __restrict__ list, typename Compute<T>::type a,
-                             const float2* __restrict__ x, T* __restrict__ y) {
+                             const float2* x, T* __restrict__ y) {
+    chain_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float2 v = x[i];
         if constexpr (std::is_same<T, double>::value) y[list[i]] = a * ff_to_double(v);
@@ -762,7 +767,7 @@ void ff_gather(long long n, const int* list, double a, const double* x, float2* 
 template <typename T>
 void ff_scatter(long long n, const int* list, double a, const float2* x, T* y, cudaStream_t s) {
     const int nb = (int)std::max<long long>(1, std::min<long long>((n + kThreads - 1) / kThreads, kMaxBlocks));
-    launch_b("k_ff_scatter", (12.0 + sizeof(T)) * n, k_ff_scatter<T>, nb, kThreads, 0, s, n, list,
+    launch_chain("k_ff_scatter", (12.0 + sizeof(T)) * n, k_ff_scatter<T>, nb, kThreads, 0, s, n, list,
              (typename Compute<T>::type)a, x, y);
 }
 template void ff_scatter<double>(long long, const int*, double, const float2*, double*, cudaStream_t);
@@ -846,13 +851,13 @@ void dcgs_step(Reducer& red, const Domain& d, int j, const float2* Q, long long 
     const float4* w4 = reinterpret_cast<const float4*>(w);
     double* coef = red.result + red.max_cols + 8;
     int nb = std::min(pair_blocks(n2, k_ff_dcgs_dots), red.cap_blocks);
-    launch_b("k_ff_dcgs_dots", 8.0 * d.live() * (j + 2), k_ff_dcgs_dots, nb, kThreads, 0, s, n2, j, q4, ld / 2,
+    launch_chain("k_ff_dcgs_dots", 8.0 * d.live() * (j + 2), k_ff_dcgs_dots, nb, kThreads, 0, s, n2, j, q4, ld / 2,
              reinterpret_cast<const float4*>(v), w4, red.partial, red.cap_blocks);
-    launch("k_dcgs_coef", k_dcgs_coef, 1, 1024, 0, s, nb, j, (const double*)red.partial, red.cap_blocks, red.result, coef);
+    launch_chain("k_dcgs_coef", 0.0, k_dcgs_coef, 1, 1024, 0, s, nb, j, (const double*)red.partial, red.cap_blocks, red.result, coef);
     nb = std::min(pair_blocks(n2, k_ff_dcgs_update), red.cap_blocks);
-    launch_b("k_ff_dcgs_update", 8.0 * d.live() * (j + 4), k_ff_dcgs_update, nb, kThreads, 0, s, n2, j, q4, ld / 2,
+    launch_chain("k_ff_dcgs_update", 8.0 * d.live() * (j + 4), k_ff_dcgs_update, nb, kThreads, 0, s, n2, j, q4, ld / 2,
              (const double*)coef, reinterpret_cast<float4*>(v), w4, reinterpret_cast<float4*>(out), red.partial);
-    launch("k_mdot_final", k_mdot_final, 1, 32, 0, s, nb, 1, (const double*)red.partial, 1, 1, red.result + m + 2);
+    launch_chain("k_mdot_final", 0.0, k_mdot_final, 1, 32, 0, s, nb, 1, (const double*)red.partial, 1, 1, red.result + m + 2);
     DM_CUDA(cudaMemcpyAsync(red.host, red.result, sizeof(double) * (m + 3), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
     for (int c = 0; c < m + 3; ++c) host_out[c] = red.host[c];

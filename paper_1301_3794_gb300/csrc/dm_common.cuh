@@ -212,6 +212,56 @@ inline void launch(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 blo
     launch_b(name, 0.0, kern, grid, block, smem, s, std::forward<Args>(args)...);
 }
 
+// Chained launches.  A kernel launched by launch_chain may be brought onto the SMs
+// while the one before it on the stream still runs its last blocks, and waits in
+// chain_wait() until that one has finished and its results are visible; what
+// comes before the wait must read nothing an earlier kernel of the call writes.
+// Every kernel so launched calls chain_wait() in every thread that goes on (so
+// that its own end implies its predecessors'), and takes pointers to what they
+// write without __restrict__: loads the compiler may treat as read-only for the
+// kernel's life would be hoisted above the wait.  The V-cycles' and Krylov steps'
+// kernels are short (3 to 10 us on the smaller grids), so the launch gap between
+// dependent kernels, about a microsecond of which this hides, is a tenth of them.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Not chained (g_chain false): the workers of a batch, whose waiting blocks would
+// keep the other workers' kernels off the SMs (six cavities on six streams:
+// 455 ms unchained, 488 chained), and FP64 cycles that fork streams (FP64 kernels
+// are long; 72 x 56 x 88 solve 16.8 ms against 17.5).  Elsewhere: projection on
+// 104 x 88 x 72 cells 3.69 -> 3.38 ms, 16^3 FP64 eigensolve 178 -> 170, 96^3 FP32
+// one 448 -> 429, 128^3 BF16 solve 17.9 -> 17.4.
+extern thread_local bool g_chain;
+struct ChainScope {
+    const bool prev;
+    explicit ChainScope(bool on) : prev(g_chain) { g_chain = prev && on; }
+    ~ChainScope() { g_chain = prev; }
+    ChainScope(const ChainScope&) = delete;
+    ChainScope& operator=(const ChainScope&) = delete;
+};
+template <typename... KArgs, typename... Args>
+inline void launch_chain(const char* name, double bytes, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                         cudaStream_t s, Args&&... args) {
+    if (!g_chain || (g_tracer && g_tracer->on && !g_untraced)) {   // (traced kernels are timed alone)
+        launch_b(name, bytes, kern, grid, block, smem, s, std::forward<Args>(args)...);
+        return;
+    }
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+    count_launch();
+    if (e != cudaSuccess) throw Error(DM_ERR_CUDA, std::string(name) + ": " + cudaGetErrorString(e));
+}
+
 // Count of the device memory, pinned host memory, CUDA events and streams the
 // library has created in this process (a diagnostic for the calls that
 // promise to create none).
@@ -466,6 +516,8 @@ struct BandNodes {
     }
 };
 bool band_nodes_fit(int brick);
+// whether a level's classes are launched side by side (wide: FP64)
+bool band_nodes_fork(int nsub, const int cls_count[kNodeClasses], bool wide);
 void band_nodes_setup(const Grid3& g, const int* band_dev, int nband, int brick, bool by_bank, NodeLayout& out,
                       cudaStream_t s);
 template <typename TC>

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const 
                                                                    const float* __restrict__ M32,
                                                                    const int* __restrict__ list,
                                                                    const unsigned char* __restrict__ zero_rows,
-                                                                   const T* __restrict__ f, T* __restrict__ x) {
+                                                                   const T* f, T* __restrict__ x) {
     using C = typename Compute<T>::type;
     extern __shared__ __align__(16) unsigned char solve_smem[];
     C* const sf = reinterpret_cast<C*>(solve_smem);
@@ -304,6 +304,7 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const 
     C v[U];
 #pragma unroll
     for (int e = 0; e < U; ++e) v[e] = lane + 32 * e < n ? m[lane + 32 * e] : C(0);
+    chain_wait();
     for (int c = threadIdx.x; c < n; c += 32 * kSolveWarps)
         sf[c] = (zero_rows && zero_rows[c]) ? C(0) : (C)to_c(f[list[c]]);
     __syncthreads();
@@ -436,7 +437,7 @@ void dense_coarse_solve(const double* Minv64, const float* Minv32, int n, const 
     using C = typename Compute<T>::type;
     if (n <= 0) return;
     // n <= 6000 FP64 values fit the 48 KB a kernel may use unasked
-    launch_b("k_coarse_solve", (double)n * n * sizeof(C) + 2.0 * n * sizeof(T), k_coarse_solve<T>,
+    launch_chain("k_coarse_solve", (double)n * n * sizeof(C) + 2.0 * n * sizeof(T), k_coarse_solve<T>,
              (n + kSolveWarps - 1) / kSolveWarps, 32 * kSolveWarps, sizeof(C) * (size_t)n, s, n, Minv64, Minv32, list,
              zero_rows, f, x);
 }

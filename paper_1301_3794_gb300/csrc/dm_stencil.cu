@@ -35,7 +35,7 @@ inline dim3 node_grid(const Grid3& g, int extra = 1) {
 // Field accessor over a padded 3-component vector in storage type T.
 template <typename T, typename C>
 struct VecAcc {
-    const T* __restrict__ x;
+    const T* x;
     int np;
     __device__ __forceinline__ C operator()(int c, int p) const { return (C)to_c(x[c * np + p]); }
 };
@@ -44,7 +44,7 @@ struct VecAcc {
 // reads its x through this instead of from a vector that pass would write.
 template <typename T, typename TC, typename C>
 struct Jac0Acc {
-    const T* __restrict__ f;
+    const T* f;
     const TC* __restrict__ invD;
     C om;
     int np;
@@ -136,7 +136,7 @@ __device__ __forceinline__ C face_K(const Coef<C, TC>& cf, const Acc& b, int c, 
 template <typename T, typename TC, int MODE, int SY, int SZ>
 __global__ void __launch_bounds__(TX * SY * SZ) k_vec_stencil_tiled(
     Grid3 g, const TC* __restrict__ A, const TC* __restrict__ L, const TC* __restrict__ invV,
-    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* __restrict__ x, const T* __restrict__ f,
+    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* x, const T* f,
     T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     constexpr int PSI_X = TX + 1, PSI_Y = SY + 1, PSI_Z = SZ + 1;   // psi: i0-1 .. i0+TX-1 (and j, k alike)
@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(TX * SY * SZ) k_vec_stencil_tiled(
                   N_EZ = EZ_X * EZ_Y * EZ_Z;
     constexpr int NT = TX * SY * SZ;
     __shared__ C s_psi[N_PSI], s_ex[N_EX], s_ey[N_EY], s_ez[N_EZ];
+    chain_wait();
     const int t = tiles[blockIdx.x];
     const int nti = (g.nx + TX) / TX, ntj = (g.ny + SY) / SY;
     const int i0 = (t % nti) * TX, j0 = ((t / nti) % ntj) * SY, k0 = (t / (nti * ntj)) * SZ;
@@ -254,7 +255,7 @@ struct CertArgs {
 template <typename T, typename TC, int MODE, int SY, int KZ, int IN = IN_PADDED>
 __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512 : 768) / (TX * SY)) k_vec_stencil_march(
     Grid3 g, const TC* __restrict__ A, const TC* __restrict__ L, const TC* __restrict__ invV,
-    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* __restrict__ x, const T* __restrict__ f,
+    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* x, const T* f,
     T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles, CertArgs ca) {
     using C = typename Compute<T>::type;
     constexpr int RW = TX + 2, RH = SY + 2, RP = RW * RH;   // ring plane: i0-1 .. i0+TX, j0-1 .. j0+SY
@@ -317,6 +318,7 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
     const int dp0 = dval ? g.idx(di, dj, 0) : 0;
     // ring entry of array a (0..2: b, 3..5: A) at node (ii, jj) of the plane in `slot`
     auto R = [&](int slot, int a, int ii, int jj) -> C { return s_ring[slot][a * RP + (jj - j0 + 1) * RW + (ii - i0 + 1)]; };
+    chain_wait();
     const C k2 = MODE == ST_CERT ? (C)ca.k2[blockIdx.y] : C(0);
     if (MODE == ST_CERT) x += blockIdx.y * ca.stride;
     C sum[kCertSums];
@@ -542,9 +544,10 @@ __global__ void k_cert_final(int nb, const double* __restrict__ part, double* __
 }
 
 template <typename T, typename TC>
-__global__ void k_jacobi_zero(Domain d, const TC* __restrict__ invD, const T* __restrict__ f, T* __restrict__ y,
+__global__ void k_jacobi_zero(Domain d, const TC* __restrict__ invD, const T* f, T* __restrict__ y,
                               typename Compute<T>::type om) {
     using C = typename Compute<T>::type;
+    chain_wait();
     for_each_entry(d, [&](long long q) { y[q] = to_store<T>(om * (C)invD[q] * (C)to_c(f[q])); });
 }
 
@@ -636,7 +639,7 @@ struct CellUnit {
 // launches; with one synchronisation less per iteration 5.4 -> 4.6 ms.
 template <typename T, typename TC, typename C>
 struct ScalJac0 {   // the first iterate from zero
-    const T* __restrict__ f;
+    const T* f;
     const TC* __restrict__ invD;
     C om;
     __device__ __forceinline__ C operator()(int p) const { return (C)to_c(to_store<T>(om * (C)invD[p] * (C)to_c(f[p]))); }
@@ -645,7 +648,7 @@ template <typename T, typename TC, typename C>
 struct ScalJac0Up {   // that iterate plus the parent's coarse correction
     ScalJac0<T, TC, C> x0;
     const unsigned char* __restrict__ active;
-    const T* __restrict__ ec;
+    const T* ec;
     Grid3 gf, gc;
     __device__ __forceinline__ C at(int p, int i, int j, int k) const {
         if (!active[p]) return C(0);
@@ -658,7 +661,7 @@ struct ScalJac0Up {   // that iterate plus the parent's coarse correction
 template <typename T, typename TC>
 __global__ void __launch_bounds__(TX * TY * TZ) k_scal_down(Grid3 g, Grid3 gc, const TC* __restrict__ A,
                                                             const unsigned char* __restrict__ active,
-                                                            const TC* __restrict__ invD, const T* __restrict__ f,
+                                                            const TC* __restrict__ invD, const T* f,
                                                             typename Compute<T>::type om,
                                                             const unsigned char* __restrict__ active_c,
                                                             T* __restrict__ fc, const int* __restrict__ tiles) {
@@ -666,6 +669,7 @@ __global__ void __launch_bounds__(TX * TY * TZ) k_scal_down(Grid3 g, Grid3 gc, c
     __shared__ C r[TZ][TY][TX];
     int i, j, k;
     block_node(g, tiles, i, j, k);
+    chain_wait();
     C v = C(0);
     if (i < g.nx && j < g.ny && k < g.nz) {
         const int p = g.idx(i, j, k);
@@ -699,12 +703,13 @@ __global__ void __launch_bounds__(TX * TY * TZ) k_scal_down(Grid3 g, Grid3 gc, c
 template <typename T, typename TC>
 __global__ void __launch_bounds__(TX * TY * TZ) k_scal_up(Grid3 g, Grid3 gc, const TC* __restrict__ A,
                                                           const unsigned char* __restrict__ active,
-                                                          const TC* __restrict__ invD, const T* __restrict__ f,
-                                                          typename Compute<T>::type om, const T* __restrict__ ec,
+                                                          const TC* __restrict__ invD, const T* f,
+                                                          typename Compute<T>::type om, const T* ec,
                                                           T* __restrict__ y, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     int i, j, k;
     block_node(g, tiles, i, j, k);
+    chain_wait();
     if (i >= g.nx || j >= g.ny || k >= g.nz) return;
     const int p = g.idx(i, j, k);
     C v = C(0);
@@ -839,7 +844,7 @@ constexpr int kFFY = 8, kFFZ = 8;
 template <typename T, bool CUBE>
 __global__ void __launch_bounds__(TX * kFFY, 3) k_vec_apply_ff(
     Grid3 g, const float2* __restrict__ A, const float2* __restrict__ L, const float2* __restrict__ invV, ffv rdx, ffv rdy,
-    ffv rdz, ffv r2, ffv sigma, const T* __restrict__ x, const int2* __restrict__ rowmap,
+    ffv rdz, ffv r2, ffv sigma, const T* x, const int2* __restrict__ rowmap,
     const unsigned char* __restrict__ rowflag, float2* __restrict__ out, T* __restrict__ zc, const int* __restrict__ tiles) {
     using O = typename FFOps<T>::type;
     using B = typename O::V;
@@ -893,6 +898,7 @@ __global__ void __launch_bounds__(TX * kFFY, 3) k_vec_apply_ff(
     }
     const bool dval = role >= 0 && di <= ilim && dj <= jlim;
     const int dp0 = dval ? g.idx(di, dj, 0) : 0;
+    chain_wait();
     const ffv one{1.f, 0.f};
     // whether the coefficients of this warp's row on plane k are all 1 (the same in the whole warp)
     auto ones = [&](int k) { return j <= g.ny && k >= 0 && k <= g.nz && (rowflag[row0 + k * rowz] & 1); };
@@ -1071,11 +1077,12 @@ __global__ void k_row_maps(Grid3 g, const double* __restrict__ A, const double* 
 // into zc alike.  A: the float-float face fractions, 1/h^2 float-float.
 template <typename T>
 __global__ void k_scal_apply_ff(Grid3 g, const float2* __restrict__ A, ffv rx2, ffv ry2, ffv rz2,
-                                const T* __restrict__ x, const int* __restrict__ cmap, float2* __restrict__ out,
+                                const T* x, const int* __restrict__ cmap, float2* __restrict__ out,
                                 T* __restrict__ zc, const int* __restrict__ tiles) {
     using O = typename FFOps<T>::type;
     int i, j, k;
     block_node(g, tiles, i, j, k);
+    chain_wait();
     if (i >= g.nx || j >= g.ny || k >= g.nz) return;
     const int p = g.idx(i, j, k);
     const int ci = cmap[p];
@@ -1141,7 +1148,7 @@ void vec_apply_ff(const FFLevel& f, double sigma, const T* x, float2* out, T* zc
     // bytes: per open face its x, A and about one L (8 each), a third of a 1/V (8), the output (8) and z
     const double bytes = (double)g.nopen * (16.0 + 8.0 / 3.0 + 8.0 + (zc ? 2.0 : 1.0) * sizeof(T));
     const bool cube = g.hx == g.hy && g.hy == g.hz;
-    launch_b("vec_apply_ff_L0", bytes, cube ? k_vec_apply_ff<T, true> : k_vec_apply_ff<T, false>, f.ntiles,
+    launch_chain("vec_apply_ff_L0", bytes, cube ? k_vec_apply_ff<T, true> : k_vec_apply_ff<T, false>, f.ntiles,
              dim3(TX, kFFY, 1), 0, s, g, f.A, f.L, f.invV, host_ff(g.rhx), host_ff(g.rhy), host_ff(g.rhz),
              host_ff(g.rhx * g.rhx), host_ff(sigma), x, f.rowmap, f.rowflag, out, zc, f.tiles);
 }
@@ -1153,7 +1160,7 @@ void scal_apply_ff(const Grid3& g, const int* tiles, int ntiles, const float2* A
     // bytes: per active cell its x, three float-float face fractions (24; six faces, each shared by two
     // cells), the output (8), its z and its compact index (4)
     const double bytes = (double)g.nact * (24.0 + 12.0 + 2.0 * sizeof(T));
-    launch_b("scal_apply_ff_L0", bytes, k_scal_apply_ff<T>, ntiles, kBlock, 0, s, g, A, host_ff(g.rhx * g.rhx),
+    launch_chain("scal_apply_ff_L0", bytes, k_scal_apply_ff<T>, ntiles, kBlock, 0, s, g, A, host_ff(g.rhx * g.rhx),
              host_ff(g.rhy * g.rhy), host_ff(g.rhz * g.rhz), x, cmap, out, zc, tiles);
 }
 
@@ -1191,7 +1198,7 @@ void vec_stencil(const VecOp<T, TC>& op, int mode, const T* x, const T* f, T* y,
     switch (op.shape * kStencilModes + mode) {
 #define DM_TILED(SH, MD, SY, SZ)                                                                              \
     case SH * kStencilModes + MD:                                                                                         \
-    launch_b(nm, bytes, k_vec_stencil_tiled<T, TC, MD, SY, SZ>, nt, dim3(TX, SY, SZ), 0, s, g, op.A, op.L,  \
+    launch_chain(nm, bytes, k_vec_stencil_tiled<T, TC, MD, SY, SZ>, nt, dim3(TX, SY, SZ), 0, s, g, op.A, op.L,  \
              op.invV, op.invD, op.sigma, x, f, y, omega, tl);                                             \
     break;
         DM_TILED(0, ST_APPLY, 4, 2) DM_TILED(0, ST_RESID, 4, 2) DM_TILED(0, ST_JACOBI, 4, 2) DM_TILED(0, ST_JACOBI2Z, 4, 2)
@@ -1200,7 +1207,7 @@ void vec_stencil(const VecOp<T, TC>& op, int mode, const T* x, const T* f, T* y,
 #undef DM_TILED
 #define DM_MARCH(SH, MD, SY, KZ)                                                                                \
     case SH * kStencilModes + MD:                                                                                         \
-    launch_b(nm, bytes, k_vec_stencil_march<T, TC, MD, SY, KZ>, nt, dim3(TX, SY, 1), 0, s, g, op.A, op.L,  \
+    launch_chain(nm, bytes, k_vec_stencil_march<T, TC, MD, SY, KZ>, nt, dim3(TX, SY, 1), 0, s, g, op.A, op.L,  \
              op.invV, op.invD, op.sigma, x, f, y, omega, tl, CertArgs{});                                 \
     break;
         DM_MARCH(3, ST_APPLY, 8, 8) DM_MARCH(3, ST_RESID, 8, 8) DM_MARCH(3, ST_JACOBI, 8, 8) DM_MARCH(3, ST_JACOBI2Z, 8, 8)
@@ -1261,7 +1268,7 @@ template <typename T, typename TC>
 void vec_jacobi_zero(const VecOp<T, TC>& op, const T* f, T* y, double omega, cudaStream_t s) {
     const Domain d{op.g, op.tiles, op.ntiles, 3};
     const int blocks = op.tiles ? std::max(op.ntiles, 1) : (int)std::min<long long>((d.len() + 255) / 256, 152 * 16);
-    launch_b(stencil_name("jacobi_zero", prec_index<T>(), ST_JACOBI, op.level == 0),
+    launch_chain(stencil_name("jacobi_zero", prec_index<T>(), ST_JACOBI, op.level == 0),
              (double)op.g.nopen * (2.0 * sizeof(T) + sizeof(TC)), k_jacobi_zero<T, TC>, blocks, 256, 0, s, d, op.invD,
              f, y, omega);
 }
@@ -1287,14 +1294,14 @@ template <typename T, typename TC>
 void scal_down(const ScalOp<T, TC>& op, const Grid3& gc, const unsigned char* active_c, const T* f, T* fc, double omega,
                cudaStream_t s) {
     // per fine cell f, 1/D, three face fractions and the flag; per coarse cell its result and flag
-    launch_b(stencil_name("scal_down", prec_index<T>(), ST_RESID, op.level == 0),
+    launch_chain(stencil_name("scal_down", prec_index<T>(), ST_RESID, op.level == 0),
              op.g.nact * (sizeof(T) + 4.0 * sizeof(TC) + 1.0) + gc.nact * (sizeof(T) + 1.0), k_scal_down<T, TC>,
              tile_grid(op.g, op.tiles, op.ntiles, 0), kBlock, 0, s, op.g, gc, op.A, op.active, op.invD, f, omega,
              active_c, fc, op.tiles);
 }
 template <typename T, typename TC>
 void scal_up(const ScalOp<T, TC>& op, const Grid3& gc, const T* f, const T* ec, T* y, double omega, cudaStream_t s) {
-    launch_b(stencil_name("scal_up", prec_index<T>(), ST_JACOBI, op.level == 0),
+    launch_chain(stencil_name("scal_up", prec_index<T>(), ST_JACOBI, op.level == 0),
              op.g.nact * (2.0 * sizeof(T) + 4.0 * sizeof(TC) + 1.0) + (double)gc.nact * sizeof(T), k_scal_up<T, TC>,
              tile_grid(op.g, op.tiles, op.ntiles, 0), kBlock, 0, s, op.g, gc, op.A, op.active, op.invD, f, omega, ec, y,
              op.tiles);

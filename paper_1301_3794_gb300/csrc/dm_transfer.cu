@@ -47,11 +47,12 @@ __device__ __forceinline__ void restrict_axis(bool normal, int c, int nc, int nf
 }
 
 template <typename T, typename TC, bool SYM>
-__global__ void k_face_restrict(Grid3 gf, Grid3 gc, const TC* __restrict__ Ac, const T* __restrict__ r,
+__global__ void k_face_restrict(Grid3 gf, Grid3 gc, const TC* __restrict__ Ac, const T* r,
                                 T* __restrict__ fc, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     int I, J, K;
     block_node(gc, tiles, I, J, K);
+    chain_wait();
     if (I > gc.nx || J > gc.ny || K > gc.nz) return;
     const int q = gc.idx(I, J, K);
 #pragma unroll
@@ -88,11 +89,12 @@ __global__ void k_face_restrict(Grid3 gf, Grid3 gc, const TC* __restrict__ Ac, c
 }
 
 template <typename T, typename TC, bool SYM>
-__global__ void k_face_prolong(Grid3 gf, Grid3 gc, const TC* __restrict__ Af, const T* __restrict__ ec,
-                               T* __restrict__ x, const int* __restrict__ tiles) {
+__global__ void k_face_prolong(Grid3 gf, Grid3 gc, const TC* __restrict__ Af, const T* ec,
+                               T* x, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     int i, j, k;
     block_node(gf, tiles, i, j, k);
+    chain_wait();
     if (i > gf.nx || j > gf.ny || k > gf.nz) return;
     const int p = gf.idx(i, j, k);
     const int nc[3] = {gc.nx, gc.ny, gc.nz};
@@ -151,10 +153,10 @@ void face_restrict(const Grid3& gf, const Grid3& gc, const TC* Ac, const T* r, T
     // every open fine face's r once; per open coarse face its A and f_c
     const double bytes = (double)gf.nopen * sizeof(T) + (double)gc.nopen * (sizeof(T) + sizeof(TC));
     if (sym)
-        launch_b("k_face_restrict", bytes, k_face_restrict<T, TC, true>, tile_grid(gc, tiles_c, ntiles_c, 1), kBlock, 0,
+        launch_chain("k_face_restrict", bytes, k_face_restrict<T, TC, true>, tile_grid(gc, tiles_c, ntiles_c, 1), kBlock, 0,
                  s, gf, gc, Ac, r, fc, tiles_c);
     else
-        launch_b("k_face_restrict", bytes, k_face_restrict<T, TC, false>, tile_grid(gc, tiles_c, ntiles_c, 1), kBlock,
+        launch_chain("k_face_restrict", bytes, k_face_restrict<T, TC, false>, tile_grid(gc, tiles_c, ntiles_c, 1), kBlock,
                  0, s, gf, gc, Ac, r, fc, tiles_c);
 }
 template <typename T, typename TC>
@@ -163,10 +165,10 @@ void face_prolong_add(const Grid3& gf, const Grid3& gc, const TC* Af, const T* e
     // every open coarse face's e_c once; per open fine face its A and x read and written
     const double bytes = (double)gc.nopen * sizeof(T) + (double)gf.nopen * (2.0 * sizeof(T) + sizeof(TC));
     if (sym)
-        launch_b("k_face_prolong", bytes, k_face_prolong<T, TC, true>, tile_grid(gf, tiles_f, ntiles_f, 1), kBlock, 0,
+        launch_chain("k_face_prolong", bytes, k_face_prolong<T, TC, true>, tile_grid(gf, tiles_f, ntiles_f, 1), kBlock, 0,
                  s, gf, gc, Af, ec, x, tiles_f);
     else
-        launch_b("k_face_prolong", bytes, k_face_prolong<T, TC, false>, tile_grid(gf, tiles_f, ntiles_f, 1), kBlock, 0,
+        launch_chain("k_face_prolong", bytes, k_face_prolong<T, TC, false>, tile_grid(gf, tiles_f, ntiles_f, 1), kBlock, 0,
                  s, gf, gc, Af, ec, x, tiles_f);
 }
 template <typename T, typename TC>
