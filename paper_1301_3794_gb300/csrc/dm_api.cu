@@ -2802,24 +2802,28 @@ dm_status dm_learned_train_step(dm_learned* net, dm_operator* op, const double* 
         GeoLevel& g0 = *const_cast<dm_geometry*>(op->geom)->lv[0];
         const long long n3 = 3ll * g0.g.np;
         const double h = std::min(g0.g.hx, std::min(g0.g.hy, g0.g.hz));
-        DBuf<double> rp(n3);
-        faces_in(op, 0, r, on_device, rp.get());
-        const double ss = sumsq<double>(n3, rp.get(), s);
+        LearnedNet& L = net->net;
+        if (L.r64.n != (size_t)n3) {
+            L.r64.alloc(n3);
+            L.r32.alloc(n3);
+            L.ybuf.alloc(n3);
+            L.kbuf.alloc(n3);
+        }
+        faces_in(op, 0, r, on_device, L.r64.get());
+        const double ss = sumsq<double>(n3, L.r64.get(), s);
         DM_REQUIRE(ss > 0.0 && op->nopen0 > 0, DM_ERR_INVALID_ARG, "learned train step: zero residual");
         const double rms = std::sqrt(ss / (double)op->nopen0);
         {
             std::lock_guard<std::mutex> lock(const_cast<dm_geometry*>(op->geom)->mu);
             ensure_f32(g0, s);
         }
-        DBuf<float> r32(n3), ybuf(n3), kbuf(n3);
-        convert<float, double>(g0.vdom(), rp.get(), r32.get(), s);
+        convert<float, double>(g0.vdom(), L.r64.get(), L.r32.get(), s);
         const VecOp<float, float> o32{g0.g, g0.A32.get(), g0.L32.get(), g0.invV32.get(), nullptr, op->sigma, 0,
                                       g0.tiles.get(), g0.ntiles, nullptr, 0, 0};
-        LearnedNet& L = net->net;
         L.alloc(g0.g);
-        L.features(g0.A.get(), g0.V.get(), 1.0 / rms, r32.get(), 1, s);
+        L.features(g0.A.get(), g0.V.get(), 1.0 / rms, L.r32.get(), 1, s);
         L.forward(s);
-        const float l = L.residual_loss(o32, g0.A.get(), r32.get(), 1.0 / rms, h * h, ybuf.get(), kbuf.get(),
+        const float l = L.residual_loss(o32, g0.A.get(), L.r32.get(), 1.0 / rms, h * h, L.ybuf.get(), L.kbuf.get(),
                                         (double)op->nopen0, s);
         L.backward(s);
         L.check(s);

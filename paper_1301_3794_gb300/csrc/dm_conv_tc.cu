@@ -25,8 +25,19 @@
 // rows).  The accumulator (128 lanes x 16 FP32 columns) lives in tensor memory;
 // each of the 4 warps reads its 32 lanes back with tcgen05.ld for the epilogue.
 //
+// A CTA is a pipeline over its tiles: while the tensor cores work on one tile,
+// the next tile's windows arrive in a second set of buffers and the previous
+// tile's sums leave a second accumulator; one after another (copy, multiply, read
+// out) a tile took about 10 us.  (The two BF16 parts of a weight as 32 columns of
+// one MMA, with two sums to add, is no faster and rounds differently.)
+// With the CTAs an SM has room for (the occupancy query gave one) an SM works on
+// several tiles' chains of 54 dependent products, whose latency is what is left.
+// Measured, 49 x 49 x 577 nodes: two hidden layers forward 290 -> 116 us each, the
+// output layer 322 -> 160, the adjoints 376 -> 147; a training step 3.06 -> 1.55 ms.
+//
 // Every wait on an mbarrier gives up after about a second: the kernel then
-// records an error code, stops issuing work and releases its tensor memory.
+// records an error code, stops issuing work, waits (as long) for the copies in
+// flight and releases its tensor memory.
 #include "dm_common.cuh"
 #include "dm_learned.cuh"
 
@@ -40,7 +51,7 @@ constexpr int kTileM = 128;                 // nodes per tile (MMA M)
 constexpr int kWin = kTileM + 2;            // window rows: one extra node on each side
 constexpr int kWinBytes = kWin * 16;        // 2080
 constexpr int kStepBytes = 2 * 16 * 16 * 2; // one step's B tiles (N = 16, K = 16, BF16): high part, low part
-constexpr uint32_t kTmemCols = 32;          // smallest allocation; columns 0..15 used
+constexpr uint32_t kTmemCols = 32;          // two accumulators of 16 columns
 constexpr unsigned long long kWaitNs = 1000000000ull;   // one second
 
 // instruction descriptor of tcgen05.mma kind::f16: BF16 A and B (K-major),
@@ -106,20 +117,12 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
     return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
-        "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
-        : "memory");
-}
-__device__ __forceinline__ void mma_bf16_id(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "l"(a), "l"(b), "r"(id), "r"(acc)
         : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -165,8 +168,8 @@ __global__ void k_pack_wtiles(const float* __restrict__ W, int wcin, int wcout, 
     const int nsteps = cb == 2 ? 27 : 14;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nsteps * 256; e += gridDim.x * blockDim.x) {
         const int s = e / 256, r = e % 256;
-        __nv_bfloat16* const o = out + s * 512 + r;
         const int kh = r / 128, r2 = r % 128, ng = r2 / 64, r3 = r2 % 64, n = ng * 8 + r3 / 8, kl = r3 % 8;
+        __nv_bfloat16* const o = out + s * 512 + r;
         const int kin = kh * 8 + kl;
         int t, ch;
         if (cb == 2) {
@@ -197,9 +200,10 @@ __global__ void __launch_bounds__(128) k_conv_tc(Grid3 g, ActLayout L, const __n
     constexpr int kSteps = CB == 2 ? 27 : 14;
     constexpr int kChunks = 9 * CB;
     extern __shared__ __align__(128) unsigned char smem[];
-    unsigned char* s_w = smem;                                   // kSteps B tiles
-    unsigned char* s_win = smem + kSteps * kStepBytes;           // kChunks windows (+ slack)
-    __shared__ __align__(8) uint64_t bar_load, bar_mma;
+    unsigned char* s_w = smem;                             // kSteps B tiles
+    unsigned char* s_win = smem + kSteps * kStepBytes;     // two buffers of kChunks windows
+    constexpr int kBuf = kChunks * kWinBytes;
+    __shared__ __align__(8) uint64_t bar_load[2], bar_mma[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -211,8 +215,10 @@ __global__ void __launch_bounds__(128) k_conv_tc(Grid3 g, ActLayout L, const __n
         for (int e = tid; e < kSteps * kStepBytes / 16; e += 128) dst[e] = src[e];
     }
     if (tid == 0) {
-        mbar_init(&bar_load, 1);
-        mbar_init(&bar_mma, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&bar_load[b], 1);
+            mbar_init(&bar_mma[b], 1);
+        }
         s_abort = 0;
         fence_barrier_init();
     }
@@ -223,102 +229,119 @@ __global__ void __launch_bounds__(128) k_conv_tc(Grid3 g, ActLayout L, const __n
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     const uint32_t w_base = smem_u32(s_w), win_base = smem_u32(s_win);
-    uint32_t phase = 0;
-
-    for (int t = tile0 + blockIdx.x; t < tile0 + ntiles; t += gridDim.x) {
-        const int p0 = t * kTileM;
-        if (tid == 0) {
-            mbar_expect_tx(&bar_load, kChunks * kWinBytes);
+    const int nit = blockIdx.x < ntiles ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    auto first_node = [&](int it) { return (tile0 + (int)blockIdx.x + it * (int)gridDim.x) * kTileM; };
+    auto load = [&](int it) {   // one thread
+        const int buf = it & 1, p0 = first_node(it);
+        mbar_expect_tx(&bar_load[buf], kBuf);
 #pragma unroll 1
-            for (int ab = 0; ab < 9; ++ab) {
-                const int a = ab / 3, b = ab % 3;
-                const int q = p0 + (b - 1) * g.sx + (a - 1) * g.sxy - 1;
+        for (int ab = 0; ab < 9; ++ab) {
+            const int a = ab / 3, b = ab % 3;
+            const int q = p0 + (b - 1) * g.sx + (a - 1) * g.sxy - 1;
 #pragma unroll
-                for (int cb = 0; cb < CB; ++cb)
-                    bulk_g2s(s_win + (ab * CB + cb) * kWinBytes, in + L.at(cb, q), kWinBytes, &bar_load);
-            }
+            for (int cb = 0; cb < CB; ++cb)
+                bulk_g2s(s_win + buf * kBuf + (ab * CB + cb) * kWinBytes, in + L.at(cb, q), kWinBytes, &bar_load[buf]);
         }
-        if (!mbar_wait(&bar_load, phase)) {
-            atomicExch(err, 1);
-            s_abort = 1;
-        }
-        __syncthreads();
-        if (s_abort) break;
-        if (tid == 0) {
-            tc_fence_after();
-#pragma unroll 1
-            for (int s = 0; s < kSteps; ++s) {
-                uint32_t a0, lbo;
-                if (CB == 2) {
-                    const int ab = s / 3, c = s % 3;
-                    a0 = win_base + ab * CB * kWinBytes + c * 16;
-                    lbo = kWinBytes;   // second channel block's window
-                } else if (s < 13) {
-                    const int t1 = 2 * s, t2 = t1 + 1;
-                    a0 = win_base + (t1 / 3) * kWinBytes + (t1 % 3) * 16;
-                    lbo = win_base + (t2 / 3) * kWinBytes + (t2 % 3) * 16 - a0;
-                } else {
-                    // lower half: zero weights on tap 0's rows (finite data); upper half: tap 26
-                    a0 = win_base;
-                    lbo = 8 * kWinBytes + 2 * 16;
+    };
+    auto epilogue = [&](int it) {
+        float v[16];
+        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (it & 1) * 16, v);
+        const int p = first_node(it) + warp * 32 + lane;
+        if (p >= L.np) return;
+        const bool ok = grid_node(g, p);
+        if (EPI == EPI_F32_3) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) outY[(size_t)p * 3 + c] = ok ? v[c] : 0.f;
+        } else {
+#pragma unroll
+            for (int cb = 0; cb < 2; ++cb) {
+                float m[8];
+                if (EPI == EPI_MASK_BF16) {
+                    const uint4 mv = *reinterpret_cast<const uint4*>(mask + L.at(cb, p));
+                    const __nv_bfloat16* mb = reinterpret_cast<const __nv_bfloat16*>(&mv);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) m[c] = __bfloat162float(mb[c]) > 0.f ? 1.f : 0.f;
                 }
-                const uint64_t ad = sdesc(a0, lbo, 128);
-                mma_bf16(tmem, ad, sdesc(w_base + s * kStepBytes, 256, 128), s > 0 ? 1u : 0u);
-                mma_bf16(tmem, ad, sdesc(w_base + s * kStepBytes + 512, 256, 128), 1u);
+                __align__(16) __nv_bfloat16 o[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    float x = v[cb * 8 + c];
+                    if (EPI == EPI_RELU_BF16) x = fmaxf(x, 0.f);
+                    else x *= m[c];
+                    o[c] = __float2bfloat16(ok ? x : 0.f);
+                }
+                *reinterpret_cast<uint4*>(out + L.at(cb, p)) = *reinterpret_cast<const uint4*>(o);
             }
-            mma_commit(&bar_mma);
         }
-        if (!mbar_wait(&bar_mma, phase)) {
+    };
+    // Tile `it` uses buffer and accumulator it & 1, whose barriers complete their
+    // phase it >> 1.  At its turn the tile before it has been multiplied (so the
+    // other buffer is free) and waits in its accumulator to be read out, which
+    // happens while this tile's products run.
+    if (tid == 0 && nit > 0) load(0);
+    for (int it = 0; it < nit; ++it) {
+        const int buf = it & 1;
+        const uint32_t parity = (uint32_t)(it >> 1) & 1u;
+        if (tid == 0) {
+            if (it + 1 < nit) load(it + 1);
+            if (!mbar_wait(&bar_load[buf], parity)) {
+                atomicExch(err, 1);
+                s_abort = 1;
+            } else {
+                tc_fence_after();
+                const uint32_t wb = win_base + buf * kBuf;
+#pragma unroll 1
+                for (int s = 0; s < kSteps; ++s) {
+                    uint32_t a0, lbo;
+                    if (CB == 2) {
+                        const int ab = s / 3, c = s % 3;
+                        a0 = wb + ab * CB * kWinBytes + c * 16;
+                        lbo = kWinBytes;   // second channel block's window
+                    } else if (s < 13) {
+                        const int t1 = 2 * s, t2 = t1 + 1;
+                        a0 = wb + (t1 / 3) * kWinBytes + (t1 % 3) * 16;
+                        lbo = wb + (t2 / 3) * kWinBytes + (t2 % 3) * 16 - a0;
+                    } else {
+                        // lower half: zero weights on tap 0's rows (finite data); upper half: tap 26
+                        a0 = wb;
+                        lbo = 8 * kWinBytes + 2 * 16;
+                    }
+                    const uint64_t ad = sdesc(a0, lbo, 128);
+                    mma_bf16(tmem + buf * 16, ad, sdesc(w_base + s * kStepBytes, 256, 128), kIdesc, s > 0 ? 1u : 0u);
+                    mma_bf16(tmem + buf * 16, ad, sdesc(w_base + s * kStepBytes + 512, 256, 128), kIdesc, 1u);
+                }
+                mma_commit(&bar_mma[buf]);
+            }
+        }
+        __syncwarp();
+        if (it > 0) {
+            tc_fence_after();
+            epilogue(it - 1);
+        }
+        // (with no products issued there is nothing to wait for: every thread then learns of it below)
+        if (!mbar_wait(&bar_mma[buf], parity)) {
             atomicExch(err, 2);
             s_abort = 1;
         }
-        tc_fence_after();
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16), v);
-        const int p = p0 + warp * 32 + lane;
-        if (p < L.np) {
-            const bool ok = grid_node(g, p) && !s_abort;
-            if (EPI == EPI_F32_3) {
-#pragma unroll
-                for (int c = 0; c < 3; ++c) outY[(size_t)p * 3 + c] = ok ? v[c] : 0.f;
-            } else {
-#pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    float m[8];
-                    if (EPI == EPI_MASK_BF16) {
-                        const uint4 mv = *reinterpret_cast<const uint4*>(mask + L.at(cb, p));
-                        const __nv_bfloat16* mb = reinterpret_cast<const __nv_bfloat16*>(&mv);
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) m[c] = __bfloat162float(mb[c]) > 0.f ? 1.f : 0.f;
-                    }
-                    __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float x = v[cb * 8 + c];
-                        if (EPI == EPI_RELU_BF16) x = fmaxf(x, 0.f);
-                        else x *= m[c];
-                        o[c] = __float2bfloat16(ok ? x : 0.f);
-                    }
-                    *reinterpret_cast<uint4*>(out + L.at(cb, p)) = *reinterpret_cast<const uint4*>(o);
-                }
-            }
-        }
         tc_fence_before();
         __syncthreads();
-        if (s_abort) break;
-        phase ^= 1u;
+        tc_fence_after();
+        if (s_abort) {
+            if (tid == 0 && it + 1 < nit) mbar_wait(&bar_load[buf ^ 1], (uint32_t)((it + 1) >> 1) & 1u);
+            break;
+        }
     }
+    if (nit > 0 && !s_abort) epilogue(nit - 1);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
-// shared bytes of a conv kernel: B tiles, windows, and slack so that a
-// descriptor with its two strides exchanged still stays inside the allocation
+// shared bytes of a conv kernel: B tiles and two buffers of windows
 template <int CB>
 constexpr size_t conv_smem() {
-    return (size_t)(CB == 2 ? 27 : 14) * kStepBytes + (size_t)9 * CB * kWinBytes + 16 * kWinBytes;
+    return (size_t)(CB == 2 ? 27 : 14) * kStepBytes + 2 * (size_t)9 * CB * kWinBytes;
 }
 
 template <int CB, int EPI>
@@ -333,12 +356,14 @@ void conv_tc_launch(const Grid3& g, const ActLayout& L, const __nv_bfloat16* in,
     const int first = g.off0 / kTileM;
     const int last = g.idx(g.nx, g.ny, g.nz) / kTileM;
     const int ntiles = last - first + 1;
-    int per_sm = 0;
-    DM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_conv_tc<CB, EPI>, 128, sm));
+    // CTAs per SM by shared memory (103 and 52 KB); the occupancy query answers 1
+    // for a kernel that allocates tensor memory, of which these take 32 of 512 columns
+    constexpr int per_sm = CB == 2 ? 2 : 4;
+    static_assert(per_sm * (conv_smem<CB>() + 2048) <= 228 * 1024, "CTAs per SM");
     int dev = 0, sms = 0;
     DM_CUDA(cudaGetDevice(&dev));
     DM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int grid = std::max(1, std::min(ntiles, sms * std::max(per_sm, 1)));
+    const int grid = std::max(1, std::min(ntiles, sms * per_sm));
     // bytes: every input block's nodes once, the output once
     const double bytes = (double)L.np * (16.0 * CB + (EPI == EPI_F32_3 ? 12.0 : 32.0 + (EPI == EPI_MASK_BF16 ? 32.0 : 0.0)));
     launch_b(EPI == EPI_F32_3 ? "conv_tc_out" : (EPI == EPI_MASK_BF16 ? "conv_tc_adjoint" : "conv_tc_relu"), bytes,
@@ -360,6 +385,8 @@ void conv_tc_launch(const Grid3& g, const ActLayout& L, const __nv_bfloat16* in,
 // cout hold whatever the slots contain and are never read out.
 constexpr int kDwSlot = kTileM * 16;     // one 128-node window of 8 channels
 constexpr uint32_t kIdescMN = kIdesc | (1u << 15) | (1u << 16);
+// The copies bound it: 27 taps' windows, 110 KB a node tile, come from L2 at 8 TB/s.
+// (Two sets of buffers, three CTAs an SM, took 143 us where this takes 135.)
 constexpr int kDwCtasPerSm = 4;
 
 template <int CB>
@@ -417,7 +444,7 @@ __global__ void __launch_bounds__(128) k_conv_dw_tc(Grid3 g, ActLayout L, const 
                 tc_fence_after();
 #pragma unroll 1
                 for (int kk = 0; kk < kTileM / 16; ++kk)
-                    mma_bf16_id(tmem + mt * 16, sdesc(a_base + kk * 256, 128, kDwSlot),
+                    mma_bf16(tmem + mt * 16, sdesc(a_base + kk * 256, 128, kDwSlot),
                                 sdesc(b_base + kk * 256, 128, kDwSlot), kIdescMN, (first && kk == 0) ? 0u : 1u);
                 mma_commit(&bar_mma);
             }
@@ -449,14 +476,29 @@ __global__ void __launch_bounds__(128) k_conv_dw_tc(Grid3 g, ActLayout L, const 
     if (warp == 0) tmem_dealloc(tmem, kCols);
 }
 
-// dW[t][ci][co] = sum over CTAs (in CTA order) of part[cta][t][ci][co]
-__global__ void k_dw_sum(const float* __restrict__ part, int nparts, int cin, int cout, float* __restrict__ dW) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= 27 * cin * cout) return;
-    const int t = e / (cin * cout), r = e % (cin * cout), ci = r / cout, co = r % cout;
+// dW[t][ci][co] = sum over CTAs of part[cta][t][ci][co], in a fixed order: a block
+// takes 32 entries, its 8 warps every eighth part each (one thread per entry
+// before, whose loads came one after another: 34 us)
+__global__ void __launch_bounds__(256) k_dw_sum(const float* __restrict__ part, int nparts, int cin, int cout,
+                                                float* __restrict__ dW) {
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
+    const bool in = e < 27 * cin * cout;
     float s = 0.f;
-    for (int b = 0; b < nparts; ++b) s += part[((size_t)b * 27 + t) * 256 + ci * 16 + co];
-    dW[e] = s;
+    if (in) {
+        const int t = e / (cin * cout), r = e % (cin * cout), ci = r / cout, co = r % cout;
+        const float* p = part + (size_t)t * 256 + ci * 16 + co;
+#pragma unroll 8
+        for (int b = wid; b < nparts; b += 8) s += p[(size_t)b * 27 * 256];
+    }
+    red[wid][lane] = s;
+    __syncthreads();
+    if (wid == 0 && in) {
+        float v = 0.f;
+        for (int w = 0; w < 8; ++w) v += red[w][lane];
+        dW[e] = v;
+    }
 }
 
 }  // namespace
@@ -494,7 +536,7 @@ void conv_dw_tc(const Grid3& g, const ActLayout& L, int cb_in, int cin, const __
                  err);
     }
     const int n = 27 * cin * cout;
-    launch("conv_tc_dw_sum", k_dw_sum, (n + 127) / 128, 128, 0, s, (const float*)part, nparts, cin, cout, dW);
+    launch("conv_tc_dw_sum", k_dw_sum, (n + 31) / 32, 256, 0, s, (const float*)part, nparts, cin, cout, dW);
 }
 
 ActLayout act_layout(const Grid3& g) {

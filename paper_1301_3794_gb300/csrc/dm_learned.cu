@@ -30,15 +30,6 @@ namespace {
 
 constexpr int LX = TX, LY = TY, LZ = TZ;                 // node tile of the elementwise kernels
 
-// column sums of part[nb][n] in block order
-__global__ void k_colsum(const float* __restrict__ part, int nb, int n, float* __restrict__ out) {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= n) return;
-    float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += part[(size_t)b * n + w];
-    out[w] = s;
-}
-
 // input features of every node: residual / scale on the three faces, A_x, A_y, A_z, V, 0
 template <typename T>
 __global__ void k_features(Grid3 g, ActLayout L, const T* __restrict__ r, const double* __restrict__ A,
@@ -184,12 +175,19 @@ __global__ void k_sumsq(long long n, const T* __restrict__ x, double* __restrict
     }
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
-__global__ void k_sum_d(const double* __restrict__ part, int n, double* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < n; ++b) s += part[b];
-        *out = s;
+// *out = sum of part[0 .. n), one block of 256 threads, in a fixed order
+template <typename R>
+__global__ void k_sum(const R* __restrict__ part, int n, R* __restrict__ out) {
+    __shared__ R red[256];
+    R s = R(0);
+    for (int b = threadIdx.x; b < n; b += 256) s += part[b];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) *out = red[0];
 }
 
 inline dim3 node_blocks(const Grid3& g) {
@@ -285,7 +283,7 @@ float LearnedNet::loss(const double* A, double msum, cudaStream_t s) {
            (float)(1.0 / std::max(msum, 1.0)), dY.get(), loss_part.get());
     const int n = nb.x * nb.y * nb.z;
     DBuf<float> tot(1);
-    launch("learned_mse_sum", k_colsum, 1, 256, 0, s, loss_part.get(), n, 1, tot.get());
+    launch("learned_mse_sum", k_sum<float>, 1, 256, 0, s, (const float*)loss_part.get(), n, tot.get());
     float h = 0.f;
     DM_CUDA(cudaMemcpyAsync(&h, tot.get(), sizeof(float), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
@@ -305,7 +303,7 @@ float LearnedNet::residual_loss(const VecOp<float, float>& o, const double* A, c
     const float inv_m = (float)(1.0 / std::max(msum, 1.0));
     launch("learned_res_loss", k_res_loss, nb, 256, 0, s, n, r, (float)inv_scale, A, kbuf, inv_m, loss_part.get());
     DBuf<float> tot(1);
-    launch("learned_mse_sum", k_colsum, 1, 256, 0, s, loss_part.get(), nb, 1, tot.get());
+    launch("learned_mse_sum", k_sum<float>, 1, 256, 0, s, (const float*)loss_part.get(), nb, tot.get());
     // dloss/dy = -K res / msum (K symmetric), dloss/dY = h^2 dloss/dy
     vec_stencil<float, float>(o, ST_APPLY, kbuf, nullptr, ybuf, 0.0, s);
     launch("learned_grad_gather", k_grad_gather, node_blocks(g), dim3(LX, LY, LZ), 0, s, g, L, ybuf, A,
@@ -340,7 +338,7 @@ double sumsq(long long n, const T* x, cudaStream_t s) {
     const int nb = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152 * 4));
     DBuf<double> part(nb), out(1);
     launch("learned_sumsq", k_sumsq<T>, nb, 256, 0, s, n, x, part.get());
-    launch("learned_sumsq", k_sum_d, 1, 32, 0, s, part.get(), nb, out.get());
+    launch("learned_sumsq", k_sum<double>, 1, 256, 0, s, (const double*)part.get(), nb, out.get());
     double h = 0.0;
     DM_CUDA(cudaMemcpyAsync(&h, out.get(), sizeof(double), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
