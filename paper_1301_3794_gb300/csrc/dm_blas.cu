@@ -502,13 +502,15 @@ __global__ void __launch_bounds__(kThreads, 2) k_ff_dcgs_dots(long long n2, int 
 //   v <- (v - Q s) / beta   (the pending vector, now finished)
 //   out <- w - Q gamma - delta v_old   and the block partial of |out|^2
 // Two entries per thread and step, as in the dots pass.
-__global__ void k_ff_dcgs_update(long long n2, int j, const float4* Q, long long ld2,
-                                 const double* coef, float4* v, const float4* w,
+__global__ void k_ff_dcgs_update(long long n2, int j, const float4* Q_in, long long ld2,
+                                 const double* coef, float4* v, const float4* w_in,
                                  float4* __restrict__ out, double* __restrict__ partial) {
     __shared__ float2 cs[128], cg[128];
     __shared__ float2 rb, dl;
     __shared__ double red[kThreads / 32];
     chain_wait();
+    const float4* __restrict__ Q = after_wait(Q_in);
+    const float4* __restrict__ w = after_wait(w_in);
     for (int c = threadIdx.x; c < j; c += blockDim.x) {
         cs[c] = ff_bits(-coef[c]);
         cg[c] = ff_bits(-coef[j + c]);
@@ -612,21 +614,30 @@ __global__ void k_ff_gather(long long n, const int* __restrict__ list, double a,
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         y[i] = ff_bits(a == 1.0 ? x[list[i]] : a * x[list[i]]);
 }
-// y[list[i]] = a x[i] in storage type T   (scatter from a compact float-float vector)
+// y[list[i]] = a x[i] in storage type T   (scatter from a compact float-float vector);
+// four entries a step, so that a thread's loads are in flight together
 template <typename T>
-__global__ void k_ff_scatter(long long n, const int* __restrict__ list, typename Compute<T>::type a,
-                             const float2* x, T* __restrict__ y) {
+__global__ void k_ff_scatter(long long n, const int* __restrict__ list, typename Compute<T>::type a, const float2* x,
+                             T* __restrict__ y) {
+    constexpr int U = 4;
+    const long long st = (long long)gridDim.x * blockDim.x;
     chain_wait();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float2 v = x[i];
-        if constexpr (std::is_same<T, double>::value) y[list[i]] = a * ff_to_double(v);
-        else y[list[i]] = to_store<T>(a * __fadd_rn(v.x, v.y));
+    for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < n; i0 += U * st) {
+        float2 v[U];
+        int q[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * st < n) {
+                v[u] = x[i0 + u * st];
+                q[u] = list[i0 + u * st];
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * st < n) {
+                if constexpr (std::is_same<T, double>::value) y[q[u]] = a * ff_to_double(v[u]);
+                else y[q[u]] = to_store<T>(a * __fadd_rn(v[u].x, v[u].y));
+            }
     }
-}
-
-inline int blocks_for(const Domain& d) {
-    const long long work = d.tiles ? (long long)d.ntiles : (d.len() + kThreads - 1) / kThreads;
-    return (int)std::max<long long>(1, std::min<long long>(work, kMaxBlocks));
 }
 
 // Grid of a grid-stride kernel: at most one full wave (the blocks that fit on

@@ -240,6 +240,13 @@ struct ChainScope {
     ChainScope(const ChainScope&) = delete;
     ChainScope& operator=(const ChainScope&) = delete;
 };
+// a pointer whose loads come after the wait (the compiler cannot see through it, so
+// the copy may be __restrict__ where the parameter may not)
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 template <typename... KArgs, typename... Args>
 inline void launch_chain(const char* name, double bytes, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                          cudaStream_t s, Args&&... args) {

@@ -35,7 +35,7 @@ inline dim3 node_grid(const Grid3& g, int extra = 1) {
 // Field accessor over a padded 3-component vector in storage type T.
 template <typename T, typename C>
 struct VecAcc {
-    const T* x;
+    const T* __restrict__ x;
     int np;
     __device__ __forceinline__ C operator()(int c, int p) const { return (C)to_c(x[c * np + p]); }
 };
@@ -44,7 +44,7 @@ struct VecAcc {
 // reads its x through this instead of from a vector that pass would write.
 template <typename T, typename TC, typename C>
 struct Jac0Acc {
-    const T* f;
+    const T* __restrict__ f;
     const TC* __restrict__ invD;
     C om;
     int np;
@@ -136,7 +136,7 @@ __device__ __forceinline__ C face_K(const Coef<C, TC>& cf, const Acc& b, int c, 
 template <typename T, typename TC, int MODE, int SY, int SZ>
 __global__ void __launch_bounds__(TX * SY * SZ) k_vec_stencil_tiled(
     Grid3 g, const TC* __restrict__ A, const TC* __restrict__ L, const TC* __restrict__ invV,
-    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* x, const T* f,
+    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* x_in, const T* f_in,
     T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     constexpr int PSI_X = TX + 1, PSI_Y = SY + 1, PSI_Z = SZ + 1;   // psi: i0-1 .. i0+TX-1 (and j, k alike)
@@ -148,6 +148,8 @@ __global__ void __launch_bounds__(TX * SY * SZ) k_vec_stencil_tiled(
     constexpr int NT = TX * SY * SZ;
     __shared__ C s_psi[N_PSI], s_ex[N_EX], s_ey[N_EY], s_ez[N_EZ];
     chain_wait();
+    const T* __restrict__ x = after_wait(x_in);
+    const T* __restrict__ f = after_wait(f_in);
     const int t = tiles[blockIdx.x];
     const int nti = (g.nx + TX) / TX, ntj = (g.ny + SY) / SY;
     const int i0 = (t % nti) * TX, j0 = ((t / nti) % ntj) * SY, k0 = (t / (nti * ntj)) * SZ;
@@ -255,7 +257,7 @@ struct CertArgs {
 template <typename T, typename TC, int MODE, int SY, int KZ, int IN = IN_PADDED>
 __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512 : 768) / (TX * SY)) k_vec_stencil_march(
     Grid3 g, const TC* __restrict__ A, const TC* __restrict__ L, const TC* __restrict__ invV,
-    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* x, const T* f,
+    const TC* __restrict__ invD, typename Compute<T>::type sigma, const T* x_in, const T* f_in,
     T* __restrict__ y, typename Compute<T>::type omega, const int* __restrict__ tiles, CertArgs ca) {
     using C = typename Compute<T>::type;
     constexpr int RW = TX + 2, RH = SY + 2, RP = RW * RH;   // ring plane: i0-1 .. i0+TX, j0-1 .. j0+SY
@@ -319,6 +321,8 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
     // ring entry of array a (0..2: b, 3..5: A) at node (ii, jj) of the plane in `slot`
     auto R = [&](int slot, int a, int ii, int jj) -> C { return s_ring[slot][a * RP + (jj - j0 + 1) * RW + (ii - i0 + 1)]; };
     chain_wait();
+    const T* __restrict__ x = after_wait(x_in);
+    const T* __restrict__ f = after_wait(f_in);
     const C k2 = MODE == ST_CERT ? (C)ca.k2[blockIdx.y] : C(0);
     if (MODE == ST_CERT) x += blockIdx.y * ca.stride;
     C sum[kCertSums];
@@ -844,7 +848,7 @@ constexpr int kFFY = 8, kFFZ = 8;
 template <typename T, bool CUBE>
 __global__ void __launch_bounds__(TX * kFFY, 3) k_vec_apply_ff(
     Grid3 g, const float2* __restrict__ A, const float2* __restrict__ L, const float2* __restrict__ invV, ffv rdx, ffv rdy,
-    ffv rdz, ffv r2, ffv sigma, const T* x, const int2* __restrict__ rowmap,
+    ffv rdz, ffv r2, ffv sigma, const T* x_in, const int2* __restrict__ rowmap,
     const unsigned char* __restrict__ rowflag, float2* __restrict__ out, T* __restrict__ zc, const int* __restrict__ tiles) {
     using O = typename FFOps<T>::type;
     using B = typename O::V;
@@ -899,6 +903,7 @@ __global__ void __launch_bounds__(TX * kFFY, 3) k_vec_apply_ff(
     const bool dval = role >= 0 && di <= ilim && dj <= jlim;
     const int dp0 = dval ? g.idx(di, dj, 0) : 0;
     chain_wait();
+    const T* __restrict__ x = after_wait(x_in);
     const ffv one{1.f, 0.f};
     // whether the coefficients of this warp's row on plane k are all 1 (the same in the whole warp)
     auto ones = [&](int k) { return j <= g.ny && k >= 0 && k <= g.nz && (rowflag[row0 + k * rowz] & 1); };

@@ -20,23 +20,18 @@ namespace {
 constexpr int BX = 32, BY = 4, BZ = 2;
 const dim3 kBlock(BX, BY, BZ);
 
-// Fine faces that a coarse face (coarse index c along an axis) gathers, with
-// the weights of P^T along that axis: along the face normal the fine planes
-// 2c-1, 2c, 2c+1 (weights 1/2, 1, 1/2); within the plane the fine cells
-// 2c-1 .. 2c+2 (weights 1/4, 3/4, 3/4, 1/4, the wall rule moving a missing
-// neighbour's 1/4 onto the nearer face).  Slots outside the grid get weight 0
-// and point at ghost positions (zero in every vector).
-__device__ __forceinline__ void restrict_axis(bool normal, int c, int nc, int nf, int idx[4], float w[4]) {
-    idx[0] = 2 * c - 1;
-    idx[1] = 2 * c;
-    idx[2] = 2 * c + 1;
-    idx[3] = 2 * c + 2;
+// Weights with which a coarse face (coarse index c along an axis) gathers the
+// fine faces 2c - 1 .. 2c + 2 of P^T along that axis: along the face normal the
+// planes 2c-1, 2c, 2c+1 (1/2, 1, 1/2); within the plane the cells 2c-1 .. 2c+2
+// (1/4, 3/4, 3/4, 1/4, the wall rule moving a missing neighbour's 1/4 onto the
+// nearer face).  Positions outside the grid get weight 0 and are ghosts (zero in
+// every vector).
+__device__ __forceinline__ void restrict_axis(bool normal, int c, int nc, int nf, float w[4]) {
     if (normal) {
         w[0] = c >= 1 ? 0.5f : 0.f;
         w[1] = 1.f;
         w[2] = 2 * c + 1 <= nf ? 0.5f : 0.f;
         w[3] = 0.f;
-        idx[3] = 2 * c;
     } else {
         const bool lo = c >= 1, hi = c + 1 < nc;
         w[0] = lo ? 0.25f : 0.f;
@@ -47,25 +42,26 @@ __device__ __forceinline__ void restrict_axis(bool normal, int c, int nc, int nf
 }
 
 template <typename T, typename TC, bool SYM>
-__global__ void k_face_restrict(Grid3 gf, Grid3 gc, const TC* __restrict__ Ac, const T* r,
+__global__ void k_face_restrict(Grid3 gf, Grid3 gc, const TC* __restrict__ Ac, const T* r_in,
                                 T* __restrict__ fc, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     int I, J, K;
     block_node(gc, tiles, I, J, K);
     chain_wait();
+    const T* __restrict__ r = after_wait(r_in);
     if (I > gc.nx || J > gc.ny || K > gc.nz) return;
     const int q = gc.idx(I, J, K);
+    const int base = gf.idx(2 * I - 1, 2 * J - 1, 2 * K - 1);
 #pragma unroll
     for (int comp = 0; comp < 3; ++comp) {
         const int oq = comp * gc.np + q;
         C acc = C(0);
         if ((C)Ac[oq] > C(0)) {
-            int ix[4], iy[4], iz[4];
             float wx[4], wy[4], wz[4];
-            restrict_axis(comp == 0, I, gc.nx, gf.nx, ix, wx);
-            restrict_axis(comp == 1, J, gc.ny, gf.ny, iy, wy);
-            restrict_axis(comp == 2, K, gc.nz, gf.nz, iz, wz);
-            const T* rc = r + comp * gf.np;
+            restrict_axis(comp == 0, I, gc.nx, gf.nx, wx);
+            restrict_axis(comp == 1, J, gc.ny, gf.ny, wy);
+            restrict_axis(comp == 2, K, gc.nz, gf.nz, wz);
+            const T* rc = r + comp * gf.np + base;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
                 if (comp == 2 && a == 3) continue;
@@ -73,11 +69,11 @@ __global__ void k_face_restrict(Grid3 gf, Grid3 gc, const TC* __restrict__ Ac, c
                 for (int b = 0; b < 4; ++b) {
                     if (comp == 1 && b == 3) continue;
                     const float wab = wz[a] * wy[b];
-                    const T* row = rc + gf.idx(0, iy[b], iz[a]);
+                    const T* row = rc + a * gf.sxy + b * gf.sx;
 #pragma unroll
                     for (int d = 0; d < 4; ++d) {
                         if (comp == 0 && d == 3) continue;
-                        acc += C(wab * wx[d]) * (C)to_c(row[ix[d]]);
+                        acc += C(wab * wx[d]) * (C)to_c(row[d]);
                     }
                 }
             }
@@ -89,36 +85,40 @@ __global__ void k_face_restrict(Grid3 gf, Grid3 gc, const TC* __restrict__ Ac, c
 }
 
 template <typename T, typename TC, bool SYM>
-__global__ void k_face_prolong(Grid3 gf, Grid3 gc, const TC* __restrict__ Af, const T* ec,
+__global__ void k_face_prolong(Grid3 gf, Grid3 gc, const TC* __restrict__ Af, const T* ec_in,
                                T* x, const int* __restrict__ tiles) {
     using C = typename Compute<T>::type;
     int i, j, k;
     block_node(gf, tiles, i, j, k);
     chain_wait();
+    const T* __restrict__ ec = after_wait(ec_in);
     if (i > gf.nx || j > gf.ny || k > gf.nz) return;
     const int p = gf.idx(i, j, k);
-    const int nc[3] = {gc.nx, gc.ny, gc.nz};
-    const int f[3] = {i, j, k};
+    // the coarse cell of the node, and per axis the offset and weights of the
+    // other face: across the plane (n) and within it (t); an axis without one has
+    // offset 0 and weight 0
+    const int nc[3] = {gc.nx, gc.ny, gc.nz}, f[3] = {i, j, k}, st[3] = {1, gc.sx, gc.sxy};
+    const int q = gc.idx(i >> 1, j >> 1, k >> 1);
+    int on[3], ot[3];
+    float wn[3][2], wt[3][2];
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        const int c = f[ax] >> 1;
+        const bool odd = f[ax] & 1;
+        const int nb = odd ? c + 1 : c - 1;
+        const bool inside = nb >= 0 && nb < nc[ax];
+        on[ax] = odd ? st[ax] : 0;
+        wn[ax][0] = odd ? 0.5f : 1.f;
+        wn[ax][1] = odd ? 0.5f : 0.f;
+        ot[ax] = inside ? (odd ? st[ax] : -st[ax]) : 0;
+        wt[ax][0] = inside ? 0.75f : 1.f;
+        wt[ax][1] = inside ? 0.25f : 0.f;
+    }
 #pragma unroll
     for (int comp = 0; comp < 3; ++comp) {
         const int op = comp * gf.np + p;
         if (!((C)Af[op] > C(0))) continue;
-        int ci[3][2];
-        float wi[3][2];
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            const int fi = f[ax];
-            if (ax == comp) {
-                if ((fi & 1) == 0) { ci[ax][0] = fi >> 1; wi[ax][0] = 1.f; ci[ax][1] = fi >> 1; wi[ax][1] = 0.f; }
-                else { ci[ax][0] = fi >> 1; wi[ax][0] = 0.5f; ci[ax][1] = (fi >> 1) + 1; wi[ax][1] = 0.5f; }
-            } else {
-                const int c = fi >> 1;
-                const int nb = (fi & 1) ? c + 1 : c - 1;
-                const bool inside = nb >= 0 && nb < nc[ax];
-                ci[ax][0] = c; wi[ax][0] = inside ? 0.75f : 1.0f;
-                ci[ax][1] = inside ? nb : c; wi[ax][1] = inside ? 0.25f : 0.f;
-            }
-        }
+        const T* e = ec + comp * gc.np + q;
         C acc = C(0);
 #pragma unroll
         for (int a = 0; a < 2; ++a)
@@ -126,8 +126,11 @@ __global__ void k_face_prolong(Grid3 gf, Grid3 gc, const TC* __restrict__ Af, co
             for (int b = 0; b < 2; ++b)
 #pragma unroll
                 for (int d = 0; d < 2; ++d) {
-                    const float w = wi[2][a] * wi[1][b] * wi[0][d];
-                    if (w != 0.f) acc += C(w) * (C)to_c(ec[comp * gc.np + gc.idx(ci[0][d], ci[1][b], ci[2][a])]);
+                    const float w = (comp == 2 ? wn[2][a] : wt[2][a]) * (comp == 1 ? wn[1][b] : wt[1][b]) *
+                                    (comp == 0 ? wn[0][d] : wt[0][d]);
+                    const int o = (d ? (comp == 0 ? on[0] : ot[0]) : 0) + (b ? (comp == 1 ? on[1] : ot[1]) : 0) +
+                                  (a ? (comp == 2 ? on[2] : ot[2]) : 0);
+                    acc += C(w) * (C)to_c(e[o]);
                 }
         if (SYM) acc /= sqrt((C)Af[op]);
         x[op] = to_store<T>((C)to_c(x[op]) + acc);
