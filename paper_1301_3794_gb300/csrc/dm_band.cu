@@ -389,19 +389,33 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_band_node(int sub0, NodeArgs<
     }
 }
 
+// One row (face component c) of node_dot: sum over the 14 couplings w of the row
+// (component block strides as there)
+template <typename C, int c, typename Ptr>
+__device__ __forceinline__ C row_dot_at(const C* w, Ptr q, int Y, int Z, int C3, C acc) {
+    constexpr int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+    const int st[3] = {1, Y, Z};
+    const int m1 = (c1 - c) * C3, m2 = (c2 - c) * C3, sc = st[c], s1 = st[c1], s2 = st[c2];
+    const int o[14] = {-1, 1, -Y, Y, -Z, Z, m1 - sc, m1 - sc + s1, m1, m1 + s1, m2 - sc, m2 - sc + s2, m2, m2 + s2};
+#pragma unroll
+    for (int e = 0; e < 14; ++e) acc += w[e] * (C)to_c(q[o[e]]);
+    return acc;
+}
+
 // FP64: a cluster of CS blocks per subdomain.  The FP64 pipe issues two FMAs
 // per clock and SM, so a subdomain's 45 FMAs per node and sweep are what its
-// time goes on; the cluster spreads them over CS SMs and leaves each thread
-// room for the couplings of its node in FP64 registers.  Every block keeps the
-// whole correction box; a node's new values go to the blocks whose nodes read
-// them (positions within one plane, row and column) through distributed shared
-// memory, and a cluster barrier closes each sweep.  Blocks of 128 threads: one
-// warp per scheduler keeps its FP64 unit busy, and three blocks fit an SM.
+// time goes on; the cluster spreads them over CS SMs.  One thread per row, not
+// per node: a warp's FMA occupies its scheduler's FP64 unit for 64 clocks, so on
+// small grids, where an SM holds few nodes, the length of a thread's chain is the
+// sweep's time (45 FMAs 1.5 us, 15 FMAs 0.5); the rows of one component share a
+// warp, and the three warps of the same nodes sit on three schedulers.  Every
+// block keeps the whole correction box; a row's new value goes to the blocks
+// whose rows read it (positions within one plane, row and column) through
+// distributed shared memory, and a cluster barrier closes each sweep.
 // Measured, one pass (one block per subdomain before): 16^3 sphere (27
-// subdomains) 190 -> 63 us; 72 x 56 x 88 ellipsoid fine level 326 -> 310 us
-// with the classes one after another, the solve with them side by side
-// 23.6 -> 15.5 ms.
-constexpr int kClusterThreads = 128;
+// subdomains) 190 -> 42 us (63 with one thread per node); 72 x 56 x 88 ellipsoid
+// fine level 326 -> 277 us with the classes one after another.
+constexpr int kClusterNodes = 128, kClusterThreads = 3 * kClusterNodes;
 template <typename T, typename TC, int CS>
 __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) k_band_node_cluster(int sub0, NodeArgs<T, TC> a) {
     using C = typename Compute<T>::type;
@@ -414,13 +428,15 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) k_
     const int sd = sub0 + blockIdx.x / CS;
     const int b0 = a.off[sd], n = a.off[sd + 1] - b0;
     const int per = (n + CS - 1) / CS;               // nodes of each block, in box order
-    const int local = rank * per + threadIdx.x;
-    const bool live = (int)threadIdx.x < per && local < n;
+    const int warp = threadIdx.x >> 5, comp = warp % 3;
+    const int inblock = (warp / 3) * 32 + (threadIdx.x & 31), local = rank * per + inblock;
     const int ct = b0 + local;
-    const int p = live ? a.node[ct] : 0;
-    const int info = live ? a.info[ct] : 0;
+    const bool node = inblock < per && local < n;
+    const int info = node ? a.info[ct] : 0;
+    const bool live = (info >> (12 + comp)) & 1;     // the node has this row
+    const int p = live ? a.node[ct] + comp * a.g.np : 0;
     const int pos = info & 4095;
-    // the blocks that hold a neighbour of this node
+    // the blocks that hold a neighbour of this row
     int r0 = CS, r1 = -1;
     if (live) {
 #pragma unroll
@@ -432,86 +448,44 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kClusterThreads) k_
             }
         }
     }
-    C v[42], cx = C(0), cy = C(0), cz = C(0);
+    C w[14], rd = C(0);
 #pragma unroll
-    for (int e = 0; e < 42; ++e) v[e] = live ? (C)a.vals[(size_t)e * a.ncopies + ct] : C(0);
+    for (int e = 0; e < 14; ++e) w[e] = live ? (C)a.vals[(size_t)(14 * comp + e) * a.ncopies + ct] : C(0);
+    if (live) rd = (C)a.vals[(size_t)(42 + comp) * a.ncopies + ct];
     for (int k = threadIdx.x; k < 2 * kNBuf; k += NT) buf[k] = C(0);
     chain_wait();
+    C c0 = C(0);
     if (live) {
         // start residual from global memory: the neighbours' loads are independent of one another
-        const int X = 1, Y = a.g.sx, Z = a.g.sxy, N = a.g.np;
         const T* q = a.x + p;
-        auto at = [&](int o) { return (C)to_c(q[o]); };
-        const C xs = at(0), ys = at(N), zs = at(2 * N);
-        cx = xs; cy = ys; cz = zs;
-        C t;
-        t = at(-X); cx += v[0] * t;
-        t = at(X); cx += v[1] * t; cy += v[14 + 13] * t; cz += v[28 + 9] * t;
-        t = at(-Y); cx += v[2] * t; cy += v[14 + 10] * t;
-        t = at(Y); cx += v[3] * t;
-        t = at(-Z); cx += v[4] * t; cz += v[28 + 6] * t;
-        t = at(Z); cx += v[5] * t;
-        t = at(X - Y); cy += v[14 + 11] * t;
-        t = at(X - Z); cz += v[28 + 7] * t;
-        cy += v[14 + 12] * xs; cz += v[28 + 8] * xs;
-        t = at(N - X); cy += v[14 + 0] * t; cx += v[6] * t;
-        t = at(N + X); cy += v[14 + 1] * t;
-        t = at(N - Y); cy += v[14 + 2] * t;
-        t = at(N + Y); cy += v[14 + 3] * t; cx += v[9] * t; cz += v[28 + 13] * t;
-        t = at(N - Z); cy += v[14 + 4] * t; cz += v[28 + 10] * t;
-        t = at(N + Z); cy += v[14 + 5] * t;
-        t = at(N + Y - X); cx += v[7] * t;
-        t = at(N + Y - Z); cz += v[28 + 11] * t;
-        cx += v[8] * ys; cz += v[28 + 12] * ys;
-        t = at(2 * N - X); cz += v[28 + 0] * t; cx += v[10] * t;
-        t = at(2 * N + X); cz += v[28 + 1] * t;
-        t = at(2 * N - Y); cz += v[28 + 2] * t; cy += v[14 + 6] * t;
-        t = at(2 * N + Y); cz += v[28 + 3] * t;
-        t = at(2 * N - Z); cz += v[28 + 4] * t;
-        t = at(2 * N + Z); cz += v[28 + 5] * t; cx += v[13] * t; cy += v[14 + 9] * t;
-        t = at(2 * N + Z - X); cx += v[11] * t;
-        t = at(2 * N + Z - Y); cy += v[14 + 7] * t;
-        cx += v[12] * zs; cy += v[14 + 8] * zs;
-        const C dx = (C)a.vals[(size_t)42 * a.ncopies + ct], dy = (C)a.vals[(size_t)43 * a.ncopies + ct],
-                dz = (C)a.vals[(size_t)44 * a.ncopies + ct];
-        cx = dx != C(0) ? a.om * (dx * (C)to_c(a.f[p]) - cx) : C(0);
-        cy = dy != C(0) ? a.om * (dy * (C)to_c(a.f[N + p]) - cy) : C(0);
-        cz = dz != C(0) ? a.om * (dz * (C)to_c(a.f[2 * N + p]) - cz) : C(0);
+        const C xs = (C)to_c(q[0]);
+        const int Y = a.g.sx, Z = a.g.sxy, N = a.g.np;
+        const C kx = comp == 0 ? row_dot_at<C, 0>(w, q, Y, Z, N, xs)
+                               : (comp == 1 ? row_dot_at<C, 1>(w, q, Y, Z, N, xs) : row_dot_at<C, 2>(w, q, Y, Z, N, xs));
+        c0 = a.om * (rd * (C)to_c(a.f[p]) - kx);
     }
 #pragma unroll
-    for (int e = 0; e < 42; ++e) v[e] *= -a.om;
+    for (int e = 0; e < 14; ++e) w[e] *= -a.om;
     cluster.sync();   // every block's buffers are zero
     const C keep = C(1) - a.om;
-    C ex = cx, ey = cy, ez = cz;
+    const int at = kN0 + comp * kNC + pos;
+    C d = c0;
     int cur = 0;      // offset of the buffer the sweep reads
-    for (int r = r0; r <= r1; ++r) {
-        C* w = cluster.map_shared_rank(buf, r) + kN0 + pos;
-        w[0] = ex;
-        w[kNC] = ey;
-        w[2 * kNC] = ez;
-    }
+    for (int r = r0; r <= r1; ++r) cluster.map_shared_rank(buf, r)[at] = d;
     for (int s = 1; s < a.sweeps; ++s) {
         cluster.sync();
         if (live) {
-            const C* q = buf + kN0 + pos + cur;
-            C ax = fma(keep, ex, cx), ay = fma(keep, ey, cy), az = fma(keep, ez, cz);
-            node_dot<C, kNX, kNXY, kNC>(v, q, ex, ey, ez, ax, ay, az);
-            ex = ax; ey = ay; ez = az;
+            const C* q = buf + at + cur;
+            const C acc = fma(keep, d, c0);
+            d = comp == 0 ? row_dot_at<C, 0>(w, q, kNX, kNXY, kNC, acc)
+                          : (comp == 1 ? row_dot_at<C, 1>(w, q, kNX, kNXY, kNC, acc)
+                                       : row_dot_at<C, 2>(w, q, kNX, kNXY, kNC, acc));
             if (s + 1 < a.sweeps)
-                for (int r = r0; r <= r1; ++r) {
-                    C* w = cluster.map_shared_rank(buf, r) + kN0 + pos + (kNBuf - cur);
-                    w[0] = ex;
-                    w[kNC] = ey;
-                    w[2 * kNC] = ez;
-                }
+                for (int r = r0; r <= r1; ++r) cluster.map_shared_rank(buf, r)[at + (kNBuf - cur)] = d;
         }
         cur = kNBuf - cur;
     }
-    if ((info >> 15) & 1) {
-        a.u[ct] = ex;
-        a.u[(size_t)a.ncopies + ct] = ey;
-        a.u[2 * (size_t)a.ncopies + ct] = ez;
-    }
+    if (live && ((info >> 15) & 1)) a.u[(size_t)comp * a.ncopies + ct] = d;
     cluster.sync();   // no block leaves while another may still write to it
 }
 
