@@ -259,15 +259,9 @@ def nvtx_mark(start):
 # (trace name, workload, grid, level-0 stencil shape) -> bytes, the shape None
 # for kernels that do not depend on it.  The profiles/ summaries hold the
 # captures and their commands; a kernel or shape without a capture reports null.
-#  - band smoother, fine level: the four size-class launches of one smoothing
-#    step of the 128^3 ellipsoid read 103.5 MB and wrote 0.2 MB (25.9 MB per
-#    launch); the 192^3 figure is that per-launch traffic scaled by the ratio of
-#    the byte model's per-launch bytes (26.27 MB / 11.64 MB), the traffic
-#    growing with the band's row copies as the byte model does.
-PROFILED_TRAFFIC = {
-    ("band_schwarz_f32_jacobi_L0", "ellipsoid", 128, None): 25_900_000,
-    ("band_schwarz_f32_jacobi_L0", "ellipsoid", 192, None): 58_450_000,
-}
+# None of the current kernels has one: the captures in profiles/ are of earlier
+# versions, and say so.
+PROFILED_TRAFFIC = {}
 
 
 def profiled_traffic(name, key):
