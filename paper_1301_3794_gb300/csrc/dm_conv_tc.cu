@@ -348,11 +348,8 @@ template <int CB, int EPI>
 void conv_tc_launch(const Grid3& g, const ActLayout& L, const __nv_bfloat16* in, const __nv_bfloat16* wt,
                     const __nv_bfloat16* mask, __nv_bfloat16* out, float* outY, int* err, cudaStream_t s) {
     const size_t sm = conv_smem<CB>();
-    static bool attr = false;   // set once per process (all devices share the kernel's attribute)
-    if (!attr) {
-        DM_CUDA(cudaFuncSetAttribute(k_conv_tc<CB, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        attr = true;
-    }
+    // above the 48 KB a kernel may use unasked; set on every call because the setting belongs to the current device
+    DM_CUDA(cudaFuncSetAttribute(k_conv_tc<CB, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     const int first = g.off0 / kTileM;
     const int last = g.idx(g.nx, g.ny, g.nz) / kTileM;
     const int ntiles = last - first + 1;
@@ -515,23 +512,16 @@ void conv_dw_tc(const Grid3& g, const ActLayout& L, int cb_in, int cin, const __
     DM_REQUIRE((cb_in == 1 || cb_in == 2) && cin <= 8 * cb_in && cout <= 8 * cb_out && cb_out >= 1 && cb_out <= 2,
                DM_ERR_INVALID_ARG, "conv_dw_tc: channel counts");
     const size_t sm = 18 * (size_t)kDwSlot + 8192;   // 16 A slots, 2 B slots, slack
-    static bool attr1 = false, attr2 = false;
     const int first = g.off0 / kTileM, last = g.idx(g.nx, g.ny, g.nz) / kTileM, ntiles = last - first + 1;
     const int nparts = std::min(conv_dw_tc_parts(), ntiles);
     // bytes: every node of the input blocks 27 times from L2 is not DRAM traffic; count the input and dy once
     const double bytes = (double)L.np * 16.0 * (cb_in + cb_out);
     if (cb_in == 2) {
-        if (!attr2) {
-            DM_CUDA(cudaFuncSetAttribute(k_conv_dw_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-            attr2 = true;
-        }
+        DM_CUDA(cudaFuncSetAttribute(k_conv_dw_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         launch_b("conv_tc_dw", bytes, k_conv_dw_tc<2>, nparts, 128, sm, s, g, L, in, cb_out, dy, first, ntiles, part,
                  err);
     } else {
-        if (!attr1) {
-            DM_CUDA(cudaFuncSetAttribute(k_conv_dw_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-            attr1 = true;
-        }
+        DM_CUDA(cudaFuncSetAttribute(k_conv_dw_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         launch_b("conv_tc_dw", bytes, k_conv_dw_tc<1>, nparts, 128, sm, s, g, L, in, cb_out, dy, first, ntiles, part,
                  err);
     }
