@@ -618,11 +618,12 @@ void face_prolong_add(const Grid3& gf, const Grid3& gc, const TC* Af, const T* e
 template <typename T, typename TC>
 void scale_sqrt_a(const Domain& d, const TC* A, bool inverse, T* x, cudaStream_t s);
 // dense (dm_dense.cu)
-// in-place inverse of the n x n row-major FP64 matrix M, n <= 6144 (work:
+constexpr int kDenseMax = 12000;   // rows of the largest coarsest level
+// in-place inverse of the n x n row-major FP64 matrix M, n <= kDenseMax (work:
 // dense_inverse_work(n) doubles).  Returns false if a column had no pivot above 1e-300.
 size_t dense_inverse_work(int n);
 bool dense_inverse(double* M, int n, double* work, int* d_flag, cudaStream_t s);
-// x[list[r]] = sum_c Minv(r, c) f[list[c]] over the rows that zero_rows does not mark (n <= 6000)
+// x[list[r]] = sum_c Minv(r, c) f[list[c]], the f of the rows that zero_rows marks taken as zero (n <= kDenseMax)
 template <typename T>
 void dense_coarse_solve(const double* Minv64, const float* Minv32, int n, const int* list, const unsigned char* zero_rows,
                         const T* f, T* x, cudaStream_t s);

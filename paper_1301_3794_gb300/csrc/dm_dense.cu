@@ -416,12 +416,16 @@ bool dense_inverse(double* M, int n, double* work, int* d_flag, cudaStream_t s) 
     int* piv = reinterpret_cast<int*>(B + kPanel * (size_t)n);
     int* src = piv + n;
     int* swaps = src + n;   // 4 kPanel entries
+    constexpr int rows = kPanelBlocks * kPanelThreads;   // of one row per thread
+    // 6,000 faces at most on the coarsest vector level, and so 12,000 cells (an active
+    // cell has an open face, a face two cells): up to six rows a thread
+    DM_REQUIRE(n <= kDenseMax && kDenseMax <= 6 * rows, DM_ERR_INVALID_ARG, "dense inverse: more rows than a panel holds");
     DM_CUDA(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
     DM_CUDA(cudaMemcpyAsync(W, M, sizeof(double) * (size_t)n * n, cudaMemcpyDeviceToDevice, s));
-    constexpr int rows = kPanelBlocks * kPanelThreads;   // of one row per thread
     if (n <= rows) gj_eliminate<1>(W, n, piv, Mt, B, swaps, d_flag, s);
     else if (n <= 2 * rows) gj_eliminate<2>(W, n, piv, Mt, B, swaps, d_flag, s);
-    else gj_eliminate<3>(W, n, piv, Mt, B, swaps, d_flag, s);
+    else if (n <= 3 * rows) gj_eliminate<3>(W, n, piv, Mt, B, swaps, d_flag, s);
+    else gj_eliminate<6>(W, n, piv, Mt, B, swaps, d_flag, s);
     int h = 0;
     DM_CUDA(cudaMemcpyAsync(&h, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
     DM_CUDA(cudaStreamSynchronize(s));
@@ -436,10 +440,13 @@ void dense_coarse_solve(const double* Minv64, const float* Minv32, int n, const 
                         const T* f, T* x, cudaStream_t s) {
     using C = typename Compute<T>::type;
     if (n <= 0) return;
-    // n <= 6000 FP64 values fit the 48 KB a kernel may use unasked
+    DM_REQUIRE(n <= kDenseMax, DM_ERR_INVALID_ARG, "coarsest solve: too many rows");
+    const size_t smem = sizeof(C) * (size_t)n;
+    // above the 48 KB a kernel may use unasked; the setting belongs to the current device
+    if (smem > 48 * 1024)
+        DM_CUDA(cudaFuncSetAttribute(k_coarse_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     launch_chain("k_coarse_solve", (double)n * n * sizeof(C) + 2.0 * n * sizeof(T), k_coarse_solve<T>,
-             (n + kSolveWarps - 1) / kSolveWarps, 32 * kSolveWarps, sizeof(C) * (size_t)n, s, n, Minv64, Minv32, list,
-             zero_rows, f, x);
+             (n + kSolveWarps - 1) / kSolveWarps, 32 * kSolveWarps, smem, s, n, Minv64, Minv32, list, zero_rows, f, x);
 }
 
 void cell_components_pin(const Grid3& g, const double* A, const int* list, int n, int* label, unsigned char* pinned,
