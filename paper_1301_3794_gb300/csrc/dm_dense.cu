@@ -278,12 +278,16 @@ void gj_eliminate(double* W, int n, int* piv, double* Mt, double* B, int* swaps,
 // nothing writes).  Every block gathers f into shared memory; one warp per row,
 // whose first loads are issued before the gather is waited for.
 // FP32 inverse (storage types FP32 and BF16): the products of two FP32 numbers
-// are summed in float-float (an error-free product and a two-sum, about 48
-// bits), because converting and adding in FP64 issues at two per clock and SM
-// where this takes nine FP32 instructions at 128; the sum is rounded to the
-// storage type either way.
+// are summed in three FP32 numbers (error-free products and sums, only the third
+// rounds: about 70 bits), because converting and adding in FP64 issues at two per
+// clock and SM where this takes two dozen FP32 instructions at 128.  An FP64 sum
+// keeps 53 bits; two FP32 numbers, about 48, leave 30 to 100 times its error where
+// a sum cancels.  Where FP32's range could show (a product or sum past its end, or
+// a result so small that its products' errors fall below it) the row is summed
+// again in FP64.
 // Measured (CUDA events, of which some 4 us a launch are the events): n = 1,990
-// in FP32, 24.9 + 6.7 + 6.4 -> 14.9 us a solve.
+// in FP32, 24.9 + 6.7 + 6.4 -> 14.9 us a solve with two FP32 numbers; the third
+// takes 2.0 us more (n = 1,817: 14.5 -> 16.5, n = 650: 8.4 -> 10.2).
 constexpr int kSolveWarps = 8;
 template <typename T>
 __global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const double* __restrict__ M64,
@@ -309,7 +313,14 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const 
         sf[c] = (zero_rows && zero_rows[c]) ? C(0) : (C)to_c(f[list[c]]);
     __syncthreads();
     if (row >= n) return;
-    C s = C(0), err = C(0);
+    C s = C(0), e1 = C(0), e2 = C(0);
+    // a + b exactly as the rounded sum (into a) and its error
+    [[maybe_unused]] auto two_sum = [](C& a, C b) {
+        const C t = a + b, bp = t - a;
+        const C err = (a - (t - bp)) + (b - bp);
+        a = t;
+        return err;
+    };
     for (int c0 = lane; c0 < n; c0 += 32 * U) {
         C cur[U];
 #pragma unroll
@@ -328,17 +339,27 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const 
                 } else {
                     const float pr = __fmul_rn(cur[e], sf[c]);
                     const float pe = fmaf(cur[e], sf[c], -pr);
-                    const float t = __fadd_rn(s, pr);
-                    const float bp = __fsub_rn(t, s);
-                    err = __fadd_rn(err, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(pr, bp)), pe));
-                    s = t;
+                    const float err = two_sum(s, pr);
+                    const float r1 = two_sum(e1, err), r2 = two_sum(e1, pe);
+                    e2 += r1 + r2;
                 }
             }
         }
     }
-    double tot = (double)s + (double)err;
+    double tot = (double)s + ((double)e1 + (double)e2);
+    auto over_lanes = [&] {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, o);
+        for (int o = 16; o > 0; o >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, o);
+    };
+    over_lanes();
+    if constexpr (!std::is_same<C, double>::value) {
+        const double mag = fabs(__shfl_sync(0xffffffffu, tot, 0));
+        if (!(mag >= 0x1p-60 && mag <= 0x1p126)) {
+            tot = 0.0;
+            for (int c = lane; c < n; c += 32) tot = fma((double)m[c], (double)sf[c], tot);
+            over_lanes();
+        }
+    }
     if (lane == 0) x[list[row]] = to_store<T>(tot);
 }
 

@@ -28,3 +28,15 @@ def run_without_device(source, tmp_path):
     r = subprocess.run([str(exe)], capture_output=True, text=True, env={**os.environ, "CUDA_VISIBLE_DEVICES": ""}, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
     return r.stdout
+
+
+def host_library(source, tmp_path):
+    """Compile the C++ source (no CUDA headers) against the library and load it."""
+    import ctypes
+    b = _builder()
+    src, so = tmp_path / "host.cpp", tmp_path / "host.so"
+    src.write_text(source)
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", str(src), b.LIB, "-Wl,-rpath," + PKG, "-o", str(so)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return ctypes.CDLL(str(so))
