@@ -842,7 +842,8 @@ template <> struct FFOps<double> { using type = FFWide; };
 // neither read nor multiplied by.  rowmap[c][row] holds the compact index of the
 // row's first open face of component c and the mask of its open faces.
 // Measured (FP32 x; 32 x 4 x 2 tiles, an FP64 copy of x and face maps of 4 bytes
-// an entry before): 192^3 ellipsoid 220 us and 33 for the copy -> 168 us; error
+// an entry before): 192^3 ellipsoid 220 us and 33 for the copy -> 161 us, 4 of them
+// the checks that keep a covered edge or cell from passing on what is not finite; error
 // against 64 bits on a 128^3 field 1.4e-14 before and after (2-norm, relative).
 constexpr int kFFY = 8, kFFZ = 8;
 template <typename T, bool CUBE>
@@ -969,18 +970,20 @@ __global__ void __launch_bounds__(TX * kFFY, 3) k_vec_apply_ff(
                   fz = s_f[s1][2][q] - s_f[s0][2][q];
         return CUBE ? fx + fy + fz : fx * rdx + fy * rdy + fz * rdz;
     };
-    auto times = [&](bool is_one, ffv c, ffv v) { return is_one ? v : c * v; };
+    // (a covered edge or cell passes nothing on, whatever x holds beside it)
+    auto scaled = [](ffv c, ffv v) { return c.hi != 0.f ? c * v : ff_zero(); };
+    auto times = [&](bool is_one, ffv c, ffv v) { return is_one ? v : scaled(c, v); };
     auto edges_xy = [&](int sm, int sp, int es) {
         s_ex[es][ty * TX + tx] = inb ? times(f_edge, cx, curl_x(i, j, sm, sp)) : ff_zero();
         s_ey[es][ty * W1 + tx] = inb ? times(f_edge, cy, curl_y(i, j, sm, sp)) : ff_zero();
-        if (role == 2) s_ex[es][dsm] = dval ? he * curl_x(di, dj, sm, sp) : ff_zero();
-        if (role == 3) s_ey[es][dsm] = dval ? he * curl_y(di, dj, sm, sp) : ff_zero();
+        if (role == 2) s_ex[es][dsm] = dval ? scaled(he, curl_x(di, dj, sm, sp)) : ff_zero();
+        if (role == 3) s_ey[es][dsm] = dval ? scaled(he, curl_y(di, dj, sm, sp)) : ff_zero();
     };
     auto psi_ez = [&](int s0, int s1) {
         s_psi[(ty + 1) * W1 + tx + 1] = inb ? times(f_cell, cv, div_at(i, j, s0, s1)) : ff_zero();
         s_ez[ty * W1 + tx] = inb ? times(f_cell, cz, curl_z(i, j, s0)) : ff_zero();
-        if (role == 0) s_psi[dsm] = dval ? hc * div_at(di, dj, s0, s1) : ff_zero();
-        if (role == 1) s_ez[dsm] = dval ? hc * curl_z(di, dj, s0) : ff_zero();
+        if (role == 0) s_psi[dsm] = dval ? scaled(hc, div_at(di, dj, s0, s1)) : ff_zero();
+        if (role == 1) s_ez[dsm] = dval ? scaled(hc, curl_z(di, dj, s0)) : ff_zero();
     };
     // (a plane below the grid's first holds ghosts only)
     fetch_ring(k0 - 1, ones(k0 - 1));
@@ -990,7 +993,7 @@ __global__ void __launch_bounds__(TX * kFFY, 3) k_vec_apply_ff(
     fetch_edges(k0, ones(k0));
     __syncthreads();
     edges_xy(0, 1, 0);
-    ffv psi_below = own ? ff_load(invV + p0 + (k0 - 1) * Z) * div_at(i, j, 0, 1) : ff_zero();
+    ffv psi_below = own ? scaled(ff_load(invV + p0 + (k0 - 1) * Z), div_at(i, j, 0, 1)) : ff_zero();
     bool o1 = ones(k0 + 1), o2 = ones(k0 + 2);
     bool ocur = ones(k0);
     fetch_ring(k0 + 1, o1);
