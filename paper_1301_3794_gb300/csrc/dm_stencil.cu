@@ -489,9 +489,10 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
                     v = bv[c] + omega * pd[c] * (pf[c] - v);
                 }
                 if constexpr (MODE == ST_CERT) {
-                    const C ab = av[c] * bv[c], r = v - k2 * ab;
-                    sum[0] += bv[c] * v;
-                    sum[1] += bv[c] * ab;
+                    // a closed face has no part in the sums, whatever x holds there
+                    const C bo = av[c] > C(0) ? bv[c] : C(0), ab = av[c] * bo, r = v - k2 * ab;
+                    sum[0] += bo * v;
+                    sum[1] += bo * ab;
                     sum[2] += ab * ab;
                     sum[3] += r * r;
                     sum[4] += r * ab;
