@@ -273,7 +273,7 @@ struct OpLevel {
     int sd_nsub = 0, sd_ncopies = 0, sd_maxrows = 0, sd_maxbox = 0;
     int sd_cls_first[kSchwarzClasses] = {}, sd_cls_count[kSchwarzClasses] = {};
     long long sd_cls_copies[kSchwarzClasses] = {}, sd_cls_owned[kSchwarzClasses] = {};
-    // the same for bricks of up to 8 nodes, which the node kernels smooth
+    // the same where the node kernels smooth the level (band_nodes_fit, band_nodes_best)
     bool by_node = false;
     DBuf<int> bn_off, bn_node, bn_info, bn_org, bn_uidx;
     DBuf<double> bn_v64;
@@ -347,7 +347,7 @@ struct dm_operator {
     int learned_streak = 0;    // consecutive shifted solves in which the correction was switched off
     long long nopen0 = 0;
     Fork fork;                 // side streams of the band smoother's class launches
-    bool forks = false;        // whether some level's classes go on them
+    bool unchained = false;    // FP64 cycles not chained (see launch_chain): some level forks or is smoothed by rows
     ~dm_operator() {
         if (vexec) cudaGraphExecDestroy(vexec);
         if (sexec) cudaGraphExecDestroy(sexec);
@@ -656,7 +656,7 @@ const T* cycle_vec(dm_operator* op, const TIn& v, double scale = 1.0) {
     T* e = reinterpret_cast<T*>(w0.e.get());
     T* r = reinterpret_cast<T*>(w0.r.get());
     mg_input<T>(D, v, scale, f, s);
-    const ChainScope chain(!(std::is_same<T, double>::value && op->forks));
+    const ChainScope chain(!(std::is_same<T, double>::value && op->unchained));
     if (graphs_allowed(op) && op->vcalls > 0) {
         if (!op->vexec && !capture_graph(op, [&] { vcycle<T, TC>(op, 0, f, e, r); }, &op->vexec, &op->vexec_kernels))
             op->graphs = false;
@@ -1236,11 +1236,13 @@ void setup_operator(dm_operator* op) {
             d.alloc(h.size(), false);
             DM_CUDA(cudaMemcpyAsync(d.get(), h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, s));
         };
-        if (g.nband > 0 && l + 1 < nl && band_nodes_fit(op->mg.band_brick)) {
-            NodeLayout nl_;
+        NodeLayout nl_;
+        if (g.nband > 0 && l + 1 < nl && band_nodes_fit(op->mg.band_brick, op->mg.precision)) {
             // (the FP64 kernel splits a subdomain by box order and is not bound by shared memory)
             band_nodes_setup(g.g, g.band.get(), g.nband, op->mg.band_brick, lowp, nl_, s);
-            o.by_node = true;
+            o.by_node = band_nodes_best(op->mg.band_brick, op->mg.precision, (int)nl_.off.size() - 1);
+        }
+        if (o.by_node) {
             o.bn_nsub = (int)nl_.off.size() - 1;
             o.bn_ncopies = (int)nl_.node.size();
             for (int k = 0; k < kNodeClasses; ++k) {
@@ -1248,7 +1250,7 @@ void setup_operator(dm_operator* op) {
                 o.bn_cls_count[k] = nl_.cls_count[k];
                 o.bn_cls_copies[k] = nl_.cls_copies[k];
             }
-            op->forks |= band_nodes_fork(o.bn_nsub, nl_.cls_count, !lowp);
+            op->unchained |= band_nodes_fork(o.bn_nsub, nl_.cls_count, !lowp);
             upload(o.bn_off, nl_.off);
             upload(o.bn_node, nl_.node);
             upload(o.bn_info, nl_.info);
@@ -1275,6 +1277,7 @@ void setup_operator(dm_operator* op) {
             band_schwarz_setup(g.g, g.band.get(), g.nband, op->mg.band_brick, sl, s);
             o.sd_nsub = (int)sl.off.size() - 1;
             o.sd_ncopies = (int)sl.copy.size();
+            op->unchained = true;
             o.sd_maxrows = sl.maxrows;
             o.sd_maxbox = sl.maxbox;
             for (int k = 0; k < kSchwarzClasses; ++k) {

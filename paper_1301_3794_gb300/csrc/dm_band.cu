@@ -10,9 +10,10 @@
 // on the owned faces.  With one brick covering the grid this is plain
 // band-restricted Jacobi.
 //
-// Bricks of up to 8 nodes (the default is 8) take k_band_node: one thread per
-// node of the subdomain, which holds the rows of the node's three faces.
-// Larger bricks take k_band_schwarz, one thread per few rows, one block per
+// Bricks of up to 8 nodes (the default is 8) take k_band_node or its FP64 form on
+// clusters: one thread per node or row of the subdomain, boxes of a fixed layout.
+// Larger and very small bricks (band_nodes_fit, band_nodes_best) take
+// k_band_schwarz, one thread per few rows, boxes clipped to the subdomain, one block per
 // subdomain.  In both the correction d lives in shared memory on the
 // subdomain's local box of nodes (all three components, zero wherever the
 // subdomain has no row), so a row's couplings are reached at fixed offsets: the
@@ -553,20 +554,18 @@ size_t schwarz_smem(int maxbox, int maxrows, int R) {
 
 }  // namespace
 
-// Size classes of subdomains (rows): each class is launched with its own
-// block size and rows per thread, so that small subdomains are not held to the
-// register and thread budget of the largest.
-// levels with at most this many subdomains are smoothed in a single launch
+// k_band_schwarz: levels with at most this many subdomains are smoothed in a single launch
 constexpr int kSingleLaunchSubdomains = 304;
 
+// Size classes of its subdomains (rows): each class is launched with its own
+// block size and rows per thread (class_shape), so that small subdomains are not held
+// to the register and thread budget of the largest.
 int schwarz_class(int rows) {
     return rows <= 256 ? 0 : (rows <= 512 ? 1 : (rows <= 1024 ? 2 : (rows <= 2048 ? 3 : 4)));
 }
 
-namespace {
-
-}  // namespace
-
+// (Counting sorts throughout: with comparison sorts of the copies an operator with bricks of
+// 2 nodes on 128^3 took 157 ms to make, now 68; 51 with the node kernels' layout.)
 void band_schwarz_setup(const Grid3& g, const int* band_dev, int nband, int brick, SchwarzLayout& out,
                         cudaStream_t s) {
     DM_REQUIRE(brick >= 1, DM_ERR_INVALID_ARG, "band brick must be >= 1 node");
@@ -579,35 +578,29 @@ void band_schwarz_setup(const Grid3& g, const int* band_dev, int nband, int bric
     // node (i, j, k) and component of every band face: q = c np + off0 + i + sx (j + sy k)
     const int n[3] = {g.nx, g.ny, g.nz};
     const int nb[3] = {(g.nx + brick) / brick, (g.ny + brick) / brick, (g.nz + brick) / brick};
-    std::vector<int> node((size_t)3 * nband);
-    std::vector<char> owner((size_t)nb[0] * nb[1] * nb[2], 0);
-    auto key = [&](int bx, int by, int bz) { return ((long long)bz * nb[1] + by) * nb[0] + bx; };
+    const size_t nbk = (size_t)nb[0] * nb[1] * nb[2];
+    struct Face {
+        int node[3];
+        int comp;
+    };
+    std::vector<Face> face(nband);
+    std::vector<char> owner(nbk, 0);
+    auto key = [&](int bx, int by, int bz) { return ((size_t)bz * nb[1] + by) * nb[0] + bx; };
     for (int t = 0; t < nband; ++t) {
-        const int q = band[t];
-        const int r = q % g.np - g.off0;
+        const int comp = band[t] / g.np, r = band[t] - comp * g.np - g.off0;
         const int k = r / g.sxy, rem = r - k * g.sxy;
         const int j = rem / g.sx, i = rem - j * g.sx;
-        node[3 * t] = i;
-        node[3 * t + 1] = j;
-        node[3 * t + 2] = k;
+        face[t] = Face{{i, j, k}, comp};
         owner[key(i / brick, j / brick, k / brick)] = 1;
     }
-    // copies (brick, face): brick B holds node P when B b - 1 <= P <= B b + b on every axis,
-    // i.e. ceil(P / b) - 1 <= B <= floor((P + 1) / b)
-    struct Copy {
-        long long brick;
-        int q, t;
-        bool owned;
-    };
-    // grouped by brick with a counting sort (two passes over the faces), then
-    // each brick's copies sorted by face index: the order of one sort by
-    // (brick, face) at a fraction of its cost
-    const size_t nbk = (size_t)nb[0] * nb[1] * nb[2];
+    // copies (brick, face), grouped by brick with a counting sort: brick B holds node P when
+    // B b - 1 <= P <= B b + b on every axis, i.e. ceil(P / b) - 1 <= B <= floor((P + 1) / b);
+    // t for the owner's copy, -1 - t for another's
     auto each_copy = [&](auto&& visit) {
         for (int t = 0; t < nband; ++t) {
             int lo[3], hi[3], own[3];
             for (int a = 0; a < 3; ++a) {
-                const int P = node[3 * t + a];
+                const int P = face[t].node[a];
                 own[a] = P / brick;
                 lo[a] = std::max((P + brick - 1) / brick - 1, 0);
                 hi[a] = std::min((P + 1) / brick, nb[a] - 1);
@@ -615,68 +608,49 @@ void band_schwarz_setup(const Grid3& g, const int* band_dev, int nband, int bric
             for (int bz = lo[2]; bz <= hi[2]; ++bz)
                 for (int by = lo[1]; by <= hi[1]; ++by)
                     for (int bx = lo[0]; bx <= hi[0]; ++bx) {
-                        const long long kb = key(bx, by, bz);
-                        if (owner[kb]) visit(kb, t, bx == own[0] && by == own[1] && bz == own[2]);
+                        const size_t kb = key(bx, by, bz);
+                        if (owner[kb]) visit(kb, bx == own[0] && by == own[1] && bz == own[2] ? t : -1 - t);
                     }
         }
     };
-    std::vector<long long> start(nbk + 1, 0);
-    each_copy([&](long long kb, int, bool) { ++start[kb + 1]; });
+    std::vector<int> start(nbk + 1, 0);
+    each_copy([&](size_t kb, int) { ++start[kb + 1]; });
     for (size_t b = 0; b < nbk; ++b) start[b + 1] += start[b];
-    std::vector<Copy> cp((size_t)start[nbk]);
+    const int nc = start[nbk];
+    std::vector<int> cp(nc);
     {
-        std::vector<long long> fill(start.begin(), start.end() - 1);
-        each_copy([&](long long kb, int t, bool owned) { cp[(size_t)fill[kb]++] = Copy{kb, band[t], t, owned}; });
+        std::vector<int> fill(start.begin(), start.end() - 1);
+        each_copy([&](size_t kb, int ct) { cp[fill[kb]++] = ct; });
     }
-    for (size_t b = 0; b < nbk; ++b)
-        std::sort(cp.begin() + start[b], cp.begin() + start[b + 1],
-                  [](const Copy& a, const Copy& c) { return a.q < c.q; });
-    const int nc = (int)cp.size();
-    // subdomains (runs of one brick), emitted class by class
-    std::vector<std::pair<int, int>> runs;
-    for (int c0 = 0; c0 < nc;) {
-        int c1 = c0;
-        while (c1 < nc && cp[c1].brick == cp[c0].brick) ++c1;
-        runs.push_back({c0, c1});
-        c0 = c1;
-    }
-    // slots of a run: its rows per component rounded up to whole warp groups
-    auto slots_of = [&](const std::pair<int, int>& r) {
-        int n[3] = {0, 0, 0};
-        for (int c = r.first; c < r.second; ++c) ++n[cp[c].q / g.np];
-        return 32 * ((n[0] + 31) / 32 + (n[1] + 31) / 32 + (n[2] + 31) / 32);
+    // subdomains class by class; slots of one: its rows per component rounded up to whole warp groups
+    struct Run {
+        size_t brick;
+        int rows[3], slots;
     };
-    std::vector<int> run_slots;
-    run_slots.reserve(runs.size());
-    for (const auto& r : runs) run_slots.push_back(slots_of(r));
-    std::vector<int> order(runs.size());
-    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return schwarz_class(run_slots[a]) < schwarz_class(run_slots[b]);
-    });
-    {
-        std::vector<std::pair<int, int>> sorted;
-        sorted.reserve(runs.size());
-        for (int i : order) sorted.push_back(runs[i]);
-        runs.swap(sorted);
-        std::vector<int> rs;
-        rs.reserve(order.size());
-        for (int i : order) rs.push_back(run_slots[i]);
-        run_slots.swap(rs);
+    std::vector<Run> runs;
+    for (size_t b = 0; b < nbk; ++b) {
+        if (start[b + 1] == start[b]) continue;
+        Run r{b, {0, 0, 0}, 0};
+        for (int c = start[b]; c < start[b + 1]; ++c) ++r.rows[face[cp[c] >= 0 ? cp[c] : -1 - cp[c]].comp];
+        for (int e : r.rows) r.slots += 32 * ((e + 31) / 32);
+        runs.push_back(r);
     }
+    std::stable_sort(runs.begin(), runs.end(),
+                     [&](const Run& x, const Run& y) { return schwarz_class(x.slots) < schwarz_class(y.slots); });
     for (int k = 0; k < kSchwarzClasses; ++k) {
         out.cls_first[k] = out.cls_count[k] = 0;
         out.cls_copies[k] = out.cls_owned[k] = 0;
     }
     out.copy.reserve((size_t)nc + 96 * runs.size());
     out.pos.reserve((size_t)nc + 96 * runs.size());
+    std::vector<int> at;   // box position of each copy of a run
     for (size_t rI = 0; rI < runs.size(); ++rI) {
-        const int c0 = runs[rI].first, c1 = runs[rI].second;
-        const int cl = schwarz_class(run_slots[rI]);
+        const size_t kb = runs[rI].brick;
+        const int c0 = start[kb], c1 = start[kb + 1];
+        const int cl = schwarz_class(runs[rI].slots);
         if (out.cls_count[cl] == 0) out.cls_first[cl] = (int)rI;
         ++out.cls_count[cl];
-        const long long kb = cp[c0].brick;
-        const int B[3] = {(int)(kb % nb[0]), (int)((kb / nb[0]) % nb[1]), (int)(kb / ((long long)nb[0] * nb[1]))};
+        const int B[3] = {(int)(kb % nb[0]), (int)((kb / nb[0]) % nb[1]), (int)(kb / ((size_t)nb[0] * nb[1]))};
         // local box: the subdomain's nodes and their neighbours (within the padded grid)
         int lo[3], l[3];
         for (int a = 0; a < 3; ++a) {
@@ -696,30 +670,31 @@ void band_schwarz_setup(const Grid3& g, const int* band_dev, int nband, int bric
         // a warp mostly sit in distinct banks; every slot offset is the same for
         // the rows of one component, so each of the 15 loads of a sweep is then
         // (nearly) free of bank conflicts.  Unfilled slots are empty lanes.
-        std::vector<std::pair<int, int>> rows[3];   // (position, copy code) per component
+        at.resize(c1 - c0);
+        int cnt[3][33] = {};
         for (int c = c0; c < c1; ++c) {
-            const int t = cp[c].t;
-            const int comp = cp[c].q / g.np;
-            if (cp[c].owned) ++out.cls_owned[cl];
-            const int li = node[3 * t] - lo[0], lj = node[3 * t + 1] - lo[1], lk = node[3 * t + 2] - lo[2];
-            rows[comp].push_back({((comp * l[2] + lk) * l[1] + lj) * l[0] + li, cp[c].owned ? t : -1 - t});
+            const Face& f = face[cp[c] >= 0 ? cp[c] : -1 - cp[c]];
+            if (cp[c] >= 0) ++out.cls_owned[cl];
+            const int p = ((f.comp * l[2] + f.node[2] - lo[2]) * l[1] + f.node[1] - lo[1]) * l[0] + f.node[0] - lo[0];
+            at[c - c0] = p;
+            ++cnt[f.comp][(p & 31) + 1];
         }
+        int ng[3];
+        size_t base[3], end = out.copy.size();
         for (int comp = 0; comp < 3; ++comp) {
-            std::vector<std::pair<int, int>>& rc = rows[comp];
-            const int n = (int)rc.size();
-            if (n == 0) continue;
-            std::stable_sort(rc.begin(), rc.end(), [](const std::pair<int, int>& a, const std::pair<int, int>& b) {
-                return (a.first & 31) < (b.first & 31);
-            });
-            const int ng = (n + 31) / 32;
-            const size_t base = out.copy.size();
-            out.copy.resize(base + 32 * (size_t)ng, kDummyCopy);
-            out.pos.resize(base + 32 * (size_t)ng, -1);
-            for (int i = 0; i < n; ++i) {
-                const size_t slot = base + (size_t)(i % ng) * 32 + i / ng;
-                out.pos[slot] = rc[i].first;
-                out.copy[slot] = rc[i].second;
-            }
+            for (int k = 0; k < 32; ++k) cnt[comp][k + 1] += cnt[comp][k];
+            ng[comp] = (runs[rI].rows[comp] + 31) / 32;
+            base[comp] = end;
+            end += 32 * (size_t)ng[comp];
+        }
+        out.copy.resize(end, kDummyCopy);
+        out.pos.resize(end, -1);
+        for (int c = c0; c < c1; ++c) {
+            const int comp = face[cp[c] >= 0 ? cp[c] : -1 - cp[c]].comp, p = at[c - c0];
+            const int rk = cnt[comp][p & 31]++;
+            const size_t slot = base[comp] + (size_t)(rk % ng[comp]) * 32 + rk / ng[comp];
+            out.pos[slot] = p;
+            out.copy[slot] = cp[c];
         }
         out.maxrows = std::max(out.maxrows, (int)out.copy.size() - out.off.back());
     }
@@ -734,7 +709,17 @@ void band_copy_vals(const int* copy, int ncopies, const double* band_vals, int n
 
 // ---- node kernels: layout and launches ----------------------------------------
 
-bool band_nodes_fit(int brick) { return brick >= 1 && brick <= kNodeBrick; }
+constexpr int kSMs = 152;
+
+// Small bricks stay with k_band_schwarz: the node kernels' local layout and x box
+// are those of 8-node bricks, whose clearing and copying outweighs the sweeps of a
+// subdomain of a few nodes, and a warp of nodes is three warps of rows.
+// Measured, a V-cycle by rows against one by nodes (96^3 / 128^3 ellipsoid, 48 x 48 x 576
+// nine-cell cavity): FP32 bricks of 2 nodes 1.11 / 1.68 / 2.20 ms against 1.20 / 1.89 / 2.40,
+// of 3 nodes 0.94 / 1.38 / 1.64 against 0.95 / 1.35 / 1.56; BF16 of 3 nodes 0.94 / 1.38 / 1.65
+// against 0.99 / 1.50 / 1.79, of 4 nodes 0.93 / 1.36 / 1.52 against 0.89 / 1.28 / 1.41; FP64 of
+// 3 nodes 3.7 / 6.0 / 8.8 against 4.5 / 7.5 / 11.4, of 6 nodes 2.8 / 4.6 / 5.8 against 2.6 / 4.2 / 5.4.
+bool band_nodes_fit(int brick, int prec) { return brick > (prec == DM_PREC_F32 ? 2 : 3) && brick <= kNodeBrick; }
 
 void band_nodes_setup(const Grid3& g, const int* band_dev, int nband, int brick, bool by_bank, NodeLayout& out,
                       cudaStream_t s) {
@@ -852,7 +837,6 @@ void band_node_vals(const int* node, const int* info, int ncopies, const Grid3& 
 
 namespace {
 
-constexpr int kSMs = 152;
 
 // A level with few subdomains goes in one launch shaped for its largest class:
 // FP32, when they fit the SMs at one block each; FP64, when clusters of eight
@@ -882,6 +866,13 @@ void launch_cluster(const char* name, double bytes, int first, int count, const 
 }
 
 }  // namespace
+
+// FP64 bricks of 4 and 5 nodes: by node while there is an SM for every subdomain, because a
+// sweep then takes as long as a thread's chain (16^3 sphere, about a hundred
+// subdomains of 4-node bricks: 0.22 ms a cycle against 0.29 by rows); with more of them the FP64 pipes are busy either way
+// (4 nodes, 32^3 / 96^3 / nine-cell: 1.21 / 3.42 / 7.61 ms by node, 1.09 / 3.05 / 6.68 by rows;
+// 5 nodes 1.18 / 2.97 / 6.03 and 1.15 / 2.88 / 6.37).
+bool band_nodes_best(int brick, int prec, int nsub) { return prec != DM_PREC_F64 || brick >= 6 || nsub <= kSMs; }
 
 bool band_nodes_fork(int nsub, const int cls_count[kNodeClasses], bool wide) {
     int nl = 0;

@@ -228,8 +228,10 @@ __device__ __forceinline__ void chain_wait() {
 }
 // Not chained (g_chain false): the workers of a batch, whose waiting blocks would
 // keep the other workers' kernels off the SMs (six cavities on six streams:
-// 455 ms unchained, 488 chained), and FP64 cycles that fork streams (FP64 kernels
-// are long; 72 x 56 x 88 solve 16.8 ms against 17.5).  Elsewhere: projection on
+// 455 ms unchained, 488 chained), and FP64 cycles that fork streams or smooth a
+// level by rows (FP64 kernels are long; 72 x 56 x 88 solve 16.8 ms against 17.5; a cycle
+// with bricks of 9 nodes on 48^3 / 64^3 / 80^3 2.19 / 2.17 / 2.74 ms against 2.26 / 2.26 / 2.79).
+// Elsewhere: projection on
 // 104 x 88 x 72 cells 3.69 -> 3.38 ms, 16^3 FP64 eigensolve 178 -> 170, 96^3 FP32
 // one 448 -> 429, 128^3 BF16 solve 17.9 -> 17.4.
 extern thread_local bool g_chain;
@@ -494,7 +496,7 @@ struct Fork {
 template <typename T, typename TC>
 void band_schwarz(const BandSchwarz<TC>& bs, const TC* invD, const Grid3& g, const int* band, int nband, const T* f,
                   T* x, double* u, double omega, int sweeps, bool fine, cudaStream_t s, const Fork* fk = nullptr);
-// Subdomains of the node kernels (bricks of up to 8 nodes, dm_band.cu): copies
+// Subdomains of the node kernels (bricks of 3 or 4 to 8 nodes, dm_band.cu): copies
 // of band nodes grouped by brick, one lane each (node -1: an empty lane), class
 // by class with the largest class first.  by_bank orders a subdomain's nodes
 // for conflict-free shared memory, else they keep box order.
@@ -522,7 +524,9 @@ struct BandNodes {
         return n;
     }
 };
-bool band_nodes_fit(int brick);
+// whether bricks of this size can be the node kernels', and whether a level of nsub such bricks is
+bool band_nodes_fit(int brick, int prec);
+bool band_nodes_best(int brick, int prec, int nsub);
 // whether a level's classes are launched side by side (wide: FP64)
 bool band_nodes_fork(int nsub, const int cls_count[kNodeClasses], bool wide);
 void band_nodes_setup(const Grid3& g, const int* band_dev, int nband, int brick, bool by_bank, NodeLayout& out,
