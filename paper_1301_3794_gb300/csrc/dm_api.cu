@@ -296,13 +296,14 @@ struct Fgmres {
     DBuf<double> w;
     void ensure(long long n_, long long nc_, int m_, size_t zbytes) {   // zbytes: of one vector of Z
         if (n == n_ && nc == nc_ && m >= m_ && Z.n >= zbytes * m_) return;
+        m = 0;   // until all are there
+        V.alloc((size_t)(m_ + 1) * nc_);
+        wf.alloc((size_t)nc_);
+        Z.alloc(zbytes * m_);
+        w.alloc((size_t)n_);
         n = n_;
         nc = nc_;
         m = m_;
-        V.alloc((size_t)(m + 1) * nc);
-        wf.alloc((size_t)nc);
-        Z.alloc(zbytes * m);
-        w.alloc((size_t)n);
     }
 };
 
@@ -594,12 +595,10 @@ void learned_correct(dm_operator* op, const T* f, T* z, T* scratch) {
     const VecOp<T, TC> o = vop<T, TC>(op, 0);
     const long long n = 3ll * g0.g.np;
     constexpr int nb = 152 * 2;
-    if (op->lc_c.n < sizeof(T) * (size_t)n) {
-        op->lc_c.alloc(sizeof(T) * (size_t)n);
-        op->lc_kc.alloc(sizeof(T) * (size_t)n);
-        op->lc_part.alloc(2 * nb);
-        op->lc_host.assign(2 * nb, 0.0);
-    }
+    op->lc_c.ensure(sizeof(T) * (size_t)n);
+    op->lc_kc.ensure(sizeof(T) * (size_t)n);
+    op->lc_part.ensure(2 * nb);
+    op->lc_host.resize(2 * nb);
     T* c = reinterpret_cast<T*>(op->lc_c.get());
     T* kc = reinterpret_cast<T*>(op->lc_kc.get());
     vec_stencil(o, ST_RESID, z, f, scratch, 0.0, s);
@@ -1077,12 +1076,13 @@ constexpr double kScalarLambdaMax = 2.0;
 void ensure_f32(GeoLevel& g, cudaStream_t s) {
     if (g.A32.get()) return;
     const long long n3 = 3ll * g.g.np, n1 = g.g.np;
-    g.A32.alloc(n3);
-    g.L32.alloc(n3);
-    g.invV32.alloc(n1);
-    convert_coeff<float>(n3, g.A.get(), g.A32.get(), s);
-    convert_coeff<float>(n3, g.L.get(), g.L32.get(), s);
-    convert_coeff<float>(n1, g.invV.get(), g.invV32.get(), s);
+    DBuf<float> A(n3), L(n3), V(n1);
+    convert_coeff<float>(n3, g.A.get(), A.get(), s);
+    convert_coeff<float>(n3, g.L.get(), L.get(), s);
+    convert_coeff<float>(n1, g.invV.get(), V.get(), s);
+    g.L32 = std::move(L);
+    g.invV32 = std::move(V);
+    g.A32 = std::move(A);
 }
 
 __global__ void k_invert_diag(long long n, const double* __restrict__ d, double* __restrict__ inv) {
@@ -2819,12 +2819,10 @@ dm_status dm_learned_train_step(dm_learned* net, dm_operator* op, const double* 
         const long long n3 = 3ll * g0.g.np;
         const double h = std::min(g0.g.hx, std::min(g0.g.hy, g0.g.hz));
         LearnedNet& L = net->net;
-        if (L.r64.n != (size_t)n3) {
-            L.r64.alloc(n3);
-            L.r32.alloc(n3);
-            L.ybuf.alloc(n3);
-            L.kbuf.alloc(n3);
-        }
+        L.r64.ensure(n3);
+        L.r32.ensure(n3);
+        L.ybuf.ensure(n3);
+        L.kbuf.ensure(n3);
         faces_in(op, 0, r, on_device, L.r64.get());
         const double ss = sumsq<double>(n3, L.r64.get(), s);
         DM_REQUIRE(ss > 0.0 && op->nopen0 > 0, DM_ERR_INVALID_ARG, "learned train step: zero residual");

@@ -291,14 +291,21 @@ struct DBuf {
         return *this;
     }
     ~DBuf() { release(); }
+    // (empty when it throws: a later call must not take a failed allocation for a buffer)
     void alloc(size_t count, bool zero = true) {
         release();
-        n = count;
         if (count) {
             note_allocation();
-            DM_CUDA(cudaMalloc(&p, count * sizeof(T)));
-            if (zero) DM_CUDA(cudaMemsetAsync(p, 0, count * sizeof(T), g_stream));
+            DBuf b;
+            DM_CUDA(cudaMalloc(&b.p, count * sizeof(T)));
+            if (zero) DM_CUDA(cudaMemsetAsync(b.p, 0, count * sizeof(T), g_stream));
+            std::swap(p, b.p);
+            n = count;
         }
+    }
+    // a buffer kept between calls: allocated again only when the size is another
+    void ensure(size_t count) {
+        if (n != count) alloc(count);
     }
     void release() {
         if (p) cudaFree(p);

@@ -200,9 +200,9 @@ inline dim3 node_blocks(const Grid3& g) {
 
 void LearnedNet::alloc(const Grid3& grid) {
     if (g.np == grid.np && g.nx == grid.nx && g.ny == grid.ny && g.nz == grid.nz && X.get()) return;
-    g = grid;
-    L = act_layout(g);
-    const size_t np = (size_t)g.np;
+    g = Grid3{};   // no grid until every buffer is there
+    L = act_layout(grid);
+    const size_t np = (size_t)grid.np;
     X.alloc(L.elems(1));
     H1.alloc(L.elems(2));
     H2.alloc(L.elems(2));
@@ -217,9 +217,10 @@ void LearnedNet::alloc(const Grid3& grid) {
     wt3a.alloc((size_t)conv_wtile_steps(1) * 512);
     wt2a.alloc((size_t)conv_wtile_steps(2) * 512);
     err.alloc(1);
-    const dim3 nb = node_blocks(g);
+    const dim3 nb = node_blocks(grid);
     loss_part.alloc((size_t)nb.x * nb.y * nb.z);
     dw_part.alloc((size_t)conv_dw_tc_parts() * 27 * 256);
+    g = grid;
 }
 
 void LearnedNet::init_params() {
