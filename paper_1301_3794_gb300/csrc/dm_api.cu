@@ -2831,7 +2831,8 @@ dm_status dm_learned_train_step(dm_learned* net, dm_operator* op, const double* 
             std::lock_guard<std::mutex> lock(const_cast<dm_geometry*>(op->geom)->mu);
             ensure_f32(g0, s);
         }
-        convert<float, double>(g0.vdom(), L.r64.get(), L.r32.get(), s);
+        // over all entries, not the active tiles alone: the kept vector may hold another geometry's off them
+        convert<float, double>(Domain{g0.g, nullptr, 0, 3}, L.r64.get(), L.r32.get(), s);
         const VecOp<float, float> o32{g0.g, g0.A32.get(), g0.L32.get(), g0.invV32.get(), nullptr, op->sigma, 0,
                                       g0.tiles.get(), g0.ntiles, nullptr, 0, 0};
         L.alloc(g0.g);
