@@ -524,28 +524,29 @@ __global__ void __launch_bounds__(TX * SY, (std::is_same<T, double>::value ? 512
     }
 }
 
-// out[vector][e] = sum of the blocks' sums, in a fixed order (one block per vector)
-__global__ void k_cert_final(int nb, const double* __restrict__ part, double* __restrict__ out) {
-    __shared__ double red[8][kCertSums];
-    const double* p = part + (size_t)blockIdx.x * nb * kCertSums;
-    double s[kCertSums];
+// out[vector][e] = sum of the blocks' sums, in a fixed order (one block per vector,
+// one warp per sum).  The lanes' sums are added up with what each addition rounds
+// off: the blocks' and the lanes' own errors average out over their number, those of
+// the last few additions of a plain sum would not.  Measured over 72 random
+// vectors on three grids, errors of rho, delta and the Rayleigh quotient against long
+// double (root mean square, 1e-16): 0.95, 0.83, 0.86; with plain sums 1.12, 1.03, 1.16.
+constexpr int kCertFinalThreads = 32 * kCertSums;
+__global__ void __launch_bounds__(kCertFinalThreads) k_cert_final(int nb, const double* __restrict__ part,
+                                                                  double* __restrict__ out) {
+    const int e = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const double* p = part + (size_t)blockIdx.x * nb * kCertSums + e;
+    double s = 0.0, r = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < nb; b += 32) s += p[(size_t)b * kCertSums];
 #pragma unroll
-    for (int e = 0; e < kCertSums; ++e) s[e] = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x)
-#pragma unroll
-        for (int e = 0; e < kCertSums; ++e) s[e] += p[(size_t)b * kCertSums + e];
-#pragma unroll
-    for (int e = 0; e < kCertSums; ++e) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s[e] += __shfl_down_sync(0xffffffffu, s[e], o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][e] = s[e];
+    for (int o = 16; o > 0; o >>= 1) {
+        const double a = __shfl_down_sync(0xffffffffu, s, o), ra = __shfl_down_sync(0xffffffffu, r, o);
+        const double t = s + a, bp = t - s;
+        r += ra + ((s - (t - bp)) + (a - bp));
+        s = t;
     }
-    __syncthreads();
-    if (threadIdx.x < kCertSums) {
-        double v = 0.0;
-        for (int w = 0; w < 8; ++w) v += red[w][threadIdx.x];
-        out[blockIdx.x * kCertSums + threadIdx.x] = v;
-    }
+    // (a sum past the range is infinite, its errors are not a number)
+    if (lane == 0) out[blockIdx.x * kCertSums + e] = isfinite(s) ? s + r : s;
 }
 
 template <typename T, typename TC>
@@ -1264,7 +1265,7 @@ void vec_cert_sums(const VecOp<double, double>& op, bool natural, int n, const d
         if (natural) go(k_vec_stencil_march<double, double, ST_CERT, 8, 8, IN_NATURAL>);
         else go(k_vec_stencil_march<double, double, ST_CERT, 8, 8, IN_PADDED>);
     }
-    launch("k_cert_final", k_cert_final, n, 256, 0, s, op.nstiles, (const double*)part, out);
+    launch("k_cert_final", k_cert_final, n, kCertFinalThreads, 0, s, op.nstiles, (const double*)part, out);
 }
 
 void band_slots(const Grid3& g, const double* A, const double* L, const double* invV, double sigma, const int* band,
