@@ -1201,6 +1201,7 @@ void vec_stencil(const VecOp<T, TC>& op, int mode, const T* x, const T* f, T* y,
     const double bytes = vec_stencil_bytes<T, TC>(g, mode);
     const int* tl = op.stiles ? op.stiles : op.tiles;
     const int nt = op.stiles ? op.nstiles : op.ntiles;
+    DM_REQUIRE(tl, DM_ERR_INVALID_ARG, "vector stencil: no tile list");
     if (nt <= 0) return;
     const char* nm = stencil_name("vec_stencil", prec_index<T>(), mode, op.level == 0);
     // tile shape: 0 = 32x4x2 (the level's active tiles), 1 = 32x2x4, 2 = 32x8x1; 3 = 32x8x8,
@@ -1235,6 +1236,7 @@ void vec_apply_natural(const VecOp<double, double>& op, const double* x, double*
     const bool march = op.stiles && op.shape >= 3;   // the level's tuned z-marching shape, else its 32x4x2 tiles
     const int* tl = march ? op.stiles : op.tiles;
     const int nt = march ? op.nstiles : op.ntiles;
+    DM_REQUIRE(tl, DM_ERR_INVALID_ARG, "vector stencil: no tile list");
     if (nt <= 0) return;
     const char* nm = traced ? stencil_name("vec_stencil", 0, ST_APPLY, op.level == 0) : "";   // (the name may allocate)
     const double bytes = traced ? vec_stencil_bytes<double, double>(g, ST_APPLY) : 0.0;
