@@ -286,9 +286,12 @@ void gj_eliminate(double* W, int n, int* piv, double* Mt, double* B, int* swaps,
 // a result so small that its products' errors fall below it) the row is summed
 // again in FP64.
 // Measured (CUDA events, of which some 4 us a launch are the events): n = 1,990
-// in FP32, 24.9 + 6.7 + 6.4 -> 14.9 us a solve with two FP32 numbers; the third
-// takes 2.0 us more (n = 1,817: 14.5 -> 16.5, n = 650: 8.4 -> 10.2).
-constexpr int kSolveWarps = 8;
+// in FP32, 24.9 + 6.7 + 6.4 -> 14.9 us a solve with two FP32 numbers.  The third took 2 us
+// more, which four gathers in flight at a time (one before) give back: n = 650 / 1,817 /
+// 2,278 with two numbers 8.5 / 14.5 / 14.5 us, with three 10.2 / 16.5 / 16.5, and now 8.8 /
+// 14.4 / 16.5; in FP64 10.6 / 19.0 / 18.8 -> 9.8 / 18.5 / 19.3.  (Eight in flight, 16 warps a
+// block or packed pairs of FP32 numbers are no faster.)
+constexpr int kSolveWarps = 8, kSolveGather = 4;
 template <typename T>
 __global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const double* __restrict__ M64,
                                                                    const float* __restrict__ M32,
@@ -308,9 +311,29 @@ __global__ void __launch_bounds__(32 * kSolveWarps) k_coarse_solve(int n, const 
     C v[U];
 #pragma unroll
     for (int e = 0; e < U; ++e) v[e] = lane + 32 * e < n ? m[lane + 32 * e] : C(0);
+    // f's places, kSolveGather at a time, so that their loads and f's are in flight together (the
+    // places need nothing from the kernels before)
+    constexpr int NT = 32 * kSolveWarps;
+    int at[kSolveGather];
+    auto places = [&](int c0) {
+#pragma unroll
+        for (int e = 0; e < kSolveGather; ++e) {
+            const int c = c0 + NT * e;
+            at[e] = c < n ? list[c] : -1;
+            if (zero_rows && c < n && zero_rows[c]) at[e] = -1;
+        }
+    };
+    places(threadIdx.x);
     chain_wait();
-    for (int c = threadIdx.x; c < n; c += 32 * kSolveWarps)
-        sf[c] = (zero_rows && zero_rows[c]) ? C(0) : (C)to_c(f[list[c]]);
+    for (int c0 = threadIdx.x; c0 < n; c0 += NT * kSolveGather) {
+        C fv[kSolveGather];
+#pragma unroll
+        for (int e = 0; e < kSolveGather; ++e) fv[e] = at[e] >= 0 ? (C)to_c(f[at[e]]) : C(0);
+        places(c0 + NT * kSolveGather);
+#pragma unroll
+        for (int e = 0; e < kSolveGather; ++e)
+            if (c0 + NT * e < n) sf[c0 + NT * e] = fv[e];
+    }
     __syncthreads();
     if (row >= n) return;
     C s = C(0), e1 = C(0), e2 = C(0);
