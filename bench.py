@@ -259,9 +259,19 @@ def nvtx_mark(start):
 # (trace name, workload, grid, level-0 stencil shape) -> bytes, the shape None
 # for kernels that do not depend on it.  The profiles/ summaries hold the
 # captures and their commands; a kernel or shape without a capture reports null.
-# None of the current kernels has one: the captures in profiles/ are of earlier
-# versions, and say so.
-PROFILED_TRAFFIC = {}
+# Captured on the 128^3 ellipsoid; the 192^3 figures are those scaled by the ratio of
+# the byte model's bytes per launch, which traffic grows with.
+#  - band smoother, fine level: the two launches of a smoothing step moved 51.9 and
+#    29.2 MB (byte model 23.50 MB a launch, 53.08 at 192^3)
+#  - float-float apply: 89.9 MB (58.59, 195.79)
+# The other captures in profiles/ are of earlier kernels, or of a shape that 128^3 and
+# 192^3 do not share.
+PROFILED_TRAFFIC = {
+    ("band_schwarz_f32_jacobi_L0", "ellipsoid", 128, None): 40_570_000,
+    ("band_schwarz_f32_jacobi_L0", "ellipsoid", 192, None): 91_650_000,
+    ("vec_apply_ff_L0", "ellipsoid", 128, None): 89_930_000,
+    ("vec_apply_ff_L0", "ellipsoid", 192, None): 300_530_000,
+}
 
 
 def profiled_traffic(name, key):

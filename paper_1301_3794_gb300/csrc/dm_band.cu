@@ -804,8 +804,10 @@ void band_nodes_setup(const Grid3& g, const int* band_dev, int nband, int brick,
         if (by_bank) {
             // Lanes of a warp in distinct shared-memory banks: the nodes sorted by
             // bank and dealt round-robin over the warps (every coupling sits at one
-            // offset for all nodes, so then all 24 loads of a sweep are nearly free
-            // of conflicts; in box order they take two to three passes each).
+            // offset for all nodes).  A bank with more nodes than the subdomain has
+            // warps still conflicts: 38% of the sweeps' load wavefronts on a 128^3
+            // ellipsoid's fine level, 39 to 47% on the next, where box order takes two
+            // to three passes for each load.
             const int ng = (n + 31) / 32;
             int cnt[33] = {};
             for (int i = 0; i < n; ++i) ++cnt[((cinfo[c0 + i] & 4095) & 31) + 1];

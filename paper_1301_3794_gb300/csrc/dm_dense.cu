@@ -15,12 +15,15 @@ namespace {
 // The steps of a panel of NB columns act on the rest of the matrix as one
 // update: with E the product of the panel's elimination steps and J its rows,
 // E v = (v with its J entries zeroed) + M v_J, and the in-place panel holds M.
-// So one block eliminates within the panel (its rows in registers), the row
-// swaps are carried to the other columns, and one rank-NB update over the whole
-// chip follows.  The n^3 FP64 FMAs of the updates bound it (two per clock and
-// SM); a step per column instead, as an n x 2n elimination of [A | I], did twice
-// those FMAs and two launches for each of the n columns, every launch waiting
-// on one block's pivot search.
+// So a cluster of blocks eliminates within the panel (its rows in registers), the
+// row swaps are carried to the other columns, and one rank-NB update over the whole
+// chip follows.  The panels bound it, 5 to 6 us a column in two cluster barriers, the
+// pivot search and a divide (89 us a panel against 20 an update on the smoke test's
+// 400 columns, 5.3 ms against 1.3 in all on the 16^3 sphere, 16.7 against 13.3 on the 96^3
+// ellipsoid); the n^3 FP64 FMAs of the updates (two per clock and SM) come next.  A
+// step per column instead, as an n x 2n elimination of [A | I], did twice those FMAs
+// and two launches for each of the n columns, every launch waiting on one block's
+// pivot search.
 // Measured (CUDA events), both coarsest inverses of an operator: 96^3 ellipsoid (2,600
 // columns in all) 80 -> 31.5 ms, 16^3 sphere (920 columns) 20 -> 7.1 ms.
 

@@ -16,7 +16,7 @@
 // tensor cores multiply BF16 copies of the weights.  The convolutions, their
 // adjoints and the weight gradients are implicit GEMMs on the tensor cores
 // (dm_conv_tc.cu); the weight gradient is reduced in a fixed order (per-CTA
-// partials, then a sum in CTA order), so training is deterministic.
+// partials, then eight interleaved sums of them), so training is deterministic.
 #include "dm_common.cuh"
 
 #include "dm_learned.cuh"

@@ -33,7 +33,7 @@ void conv_tc(const Grid3& g, const ActLayout& L, int cb, int epi, const __nv_bfl
 // weight gradient dW[t][ci][co] = sum_p in[p + d_t, ci] dy[p, co] on tensor
 // cores: cb_in input channel blocks (cin channels), dy with cout <= 16
 // channels in cb_out blocks; part: per-CTA partials (conv_dw_tc_parts() x
-// 27 x 16 x 16 floats), summed in CTA order into dW ([27][cin][cout]).
+// 27 x 16 x 16 floats), summed in a fixed order into dW ([27][cin][cout]).
 int conv_dw_tc_parts();
 void conv_dw_tc(const Grid3& g, const ActLayout& L, int cb_in, int cin, const __nv_bfloat16* in, int cb_out, int cout,
                 const __nv_bfloat16* dy, float* part, float* dW, int* err, cudaStream_t s);
